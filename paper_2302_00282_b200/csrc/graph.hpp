@@ -74,6 +74,7 @@ struct ASeg {
     int k = 1, stride = 1, pad = 0;
     int kelems = 0;               // K elements this segment contributes (taps * C, before padding)
     int kblocks = 0;              // 64-wide K blocks (each segment starts block aligned)
+    int cbox = 64, cpad = 0;      // conv_tc_kernel: channels per copy-engine box (64, 32, 16); channels per tap in the packed K order
     int src_dtype = XENOS_DTYPE_BF16;   // AM_STEM only: F32 or BF16 NCHW
     // AM_DW: depthwise parameters in the workspace (fp32 [9][C] tap-major, bias [C]) and its act
     size_t dw_w_off = 0, dw_b_off = 0;
@@ -141,6 +142,8 @@ struct Launch {
     int a_tma = 0, a_box_bytes = 0;                                // activation operand by TMA: 1 matrix rows, 2 shifted patch
     int fc_small = 0;                                              // 1: fully connected layer of a small batch on the CUDA cores (fc_small_kernel)
     int dw_workers = 0;                                            // > 0: depthwise -> pointwise in dwpw_kernel with that many worker warps
+    // convolution, product or fc in conv_tc_kernel: its epilogue kind, rows of an operand box, resident weights, column chunks
+    int conv_tc = 0, cv_epi = 0, a_rows = 128, b_resident = 0, b_group = 0, chunk = 0, nchunks = 0, off_b = 0;
     int n_acc = 1;                                                 // dwpw_kernel: channel tiles of tile_n columns per CTA (2: both accumulators hold one tile)
     // ---- two linked convolutions (LK_GEMM2): producer tile rh1 x rw1 = patch_rh x patch_rw, consumer tile rh2 x rw2
     int k2 = 1, kblocks2 = 0, n1pad = 0, halo2 = 0, rh2 = 0, rw2 = 0, act3 = 0, off_mid = 0, stage_bytes = 0;

@@ -669,7 +669,84 @@ struct Lower {
     // ---- bf16 tensor-core lowering ---------------------------------------------------------
     // Packs the [npad][kpad] bf16 weight matrix of an implicit GEMM: row n = output channel,
     // K order = (tap r*k+s, input channel c) per segment, each segment padded to 64.
-    struct WSrc { const Node *n; int row0; int seg; bool centre_only; };
+    // ---- tiles of conv_tc_kernel ------------------------------------------------------------------------------------
+    // Modelled cycles of a plan with tile_n columns and ksplit chunks on `units` SMs.  Per 64-wide K block a CTA waits for
+    // the slower of the tensor pipe (max(48, tile_n / 2) cycles per K = 16 step) and the operand traffic from L2 (75
+    // bytes per cycle and SM); a tile's epilogue overlaps the next tile's product; a split adds the exchange of the partial
+    // sums.  The constants are measurements on B200 (see conv_tc.cuh).
+    double conv_cycles(const Launch &L, int tile_n, int n_tiles, int ksplit) const {
+        const double units = g.hw.sm_count;
+        const double tiles = (double)L.m_tiles * n_tiles * ksplit;
+        const double waves = std::ceil(tiles / units);
+        const int kb = ceil_div(L.kblocks, ksplit);
+        const double mma = 4.0 * std::max(48.0, tile_n / 2.0);
+        const double load = (L.a_rows * 128.0 + tile_n * 128.0) / 75.0;
+        const double main = kb * std::max(mma, std::max(load, 150.0));
+        const double epi = 400.0 + 5.0 * tile_n;
+        double t = waves * std::max(main, epi) + std::min(main, epi);
+        if (ksplit > 1) t += 2600.0 + L.a_rows * tile_n * 8.0 / 40.0;
+        return t;
+    }
+    // Widths are the equal cuts of the output channels (Section 4.2.1) down to 32 columns; the reduction is cut (Section
+    // 4.2.2) only where that is modelled to be faster, into chunks of at least two K blocks that run at the same time.
+    void choose_conv_tiles(Launch &L, int N16, const SplitRequest &rq, bool fc, int &ksplit) const {
+        double best = -1;
+        const bool can_split = L.epi == EPI_STORE && !rq.user;
+        ksplit = 1;
+        for (int nt = ceil_div(N16, 256); nt <= N16 / 16; ++nt) {
+            const int tn = round_up(ceil_div(N16, nt), 16);
+            if ((nt - 1) * tn >= N16) continue;                    // an empty last tile
+            if (tn < 32 && nt > ceil_div(N16, 256)) break;
+            for (int ks : {1, 2, 3, 4, 6, 8, 12, 16}) {
+                if (ks > 1 && (!can_split || L.kblocks < 2 * ks || (long)L.m_tiles * nt * ks > g.hw.sm_count)) break;
+                const int per = ceil_div(L.kblocks, ks);
+                if (ks > 1 && ceil_div(L.kblocks, per) != ks) continue;
+                // (a fully connected layer of few rows is a pass over its weights: it always spreads over the units)
+                const double c = conv_cycles(L, tn, nt, ks) + (fc && ks == 1 && L.m_tiles == 1 && L.kblocks >= 4 ? 1e6 : 0);
+                if (best < 0 || c < best) { best = c; L.n_tiles = nt; L.tile_n = tn; ksplit = ks; }
+            }
+        }
+    }
+    // Shared memory and epilogue shape of conv_tc_kernel.
+    xenos_status_t layout_conv(Launch &L, const Tensor &ot) {
+        const bool vec = L.out_dtype == XENOS_DTYPE_F32 || ot.c % 8;
+        L.cv_epi = L.epi == EPI_GAP ? 3 : L.ksplit > 1 ? 4 : vec ? 2 : L.skip >= 0 ? 1 : 0;
+        if (L.cv_epi == 2 && L.skip >= 0) return fail(g, XENOS_E_UNSUPPORTED, "internal: shortcut on a vector result");
+        int stg = 0;
+        L.chunk = 16;
+        if (L.cv_epi == 0 || L.cv_epi == 1) {
+            // the widest column chunk that gives both warps of a quarter the same number of chunks
+            // (at tile_n = 256 the 64-column boxes would take the fourth stage of the ring)
+            for (int c : {64, 32, 16})
+                if (L.tile_n % c == 0 && (L.tile_n / c) % 2 == 0 && !(c == 64 && L.tile_n > 160)) { L.chunk = c; break; }
+            stg = 16 * L.chunk * 64;                 // two 32-row boxes for each of eight warps
+        } else if (L.cv_epi == 3) {
+            L.chunk = 32;
+            stg = 2 * (128 * 33 + 128) * 4;
+        }
+        L.nchunks = ceil_div(L.tile_n, L.chunk);
+        stg = (int)align_up((size_t)stg, 1024);
+        const int bias = (int)align_up((size_t)L.npad * 4, 128);
+        const int room = std::min(g.hw.smem_bytes_per_cta, 227 * 1024) - 1024 - 512 - bias - stg;
+        const int bbytes = L.kblocks * L.tile_n * 128;
+        // weights stay in shared memory when a CTA meets more than one tile of its channel tile and four operand stages
+        // still fit beside them
+        const int rgrid = g.hw.sm_count / L.n_tiles * L.n_tiles;
+        L.b_resident = L.ksplit == 1 && rgrid > 0 && (long)L.m_tiles * L.n_tiles > rgrid && room - bbytes >= 4 * 16384;
+        const int stage = 16384 + (L.b_resident ? 0 : L.tile_n * 128);
+        L.stage_bytes = stage;
+        L.stages = std::min(6, (room - (L.b_resident ? bbytes : 0)) / stage);
+        if (L.stages < 2) return fail(g, XENOS_E_BAD_SPLIT, "split: pipeline does not fit shared memory");
+        L.b_group = ceil_div(L.kblocks, 4);
+        L.off_b = L.stages * stage;
+        L.off_stg = L.off_b + (L.b_resident ? bbytes : 0);
+        L.off_bias = L.off_stg + stg;
+        L.off_bar = L.off_bias + bias;
+        L.smem_bytes = L.off_bar + 512 + 1024;
+        L.grid = std::min(L.m_tiles * L.n_tiles * L.ksplit, L.b_resident ? rgrid : g.hw.sm_count);
+        L.block = 384;
+        return XENOS_OK;
+    }
 
     xenos_status_t make_gemm(int ci, const std::vector<int> &cover, const Node *dw, const Node *mainc,
                              const Node *shortcut, const Node *expand2, const Node *addn, const Node *pooln,
@@ -715,12 +792,23 @@ struct Lower {
             s0.mode = AM_GATHER; s0.k = kk; s0.stride = M.stride; s0.pad = expand2 ? kpadg : M.pad;
             s0.kelems = kk * kk * src.c;
         }
+        // Everything that gathers an NHWC window and stores rows, vectors or averages runs in conv_tc_kernel: the copy
+        // engine brings a tap's channels in boxes of 64, 32 or 16, so the packed K order gives every tap whole boxes.
+        const bool tc = s0.mode == AM_GATHER && !pooln;
+        auto boxes = [&](ASeg &a) {
+            a.cbox = a.C > 32 ? 64 : a.C > 16 ? 32 : 16;
+            a.cpad = a.cbox == 64 ? round_up(a.C, 64) : a.cbox;
+            a.kelems = a.k * a.k * a.cpad;
+        };
+        if (tc) boxes(s0);
         s0.kblocks = ceil_div(s0.kelems, 64);
         ASeg &s1 = L.seg[1];
         if (shortcut) {
             const Tensor &ss = g.tensors[shortcut->in[0]];
             s1.mode = AM_GATHER; s1.tensor = shortcut->in[0]; s1.C = ss.c; s1.H = ss.h; s1.W = ss.w;
-            s1.k = 1; s1.stride = shortcut->stride; s1.pad = 0; s1.kelems = ss.c; s1.kblocks = ceil_div(ss.c, 64);
+            s1.k = 1; s1.stride = shortcut->stride; s1.pad = 0; s1.kelems = ss.c;
+            if (tc) boxes(s1);
+            s1.kblocks = ceil_div(s1.kelems, 64);
         }
         L.kblocks = s0.kblocks + s1.kblocks;
         L.kpad = 64 * L.kblocks;
@@ -762,35 +850,12 @@ struct Lower {
                 L.gap_imgs = 1; L.gap_area = 128;
             }
         }
-        // Where a 64-channel K block of the activation operand is a box of the NHWC tensor (stride 1, channels a
-        // multiple of 64, no second K segment), TMA fetches it and writes the operand layout itself: the rows of
-        // the [pixels][C] matrix for a 1x1 convolution or fc, the tile's patch shifted by the tap for k x k.
-        if (s0.mode == AM_GATHER && !expand2 && !shortcut && !pooln && src.c % 64 == 0 && M.stride == 1) {
-            if (M.k == 1 && M.pad == 0) {
-                L.a_tma = 1;
-                L.a_box_bytes = 128 * 128;
-            } else if (!gapn && !fc) {
-                // patch tiles: ni whole images when one fits 128 rows, else rh x rw output pixels with the fewest tiles
-                L.a_tma = 2;
-                L.map_mode = MAP_PATCH;
-                if (L.P * L.Q <= 128) {
-                    L.patch_rh = L.P; L.patch_rw = L.Q; L.ni = std::min(128 / (L.P * L.Q), g.max_batch);
-                    // (fewer images per tile while units would idle, as for the depthwise chains)
-                    while (L.ni > 1 && (long)ceil_div(g.max_batch, L.ni) * ceil_div(round_up(N, 16), 256) * 2 <= g.hw.sm_count) --L.ni;
-                } else {
-                    L.ni = 1;
-                    long best = -1;
-                    for (int tw = 1; tw <= std::min(L.Q, 128); ++tw) {
-                        int th = std::min(L.P, 128 / tw);
-                        long tiles = (long)ceil_div(L.P, th) * ceil_div(L.Q, tw);
-                        if (best < 0 || tiles < best || (tiles == best && tw > L.patch_rw)) { best = tiles; L.patch_rh = th; L.patch_rw = tw; }
-                    }
-                }
-                L.tiles_y = ceil_div(L.P, L.patch_rh); L.tiles_x = ceil_div(L.Q, L.patch_rw);
-                L.step_y = L.patch_rh; L.step_x = L.patch_rw; L.off_y = L.off_x = 0;
-                L.tile_rows = L.ni * L.patch_rh * L.patch_rw;
-                L.a_box_bytes = L.tile_rows * 128;
-            }
+        // (which activation operands are plain boxes of the tensor: 1 rows of the [pixels][C] matrix, 2 a patch per tap;
+        // the others need the im2col form, or share a K block between taps)
+        if (tc) {
+            if (!expand2 && !shortcut && src.c % 64 == 0 && M.stride == 1) L.a_tma = (M.k == 1 && M.pad == 0) ? 1 : (!gapn && !fc) ? 2 : 0;
+            L.conv_tc = 1;
+            L.a_rows = gapn ? 128 : std::min(128, round_up(g.max_batch * L.rows_per_image, 16));
         }
         if (s0.mode == AM_STEM) {
             // The stem stages the tile's input patch in shared memory, so its tile is a patch too:
@@ -889,7 +954,10 @@ struct Lower {
         else L.m_tiles = ceil_div(g.max_batch * L.rows_per_image, 128);
         if (rq.user && (rq.h > 1 || rq.w > 1))
             return fail(g, XENOS_E_BAD_SPLIT, "split: tensor-core chains cut rows / columns into 128-row tiles themselves; only parts_outc can be set");
-        if (rq.user && rq.outc > 0) {
+        int tc_ksplit = 1;
+        if (L.conv_tc && !(rq.user && rq.outc > 0)) {
+            choose_conv_tiles(L, N16, rq, fc, tc_ksplit);
+        } else if (rq.user && rq.outc > 0) {
             L.n_tiles = rq.outc;
             L.tile_n = round_up(ceil_div(N16, rq.outc), 16);
             if (L.tile_n > 256 || (rq.outc - 1) * L.tile_n >= N)
@@ -922,18 +990,16 @@ struct Lower {
             if (fc && !rq.user && g.max_batch <= 8 && L.epi == EPI_STORE && L.skip < 0 && !shortcut && src.c % 8 == 0 &&
                 (long)g.max_batch * src.c * 2 <= 160 * 1024 && !(src.input_slot >= 0 && src.io_dtype != XENOS_DTYPE_BF16))
                 L.fc_small = 1;
-            const bool plain = !L.fc_small && s0.mode == AM_GATHER && (L.map_mode == MAP_FLAT || L.a_tma == 2);
-            // (a linked shortcut convolution, the second K segment of a gathered convolution, is cut with it: the chunks
-            // are blocks of the concatenated K)
-            const bool can = ((plain || s0.mode == AM_DW) && s1.mode == AM_NONE && L.epi == EPI_STORE) ||
-                             (plain && L.map_mode == MAP_FLAT && !L.a_tma && s1.mode == AM_GATHER && L.epi == EPI_STORE);
+            // (a linked shortcut convolution, the second K segment, is cut with its block: the chunks are blocks of the
+            // concatenated K)
+            const bool can = ((L.conv_tc && !L.fc_small) || (s0.mode == AM_DW && s1.mode == AM_NONE)) && L.epi == EPI_STORE;
             int want = 1;
             if (rq.user && rq.k > 1) {
                 if (!can) return fail(g, XENOS_E_UNSUPPORTED, "split: parts_k applies to a convolution, depthwise -> pointwise chain or fc that stores its tile (no image stem or pooling epilogue)");
                 if (rq.k > L.kblocks) return fail(g, XENOS_E_BAD_SPLIT, "split: parts_k exceeds the number of 64-element K blocks");
                 want = rq.k;
-            } else if (!rq.user && can && plain && L.kblocks >= 4 && (long)L.m_tiles * L.n_tiles * 2 <= g.hw.sm_count) {
-                want = std::min(L.kblocks / 2, g.hw.sm_count / (L.m_tiles * L.n_tiles));
+            } else if (!rq.user && can && L.conv_tc) {
+                want = tc_ksplit;
             }
             if (want > 1) {
                 L.kb_per = ceil_div(L.kblocks, want);
@@ -969,6 +1035,10 @@ struct Lower {
         L.tmem_cols = 32;
         while (L.tmem_cols < 2 * L.acc_stride) L.tmem_cols *= 2;
         if (L.tmem_cols > g.hw.tmem_columns) return fail(g, XENOS_E_BAD_SPLIT, "split: accumulator tiles exceed tensor memory columns");
+        if (L.conv_tc) {
+            const xenos_status_t lst = layout_conv(L, ot);
+            if (lst != XENOS_OK) return lst;
+        } else {
         // shared memory of the one persistent CTA per SM: [A|B ring][halo ring][epilogue staging][barriers]
         int stage_bytes = 16384 + L.n_acc * L.tile_n * 128;
         int stg_bytes = L.epi == EPI_POOL ? 128 * (L.tile_n * 2 + 16) : (L.epi == EPI_GAP ? 128 * 33 * 4 + 512 : 0);
@@ -1009,12 +1079,13 @@ struct Lower {
             L.dw_workers = L.halo_cb > 32 ? 16 : 8;
             L.block = 64 + 32 * L.dw_workers;
         }
+        }
         // --- pack weights + bias
         L.w_off = blob_reserve(g, (size_t)L.npad * L.kpad * 2);
         L.b_off = blob_reserve(g, (size_t)L.npad * 4);
         uint16_t *wp = reinterpret_cast<uint16_t *>(g.param_blob.data() + L.w_off);
         float *bp = reinterpret_cast<float *>(g.param_blob.data() + L.b_off);
-        auto pack_conv = [&](const Node &n, int row0, int kbase, int kwin, int C) {
+        auto pack_conv = [&](const Node &n, int row0, int kbase, int kwin, int C, int Cp) {
             // n.w is [cout][C][n.k][n.k]; it sits centred in a kwin x kwin window
             int shift = (kwin - n.k) / 2;
             for (int o = 0; o < n.cout; ++o)
@@ -1022,7 +1093,7 @@ struct Lower {
                     for (int r = 0; r < n.k; ++r)
                         for (int s = 0; s < n.k; ++s) {
                             int tap = (r + shift) * kwin + (s + shift);
-                            wp[(size_t)(row0 + o) * L.kpad + kbase + tap * C + c] =
+                            wp[(size_t)(row0 + o) * L.kpad + kbase + tap * Cp + c] =
                                 f32_to_bf16_rne(n.w[(((size_t)o * C + c) * n.k + r) * n.k + s]);
                         }
             for (int o = 0; o < n.cout; ++o) bp[row0 + o] += n.b[o];
@@ -1034,8 +1105,9 @@ struct Lower {
             }
         } else if (expand2) {
             // concat order decides the row offsets; both read the same kk x kk window
-            pack_conv(M, 0, 0, kk, src.c);
-            pack_conv(*expand2, M.cout, 0, kk, src.c);
+            const int cp = tc ? s0.cpad : src.c;
+            pack_conv(M, 0, 0, kk, src.c, cp);
+            pack_conv(*expand2, M.cout, 0, kk, src.c, cp);
         } else if (s0.mode == AM_STEM && M.k > 4) {
             const int kp = 8;
             for (int o = 0; o < M.cout; ++o) {
@@ -1047,9 +1119,9 @@ struct Lower {
                 bp[o] += M.b[o];
             }
         } else {
-            pack_conv(M, 0, 0, M.k, src.c);
+            pack_conv(M, 0, 0, M.k, src.c, tc ? s0.cpad : src.c);
         }
-        if (shortcut) pack_conv(*shortcut, 0, 64 * s0.kblocks, 1, s1.C);
+        if (shortcut) pack_conv(*shortcut, 0, 64 * s0.kblocks, 1, s1.C, s1.C);
         // --- modelled work
         for (int ni : cover) L.flops += 2.0 * node_macs(g.nodes[ni]);
         L.bytes = tbytes(L.in0) + tbytes(L.out) + (double)L.npad * L.kpad * 2 + 4.0 * L.npad;
@@ -1460,7 +1532,7 @@ void emit_plan_json(Graph &g) {
             jint(s, "ni", L.ni); jint(s, "step_y", L.step_y); jint(s, "step_x", L.step_x); jint(s, "off_y", L.off_y); jint(s, "off_x", L.off_x);
             jint(s, "hstages", L.hstages); jint(s, "halo_h", L.halo_h); jint(s, "halo_w", L.halo_w); jint(s, "halo_cb", L.halo_cb);
             jint(s, "halo_bytes", L.halo_bytes);
-            jint(s, "ksplit", L.ksplit); jint(s, "kb_per", L.kb_per); jint(s, "a_tma", L.a_tma); jint(s, "fc_small", L.fc_small); jint(s, "dw_workers", L.dw_workers); jint(s, "n_acc", L.n_acc); jint(s, "gap_parts", L.gap_parts);
+            jint(s, "ksplit", L.ksplit); jint(s, "kb_per", L.kb_per); jint(s, "a_tma", L.a_tma); jint(s, "fc_small", L.fc_small); jint(s, "dw_workers", L.dw_workers); jint(s, "n_acc", L.n_acc); jint(s, "gap_parts", L.gap_parts); jint(s, "conv_tc", L.conv_tc); jint(s, "b_resident", L.b_resident);
         }
         if (L.kind == LK_GEMM2) {
             jint(s, "k2", L.k2); jint(s, "cmid", L.Cmid); jint(s, "n1pad", L.n1pad); jint(s, "kblocks", L.kblocks); jint(s, "kblocks2", L.kblocks2);

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "chain2_tc.cuh"
+#include "conv_tc.cuh"
 #include "dwpw_tc.cuh"
 #include "gemm_tc.cuh"
 #include "graph.hpp"
@@ -21,13 +22,17 @@
 
 namespace xenos {
 
+struct ConvMaps { CUtensorMap a0, a1, o, s; };      // operand segments, result, shortcut of a conv_tc_kernel launch
+
 struct Runtime {
     int device = -1;
     int sm_count = 0;
     std::vector<CUtensorMap> tmaps;     // one per launch record (used by gemm launches only)
     std::vector<CUtensorMap> hmaps;     // halo maps of linked depthwise stages / activation operand maps
     std::vector<CUtensorMap> tmaps2;    // second weight matrix of two linked convolutions
+    std::vector<ConvMaps> conv;
     PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+    PFN_cuTensorMapEncodeIm2col_v12000 encode_im2col = nullptr;
 };
 
 static xenos_status_t cuda_fail(const Graph &g, const char *what, cudaError_t e) {
@@ -64,31 +69,82 @@ static xenos_status_t encode_halo_map(const Graph &g, Runtime *rt, const Launch 
     return XENOS_OK;
 }
 
-// Activation operand by TMA: the [pixels][C] matrix of an NHWC tensor (box = 128 rows of one 64-channel block), or the
-// tensor itself as (C, W, H, N) with a box of one tile's patch; 128-byte swizzle, the layout the MMA descriptor reads.
-static xenos_status_t encode_a_map(const Graph &g, Runtime *rt, const Launch &L, void *base, int images, CUtensorMap *out) {
-    const ASeg &a = L.seg[0];
-    CUresult r;
-    if (((uintptr_t)base & 15u) || (a.C % 64)) return fail(g, XENOS_E_CUDA, "internal: activation operand is not addressable by TMA");
-    if (L.a_tma == 1) {
-        cuuint64_t dims[2] = {(cuuint64_t)a.C, (cuuint64_t)images * a.H * a.W};
-        cuuint64_t strides[1] = {(cuuint64_t)a.C * 2};
-        cuuint32_t box[2] = {64u, 128u};
-        cuuint32_t estr[2] = {1u, 1u};
-        r = rt->encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                       CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    } else {
-        cuuint64_t dims[4] = {(cuuint64_t)a.C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)images};
-        cuuint64_t strides[3] = {(cuuint64_t)a.C * 2, (cuuint64_t)a.W * a.C * 2, (cuuint64_t)a.H * a.W * a.C * 2};
-        cuuint32_t box[4] = {64u, (cuuint32_t)L.patch_rw, (cuuint32_t)L.patch_rh, (cuuint32_t)L.ni};
-        cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
-        if (box[1] > 256u || box[2] > 256u || box[3] > 256u || box[1] * box[2] * box[3] > 128u)
-            return fail(g, XENOS_E_CUDA, "internal: activation patch exceeds the TMA box limits");
-        r = rt->encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                       CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    }
-    if (r != CUDA_SUCCESS) return fail(g, XENOS_E_CUDA, "cuTensorMapEncodeTiled (activation operand) failed with code " + std::to_string((int)r));
+// ---- maps of conv_tc_kernel ------------------------------------------------------------------------------------------
+static CUtensorMapSwizzle swizzle_of(int cols) {
+    return cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
+}
+static bool conv_seg_im2col(const ASeg &a) { return !(a.k == 1 && a.stride == 1 && a.pad == 0); }
+
+// Rows of a dense [rows][C] bf16 matrix in boxes of `rows_box` x `cols`, swizzled by the box's width.
+static xenos_status_t encode_rows_map(const Graph &g, Runtime *rt, void *base, int C, long long rows, int cols, int rows_box, CUtensorMap *out) {
+    cuuint64_t dims[2] = {(cuuint64_t)C, (cuuint64_t)rows};
+    cuuint64_t strides[1] = {(cuuint64_t)C * 2};
+    cuuint32_t box[2] = {(cuuint32_t)cols, (cuuint32_t)rows_box};
+    cuuint32_t estr[2] = {1u, 1u};
+    if (((uintptr_t)base & 15u) || C % 8 || rows_box > 256) return fail(g, XENOS_E_CUDA, "internal: a matrix is not addressable by TMA");
+    CUresult r = rt->encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            swizzle_of(cols), CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(g, XENOS_E_CUDA, "cuTensorMapEncodeTiled (rows) failed with code " + std::to_string((int)r));
     return XENOS_OK;
+}
+
+// One segment of the activation operand: matrix rows, or the im2col walk over the window origins of an NHWC tensor
+// (bounding box from -pad to the last window origin, traversed with the convolution's stride; padding reads zeros).
+static xenos_status_t encode_conv_a(const Graph &g, Runtime *rt, const Launch &L, const ASeg &a, void *base, int images, CUtensorMap *out) {
+    if (!conv_seg_im2col(a)) return encode_rows_map(g, rt, base, a.C, (long long)images * a.H * a.W, a.cbox, L.a_rows, out);
+    const int hi = a.pad - (a.k - 1);
+    cuuint64_t dims[4] = {(cuuint64_t)a.C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)images};
+    cuuint64_t strides[3] = {(cuuint64_t)a.C * 2, (cuuint64_t)a.W * a.C * 2, (cuuint64_t)a.H * a.W * a.C * 2};
+    int lower[2] = {-a.pad, -a.pad}, upper[2] = {hi, hi};
+    cuuint32_t estr[4] = {1u, (cuuint32_t)a.stride, (cuuint32_t)a.stride, 1u};
+    if (((uintptr_t)base & 15u) || a.C % 8 || a.pad > 127 || hi < -127 || a.stride > 8)
+        return fail(g, XENOS_E_UNSUPPORTED, "a convolution window, stride or padding exceeds the copy engine's im2col limits");
+    CUresult r = rt->encode_im2col(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, lower, upper, (cuuint32_t)a.cbox,
+                                   (cuuint32_t)L.a_rows, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(a.cbox),
+                                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(g, XENOS_E_CUDA, "cuTensorMapEncodeIm2col failed with code " + std::to_string((int)r));
+    return XENOS_OK;
+}
+
+// The maps of a launch whose tensors sit where `ptr` says; `want_external` selects those on caller buffers (run time, for
+// the batch at hand) or those on the workspace (bind time, for max_batch images).
+template <class Ptr>
+static xenos_status_t encode_conv_maps(const Graph &g, Runtime *rt, const Launch &L, Ptr ptr, int images, bool want_external, ConvMaps *m) {
+    auto external = [&](int t) { return g.tensors[t].input_slot >= 0 || g.tensors[t].output_slot >= 0; };
+    const ASeg &a0 = L.seg[0], &a1 = L.seg[1];
+    xenos_status_t st = XENOS_OK;
+    if (external(a0.tensor) == want_external) st = encode_conv_a(g, rt, L, a0, ptr(a0.tensor), images, &m->a0);
+    if (st == XENOS_OK && a1.mode != AM_NONE && external(a1.tensor) == want_external) st = encode_conv_a(g, rt, L, a1, ptr(a1.tensor), images, &m->a1);
+    const long long rows = (long long)images * L.rows_per_image;
+    if (st == XENOS_OK && (L.cv_epi == xk::CE_STORE || L.cv_epi == xk::CE_SKIP) && external(L.out) == want_external)
+        st = encode_rows_map(g, rt, ptr(L.out), L.out_ctot, rows, L.chunk, 32, &m->o);
+    if (st == XENOS_OK && L.cv_epi == xk::CE_SKIP && external(L.skip) == want_external)
+        st = encode_rows_map(g, rt, ptr(L.skip), g.tensors[L.skip].c, rows, L.chunk, 32, &m->s);
+    return st;
+}
+static bool conv_has_external(const Graph &g, const Launch &L) {
+    auto external = [&](int t) { return t >= 0 && (g.tensors[t].input_slot >= 0 || g.tensors[t].output_slot >= 0); };
+    return external(L.seg[0].tensor) || (L.seg[1].mode != AM_NONE && external(L.seg[1].tensor)) || external(L.out) || external(L.skip);
+}
+
+static xk::ConvSegment conv_segment(const Launch &L, const ASeg &a) {
+    xk::ConvSegment s;
+    std::memset(&s, 0, sizeof s);
+    if (a.mode == AM_NONE) { s.per_stage = 1; s.k = 1; s.cblocks = 1; s.spb = 4; return s; }
+    s.im2col = conv_seg_im2col(a);
+    s.k = a.k; s.stride = a.stride; s.low = -a.pad;
+    s.taps = a.k * a.k;
+    s.kblocks = a.kblocks;
+    s.cblocks = a.cbox == 64 ? a.cpad / 64 : 1;
+    s.last_steps = a.cbox == 64 ? (a.C - 64 * (s.cblocks - 1) + 15) / 16 : 4;
+    s.per_stage = 64 / a.cbox;
+    s.spb = a.cbox / 16;
+    s.box_bytes = (uint32_t)(L.a_rows * a.cbox * 2);
+    s.box_stride = (uint32_t)(128 * a.cbox * 2);
+    // version bit, group stride (8 rows of the box), swizzle mode
+    const uint32_t mode = a.cbox == 64 ? 2u : a.cbox == 32 ? 4u : 6u;
+    s.desc_hi = (uint32_t)((8 * a.cbox * 2) >> 4) | (1u << 14) | (mode << 29);
+    return s;
 }
 
 // Maps of two linked convolutions: the first one's input (C, W, H, N) with a box of the producer tile, and the two
@@ -177,6 +233,8 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
     rt->tmaps.resize(g.launches.size());
     rt->hmaps.resize(g.launches.size());
     rt->tmaps2.resize(g.launches.size());
+    rt->conv.resize(g.launches.size());
+    std::memset(rt->conv.data(), 0, rt->conv.size() * sizeof(ConvMaps));
     if (any_gemm) {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult qres;
@@ -184,6 +242,10 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
         if (e != cudaSuccess || !fn || qres != cudaDriverEntryPointSuccess)
             return fail(g, XENOS_E_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
         rt->encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+        e = cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &fn, cudaEnableDefault, &qres);
+        if (e != cudaSuccess || !fn || qres != cudaDriverEntryPointSuccess)
+            return fail(g, XENOS_E_CUDA, "cuTensorMapEncodeIm2col is not available from the driver");
+        rt->encode_im2col = reinterpret_cast<PFN_cuTensorMapEncodeIm2col_v12000>(fn);
         for (size_t i = 0; i < g.launches.size(); ++i) {
             const Launch &L = g.launches[i];
             if (L.kind == LK_GEMM2) {
@@ -207,9 +269,11 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
                                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r != CUDA_SUCCESS) return fail(g, XENOS_E_CUDA, "cuTensorMapEncodeTiled failed with code " + std::to_string((int)r));
-            if (L.a_tma && g.tensors[L.seg[0].tensor].input_slot < 0) {
-                xenos_status_t st = encode_a_map(g, rt, L, static_cast<uint8_t *>(ws) + g.place[L.seg[0].tensor].off, g.max_batch, &rt->hmaps[i]);
+            if (L.conv_tc) {
+                if (L.fc_small) continue;
+                xenos_status_t st = encode_conv_maps(g, rt, L, [&](int t) -> void * { return static_cast<uint8_t *>(ws) + g.place[t].off; }, g.max_batch, false, &rt->conv[i]);
                 if (st != XENOS_OK) return st;
+                continue;
             }
             if (L.seg[0].mode == AM_DW && g.tensors[L.seg[0].tensor].input_slot < 0) {
                 xenos_status_t st = encode_halo_map(g, rt, L, static_cast<uint8_t *>(ws) + g.place[L.seg[0].tensor].off, g.max_batch, &rt->hmaps[i]);
@@ -226,6 +290,13 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
         if ((e = cudaFuncSetAttribute(xk::gemm_chain_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(xk::gemm_chain_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(gemm)", e);
+    if (any_gemm)
+        if ((e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_SKIP>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_GAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
+            return cuda_fail(g, "cudaFuncSetAttribute(conv)", e);
     if (any_gemm)
         if ((e = cudaFuncSetAttribute(xk::dwpw_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(xk::dwpw_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
@@ -434,6 +505,55 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
                     L.kpad, L.K, L.act, L.out_dtype == XENOS_DTYPE_F32, L.out_ctot, L.out_coff);
                 break;
             }
+            if (L.conv_tc) {
+                xk::ConvParams p;
+                std::memset(&p, 0, sizeof p);
+                p.seg[0] = conv_segment(L, L.seg[0]); p.seg[1] = conv_segment(L, L.seg[1]);
+                p.bias = (const float *)(ws + L.b_off); p.out = ptr(L.out); p.status = status;
+                p.rows = N * L.rows_per_image;
+                p.tile_rows = L.epi == EPI_GAP ? L.tile_rows : 128;
+                const int mt = L.gap_parts > 1 ? N * L.gap_parts : (p.rows + p.tile_rows - 1) / p.tile_rows;
+                p.d_rpi = xk::make_fastdiv((uint32_t)L.rows_per_image); p.d_q = xk::make_fastdiv((uint32_t)L.Q);
+                p.d_nt = xk::make_fastdiv((uint32_t)L.n_tiles); p.d_ks = xk::make_fastdiv((uint32_t)L.ksplit);
+                p.total = mt * L.n_tiles * L.ksplit; p.tile_n = L.tile_n; p.npad = L.npad; p.N = L.K;
+                p.kblocks = L.kblocks; p.stages = L.stages; p.stage_bytes = L.stage_bytes; p.b_resident = L.b_resident; p.b_group = L.b_group;
+                p.acc_stride = L.acc_stride; p.tmem_cols = L.tmem_cols;
+                p.chunk = L.chunk; p.nchunks = L.nchunks; p.box_bytes = L.chunk * 64;
+                // (two clamps in a row with no shortcut between them are one: none < ReLU < ReLU6)
+                p.act = L.skip >= 0 ? L.act : std::max(L.act, L.act2); p.act2 = L.skip >= 0 ? L.act2 : 0; p.out_ctot = L.out_ctot; p.out_f32 = L.out_dtype == XENOS_DTYPE_F32;
+                p.idesc = make_idesc(L.tile_n);
+                p.off_b = L.off_b; p.off_stage = L.off_stg; p.off_bias = L.off_bias; p.off_bar = L.off_bar;
+                p.launch_id = (int)li;
+                p.gap_imgs = L.gap_imgs; p.gap_rpi = L.gap_rpi; p.gap_parts = L.gap_parts; p.batch = N;
+                p.ksplit = L.ksplit; p.kb_per = L.ksplit > 1 ? L.kb_per : L.kblocks; p.split_ld = L.npad;
+                p.split_stride = (long long)p.rows * L.npad;
+                p.split_part = reinterpret_cast<float *>(ws + g.split_off);
+                p.split_cnt = reinterpret_cast<unsigned int *>(ws + L.split_cnt_off);
+                p.skip = (const __nv_bfloat16 *)ptr(L.skip); p.skip_ctot = L.skip >= 0 ? g.tensors[L.skip].c : 0;
+                const ConvMaps *maps = &rt->conv[li];
+                ConvMaps now;
+                if (conv_has_external(g, L)) {
+                    now = *maps;
+                    xenos_status_t st = encode_conv_maps(g, rt, L, ptr, N, true, &now);
+                    if (st != XENOS_OK) return st;
+                    maps = &now;
+                }
+                int limit = sms;
+                if (L.b_resident) limit = std::max(1, sms / L.n_tiles) * L.n_tiles;
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)std::min(p.total, limit)); cfg.blockDim = dim3((unsigned)xk::kCvThreads);
+                cfg.dynamicSmemBytes = (size_t)L.smem_bytes; cfg.stream = stream;
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+                at[0].val.programmaticStreamSerializationAllowed = 1;
+                cfg.attrs = at; cfg.numAttrs = 1;
+                auto *k = L.cv_epi == xk::CE_STORE ? xk::conv_tc_kernel<xk::CE_STORE> : L.cv_epi == xk::CE_SKIP ? xk::conv_tc_kernel<xk::CE_SKIP>
+                        : L.cv_epi == xk::CE_VEC ? xk::conv_tc_kernel<xk::CE_VEC> : L.cv_epi == xk::CE_GAP ? xk::conv_tc_kernel<xk::CE_GAP>
+                        : xk::conv_tc_kernel<xk::CE_SPLIT>;
+                cudaError_t le = cudaLaunchKernelEx(&cfg, k, maps->a0, maps->a1, rt->tmaps[li], maps->o, maps->s, p);
+                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+                break;
+            }
             xk::GemmParams p;
             std::memset(&p, 0, sizeof p);
             for (int s = 0; s < 2; ++s) {
@@ -462,7 +582,6 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
             p.hstages = L.hstages; p.halo_bytes = L.halo_bytes; p.halo_stride = L.halo_stride;
             p.halo_h = L.halo_h; p.halo_w = L.halo_w; p.halo_cb = L.halo_cb;
             p.stem_tma = L.stem_tma; p.stem_align = L.stem_align;
-            p.a_tma = L.a_tma; p.a_box_bytes = L.a_box_bytes; p.a_cpb = L.seg[0].C / 64;
             p.off_halo = L.off_halo; p.off_stg = L.off_stg; p.off_dww = L.off_dww; p.off_bias = L.off_bias; p.off_bar = L.off_bar;
             p.n_acc = L.n_acc; p.gap_parts = L.gap_parts;
             p.act = L.act; p.act2 = L.act2; p.epi = L.epi; p.out_ctot = L.out_ctot; p.out_coff = L.out_coff;
@@ -483,16 +602,6 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
                     xenos_status_t st = encode_stem_map(g, rt, L, ptr(L.seg[0].tensor), N, &tmh_now);
                     if (st != XENOS_OK) return st;
                     tmh = &tmh_now;
-                }
-            }
-            if (L.a_tma) {
-                if (g.tensors[L.seg[0].tensor].input_slot >= 0) {
-                    // the operand is a caller buffer: its map is encoded now (rows / images beyond the batch read zeros)
-                    xenos_status_t st = encode_a_map(g, rt, L, ptr(L.seg[0].tensor), N, &tmh_now);
-                    if (st != XENOS_OK) return st;
-                    tmh = &tmh_now;
-                } else {
-                    tmh = &rt->hmaps[li];
                 }
             }
             if (L.seg[0].mode == AM_DW) {
