@@ -145,6 +145,7 @@ struct Launch {
     // convolution, product or fc in conv_tc_kernel: its epilogue kind, rows of an operand box, resident weights, column chunks
     int conv_tc = 0, cv_epi = 0, a_rows = 128, b_resident = 0, b_group = 0, chunk = 0, nchunks = 0, off_b = 0;
     int n_acc = 1;                                                 // dwpw_kernel: channel tiles of tile_n columns per CTA (2: both accumulators hold one tile)
+    int pair = 0, a_slots = 0, b_slots = 0, off_b2 = 0;            // LK_GEMM2 with a 1x1 consumer: pair_tc_kernel and its rings
     // ---- two linked convolutions (LK_GEMM2): producer tile rh1 x rw1 = patch_rh x patch_rw, consumer tile rh2 x rw2
     int k2 = 1, kblocks2 = 0, n1pad = 0, halo2 = 0, rh2 = 0, rw2 = 0, act3 = 0, off_mid = 0, stage_bytes = 0;
     int off_halo = 0, off_stg = 0, off_dww = 0, off_bias = 0, off_bar = 0;                    // shared-memory layout

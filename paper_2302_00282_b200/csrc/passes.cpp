@@ -1149,7 +1149,8 @@ struct Lower {
         L.k = A.k; L.stride = 1; L.pad = A.pad; L.k2 = k2; L.halo2 = h;
         L.Cmid = A.cout; L.n1pad = round_up(A.cout, 64);
         L.seg[0].tensor = L.in0; L.seg[0].C = src.c; L.seg[0].H = src.h; L.seg[0].W = src.w; L.seg[0].k = A.k; L.seg[0].pad = A.pad;
-        L.kblocks = A.k * A.k * (src.c / 64);
+        L.seg[0].mode = AM_GATHER; L.seg[0].cbox = 64; L.seg[0].cpad = src.c;
+        L.kblocks = L.seg[0].kblocks = A.k * A.k * (src.c / 64);
         L.kblocks2 = k2 * k2 * (L.n1pad / 64);
         L.act = A.act; L.act2 = B ? B->act : E0->act;
         if (addn) {
@@ -1164,22 +1165,48 @@ struct Lower {
         L.tiles_y = ceil_div(L.P, L.rh2); L.tiles_x = ceil_div(L.Q, L.rw2);
         L.m_tiles = g.max_batch * L.tiles_y * L.tiles_x;
         L.a_box_bytes = L.patch_rh * L.patch_rw * 128;
-        const int N216 = round_up(N2, 16);
-        L.n_tiles = ceil_div(N216, 256);
-        L.tile_n = round_up(ceil_div(N216, L.n_tiles), 16);
-        L.npad = L.n_tiles * L.tile_n;
+        const int cap = std::min(g.hw.smem_bytes_per_cta, 227 * 1024) - 1024;
         L.out_ctot = ot.c; L.out_coff = 0;
-        L.stage_bytes = 16384 + std::max(L.n1pad, L.tile_n) * 128;
-        const int mid_bytes = (L.n1pad / 64) * (128 + 64) * 128;
-        const int cap = std::min(g.hw.smem_bytes_per_cta, 227 * 1024) - 1024 - 256;
-        L.stages = std::min(6, (cap - mid_bytes) / L.stage_bytes);
-        if (L.stages < 2) return fail(g, XENOS_E_BAD_SPLIT, "split: two linked convolutions do not fit shared memory");
-        L.off_mid = L.stages * L.stage_bytes;
-        L.off_bar = L.off_mid + mid_bytes;
-        L.smem_bytes = L.off_bar + 256 + 1024;
+        if (k2 == 1) {
+            // pair_tc_kernel: tiles of 128 consecutive pixels, 128 output channels at a time; 16 KB slots for activation and
+            // weight blocks share what the middle tile, the staging boxes and the biases leave
+            L.pair = 1;
+            L.m_tiles = ceil_div(g.max_batch * L.rows_per_image, 128);
+            L.tile_n = 128; L.n_tiles = ceil_div(N2, 128); L.npad = L.n_tiles * 128;
+            const int mid = (L.n1pad / 64) * 16384, stg = 16 * 2048, bias = (int)align_up((size_t)(L.n1pad + L.npad) * 4, 128);
+            const int room = cap - 512 - mid - stg - bias;
+            const int weights = L.kblocks * L.n1pad * 128 + L.kblocks2 * L.n_tiles * 16384;
+            L.b_resident = room - weights >= 4 * 16384;
+            const int slots = (room - (L.b_resident ? weights : 0)) / 16384;
+            L.a_slots = L.b_resident ? std::min(8, slots) : slots * 2 / 5;
+            L.b_slots = L.b_resident ? 0 : std::min(8, slots - L.a_slots);
+            L.a_slots = std::min(8, L.a_slots);
+            if (L.a_slots < 2 || (!L.b_resident && L.b_slots < 2)) return fail(g, XENOS_E_BAD_SPLIT, "split: two linked convolutions do not fit shared memory");
+            L.off_b2 = L.a_slots * 16384;
+            L.off_mid = L.off_b2 + (L.b_resident ? weights : L.b_slots * 16384);
+            L.off_stg = L.off_mid + mid;
+            L.off_bias = L.off_stg + stg;
+            L.off_bar = L.off_bias + bias;
+            L.smem_bytes = L.off_bar + 512 + 1024;
+            L.stages = L.a_slots;
+            L.a_rows = 128;
+            L.block = 384;
+        } else {
+            const int N216 = round_up(N2, 16);
+            L.n_tiles = ceil_div(N216, 256);
+            L.tile_n = round_up(ceil_div(N216, L.n_tiles), 16);
+            L.npad = L.n_tiles * L.tile_n;
+            L.stage_bytes = 16384 + std::max(L.n1pad, L.tile_n) * 128;
+            const int mid_bytes = (L.n1pad / 64) * (128 + 64) * 128;
+            L.stages = std::min(6, (cap - 256 - mid_bytes) / L.stage_bytes);
+            if (L.stages < 2) return fail(g, XENOS_E_BAD_SPLIT, "split: two linked convolutions do not fit shared memory");
+            L.off_mid = L.stages * L.stage_bytes;
+            L.off_bar = L.off_mid + mid_bytes;
+            L.smem_bytes = L.off_bar + 256 + 1024;
+            L.block = 320;
+        }
         L.tmem_cols = 512;
         L.grid = std::min(L.m_tiles, g.hw.sm_count);
-        L.block = 320;
         if (g.chains[ci].split.user && (g.chains[ci].split.outc > 1 || g.chains[ci].split.h > 1 || g.chains[ci].split.w > 1 || g.chains[ci].split.k > 1))
             return fail(g, XENOS_E_BAD_SPLIT, "split: two linked convolutions keep all output channels of a tile in one CTA; no explicit split");
         // --- parameters: W1 [n1pad][K1], bias1 [n1pad]; W2 [npad][k2*k2*n1pad], bias2 [npad]; K order (tap, channel)

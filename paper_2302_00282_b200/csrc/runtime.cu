@@ -19,6 +19,7 @@
 #include "graph.hpp"
 #include "kernels_bf16.cuh"
 #include "kernels_f32.cuh"
+#include "pair_tc.cuh"
 
 namespace xenos {
 
@@ -116,10 +117,10 @@ static xenos_status_t encode_conv_maps(const Graph &g, Runtime *rt, const Launch
     if (external(a0.tensor) == want_external) st = encode_conv_a(g, rt, L, a0, ptr(a0.tensor), images, &m->a0);
     if (st == XENOS_OK && a1.mode != AM_NONE && external(a1.tensor) == want_external) st = encode_conv_a(g, rt, L, a1, ptr(a1.tensor), images, &m->a1);
     const long long rows = (long long)images * L.rows_per_image;
-    if (st == XENOS_OK && (L.cv_epi == xk::CE_STORE || L.cv_epi == xk::CE_SKIP) && external(L.out) == want_external)
-        st = encode_rows_map(g, rt, ptr(L.out), L.out_ctot, rows, L.chunk, 32, &m->o);
-    if (st == XENOS_OK && L.cv_epi == xk::CE_SKIP && external(L.skip) == want_external)
-        st = encode_rows_map(g, rt, ptr(L.skip), g.tensors[L.skip].c, rows, L.chunk, 32, &m->s);
+    if (st == XENOS_OK && (L.pair || L.cv_epi == xk::CE_STORE || L.cv_epi == xk::CE_SKIP) && external(L.out) == want_external)
+        st = encode_rows_map(g, rt, ptr(L.out), L.out_ctot, rows, L.pair ? 32 : L.chunk, 32, &m->o);
+    if (st == XENOS_OK && L.skip >= 0 && (L.pair || L.cv_epi == xk::CE_SKIP) && external(L.skip) == want_external)
+        st = encode_rows_map(g, rt, ptr(L.skip), g.tensors[L.skip].c, rows, L.pair ? 32 : L.chunk, 32, &m->s);
     return st;
 }
 static bool conv_has_external(const Graph &g, const Launch &L) {
@@ -248,6 +249,13 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
         rt->encode_im2col = reinterpret_cast<PFN_cuTensorMapEncodeIm2col_v12000>(fn);
         for (size_t i = 0; i < g.launches.size(); ++i) {
             const Launch &L = g.launches[i];
+            if (L.kind == LK_GEMM2 && L.pair) {
+                xenos_status_t st = encode_weight_map(g, rt, static_cast<uint8_t *>(ws) + L.w_off, L.kblocks * 64, L.n1pad, std::min(128, L.n1pad), &rt->tmaps[i]);
+                if (st == XENOS_OK) st = encode_weight_map(g, rt, static_cast<uint8_t *>(ws) + L.w2_off, L.kblocks2 * 64, L.npad, 128, &rt->tmaps2[i]);
+                if (st == XENOS_OK) st = encode_conv_maps(g, rt, L, [&](int t) -> void * { return static_cast<uint8_t *>(ws) + g.place[t].off; }, g.max_batch, false, &rt->conv[i]);
+                if (st != XENOS_OK) return st;
+                continue;
+            }
             if (L.kind == LK_GEMM2) {
                 xenos_status_t st = encode_weight_map(g, rt, static_cast<uint8_t *>(ws) + L.w_off, L.kblocks * 64, L.n1pad, L.n1pad, &rt->tmaps[i]);
                 if (st == XENOS_OK) st = encode_weight_map(g, rt, static_cast<uint8_t *>(ws) + L.w2_off, L.kblocks2 * 64, L.npad, L.tile_n, &rt->tmaps2[i]);
@@ -304,6 +312,10 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
     if (any_gemm)
         if ((e = cudaFuncSetAttribute(xk::fc_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(fc)", e);
+    if (any_gemm2)
+        if ((e = cudaFuncSetAttribute(xk::pair_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::pair_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
+            return cuda_fail(g, "cudaFuncSetAttribute(pair)", e);
     if (any_gemm2)
         if ((e = cudaFuncSetAttribute(xk::chain2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(chain2)", e);
@@ -463,6 +475,39 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
             break;
         }
         case LK_GEMM2: {
+            if (L.pair) {
+                xk::PairParams p;
+                std::memset(&p, 0, sizeof p);
+                p.seg = conv_segment(L, L.seg[0]);
+                p.bias1 = (const float *)(ws + L.b_off); p.bias2 = (const float *)(ws + L.b2_off); p.status = status;
+                p.rows = N * L.rows_per_image; p.tiles = (p.rows + 127) / 128;
+                p.d_rpi = xk::make_fastdiv((uint32_t)L.rows_per_image); p.d_q = xk::make_fastdiv((uint32_t)L.Q);
+                p.n1pad = L.n1pad; p.n1_slots = (L.n1pad + 127) / 128; p.kblocks2 = L.kblocks2; p.n2_blocks = L.n_tiles; p.npad2 = L.npad;
+                p.a_slots = L.a_slots; p.b_slots = L.b_slots; p.resident = L.b_resident; p.dbl = L.n1pad <= 128;
+                // (without a shortcut the two last clamps are one)
+                p.act1 = L.act; p.act2 = L.skip >= 0 ? L.act2 : std::max(L.act2, L.act3); p.act3 = L.act3;
+                p.idesc1 = make_idesc(std::min(128, L.n1pad)); p.idesc2 = make_idesc(128);
+                p.off_b = L.off_b2; p.off_mid = L.off_mid; p.off_stage = L.off_stg; p.off_bias = L.off_bias; p.off_bar = L.off_bar;
+                p.launch_id = (int)li;
+                const ConvMaps *maps = &rt->conv[li];
+                ConvMaps now;
+                if (conv_has_external(g, L)) {
+                    now = *maps;
+                    xenos_status_t st = encode_conv_maps(g, rt, L, ptr, N, true, &now);
+                    if (st != XENOS_OK) return st;
+                    maps = &now;
+                }
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)std::min(p.tiles, sms)); cfg.blockDim = dim3((unsigned)xk::kCvThreads);
+                cfg.dynamicSmemBytes = (size_t)L.smem_bytes; cfg.stream = stream;
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+                at[0].val.programmaticStreamSerializationAllowed = 1;
+                cfg.attrs = at; cfg.numAttrs = 1;
+                cudaError_t le = cudaLaunchKernelEx(&cfg, L.skip >= 0 ? xk::pair_tc_kernel<true> : xk::pair_tc_kernel<false>, maps->a0, rt->tmaps[li], rt->tmaps2[li], maps->o, maps->s, p);
+                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+                break;
+            }
             xk::Chain2Params p;
             std::memset(&p, 0, sizeof p);
             p.bias1 = (const float *)(ws + L.b_off); p.bias2 = (const float *)(ws + L.b2_off);
