@@ -155,6 +155,7 @@ struct Launch {
     size_t split_cnt_off = 0;
     // ---- fp32 linked chain (conv kxk -> conv1x1 -> pool)
     int Cmid = 0, K2 = 0, act2 = 0;
+    int f32_big = 0, f32_ws = 0, f32_iwp = 0, f32_hp = 0;       // register tile 8 x 4 or 2 x 1, weights in shared memory, row pitches
     int parts_outc = 1, tile_h = 0, tile_w = 0, tiles_h = 0, tiles_w = 0;   // tile of POOL outputs
     int halo_h = 0, halo_w = 0;   // stage-1 region a full tile needs (rows, cols)
     // ---- launch shape and modelled work

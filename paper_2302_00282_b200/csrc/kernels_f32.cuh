@@ -136,93 +136,315 @@ __global__ void f32_fc_kernel(const float *__restrict__ x, const float *__restri
 }
 
 // ------------------------------------------------------------------------------------------------
-// Linked chain ConvX(+act) -> Conv1x1(+act) -> pool, one CTA per (image, outC part, pool tile).
-//   stage 0: the input patch the tile needs goes to shared memory, zero-filled outside the image
-//   stage 1: ConvX on the patch -> shared memory [Cmid][rh][rw], i.e. channel-major so that
-//            stage 2 reads a pixel's channels at a fixed stride and neighbouring threads read
-//            neighbouring pixels (the consumer's read order)
+// Linked chain ConvX(+act) -> Conv1x1(+act) -> pool (Table 1), a CTA per (image, outC part, pool tile), walking over
+// them when there are more than fit.
+//   stage 0: the input patch the tile needs goes to shared memory (cp.async, zeros outside the image and in the padding of
+//            the row pitch)
+//   stage 1: ConvX on the patch -> shared memory [Cmid][row][column % pool_stride][column / pool_stride], so that the
+//            outputs of one pool tap are adjacent: the order stage 2 reads
 //   stage 2: Conv1x1 over the CTA's slice of output channels, pooled in registers
-// Every index is checked against the buffer extents; a failed check sets the status word and
-// skips the access.
+// Both stages are register-tiled: a thread owns TM channels x TP adjacent pixels (pool outputs), lanes of a warp take
+// neighbouring pixels of the same channels (weights are broadcast reads), products are packed fp32 pairs over channels.
+// Every sum runs over (channel, row, column) in ascending order whatever the tile: a split changes no value.
+// Bound by the FMA pipes (8 x 4 tiles: 6 shared-memory reads for 32 multiply-adds); 2 x 1 tiles spread a small map over
+// many threads, where latency decides.  Weights sit in shared memory when they fit (kWS), else they are read through L1.
+// Measured: 32 -> 64 -> 64 channels, 75 x 75, batch 32: 0.24 ms (34 TFLOP/s, half of the FMA pipes' rate; plain fmaf
+// instead of pairs 0.26 ms), 4.37 ms with one output per thread and iteration before.
 // ------------------------------------------------------------------------------------------------
 struct F32ChainParams {
-    const float *x, *w1, *b1, *w2, *b2;
+    const float *x, *w1, *b1, *w2, *b2;      // w1 [C][k][k][mpad], w2 [part][Cmid][kperp]: output channels padded to 8 with zeros
     float *y;
     int N, C, H, W;          // input
-    int Cmid, P, Q;          // stage-1 output
+    int Cmid, mpad, P, Q;    // stage-1 output
     int k, stride, pad, act1;
     int K2, act2;
     int pool_kind, pool_k, pool_stride, PP, PQ;
     int parts_outc, tile_h, tile_w, tiles_h, tiles_w, halo_h, halo_w;
+    int iwp, hp;             // row pitch of the patch; pitch of one column residue of the middle map
     unsigned int *status;
 };
 
-__global__ void f32_conv_conv_pool_kernel(F32ChainParams p) {
-    extern __shared__ float smem[];
-    int cta = blockIdx.x;
-    int tx = cta % p.tiles_w; cta /= p.tiles_w;
-    int ty = cta % p.tiles_h; cta /= p.tiles_h;
-    int part = cta % p.parts_outc;
-    int n = cta / p.parts_outc;
-    if (n >= p.N) return;
-    // pool tile -> stage-1 patch -> input patch
-    int py0 = ty * p.tile_h, px0 = tx * p.tile_w;
-    int th = min(p.tile_h, p.PP - py0), tw = min(p.tile_w, p.PQ - px0);
-    int rh = (th - 1) * p.pool_stride + p.pool_k, rw = (tw - 1) * p.pool_stride + p.pool_k;
-    int r0 = py0 * p.pool_stride, c0 = px0 * p.pool_stride;                 // stage-1 origin (pool pad is 0)
-    int ih = (rh - 1) * p.stride + p.k, iw = (rw - 1) * p.stride + p.k;
-    int i0 = r0 * p.stride - p.pad, j0 = c0 * p.stride - p.pad;             // input origin, may be negative
-    int max_ih = (p.halo_h - 1) * p.stride + p.k, max_iw = (p.halo_w - 1) * p.stride + p.k;
-    float *s_in = smem;                                                      // [C][ih][iw]
-    float *s_mid = smem + (size_t)p.C * max_ih * max_iw;                     // [Cmid][rh][rw]
-    if (rh > p.halo_h || rw > p.halo_w || ih > max_ih || iw > max_iw) {
-        if (threadIdx.x == 0) atomicCAS(p.status, 0u, 0x80000000u | 10u);
-        return;
-    }
-    for (int i = threadIdx.x; i < p.C * ih * iw; i += blockDim.x) {
-        int c = i / (ih * iw), r = i % (ih * iw);
-        int a = i0 + r / iw, b = j0 + r % iw;
-        float v = 0.0f;
-        if (a >= 0 && a < p.H && b >= 0 && b < p.W) v = p.x[(((size_t)n * p.C + c) * p.H + a) * p.W + b];
-        s_in[i] = v;
-    }
-    __syncthreads();
-    // stage 1: one (channel, pixel) per thread-iteration; pixels fastest so threads read s_in contiguously
-    for (int i = threadIdx.x; i < p.Cmid * rh * rw; i += blockDim.x) {
-        int m = i / (rh * rw), r = i % (rh * rw);
-        int a = r / rw, b = r % rw;
-        float acc = 0.0f;
-        const float *wm = p.w1 + (size_t)m * p.C * p.k * p.k;
-        for (int c = 0; c < p.C; ++c) {
-            const float *sc = s_in + ((size_t)c * ih + a * p.stride) * iw + b * p.stride;
-            const float *wc = wm + c * p.k * p.k;
-            for (int r1 = 0; r1 < p.k; ++r1)
-                for (int s1 = 0; s1 < p.k; ++s1) acc = fmaf(sc[r1 * iw + s1], wc[r1 * p.k + s1], acc);
+__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool live) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(live ? 4u : 0u) : "memory");
+}
+
+__device__ __forceinline__ void cp_async16_f32(float *dst, const float *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+template <int TM>
+__device__ __forceinline__ void f32_load_w(float2 (&w)[TM / 2], const float *src) {
+    if (TM % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < TM / 4; ++i) {
+            const float4 v = *reinterpret_cast<const float4 *>(src + 4 * i);
+            w[2 * i] = make_float2(v.x, v.y); w[2 * i + 1] = make_float2(v.z, v.w);
         }
-        // positions of the patch outside the stage-1 extent are never read by a pool window
-        s_mid[i] = apply_act(acc + p.b1[m], p.act1);
+    } else {
+#pragma unroll
+        for (int i = 0; i < TM / 2; ++i) w[i] = *reinterpret_cast<const float2 *>(src + 2 * i);
     }
-    __syncthreads();
-    // stage 2 + pool: one (output channel, pool output) per thread-iteration
-    int kper = p.K2 / p.parts_outc, k0 = part * kper;
-    for (int i = threadIdx.x; i < kper * th * tw; i += blockDim.x) {
-        int kk = k0 + i / (th * tw), r = i % (th * tw);
-        int oy = r / tw, ox = r % tw;
-        const float *w2 = p.w2 + (size_t)kk * p.Cmid;
-        float bias = p.b2[kk];
-        float m = -INFINITY, sum = 0.0f;
-        for (int dy = 0; dy < p.pool_k; ++dy)
-            for (int dx = 0; dx < p.pool_k; ++dx) {
-                int a = oy * p.pool_stride + dy, b = ox * p.pool_stride + dx;
-                float acc = 0.0f;
-                for (int c = 0; c < p.Cmid; ++c) acc = fmaf(s_mid[((size_t)c * rh + a) * rw + b], w2[c], acc);
-                float v = apply_act(acc + bias, p.act2);
-                m = fmaxf(m, v);
-                sum += v;
+}
+
+template <int TM, int TP>
+__device__ __forceinline__ void f32_fma(float2 (&acc)[TM / 2][TP], const float2 (&w)[TM / 2], const float *x) {
+#pragma unroll
+    for (int j = 0; j < TP; ++j) {
+        const float2 xx = make_float2(x[j], x[j]);
+#pragma unroll
+        for (int i = 0; i < TM / 2; ++i) acc[i][j] = __ffma2_rn(xx, w[i], acc[i][j]);
+    }
+}
+
+template <int TM, int TP, bool kWS>
+__global__ void __launch_bounds__(TP == 4 ? 512 : 256)
+f32_chain_kernel(const F32ChainParams p) {
+    extern __shared__ __align__(16) float f32_smem[];
+    const int T = blockDim.x;
+    const int max_ih = (p.halo_h - 1) * p.stride + p.k;
+    const int rp = p.pool_stride * p.hp, mp = p.halo_h * rp;      // pitches of a middle row and of a middle channel
+    float *s_in = f32_smem;                                       // [C][max_ih][iwp]
+    float *s_mid = s_in + p.C * max_ih * p.iwp;                   // [mpad][halo_h][pool_stride][hp]
+    float *s_w1 = s_mid + p.mpad * mp;                            // [C][k][k][mpad]
+    const int kper = p.K2 / p.parts_outc, kperp = (kper + 7) & ~7;
+    float *s_w2 = s_w1 + p.C * p.k * p.k * p.mpad;               // [Cmid][kperp], the part's slice
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (kWS) {
+        const int n4 = p.C * p.k * p.k * p.mpad / 4;
+        for (int i = threadIdx.x; i < n4; i += T) cp_async16_f32(s_w1 + 4 * i, p.w1 + 4 * i);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // (the image may be the predecessor's result)
+    int cur_part = -1;
+    const int total = p.N * p.parts_outc * p.tiles_h * p.tiles_w;
+    for (int cta0 = blockIdx.x; cta0 < total; cta0 += gridDim.x) {
+        int cta = cta0;
+        const int tx = cta % p.tiles_w; cta /= p.tiles_w;
+        const int ty = cta % p.tiles_h; cta /= p.tiles_h;
+        const int part = cta % p.parts_outc, n = cta / p.parts_outc;
+        // pool tile -> stage-1 patch -> input patch
+        const int py0 = ty * p.tile_h, px0 = tx * p.tile_w;
+        const int th = min(p.tile_h, p.PP - py0), tw = min(p.tile_w, p.PQ - px0);
+        const int rh = (th - 1) * p.pool_stride + p.pool_k, rw = (tw - 1) * p.pool_stride + p.pool_k;
+        const int ih = (rh - 1) * p.stride + p.k;
+        const int i0 = py0 * p.pool_stride * p.stride - p.pad, j0 = px0 * p.pool_stride * p.stride - p.pad;      // may be negative
+        if (rh > p.halo_h || rw > p.halo_w || ih > max_ih) {
+            if (threadIdx.x == 0) atomicCAS(p.status, 0u, 0x80000000u | 10u);
+            return;
+        }
+        {
+            // a warp per (channel, row): lanes along the row
+            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = T >> 5;
+            for (int cr = warp; cr < p.C * ih; cr += warps) {
+                const int c = cr / ih, a = cr - c * ih, gy = i0 + a;
+                const bool row_in = gy >= 0 && gy < p.H;
+                const float *src = p.x + (((size_t)n * p.C + c) * p.H + (row_in ? gy : 0)) * p.W;
+                float *dst = s_in + (c * max_ih + a) * p.iwp;
+                for (int b = lane; b < p.iwp; b += 32) {
+                    const int gx = j0 + b;
+                    const bool live = row_in && gx >= 0 && gx < p.W;
+                    cp_async4(dst + b, live ? src + gx : p.x, live);
+                }
             }
-        float o = p.pool_kind == 0 ? m : sum / (float)(p.pool_k * p.pool_k);
-        size_t oi = (((size_t)n * p.K2 + kk) * p.PP + (py0 + oy)) * p.PQ + (px0 + ox);
-        p.y[oi] = o;
+        }
+        const float *w2 = p.w2 + (size_t)part * p.Cmid * kperp;
+        if (kWS && part != cur_part) {
+            cur_part = part;
+            for (int i = threadIdx.x; i < p.Cmid * kperp / 4; i += T) cp_async16_f32(s_w2 + 4 * i, w2 + 4 * i);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        // stage 1
+        {
+            const int gpr = (rw + TP - 1) / TP, npg = rh * gpr, units = npg * (p.mpad / TM);
+            for (int u = threadIdx.x; u < units; u += T) {
+                const int mg = u / npg, pg = u - mg * npg, a = pg / gpr, b = (pg - a * gpr) * TP;
+                float2 acc[TM / 2][TP];
+#pragma unroll
+                for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < TP; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+                const float *in0 = s_in + a * p.stride * p.iwp + b * p.stride;
+                const float *wp = (kWS ? s_w1 : p.w1) + mg * TM;
+                if (TP == 4 && p.k == 3 && p.stride == 1) {
+                    for (int c = 0; c < p.C; ++c)
+#pragma unroll
+                        for (int r = 0; r < 3; ++r) {
+                            const float *row = in0 + (c * max_ih + r) * p.iwp;
+                            const float4 x0 = *reinterpret_cast<const float4 *>(row);
+                            const float2 x1 = *reinterpret_cast<const float2 *>(row + 4);
+                            const float xs[6] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y};
+#pragma unroll
+                            for (int s = 0; s < 3; ++s) {
+                                float2 w[TM / 2];
+                                f32_load_w<TM>(w, wp);
+                                wp += p.mpad;
+                                f32_fma<TM, TP>(acc, w, xs + s);
+                            }
+                        }
+                } else if (TP == 1 && p.k == 3) {
+                    for (int c = 0; c < p.C; ++c) {
+                        // (all of a channel's reads before its products: one warp per scheduler has nothing else to hide them)
+                        float xs[9];
+                        float2 w[9][TM / 2];
+#pragma unroll
+                        for (int t = 0; t < 9; ++t) {
+                            xs[t] = in0[(c * max_ih + t / 3) * p.iwp + t % 3];
+                            f32_load_w<TM>(w[t], wp + t * p.mpad);
+                        }
+#pragma unroll
+                        for (int t = 0; t < 9; ++t) f32_fma<TM, TP>(acc, w[t], xs + t);
+                        wp += 9 * p.mpad;
+                    }
+                } else {
+                    for (int c = 0; c < p.C; ++c)
+                        for (int r = 0; r < p.k; ++r) {
+                            const float *row = in0 + (c * max_ih + r) * p.iwp;
+#pragma unroll 3
+                            for (int s = 0; s < p.k; ++s) {
+                                float2 w[TM / 2];
+                                float xs[TP];
+                                f32_load_w<TM>(w, wp);
+                                wp += p.mpad;
+#pragma unroll
+                                for (int j = 0; j < TP; ++j) xs[j] = row[s + j * p.stride];
+                                f32_fma<TM, TP>(acc, w, xs);
+                            }
+                        }
+                }
+#pragma unroll
+                for (int i = 0; i < TM / 2; ++i) {
+                    const int m = mg * TM + 2 * i;
+                    const float b0 = m < p.Cmid ? __ldg(p.b1 + m) : 0.0f, b1 = m + 1 < p.Cmid ? __ldg(p.b1 + m + 1) : 0.0f;
+                    float *o = s_mid + m * mp + a * rp;
+#pragma unroll
+                    for (int j = 0; j < TP; ++j) {
+                        const int x = b + j;
+                        if (x >= rw) break;
+                        const int q = p.pool_stride == 2 ? (x & 1) * p.hp + (x >> 1) : (x % p.pool_stride) * p.hp + x / p.pool_stride;
+                        o[q] = apply_act(acc[i][j].x + b0, p.act1);
+                        o[mp + q] = apply_act(acc[i][j].y + b1, p.act1);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        // stage 2 + pool
+        if (p.pool_k == 2) {
+            // a thread takes TM channels of one pool output: the window's four pixels are its pixel tile
+            const int npg = th * tw, units = npg * (kperp / TM);
+            for (int u = threadIdx.x; u < units; u += T) {
+                const int kg = u / npg, pg = u - kg * npg, oy = pg / tw, ox = pg - oy * tw, kk0 = part * kper + kg * TM;
+                const float *src[4];
+#pragma unroll
+                for (int d = 0; d < 4; ++d) {
+                    const int dx = d & 1, sh = dx / p.pool_stride;
+                    src[d] = s_mid + (oy * p.pool_stride + (d >> 1)) * rp + (dx - sh * p.pool_stride) * p.hp + sh + ox;
+                }
+                const float *wp = (kWS ? s_w2 : w2) + kg * TM;
+                float2 acc[TM / 2][4];
+#pragma unroll
+                for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) acc[i][d] = make_float2(0.0f, 0.0f);
+#pragma unroll 4
+                for (int m = 0; m < p.Cmid; ++m) {
+                    float2 w[TM / 2];
+                    float xs[4];
+                    f32_load_w<TM>(w, wp);
+                    wp += kperp;
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) xs[d] = src[d][m * mp];
+                    f32_fma<TM, 4>(acc, w, xs);
+                }
+#pragma unroll
+                for (int i = 0; i < TM / 2; ++i) {
+                    const int kl = kg * TM + 2 * i;
+                    const float bx = kl < kper ? __ldg(p.b2 + kk0 + 2 * i) : 0.0f, by = kl + 1 < kper ? __ldg(p.b2 + kk0 + 2 * i + 1) : 0.0f;
+                    const float pool0 = p.pool_kind == 0 ? -INFINITY : 0.0f;
+                    float2 res = make_float2(pool0, pool0);
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) {
+                        const float vx = apply_act(acc[i][d].x + bx, p.act2), vy = apply_act(acc[i][d].y + by, p.act2);
+                        res.x = p.pool_kind == 0 ? fmaxf(res.x, vx) : res.x + vx;
+                        res.y = p.pool_kind == 0 ? fmaxf(res.y, vy) : res.y + vy;
+                    }
+                    if (p.pool_kind != 0) { res.x /= 4.0f; res.y /= 4.0f; }
+                    const size_t oi = (((size_t)n * p.K2 + kk0 + 2 * i) * p.PP + (py0 + oy)) * p.PQ + (px0 + ox);
+                    if (kl < kper) p.y[oi] = res.x;
+                    if (kl + 1 < kper) p.y[oi + (size_t)p.PP * p.PQ] = res.y;
+                }
+            }
+        } else {
+            const int gpr = (tw + TP - 1) / TP, npg = th * gpr, units = npg * (kperp / TM);
+            for (int u = threadIdx.x; u < units; u += T) {
+                const int kg = u / npg, pg = u - kg * npg, oy = pg / gpr, ox = (pg - oy * gpr) * TP;
+                const int kk0 = part * kper + kg * TM;
+                const bool is_max = p.pool_kind == 0;
+                const float pool0 = is_max ? -INFINITY : 0.0f;
+                float2 res[TM / 2][TP], bias[TM / 2];
+#pragma unroll
+                for (int i = 0; i < TM / 2; ++i) {
+                    bias[i].x = kg * TM + 2 * i < kper ? __ldg(p.b2 + kk0 + 2 * i) : 0.0f;
+                    bias[i].y = kg * TM + 2 * i + 1 < kper ? __ldg(p.b2 + kk0 + 2 * i + 1) : 0.0f;
+#pragma unroll
+                    for (int j = 0; j < TP; ++j) res[i][j] = make_float2(pool0, pool0);
+                }
+                for (int dy = 0; dy < p.pool_k; ++dy)
+                    for (int dx = 0; dx < p.pool_k; ++dx) {
+                        const int sh = dx / p.pool_stride;
+                        const float *src = s_mid + (oy * p.pool_stride + dy) * rp + (dx - sh * p.pool_stride) * p.hp + sh + ox;
+                        const float *wp = (kWS ? s_w2 : w2) + kg * TM;
+                        float2 acc[TM / 2][TP];
+#pragma unroll
+                        for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+                            for (int j = 0; j < TP; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+                        if (TP == 4 && sh == 0) {
+#pragma unroll 4
+                            for (int m = 0; m < p.Cmid; ++m) {
+                                float2 w[TM / 2];
+                                f32_load_w<TM>(w, wp);
+                                wp += kperp;
+                                const float4 x4 = *reinterpret_cast<const float4 *>(src + m * mp);
+                                const float xs[4] = {x4.x, x4.y, x4.z, x4.w};
+                                f32_fma<TM, TP>(acc, w, xs);
+                            }
+                        } else {
+#pragma unroll 4
+                            for (int m = 0; m < p.Cmid; ++m) {
+                                float2 w[TM / 2];
+                                float xs[TP];
+                                f32_load_w<TM>(w, wp);
+                                wp += kperp;
+#pragma unroll
+                                for (int j = 0; j < TP; ++j) xs[j] = src[m * mp + j];
+                                f32_fma<TM, TP>(acc, w, xs);
+                            }
+                        }
+#pragma unroll
+                        for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+                            for (int j = 0; j < TP; ++j) {
+                                const float vx = apply_act(acc[i][j].x + bias[i].x, p.act2), vy = apply_act(acc[i][j].y + bias[i].y, p.act2);
+                                res[i][j].x = is_max ? fmaxf(res[i][j].x, vx) : res[i][j].x + vx;
+                                res[i][j].y = is_max ? fmaxf(res[i][j].y, vy) : res[i][j].y + vy;
+                            }
+                    }
+                const float area = (float)(p.pool_k * p.pool_k);
+#pragma unroll
+                for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < TP; ++j) {
+                        if (ox + j >= tw) break;
+                        const int kl = kg * TM + 2 * i;
+                        const size_t oi = (((size_t)n * p.K2 + kk0 + 2 * i) * p.PP + (py0 + oy)) * p.PQ + (px0 + ox + j);
+                        if (kl < kper) p.y[oi] = is_max ? res[i][j].x : res[i][j].x / area;
+                        if (kl + 1 < kper) p.y[oi + (size_t)p.PP * p.PQ] = is_max ? res[i][j].y : res[i][j].y / area;
+                    }
+            }
+        }
+        __syncthreads();      // the patch and the middle map are rewritten for the next tile
     }
 }
 

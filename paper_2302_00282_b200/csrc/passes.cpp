@@ -611,19 +611,21 @@ struct Lower {
         L.pool_kind = C.kind == NK_MAXPOOL ? 0 : 1;
         L.pool_k = C.k; L.pool_stride = C.stride; L.pool_pad = 0; L.PP = po.h; L.PQ = po.w;
         L.out_ctot = B.cout;
-        L.w_off = put_f32(A.w); L.b_off = put_f32(A.b);
-        L.w2_off = put_f32(B.w); L.b2_off = put_f32(B.b);
         const SplitRequest &rq = ch.split;
         if (rq.user && rq.k > 1)
             return fail(g, XENOS_E_UNSUPPORTED, "split: the fp32 CUDA-core chain keeps every reduction inside one thread; parts_k applies to tensor-core convolutions and fc");
         const int smem_cap = std::min(g.hw.smem_bytes_per_cta, 227 * 1024) - 1024;
         auto region = [&](int t) { return (t - 1) * C.stride + C.k; };        // conv-output rows a tile of t pool rows reads
-        auto smem_need = [&](int th, int tw) {
-            int rh = region(th), rw = region(tw);
-            int ih = (rh - 1) * A.stride + A.k, iw = (rw - 1) * A.stride + A.k;
-            return (size_t)4 * ((size_t)A.cin * ih * iw + (size_t)A.cout * rh * rw);
+        const int mpad = round_up(A.cout, 8), taps = A.cin * A.k * A.k;
+        auto patch_pitch = [&](int tw) { return round_up((round_up(region(tw), 4) - 1) * A.stride + A.k, 4); };
+        auto mid_pitch = [&](int tw) { return round_up(tw, 4) + round_up((C.k - 1) / C.stride, 4); };
+        auto smem_need = [&](int th, int tw, int po, bool ws) {
+            const int rh = region(th), ih = (rh - 1) * A.stride + A.k;
+            size_t f = (size_t)A.cin * ih * patch_pitch(tw) + (size_t)mpad * rh * C.stride * mid_pitch(tw);
+            if (ws) f += (size_t)taps * mpad + (size_t)A.cout * round_up(B.cout / po, 8);
+            return 4 * f;
         };
-        int best_po = 0, best_th = 0, best_tw = 0;
+        int best_po = 0, best_th = 0, best_tw = 0, best_var = 0;
         double best_cost = 0;
         std::vector<int> po_cands, th_cands, tw_cands;
         if (rq.user && rq.outc > 0) {
@@ -642,24 +644,50 @@ struct Lower {
         };
         if (!dim_cands(rq.h, po.h, th_cands)) return fail(g, XENOS_E_BAD_SPLIT, "split: parts_h does not divide the output rows into equal-height tiles");
         if (!dim_cands(rq.w, po.w, tw_cands)) return fail(g, XENOS_E_BAD_SPLIT, "split: parts_w does not divide the output columns into equal-width tiles");
+        // Modelled cycles of a plan: waves over the units, per tile the patch's copy and, per stage, the warp-sized groups of
+        // register tiles that a scheduler runs in turn (8 x 4 tiles: 32 cycles of the FMA pipe per product step, at least four
+        // groups' worth because one warp alone waits for its own results; 2 x 1 tiles: 8 cycles, latency included).
+        // bit 0 of a variant: 8 x 4 tiles, bit 1: weights in shared memory.
         for (int p : po_cands)
             for (int th : th_cands)
-                for (int tw : tw_cands) {
-                    if (smem_need(th, tw) > (size_t)smem_cap) continue;
-                    int ctas = p * ceil_div(po.h, th) * ceil_div(po.w, tw);
-                    double s1 = (double)region(th) * region(tw) * A.cout * A.cin * A.k * A.k;
-                    double s2 = (double)region(th) * region(tw) * (B.cout / p) * A.cout;
-                    // modelled time: waves over the units, plus a fixed per-CTA overhead worth 2048 MACs
-                    double cost = (double)ceil_div(ctas * g.max_batch, g.hw.sm_count) * (s1 + s2 + 2048.0);
-                    if (best_po == 0 || cost < best_cost) { best_cost = cost; best_po = p; best_th = th; best_tw = tw; }
-                }
+                for (int tw : tw_cands)
+                    for (int var = 0; var < 4; ++var) {
+                        const bool big = var & 1, ws = var & 2;
+                        const size_t need = smem_need(th, tw, p, ws);
+                        if (need > (size_t)smem_cap) continue;
+                        const int rh = region(th), rw = region(tw), tm = big ? 8 : 2, tp = big ? 4 : 1;
+                        const double step = (big ? 32.0 : 8.0) * (ws ? 1.0 : 1.6), least = big ? 4.0 : 1.0;
+                        auto groups = [&](double units) { return std::max(least, std::ceil(std::ceil(units / 32.0) / 4.0)); };
+                        const double s1 = taps * step * groups((double)(mpad / tm) * rh * ceil_div(rw, tp));
+                        const double wide = round_up(B.cout / p, 8) / tm;
+                        const double s2 = C.k == 2 ? A.cout * (big ? step : 3.0 * step) * groups(wide * th * tw)      // (four window pixels at a time)
+                                                   : (double)C.k * C.k * A.cout * step * groups(wide * th * ceil_div(tw, tp));
+                        const double copy = 800.0 + (double)A.cin * ((rh - 1) * A.stride + A.k) * patch_pitch(tw) / 16.0;
+                        const long ctas = (long)p * ceil_div(po.h, th) * ceil_div(po.w, tw) * g.max_batch;
+                        const double cost = std::ceil((double)ctas / g.hw.sm_count) * (s1 + s2 + copy) + (ws ? (taps * mpad + A.cout * B.cout / p) * 4.0 / 50.0 : 0.0);
+                        if (best_po == 0 || cost < best_cost) { best_cost = cost; best_po = p; best_th = th; best_tw = tw; best_var = var; }
+                    }
         if (best_po == 0) return fail(g, XENOS_E_BAD_SPLIT, "split: no tile of the linked chain fits shared memory");
         L.parts_outc = best_po; L.tile_h = best_th; L.tile_w = best_tw;
         L.tiles_h = ceil_div(po.h, best_th); L.tiles_w = ceil_div(po.w, best_tw);
         L.halo_h = region(best_th); L.halo_w = region(best_tw);
-        L.smem_bytes = (int)smem_need(best_th, best_tw);
+        L.f32_big = best_var & 1; L.f32_ws = (best_var >> 1) & 1;
+        L.f32_iwp = patch_pitch(best_tw); L.f32_hp = mid_pitch(best_tw); L.npad = mpad;
+        L.smem_bytes = (int)smem_need(best_th, best_tw, best_po, L.f32_ws);
         L.grid = L.parts_outc * L.tiles_h * L.tiles_w;   // per image
-        L.block = 128;
+        L.block = L.f32_big ? 512 : 256;
+        {
+            // w1 [channel][row][column][Cmid], w2 [part][Cmid][channels of the part]: output channels innermost, padded to 8
+            std::vector<float> w1((size_t)taps * mpad, 0.0f);
+            for (int m = 0; m < A.cout; ++m)
+                for (int t = 0; t < taps; ++t) w1[(size_t)t * mpad + m] = A.w[(size_t)m * taps + t];
+            const int kper = B.cout / best_po, kperp = round_up(kper, 8);
+            std::vector<float> w2((size_t)best_po * A.cout * kperp, 0.0f);
+            for (int k = 0; k < B.cout; ++k)
+                for (int m = 0; m < A.cout; ++m) w2[((size_t)(k / kper) * A.cout + m) * kperp + k % kper] = B.w[(size_t)k * A.cout + m];
+            L.w_off = put_f32(w1); L.b_off = put_f32(A.b);
+            L.w2_off = put_f32(w2); L.b2_off = put_f32(B.b);
+        }
         L.flops = 2.0 * (node_macs(A) + node_macs(B));
         L.bytes = tbytes(A.in[0]) + tbytes(C.out) + node_param_bytes(A) + node_param_bytes(B);
         push(L, ci);

@@ -10,6 +10,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "chain2_tc.cuh"
@@ -320,9 +321,26 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
         if ((e = cudaFuncSetAttribute(xk::chain2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(chain2)", e);
     if (max_chain_smem > 0)
-        if ((e = cudaFuncSetAttribute(xk::f32_conv_conv_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
+        if ((e = cudaFuncSetAttribute(xk::f32_chain_kernel<8, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::f32_chain_kernel<8, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::f32_chain_kernel<2, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::f32_chain_kernel<2, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(f32 chain)", e);
     return XENOS_OK;
+}
+
+// Programmatic dependent launch: the kernel may be scheduled while its predecessor in the stream drains, runs its set-up
+// and then waits (griddepcontrol.wait) before it touches the predecessor's results.
+template <class... P, class... A>
+static cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t stream, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 static int ew_grid(long long total, int block, int sms) {
@@ -395,12 +413,18 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
             p.x = (const float *)ptr(L.in0); p.y = (float *)ptr(L.out);
             p.w1 = (const float *)(ws + L.w_off); p.b1 = (const float *)(ws + L.b_off);
             p.w2 = (const float *)(ws + L.w2_off); p.b2 = (const float *)(ws + L.b2_off);
-            p.N = N; p.C = L.C; p.H = L.H; p.W = L.W; p.Cmid = L.Cmid; p.P = L.P; p.Q = L.Q;
+            p.N = N; p.C = L.C; p.H = L.H; p.W = L.W; p.Cmid = L.Cmid; p.mpad = L.npad; p.P = L.P; p.Q = L.Q;
             p.k = L.k; p.stride = L.stride; p.pad = L.pad; p.act1 = L.act; p.K2 = L.K2; p.act2 = L.act2;
             p.pool_kind = L.pool_kind; p.pool_k = L.pool_k; p.pool_stride = L.pool_stride; p.PP = L.PP; p.PQ = L.PQ;
             p.parts_outc = L.parts_outc; p.tile_h = L.tile_h; p.tile_w = L.tile_w; p.tiles_h = L.tiles_h; p.tiles_w = L.tiles_w;
-            p.halo_h = L.halo_h; p.halo_w = L.halo_w; p.status = status;
-            xk::f32_conv_conv_pool_kernel<<<N * L.grid, L.block, L.smem_bytes, stream>>>(p);
+            p.halo_h = L.halo_h; p.halo_w = L.halo_w; p.iwp = L.f32_iwp; p.hp = L.f32_hp; p.status = status;
+            // a CTA keeps its weights and walks over tiles when there are more tiles than resident CTAs
+            const int occ = std::max(1, std::min(2048 / L.block, (228 * 1024) / (L.smem_bytes + 1024)));
+            const int grid = (int)std::min<long long>((long long)N * L.grid, (long long)sms * occ);
+            auto *k = L.f32_big ? (L.f32_ws ? xk::f32_chain_kernel<8, 4, true> : xk::f32_chain_kernel<8, 4, false>)
+                                : (L.f32_ws ? xk::f32_chain_kernel<2, 1, true> : xk::f32_chain_kernel<2, 1, false>);
+            cudaError_t le = launch_pdl(k, grid, L.block, L.smem_bytes, stream, p);
+            if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
         }
         case LK_STEM3X3: {
@@ -497,14 +521,8 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
                     if (st != XENOS_OK) return st;
                     maps = &now;
                 }
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3((unsigned)std::min(p.tiles, sms)); cfg.blockDim = dim3((unsigned)xk::kCvThreads);
-                cfg.dynamicSmemBytes = (size_t)L.smem_bytes; cfg.stream = stream;
-                cudaLaunchAttribute at[1];
-                at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-                at[0].val.programmaticStreamSerializationAllowed = 1;
-                cfg.attrs = at; cfg.numAttrs = 1;
-                cudaError_t le = cudaLaunchKernelEx(&cfg, L.skip >= 0 ? xk::pair_tc_kernel<true> : xk::pair_tc_kernel<false>, maps->a0, rt->tmaps[li], rt->tmaps2[li], maps->o, maps->s, p);
+                const int lgrid = (int)std::min(p.tiles, sms), lblock = (int)xk::kCvThreads;
+                cudaError_t le = launch_pdl(L.skip >= 0 ? xk::pair_tc_kernel<true> : xk::pair_tc_kernel<false>, lgrid, lblock, L.smem_bytes, stream, maps->a0, rt->tmaps[li], rt->tmaps2[li], maps->o, maps->s, p);
                 if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
                 break;
             }
@@ -531,14 +549,8 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
                 if (st != XENOS_OK) return st;
                 tma = &tma_now;
             }
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)std::min(p.m_tiles, sms)); cfg.blockDim = dim3((unsigned)xk::kC2Threads);
-            cfg.dynamicSmemBytes = (size_t)L.smem_bytes; cfg.stream = stream;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            at[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = at; cfg.numAttrs = 1;
-            cudaError_t le = cudaLaunchKernelEx(&cfg, xk::chain2_kernel, *tma, rt->tmaps[li], rt->tmaps2[li], p);
+            const int lgrid = (int)std::min(p.m_tiles, sms), lblock = (int)xk::kC2Threads;
+            cudaError_t le = launch_pdl(xk::chain2_kernel, lgrid, lblock, L.smem_bytes, stream, *tma, rt->tmaps[li], rt->tmaps2[li], p);
             if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
         }
@@ -585,17 +597,11 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
                 }
                 int limit = sms;
                 if (L.b_resident) limit = std::max(1, sms / L.n_tiles) * L.n_tiles;
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3((unsigned)std::min(p.total, limit)); cfg.blockDim = dim3((unsigned)xk::kCvThreads);
-                cfg.dynamicSmemBytes = (size_t)L.smem_bytes; cfg.stream = stream;
-                cudaLaunchAttribute at[1];
-                at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-                at[0].val.programmaticStreamSerializationAllowed = 1;
-                cfg.attrs = at; cfg.numAttrs = 1;
+                const int lgrid = (int)std::min(p.total, limit), lblock = (int)xk::kCvThreads;
                 auto *k = L.cv_epi == xk::CE_STORE ? xk::conv_tc_kernel<xk::CE_STORE> : L.cv_epi == xk::CE_SKIP ? xk::conv_tc_kernel<xk::CE_SKIP>
                         : L.cv_epi == xk::CE_VEC ? xk::conv_tc_kernel<xk::CE_VEC> : L.cv_epi == xk::CE_GAP ? xk::conv_tc_kernel<xk::CE_GAP>
                         : xk::conv_tc_kernel<xk::CE_SPLIT>;
-                cudaError_t le = cudaLaunchKernelEx(&cfg, k, maps->a0, maps->a1, rt->tmaps[li], maps->o, maps->s, p);
+                cudaError_t le = launch_pdl(k, lgrid, lblock, L.smem_bytes, stream, maps->a0, maps->a1, rt->tmaps[li], maps->o, maps->s, p);
                 if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
                 break;
             }
@@ -663,18 +669,12 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
             // Programmatic dependent launch: the kernel may be scheduled while its predecessor in the
             // stream drains, runs its set-up (barriers, tensor memory, constant staging) and then
             // waits (griddepcontrol.wait) before it touches any activation.
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)L.block);
-            cfg.dynamicSmemBytes = (size_t)L.smem_bytes; cfg.stream = stream;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            at[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = at; cfg.numAttrs = 1;
+            const int lgrid = (int)grid, lblock = (int)L.block;
             cudaError_t le;
-            if (L.dw_workers == 16) le = cudaLaunchKernelEx(&cfg, xk::dwpw_kernel<16>, rt->tmaps[li], *tmh, p);
-            else if (L.dw_workers == 8) le = cudaLaunchKernelEx(&cfg, xk::dwpw_kernel<8>, rt->tmaps[li], *tmh, p);
-            else if (L.ksplit > 1 || L.gap_parts > 1) le = cudaLaunchKernelEx(&cfg, xk::gemm_chain_kernel<1>, rt->tmaps[li], *tmh, p);
-            else le = cudaLaunchKernelEx(&cfg, xk::gemm_chain_kernel<0>, rt->tmaps[li], *tmh, p);
+            if (L.dw_workers == 16) le = launch_pdl(xk::dwpw_kernel<16>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
+            else if (L.dw_workers == 8) le = launch_pdl(xk::dwpw_kernel<8>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
+            else if (L.ksplit > 1 || L.gap_parts > 1) le = launch_pdl(xk::gemm_chain_kernel<1>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
+            else le = launch_pdl(xk::gemm_chain_kernel<0>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
             if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
         }
