@@ -149,6 +149,7 @@ __device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorM
     const ConvSegment &sg = g.seg[kSeg];
     const uint32_t box = in_reg(sg.box_bytes);
     if (!sg.im2col && sg.per_stage == 1) {
+#pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
             if (!mbar_wait(st.empty(), st.ph ^ 1u)) return false;
             mbar_arrive_expect_tx(st.fb, box);
@@ -166,6 +167,7 @@ __device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorM
             const int tap = kb0 / sg.cblocks;
             c = (kb0 - tap * sg.cblocks) * kTileK; r = tap / k; s = tap - r * k;
         }
+#pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
             if (!mbar_wait(st.empty(), st.ph ^ 1u)) return false;
             mbar_arrive_expect_tx(st.fb, box);
@@ -180,10 +182,12 @@ __device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorM
     const int per = in_reg(sg.per_stage), taps = in_reg(sg.taps);
     const uint32_t stride = in_reg(sg.box_stride);
     int tap = kb0 * per, r = tap / k, s = tap - r * k;
+#pragma unroll 1
     for (int kb = kb0; kb < kb1; ++kb) {
         const int nb = min(per, taps - tap);
         if (!mbar_wait(st.empty(), st.ph ^ 1u)) return false;
         mbar_arrive_expect_tx(st.fb, box * nb);
+#pragma unroll 1
         for (int b = 0; b < nb; ++b) {
             if (sg.im2col) tma_load_im2col(st.data + b * stride, tm, 0, w0, h0, n, st.fb, s, r);
             else tma_load_2d(st.data + b * stride, tm, 0, m0, st.fb);
@@ -224,6 +228,7 @@ __device__ __forceinline__ bool conv_mma(const ConvParams &g, ConvRing &st, uint
     if (per == 1) {
         const int cblocks = in_reg(sg.cblocks), last = in_reg(sg.last_steps);
         int cb = kb0 ? kb0 % cblocks : 0;
+#pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
             const uint32_t a4 = 0x10000u | (st.data >> 4);      // (shared addresses are below 2^18)
             if (!kRes) b4 = a4 + (kABytes >> 4);
@@ -237,6 +242,7 @@ __device__ __forceinline__ bool conv_mma(const ConvParams &g, ConvRing &st, uint
                 umma_bf16_acc(d_tmem, a_hi | (a4 + 4), b_hi | (b4 + 4), idesc);
                 umma_bf16_acc(d_tmem, a_hi | (a4 + 6), b_hi | (b4 + 6), idesc);
             } else {
+#pragma unroll 1
                 for (int x = 1; x < steps; ++x) umma_bf16_acc(d_tmem, a_hi | (a4 + 2 * x), b_hi | (b4 + 2 * x), idesc);
             }
             umma_commit(st.empty());
@@ -250,6 +256,7 @@ __device__ __forceinline__ bool conv_mma(const ConvParams &g, ConvRing &st, uint
         const uint32_t box16 = in_reg(sg.box_stride >> 4);
         const uint32_t s1 = spb == 1 ? box16 : 2u, s2 = spb == 1 ? 2 * box16 : box16;
         int left = sg.taps - kb0 * per;
+#pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
             const uint32_t a4 = 0x10000u | (st.data >> 4);
             if (!kRes) b4 = a4 + (kABytes >> 4);
@@ -276,6 +283,7 @@ __device__ __forceinline__ bool conv_mma_loop(const ConvParams &g, uint32_t sbas
     int i = 0, bseen = 0;
     const int k0 = in_reg(g.seg[0].kblocks), total = in_reg(g.total);
     const uint32_t b_res = sbase + g.off_b, acc_stride = in_reg((uint32_t)g.acc_stride), accf = bar + 8u * (2 * kCvMaxStages);
+#pragma unroll 1
     for (int ti = blockIdx.x; ti < total; ti += gridDim.x, ++i) {
         const int b = i & 1;
         const ConvTile t = conv_tile(g, ti);
@@ -352,6 +360,7 @@ __device__ __forceinline__ bool conv_epilogue_gap(const ConvParams &g, uint8_t *
         else reinterpret_cast<__nv_bfloat16 *>(g.out)[oi] = __float2bfloat16_rn(sum);
     };
     int i = 0;
+#pragma unroll 1
     for (int ti = blockIdx.x; ti < g.total; ti += gridDim.x, ++i) {
         const ConvTile t = conv_tile(g, ti);
         const int b = i & 1, n0 = t.nt * g.tile_n;
@@ -364,6 +373,7 @@ __device__ __forceinline__ bool conv_epilogue_gap(const ConvParams &g, uint8_t *
         if (fail_flag[0]) return false;
         tc_fence_after();
         const int per = g.gap_imgs * 32, parts = per >= 128 ? 1 : (per >= 64 ? 2 : 4);
+#pragma unroll 1
         for (int j = half; j < g.nchunks; j += 2) {
             float v[32];
             const int ncols = min(32, g.tile_n - j * 32), nc0 = n0 + j * 32;
@@ -387,6 +397,7 @@ __device__ __forceinline__ bool conv_epilogue_gap(const ConvParams &g, uint8_t *
             for (int c = 0; c < 32; ++c)
                 if (c < ncols) slab[row * 33 + c] = valid ? (g.act2 ? fminf(fmaxf(v[c], lo2), hi2) : v[c]) : 0.0f;
             asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");
+#pragma unroll 1
             for (int item = ht; item < per * parts; item += 128) {
                 const int c = item & 31, rest = item >> 5, img = rest / parts, pa = rest - img * parts;
                 float acc = 0.0f;
@@ -396,6 +407,7 @@ __device__ __forceinline__ bool conv_epilogue_gap(const ConvParams &g, uint8_t *
             }
             asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");
             if (parts > 1)
+#pragma unroll 1
                 for (int item = ht; item < per; item += 128) {
                     const int c = item & 31, img = item >> 5;
                     if (c >= ncols || nc0 + c >= g.N || img0 + img >= g.batch) continue;
@@ -417,6 +429,7 @@ __device__ __forceinline__ bool conv_epilogue_gap(const ConvParams &g, uint8_t *
                 for (int col = threadIdx.x - 128; col < g.tile_n; col += 256) {
                     if (n0 + col >= g.N || img0 >= g.batch) continue;
                     float acc = 0.0f;
+#pragma unroll 1
                     for (int q = 0; q < g.gap_parts; ++q) acc += __ldcg(g.split_part + ((size_t)img0 * g.gap_parts + q) * g.split_ld + n0 + col);
                     store(img0, n0 + col, acc);
                 }
@@ -466,6 +479,7 @@ __device__ __forceinline__ bool conv_epilogue_split(const ConvParams &g, uint8_t
     const uint32_t bias_s = smem_u32(sm) + g.off_bias;
     const uint32_t t_warp = tmem_base + ((uint32_t)(quarter * 32) << 16);
     int i = 0;
+#pragma unroll 1
     for (int ti = blockIdx.x; ti < g.total; ti += gridDim.x, ++i) {
         const ConvTile t = conv_tile(g, ti);
         const int b = i & 1, n0 = t.nt * g.tile_n, m0 = t.mt * g.tile_rows;
@@ -474,6 +488,7 @@ __device__ __forceinline__ bool conv_epilogue_split(const ConvParams &g, uint8_t
         if (fail_flag[0]) return false;
         tc_fence_after();
         float *part = g.split_part + (size_t)t.ks * g.split_stride + (size_t)(m0 + row) * g.split_ld + n0;
+#pragma unroll 1
         for (int j = half; j < g.nchunks; j += 2) {
             float v[16];
             tmem_ld16(t_warp + b * g.acc_stride + j * 16, v);
@@ -489,6 +504,7 @@ __device__ __forceinline__ bool conv_epilogue_split(const ConvParams &g, uint8_t
         if (et == 0) {
             atomicAdd(cnt, 1u);
             int seen = 0;
+#pragma unroll 1
             for (int spin = 0; spin < (1 << 22); ++spin) {
                 if (*reinterpret_cast<volatile unsigned int *>(cnt) >= (unsigned int)g.ksplit) { seen = 1; break; }
                 __nanosleep(32);
@@ -500,6 +516,7 @@ __device__ __forceinline__ bool conv_epilogue_split(const ConvParams &g, uint8_t
         __threadfence();
         const int live = min(kTileM, g.rows - m0), rows_per = (live + g.ksplit - 1) / g.ksplit;
         const int r0 = t.ks * rows_per, r1 = min(live, r0 + rows_per), c4n = g.tile_n >> 2;
+#pragma unroll 1
         for (int idx = et; idx < (r1 - r0) * c4n; idx += 256) {
             const int rr = r0 + idx / c4n, c4 = idx - (rr - r0) * c4n, nc = n0 + c4 * 4;
             if (nc >= g.N) continue;
@@ -575,6 +592,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
             ConvRing st;
             st.init(g, sbase, bar);
             const int k0 = in_reg(g.seg[0].kblocks), total = in_reg(g.total);
+#pragma unroll 1
             for (int ti = blockIdx.x; ti < total && ok; ti += gridDim.x) {
                 const ConvTile t = conv_tile(g, ti);
                 const int m0 = conv_row0(g, t.mt);
@@ -601,15 +619,18 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                 for (int q = 0; q < 4; ++q) {
                     const int k0 = q * g.b_group, k1 = min(g.kblocks, k0 + g.b_group);
                     mbar_arrive_expect_tx(bres_bar(q), k1 > k0 ? (uint32_t)(k1 - k0) * bytes : 0u);
+#pragma unroll 1
                     for (int kb = k0; kb < k1; ++kb) tma_load_2d(sbase + g.off_b + kb * bytes, &tmB, kb * kTileK, t.nt * tile_n, bres_bar(q));
                 }
             } else {
                 ConvRing st;
                 st.init(g, sbase, bar);
                 const int total = in_reg(g.total);
+#pragma unroll 1
                 for (int ti = blockIdx.x; ti < total && ok; ti += gridDim.x) {
                     const ConvTile t = conv_tile(g, ti);
                     const int row = t.nt * tile_n;
+#pragma unroll 1
                     for (int kb = t.kb0; kb < t.kb1; ++kb) {
                         ok = mbar_wait(st.empty(), st.ph ^ 1u);
                         if (!ok) break;
@@ -641,12 +662,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                 }
                 __syncwarp();
             }
+#pragma unroll 1
             for (int ti = blockIdx.x; ti < g.total && ok; ti += gridDim.x, ++i) {
                 const ConvTile t = conv_tile(g, ti);
                 const int b = i & 1, y = t.mt * g.tile_rows + quarter * 32;
                 if (!mbar_wait(accf_bar(b), (i >> 1) & 1)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t t_acc = t_warp + b * g.acc_stride;
+#pragma unroll 1
                 for (int j = half; j < g.nchunks; j += 2, ++cnt) {
                     const uint32_t buf = stage0 + (uint32_t)(cnt & 1) * g.box_bytes;
                     const int x = t.nt * g.tile_n + j * g.chunk;
@@ -658,6 +681,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                         ok = mbar_wait(skip_bar(e, cnt & 1), (cnt >> 1) & 1);
                         if (!ok) break;
                     }
+#pragma unroll 1
                     for (int c0 = 0; c0 < g.chunk; c0 += 32) {
                         const bool wide = g.chunk - c0 >= 32;
                         float v[32];
@@ -712,11 +736,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
         } else if (kEpi == CE_VEC) {
             // vectors (fp32 results, channel counts that are no multiple of 8): plain stores
             int i = 0;
+#pragma unroll 1
             for (int ti = blockIdx.x; ti < g.total && ok; ti += gridDim.x, ++i) {
                 const ConvTile t = conv_tile(g, ti);
                 const int b = i & 1, m = t.mt * g.tile_rows + row;
                 if (!mbar_wait(accf_bar(b), (i >> 1) & 1)) { ok = false; break; }
                 tc_fence_after();
+#pragma unroll 1
                 for (int j = half; j < g.nchunks; j += 2) {
                     const int x = t.nt * g.tile_n + j * 16;
                     float v[16];

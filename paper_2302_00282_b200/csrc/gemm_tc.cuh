@@ -131,6 +131,7 @@ __device__ __forceinline__ bool mbar_wait_limited(uint32_t bar, uint32_t parity,
             : "=r"(done) : "r"(bar), "r"(parity) : "memory");
         if (done) return true;
     }
+#pragma unroll 1
     for (int i = 0; i < limit; ++i) {
         uint32_t done;
         asm volatile(

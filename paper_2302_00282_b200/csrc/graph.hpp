@@ -141,10 +141,11 @@ struct Launch {
     int stem_tma = 0, stem_align = 1;                              // stem: image patch by TMA, x alignment in elements
     int a_tma = 0, a_box_bytes = 0;                                // activation operand by TMA: 1 matrix rows, 2 shifted patch
     int fc_small = 0;                                              // 1: fully connected layer of a small batch on the CUDA cores (fc_small_kernel)
-    int dw_workers = 0;                                            // > 0: depthwise -> pointwise in dwpw_kernel with that many worker warps
+    int dw_workers = 0;                                            // depthwise -> pointwise (dw_tc_kernel): worker warps
+    int dw_groups = 0, dw_wpg_log2 = 0, dw_br = 1, dw_batch = 1, h_slots = 0, out_bufs = 1;      // ... their groups, a thread's block rows, halo slots, result boxes
     // convolution, product or fc in conv_tc_kernel: its epilogue kind, rows of an operand box, resident weights, column chunks
     int conv_tc = 0, cv_epi = 0, a_rows = 128, b_resident = 0, b_group = 0, chunk = 0, nchunks = 0, off_b = 0;
-    int n_acc = 1;                                                 // dwpw_kernel: channel tiles of tile_n columns per CTA (2: both accumulators hold one tile)
+    int n_acc = 1;                                                 // dw_tc_kernel: channel tiles of tile_n columns per CTA (2: both accumulators hold one tile)
     int pair = 0, a_slots = 0, b_slots = 0, off_b2 = 0;            // LK_GEMM2 with a 1x1 consumer: pair_tc_kernel and its rings
     // ---- two linked convolutions (LK_GEMM2): producer tile rh1 x rw1 = patch_rh x patch_rw, consumer tile rh2 x rw2
     int k2 = 1, kblocks2 = 0, n1pad = 0, halo2 = 0, rh2 = 0, rw2 = 0, act3 = 0, off_mid = 0, stage_bytes = 0;

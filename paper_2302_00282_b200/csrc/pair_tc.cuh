@@ -50,9 +50,11 @@ __device__ __forceinline__ bool pair_gemm1(const PairParams &g, PairRing &ra, Pa
     constexpr uint64_t hi = (uint64_t)(64u | (1u << 14) | (2u << 29)) << 32;
     const uint32_t b0 = sbase + g.off_b;
     uint32_t acc = 0u;
+#pragma unroll 1
     for (int kb = 0; kb < n; ++kb) {
         if (!mbar_wait(a_full + 8u * ra.s, ra.ph)) return false;
         const uint32_t a4 = 0x10000u | ((sbase + ra.s * kABytes) >> 4);
+#pragma unroll 1
         for (int h = 0; h < slots; ++h) {
             uint32_t b4;
             if (resident) b4 = 0x10000u | ((b0 + kb * n1pad * 128) >> 4);
@@ -129,6 +131,7 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             pdl_wait();
             PairRing ra = {0, in_reg(g.a_slots), 0u};
             const int tiles = in_reg(g.tiles), n_kb = in_reg(g.seg.kblocks), cend = in_reg(g.seg.cblocks * kTileK), k = in_reg(g.seg.k);
+#pragma unroll 1
             for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
                 const int m0 = t * kTileM;
                 const int n = (int)g.d_rpi.div((uint32_t)m0), rem = m0 - n * (int)g.d_rpi.d;
@@ -136,6 +139,7 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 const int h0 = p * g.seg.stride + g.seg.low, w0 = q * g.seg.stride + g.seg.low;
                 const bool im2col = g.seg.im2col != 0;
                 int c = 0, r = 0, s = 0;
+#pragma unroll 1
                 for (int kb = 0; kb < n_kb; ++kb) {
                     const uint32_t fb = a_full + 8u * ra.s;
                     ok = mbar_wait(fb + 8u * kPairMaxSlots, ra.ph ^ 1u);
@@ -157,14 +161,19 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const int n_kb = in_reg(g.seg.kblocks), n1pad = in_reg(g.n1pad), slots = in_reg(g.n1_slots), kb2n = in_reg(g.kblocks2), n2 = in_reg(g.n2_blocks);
             if (g.resident) {
                 mbar_arrive_expect_tx(bres, (uint32_t)(n_kb * n1pad + kb2n * n2 * 128) * 128u);
+#pragma unroll 1
                 for (int kb = 0; kb < n_kb; ++kb) tma_load_2d(b0 + kb * n1pad * 128, &tmB1, kb * kTileK, 0, bres);
+#pragma unroll 1
                 for (int c = 0; c < n2; ++c)
+#pragma unroll 1
                     for (int kb = 0; kb < kb2n; ++kb) tma_load_2d(b0 + n_kb * n1pad * 128 + (c * kb2n + kb) * kABytes, &tmB2, kb * kTileK, c * 128, bres);
             } else {
                 PairRing rb = {0, in_reg(g.b_slots), 0u};
                 const uint32_t bytes1 = (uint32_t)min(n1pad, 128) * 128u;
                 auto first = [&]() {
+#pragma unroll 1
                     for (int kb = 0; kb < n_kb && ok; ++kb)
+#pragma unroll 1
                         for (int h = 0; h < slots; ++h) {
                             const uint32_t fb = b_full + 8u * rb.s;
                             ok = mbar_wait(fb + 8u * kPairMaxSlots, rb.ph ^ 1u);
@@ -175,7 +184,9 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         }
                 };
                 auto second = [&]() {
+#pragma unroll 1
                     for (int c = 0; c < n2 && ok; ++c)
+#pragma unroll 1
                         for (int kb = 0; kb < kb2n; ++kb) {
                             const uint32_t fb = b_full + 8u * rb.s;
                             ok = mbar_wait(fb + 8u * kPairMaxSlots, rb.ph ^ 1u);
@@ -187,6 +198,7 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 };
                 const int step = gridDim.x;
                 if (g.dbl) first();
+#pragma unroll 1
                 for (int t = blockIdx.x; t < g.tiles && ok; t += step) {
                     if (!g.dbl || t + step < g.tiles) first();
                     if (ok) second();
@@ -214,14 +226,17 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (resident) ok = mbar_wait(bres, 0u);
             if (ok && dbl && (int)blockIdx.x < tiles) ok = first();
             int i = 0;
+#pragma unroll 1
             for (int t = blockIdx.x; t < tiles && ok; t += step, ++i) {
                 if (!dbl || t + step < tiles) { ok = first(); if (!ok) break; }
                 ok = mbar_wait(midf, i & 1);
+#pragma unroll 1
                 for (int c = 0; c < n2 && ok; ++c, ++c2) {
                     const int b = c2 & 1;
                     ok = mbar_wait(d2e + 8u * b, ((c2 >> 1) & 1) ^ 1u);
                     if (!ok) break;
                     const uint32_t d = tmem_base + 256 + b * 128;
+#pragma unroll 1
                     for (int kb = 0; kb < kb2n; ++kb) {
                         const uint32_t a4 = 0x10000u | ((mid + kb * kABytes) >> 4);
                         uint32_t b4;
@@ -273,12 +288,14 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         int i = 0, c2 = 0, cnt = 0;
         if (kSkip && (int)blockIdx.x < tiles && elect_one()) ask_skip(0, blockIdx.x, 0, 0);
         __syncwarp();
+#pragma unroll 1
         for (int t = blockIdx.x; t < tiles && ok; t += step, ++i) {
             // middle: first accumulator -> operand layout of the second product
             const int b1 = dbl ? i & 1 : 0, use = dbl ? i >> 1 : i;
             ok = mbar_wait(mide, (i & 1) ^ 1u) && mbar_wait(d1f + 8u * b1, use & 1);      // GEMM 2 has read the previous tile's middle
             if (!ok) break;
             tc_fence_after();
+#pragma unroll 1
             for (int j = half; j < (n1pad >> 5); j += 2) {
                 float v[32];
                 tmem_ld32(t_warp + b1 * 128 + j * 32, v);
@@ -300,6 +317,7 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             __syncwarp();
             if (lane == 0) { mbar_arrive(d1e + 8u * b1); mbar_arrive(midf); }
             // final
+#pragma unroll 1
             for (int c = 0; c < n2 && ok; ++c, ++c2) {
                 const int b = c2 & 1;
                 ok = mbar_wait(d2f + 8u * b, (c2 >> 1) & 1);

@@ -776,6 +776,95 @@ struct Lower {
         return XENOS_OK;
     }
 
+    // Worker groups, rings and shared memory of dw_tc_kernel for the tile geometry at hand.  A group of 2^w warps covers a
+    // tile's units (a lane owns br x 4 pixels of a channel pair); an item takes the slower of the issue slots of its warps
+    // (a scheduler runs a quarter of the 16 warps) and its own latency shared by the groups.  The configuration with the least time whose rings fit is taken; what is left goes to deeper rings.
+    xenos_status_t layout_dw(Launch &L) {
+        const ASeg &s0 = L.seg[0];
+        const int C = s0.C, cols = L.n_acc * L.tile_n, pairs = L.halo_cb > 32 ? 32 : 16;
+        const long tiles = (long)L.m_tiles * L.n_tiles * L.ksplit;
+        const bool one = tiles <= g.hw.sm_count;                  // a CTA's only tile: results leave through the operand ring
+        const int dww = (int)align_up((size_t)40 * C, 1024), bias = (int)align_up((size_t)L.npad * 4, 128);
+        const int room = std::min(g.hw.smem_bytes_per_cta, 227 * 1024) - 2048 - 512 - dww - bias;
+        const int bslot = cols * 128;
+        // (the window covers whole blocks of br rows)
+        auto window_h = [&](int br) { return (round_up(L.patch_rh, br) - 1) * s0.stride + 3; };
+        auto window = [&](int br) { return (int)align_up((size_t)L.ni * window_h(br) * L.halo_w * L.halo_cb * 2, 128); };
+        const int rgrid = g.hw.sm_count / L.n_tiles * L.n_tiles;
+        L.cv_epi = L.epi == EPI_GAP ? 1 : L.ksplit > 1 ? 2 : 0;
+        auto staging = [&](int chunk, int bufs) {
+            if (L.cv_epi == 2) return 0;
+            if (L.cv_epi == 1) {
+                const int per = 4 * L.gap_imgs * 32, parts = per * 4 <= 512 ? 4 : (per * 2 <= 512 ? 2 : 1);
+                return (int)align_up((size_t)4 * 128 * 33 * 4 + (size_t)per * parts * 4, 1024);
+            }
+            return 4 * bufs * 128 * chunk * 2;
+        };
+        double best = -1;
+        for (int br : {4, 2, 1}) {
+            if (br > 1 && L.patch_rh <= br / 2) continue;
+            const int units = L.ni * ceil_div(L.patch_rh, br) * (L.patch_rw / 4) * pairs, hstride = window(br);
+            const double issue = s0.stride == 1 ? (br == 4 ? 340.0 : br == 2 ? 200.0 : 125.0) : (br == 4 ? 460.0 : br == 2 ? 270.0 : 160.0);
+            if (window_h(br) > 256) continue;
+            for (int w = 0; w <= 4; ++w) {
+                if ((32 << w) < units) continue;
+                const int groups = 16 >> w;
+                for (int res = 1; res >= 0; --res)
+                    for (int chunk : {64, 32, 16})
+                        for (int bufs = 2; bufs >= 1; --bufs) {
+                            if (L.cv_epi == 0 && (cols % chunk || (chunk > 16 && cols / chunk < 4))) continue;
+                            if (L.cv_epi != 0 && (chunk != (L.cv_epi == 1 ? 32 : 16) || bufs == 2)) continue;
+                            if (res && (one || L.ksplit > 1 || rgrid == 0)) continue;
+                            const int a_min = std::max(2, groups), h_min = std::max(2, groups), b_min = res ? 0 : 2;
+                            const int ops = a_min * 16384 + (res ? L.kblocks * bslot : b_min * bslot), st = staging(chunk, bufs);
+                            const int need = (one ? std::max(ops, st) : ops + st) + h_min * hstride;
+                            if (a_min > 8 || h_min > 8 || need > room) continue;
+                            const double t = std::max((1 << w) * issue / 4.0, (300.0 + 2.2 * issue) / groups) +
+                                             (res ? 0.0 : 20.0) + (chunk == 16 ? 15.0 : 0.0) + (bufs == 1 ? 10.0 : 0.0);
+                            if (best >= 0 && t >= best) continue;
+                            best = t;
+                            L.chunk = chunk;
+                            L.dw_br = br; L.dw_wpg_log2 = w; L.dw_groups = groups; L.b_resident = res; L.out_bufs = bufs;
+                            L.a_slots = a_min; L.h_slots = h_min; L.b_slots = b_min;
+                        }
+            }
+        }
+        if (best < 0) return fail(g, XENOS_E_BAD_SPLIT, "split: pipeline does not fit shared memory");
+        const int st = staging(L.chunk, L.out_bufs), groups = L.dw_groups, hstride = window(L.dw_br);
+        L.halo_h = window_h(L.dw_br);
+        L.halo_bytes = L.ni * L.halo_h * L.halo_w * L.halo_cb * 2;
+        L.halo_stride = hstride;
+        auto used = [&]() {
+            const int ops = L.a_slots * 16384 + (L.b_resident ? L.kblocks * bslot : L.b_slots * bslot);
+            return (one ? std::max(ops, st) : ops + st) + L.h_slots * hstride;
+        };
+        // deeper rings with what is left: windows first (they come from the predecessor's tensor), then weights, then operands
+        auto grow = [&](int &slots, int by, int most) { while (slots + by <= most) { slots += by; if (used() > room) { slots -= by; break; } } };
+        grow(L.h_slots, groups, std::min(8, 2 * std::max(2, groups)));
+        if (!L.b_resident) grow(L.b_slots, 1, std::min(4, std::max(2, L.kblocks)));
+        grow(L.a_slots, groups, std::min(8, 2 * std::max(2, groups)));
+        L.nchunks = ceil_div(cols, L.chunk);
+        L.off_b = L.a_slots * 16384;
+        const int ops = L.off_b + (L.b_resident ? L.kblocks * bslot : L.b_slots * bslot);
+        L.off_stg = one ? 0 : ops;
+        L.off_halo = (int)align_up((size_t)(one ? std::max(ops, st) : ops + st), 1024);
+        L.off_dww = (int)align_up((size_t)L.off_halo + (size_t)L.h_slots * hstride, 128);
+        L.off_bias = L.off_dww + dww;
+        L.off_bar = L.off_bias + bias;
+        L.smem_bytes = L.off_bar + 512 + 1024;
+        L.stages = std::min(6, L.a_slots); L.hstages = L.h_slots;
+        L.dw_workers = 16;
+        L.grid = (int)std::min<long>(tiles, L.b_resident ? rgrid : g.hw.sm_count);
+        L.block = 64 + 32 * 16;
+        // tiles of a batch: enough items for every group, an accumulator pair each
+        L.dw_batch = 1;
+        if (L.cv_epi == 0 && L.n_acc == 1 && !one)
+            L.dw_batch = std::max(1, std::min(std::min(ceil_div(groups, L.kblocks), g.hw.tmem_columns / (2 * L.acc_stride)), 4));
+        L.tmem_cols = 32;
+        while (L.tmem_cols < (L.n_acc == 2 ? 2 : 2 * L.dw_batch) * L.acc_stride) L.tmem_cols *= 2;
+        return XENOS_OK;
+    }
+
     xenos_status_t make_gemm(int ci, const std::vector<int> &cover, const Node *dw, const Node *mainc,
                              const Node *shortcut, const Node *expand2, const Node *addn, const Node *pooln,
                              const Node *gapn, const Node *catn, bool fc) {
@@ -951,7 +1040,7 @@ struct Lower {
             // the depthwise stage is recomputed per channel tile and its time grows with the tile's pixels:
             // while SMs would stay idle, fewer images per tile spread it over more of them
             while (L.ni > 1 && (long)ceil_div(g.max_batch, L.ni) * ceil_div(round_up(N, 16), 256) * 2 <= g.hw.sm_count) --L.ni;
-            while (!gapn && L.patch_rh > 1 && halo_of(L.ni, L.patch_rh, L.patch_rw) > 76 * 1024) --L.patch_rh;
+            while (!gapn && L.patch_rh > 1 && halo_of(L.ni, L.patch_rh, L.patch_rw) > 44 * 1024) --L.patch_rh;
             // Small batches leave most units idle while each tile's depthwise stage runs its K blocks one after the
             // other, at a pace set by the pixels per tile: while at least half of the units would stay idle, halve the
             // tile's rows (the MMA tile is then partly empty, which costs nothing there).
@@ -1066,6 +1155,9 @@ struct Lower {
         if (L.conv_tc) {
             const xenos_status_t lst = layout_conv(L, ot);
             if (lst != XENOS_OK) return lst;
+        } else if (dw) {
+            const xenos_status_t lst = layout_dw(L);
+            if (lst != XENOS_OK) return lst;
         } else {
         // shared memory of the one persistent CTA per SM: [A|B ring][halo ring][epilogue staging][barriers]
         int stage_bytes = 16384 + L.n_acc * L.tile_n * 128;
@@ -1094,19 +1186,6 @@ struct Lower {
         L.smem_bytes = L.off_bar + 256 + 1024;     // + barriers, alignment slack
         L.grid = std::min(L.m_tiles * L.n_tiles * L.ksplit, g.hw.sm_count);
         L.block = 448;
-        // A depthwise -> pointwise chain that stores its tile and has one tile per CTA at most runs in the kernel whose
-        // warps all work on the stencil and then on the store (dwpw_kernel: 16 worker warps for 64-channel blocks, 8
-        // for narrower ones): with a single tile the separate producer and epilogue warps of gemm_chain_kernel
-        // would take turns waiting.  Measured on MobileNet at batch 32: 18.8 against 20.1 us per 14 x 14 chain; the
-        // chains with many tiles per CTA are faster in gemm_chain_kernel (44 against 48 us for the first one).
-        // (a global-average epilogue parks its slabs in the A|B ring, which a CTA's only tile has left free)
-        const int gap_workers = L.halo_cb > 32 ? 16 : 8;
-        const long gap_need = (long)(gap_workers / 4) * 128 * 33 * 4 + 4L * std::max(32 * gap_workers, (gap_workers / 4) * L.gap_imgs * 32);
-        const bool gap_fits = L.epi == EPI_GAP && L.skip < 0 && L.act2 == 0 && (long)L.stages * stage_bytes >= gap_need;
-        if (dw && (L.epi == EPI_STORE || gap_fits) && L.ksplit == 1 && s1.mode == AM_NONE && L.m_tiles * L.n_tiles <= g.hw.sm_count) {
-            L.dw_workers = L.halo_cb > 32 ? 16 : 8;
-            L.block = 64 + 32 * L.dw_workers;
-        }
         }
         // --- pack weights + bias
         L.w_off = blob_reserve(g, (size_t)L.npad * L.kpad * 2);
@@ -1587,7 +1666,7 @@ void emit_plan_json(Graph &g) {
             jint(s, "ni", L.ni); jint(s, "step_y", L.step_y); jint(s, "step_x", L.step_x); jint(s, "off_y", L.off_y); jint(s, "off_x", L.off_x);
             jint(s, "hstages", L.hstages); jint(s, "halo_h", L.halo_h); jint(s, "halo_w", L.halo_w); jint(s, "halo_cb", L.halo_cb);
             jint(s, "halo_bytes", L.halo_bytes);
-            jint(s, "ksplit", L.ksplit); jint(s, "kb_per", L.kb_per); jint(s, "a_tma", L.a_tma); jint(s, "fc_small", L.fc_small); jint(s, "dw_workers", L.dw_workers); jint(s, "n_acc", L.n_acc); jint(s, "gap_parts", L.gap_parts); jint(s, "conv_tc", L.conv_tc); jint(s, "b_resident", L.b_resident);
+            jint(s, "ksplit", L.ksplit); jint(s, "kb_per", L.kb_per); jint(s, "a_tma", L.a_tma); jint(s, "fc_small", L.fc_small); jint(s, "dw_workers", L.dw_workers); jint(s, "dw_groups", L.dw_groups); jint(s, "dw_br", L.dw_br); jint(s, "chunk", L.chunk); jint(s, "out_bufs", L.out_bufs); jint(s, "b_slots", L.b_slots); jint(s, "n_acc", L.n_acc); jint(s, "gap_parts", L.gap_parts); jint(s, "conv_tc", L.conv_tc); jint(s, "b_resident", L.b_resident);
         }
         if (L.kind == LK_GEMM2) {
             jint(s, "k2", L.k2); jint(s, "cmid", L.Cmid); jint(s, "n1pad", L.n1pad); jint(s, "kblocks", L.kblocks); jint(s, "kblocks2", L.kblocks2);

@@ -15,7 +15,7 @@
 
 #include "chain2_tc.cuh"
 #include "conv_tc.cuh"
-#include "dwpw_tc.cuh"
+#include "dw_tc.cuh"
 #include "gemm_tc.cuh"
 #include "graph.hpp"
 #include "kernels_bf16.cuh"
@@ -124,6 +124,24 @@ static xenos_status_t encode_conv_maps(const Graph &g, Runtime *rt, const Launch
         st = encode_rows_map(g, rt, ptr(L.skip), g.tensors[L.skip].c, rows, L.pair ? 32 : L.chunk, 32, &m->s);
     return st;
 }
+// Depthwise chains: input windows (a0) and result boxes (o: (channel, column, row, image) with a box of one tile).
+template <class Ptr>
+static xenos_status_t encode_dw_maps(const Graph &g, Runtime *rt, const Launch &L, Ptr ptr, int images, bool want_external, ConvMaps *m) {
+    auto external = [&](int t) { return g.tensors[t].input_slot >= 0 || g.tensors[t].output_slot >= 0; };
+    xenos_status_t st = XENOS_OK;
+    if (external(L.seg[0].tensor) == want_external) st = encode_halo_map(g, rt, L, ptr(L.seg[0].tensor), images, &m->a0);
+    if (st != XENOS_OK || L.cv_epi != xk::DE_STORE || external(L.out) != want_external) return st;
+    void *base = ptr(L.out);
+    const cuuint64_t C = (cuuint64_t)L.out_ctot, W = (cuuint64_t)L.Q, H = (cuuint64_t)L.P;
+    cuuint64_t dims[4] = {C, W, H, (cuuint64_t)images}, strides[3] = {C * 2, W * C * 2, H * W * C * 2};
+    cuuint32_t box[4] = {(cuuint32_t)L.chunk, (cuuint32_t)L.patch_rw, (cuuint32_t)L.patch_rh, (cuuint32_t)L.ni}, estr[4] = {1u, 1u, 1u, 1u};
+    if (((uintptr_t)base & 15u) || (C & 7) || L.patch_rw * L.patch_rh * L.ni > 128) return fail(g, XENOS_E_CUDA, "internal: depthwise result tile violates the TMA limits");
+    CUresult r = rt->encode(&m->o, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            swizzle_of(L.chunk), CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(g, XENOS_E_CUDA, "cuTensorMapEncodeTiled (depthwise result) failed with code " + std::to_string((int)r));
+    return XENOS_OK;
+}
+
 static bool conv_has_external(const Graph &g, const Launch &L) {
     auto external = [&](int t) { return t >= 0 && (g.tensors[t].input_slot >= 0 || g.tensors[t].output_slot >= 0); };
     return external(L.seg[0].tensor) || (L.seg[1].mode != AM_NONE && external(L.seg[1].tensor)) || external(L.out) || external(L.skip);
@@ -194,6 +212,16 @@ static xenos_status_t encode_stem_map(const Graph &g, Runtime *rt, const Launch 
                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(g, XENOS_E_CUDA, "cuTensorMapEncodeTiled (stem) failed with code " + std::to_string((int)r));
     return XENOS_OK;
+}
+
+typedef void (*DwKernel)(CUtensorMap, CUtensorMap, CUtensorMap, xk::DwParams);
+template <int kEpi>
+static DwKernel dw_kernel_of(int stride, int br) {
+    if (stride == 1) return br == 4 ? xk::dw_tc_kernel<kEpi, 1, 4> : br == 2 ? xk::dw_tc_kernel<kEpi, 1, 2> : xk::dw_tc_kernel<kEpi, 1, 1>;
+    return br == 4 ? xk::dw_tc_kernel<kEpi, 2, 4> : br == 2 ? xk::dw_tc_kernel<kEpi, 2, 2> : xk::dw_tc_kernel<kEpi, 2, 1>;
+}
+static DwKernel dw_kernel(int epi, int stride, int br) {
+    return epi == xk::DE_STORE ? dw_kernel_of<xk::DE_STORE>(stride, br) : epi == xk::DE_GAP ? dw_kernel_of<xk::DE_GAP>(stride, br) : dw_kernel_of<xk::DE_SPLIT>(stride, br);
 }
 
 void runtime_free(Graph &g) {
@@ -284,8 +312,8 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
                 if (st != XENOS_OK) return st;
                 continue;
             }
-            if (L.seg[0].mode == AM_DW && g.tensors[L.seg[0].tensor].input_slot < 0) {
-                xenos_status_t st = encode_halo_map(g, rt, L, static_cast<uint8_t *>(ws) + g.place[L.seg[0].tensor].off, g.max_batch, &rt->hmaps[i]);
+            if (L.seg[0].mode == AM_DW) {
+                xenos_status_t st = encode_dw_maps(g, rt, L, [&](int t) -> void * { return static_cast<uint8_t *>(ws) + g.place[t].off; }, g.max_batch, false, &rt->conv[i]);
                 if (st != XENOS_OK) return st;
             }
         }
@@ -307,9 +335,11 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
             (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(conv)", e);
     if (any_gemm)
-        if ((e = cudaFuncSetAttribute(xk::dwpw_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::dwpw_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
-            return cuda_fail(g, "cudaFuncSetAttribute(dwpw)", e);
+        for (int epi = 0; epi < 3; ++epi)
+            for (int stride = 1; stride <= 2; ++stride)
+                for (int br : {1, 2, 4})
+                    if ((e = cudaFuncSetAttribute(dw_kernel(epi, stride, br), cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
+                        return cuda_fail(g, "cudaFuncSetAttribute(dw)", e);
     if (any_gemm)
         if ((e = cudaFuncSetAttribute(xk::fc_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(fc)", e);
@@ -605,6 +635,46 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
                 if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
                 break;
             }
+            if (L.seg[0].mode == AM_DW) {
+                const ASeg &a = L.seg[0];
+                xk::DwParams p;
+                std::memset(&p, 0, sizeof p);
+                p.dw_w = (const float *)(ws + a.dw_w_off); p.dw_b = (const float *)(ws + a.dw_b_off); p.bias = (const float *)(ws + L.b_off);
+                p.out = ptr(L.out); p.status = status;
+                p.d_nt = xk::make_fastdiv((uint32_t)L.n_tiles); p.d_ks = xk::make_fastdiv((uint32_t)L.ksplit);
+                p.d_tx = xk::make_fastdiv((uint32_t)L.tiles_x); p.d_ty = xk::make_fastdiv((uint32_t)L.tiles_y);
+                p.batch = N; p.P = L.P; p.Q = L.Q; p.C = a.C; p.stride = a.stride; p.pad = a.pad; p.dw_act = a.dw_act;
+                p.ni = L.ni; p.rh = L.patch_rh; p.rw = L.patch_rw; p.tile_rows = L.tile_rows;
+                p.total = (N + L.ni - 1) / L.ni * L.tiles_y * L.tiles_x * L.n_tiles * L.ksplit;
+                p.kblocks = L.kblocks; p.last_steps = (a.C - 64 * (L.kblocks - 1) + 15) / 16; p.tile_n = L.tile_n; p.n_acc = L.n_acc; p.N = L.K;
+                p.kb_per = L.ksplit > 1 ? L.kb_per : L.kblocks;
+                p.groups = L.dw_groups; p.wpg_log2 = L.dw_wpg_log2; p.pairs = L.halo_cb > 32 ? 32 : 16;
+                p.batch_tiles = L.dw_batch; p.n_bufs = L.n_acc == 2 ? 1 : 2 * L.dw_batch;
+                p.a_slots = L.a_slots; p.b_slots = L.b_slots; p.h_slots = L.h_slots; p.b_resident = L.b_resident;
+                p.halo_bytes = L.halo_bytes; p.halo_stride = L.halo_stride; p.halo_h = L.halo_h; p.halo_w = L.halo_w; p.halo_cb = L.halo_cb;
+                p.acc_stride = L.acc_stride; p.tmem_cols = L.tmem_cols;
+                p.chunk = L.chunk; p.nchunks = L.nchunks; p.box_bytes = 128 * L.chunk * 2; p.out_bufs = L.out_bufs;
+                p.act = L.act; p.out_ctot = L.out_ctot; p.out_f32 = L.out_dtype == XENOS_DTYPE_F32;
+                p.idesc = make_idesc(L.tile_n);
+                p.off_b = L.off_b; p.off_halo = L.off_halo; p.off_dww = L.off_dww; p.off_stage = L.off_stg; p.off_bias = L.off_bias; p.off_bar = L.off_bar;
+                p.gap_imgs = L.gap_imgs; p.gap_area = L.gap_area; p.gap_rpi = L.gap_rpi;
+                p.ksplit = L.ksplit; p.split_ld = L.npad; p.split_stride = (long long)N * L.rows_per_image * L.npad;
+                p.split_part = reinterpret_cast<float *>(ws + g.split_off); p.split_cnt = reinterpret_cast<unsigned int *>(ws + L.split_cnt_off);
+                p.launch_id = (int)li;
+                const ConvMaps *maps = &rt->conv[li];
+                ConvMaps now;
+                if (conv_has_external(g, L)) {
+                    now = *maps;
+                    xenos_status_t st = encode_dw_maps(g, rt, L, ptr, N, true, &now);
+                    if (st != XENOS_OK) return st;
+                    maps = &now;
+                }
+                const int limit = L.b_resident ? std::max(1, sms / L.n_tiles) * L.n_tiles : sms;
+                auto *k = dw_kernel(L.cv_epi, a.stride, L.dw_br);
+                cudaError_t le = launch_pdl(k, std::min(p.total, limit), L.block, L.smem_bytes, stream, maps->a0, rt->tmaps[li], maps->o, p);
+                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+                break;
+            }
             xk::GemmParams p;
             std::memset(&p, 0, sizeof p);
             for (int s = 0; s < 2; ++s) {
@@ -655,25 +725,9 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
                     tmh = &tmh_now;
                 }
             }
-            if (L.seg[0].mode == AM_DW) {
-                const Tensor &hx = g.tensors[L.seg[0].tensor];
-                if (hx.input_slot >= 0) {
-                    xenos_status_t st = encode_halo_map(g, rt, L, ptr(L.seg[0].tensor), N, &tmh_now);
-                    if (st != XENOS_OK) return st;
-                    tmh = &tmh_now;
-                } else {
-                    tmh = &rt->hmaps[li];
-                }
-            }
-            const int grid = std::min(p.m_tiles * p.n_tiles, sms);
-            // Programmatic dependent launch: the kernel may be scheduled while its predecessor in the
-            // stream drains, runs its set-up (barriers, tensor memory, constant staging) and then
-            // waits (griddepcontrol.wait) before it touches any activation.
-            const int lgrid = (int)grid, lblock = (int)L.block;
+            const int lgrid = std::min(p.m_tiles * p.n_tiles, sms), lblock = L.block;
             cudaError_t le;
-            if (L.dw_workers == 16) le = launch_pdl(xk::dwpw_kernel<16>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
-            else if (L.dw_workers == 8) le = launch_pdl(xk::dwpw_kernel<8>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
-            else if (L.ksplit > 1 || L.gap_parts > 1) le = launch_pdl(xk::gemm_chain_kernel<1>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
+            if (L.ksplit > 1 || L.gap_parts > 1) le = launch_pdl(xk::gemm_chain_kernel<1>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
             else le = launch_pdl(xk::gemm_chain_kernel<0>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
             if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
