@@ -26,7 +26,23 @@ namespace xenos {
 
 struct ConvMaps { CUtensorMap a0, a1, o, s; };      // operand segments, result, shortcut of a conv_tc_kernel launch
 
+// One recorded pass: the launches of a graph for one batch size and one set of caller buffers, replayed as a CUDA graph.
+struct Replay {
+    std::vector<const void *> key;      // batch, inputs, outputs
+    cudaGraphExec_t exec = nullptr;     // null: seen once, not recorded
+    uint64_t used = 0;
+};
+constexpr size_t kReplays = 8;          // passes remembered per binding; the least recently used one makes room
+
 struct Runtime {
+    std::vector<Replay> replays;
+    cudaStream_t record_stream = nullptr;      // records replays (never runs anything)
+    uint64_t tick = 0;
+    bool replay_ok = true;              // cleared when recording fails: passes are then launched one kernel at a time
+    ~Runtime() {
+        for (Replay &r : replays) if (r.exec) cudaGraphExecDestroy(r.exec);
+        if (record_stream) cudaStreamDestroy(record_stream);
+    }
     int device = -1;
     int sm_count = 0;
     std::vector<CUtensorMap> tmaps;     // one per launch record (used by gemm launches only)
@@ -381,8 +397,8 @@ static int ew_grid(long long total, int block, int sms) {
     return (int)b;
 }
 
-xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *const *out, void *stream_v,
-                           float *ms_per_launch) {
+static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, void *const *out, void *stream_v,
+                                  float *ms_per_launch) {
     Runtime *rt = static_cast<Runtime *>(g.rt);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
     uint8_t *ws = static_cast<uint8_t *>(g.ws);
@@ -751,6 +767,64 @@ xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *con
     return XENOS_OK;
 }
 
+// A pass of several launches that comes again with the same batch and buffers is recorded on its second call and from then
+// on replayed as one CUDA graph (programmatic dependencies between the kernels included).  Single launches cost the host 2.3
+// to 4.5 us each, more than many of these kernels run on a small batch; a replay costs one call.  Passes whose buffers
+// change from call to call, passes inside a caller's own stream capture and single launches go to the stream directly (a
+// graph of one kernel takes 2.5 us longer than the kernel).
+xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *const *out, void *stream_v, float *ms_per_launch) {
+    Runtime *rt = static_cast<Runtime *>(g.rt);
+    cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
+    if (ms_per_launch || !rt->replay_ok || g.launches.size() < 2) return launch_pass(g, batch, in, out, stream_v, ms_per_launch);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return launch_pass(g, batch, in, out, stream_v, nullptr);
+    }
+    const size_t ni = g.inputs.size(), no = g.outputs.size();
+    auto same = [&](const Replay &r) {
+        if (r.key[0] != (const void *)(uintptr_t)batch) return false;
+        for (size_t i = 0; i < ni; ++i) if (r.key[1 + i] != in[i]) return false;
+        for (size_t i = 0; i < no; ++i) if (r.key[1 + ni + i] != out[i]) return false;
+        return true;
+    };
+    Replay *hit = nullptr;
+    for (Replay &r : rt->replays) if (same(r)) { hit = &r; break; }
+    if (!hit) {
+        // first call with these buffers: remember it (in the slot of the least recently used pass), launch directly
+        if (rt->replays.size() < kReplays) rt->replays.emplace_back();
+        hit = &rt->replays[0];
+        for (Replay &r : rt->replays) if (r.used < hit->used) hit = &r;
+        if (hit->exec) { cudaGraphExecDestroy(hit->exec); hit->exec = nullptr; }
+        hit->key.assign(1, (const void *)(uintptr_t)batch);
+        hit->key.insert(hit->key.end(), in, in + ni);
+        for (size_t i = 0; i < no; ++i) hit->key.push_back(out[i]);
+        hit->used = ++rt->tick;
+        return launch_pass(g, batch, in, out, stream_v, nullptr);
+    }
+    hit->used = ++rt->tick;
+    if (!hit->exec) {
+        cudaGraph_t graph = nullptr;
+        bool good = rt->record_stream || cudaStreamCreateWithFlags(&rt->record_stream, cudaStreamNonBlocking) == cudaSuccess;
+        good = good && cudaStreamBeginCapture(rt->record_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+        if (good) {
+            const xenos_status_t st = launch_pass(g, batch, in, out, rt->record_stream, nullptr);
+            good = cudaStreamEndCapture(rt->record_stream, &graph) == cudaSuccess && st == XENOS_OK && graph;
+            good = good && cudaGraphInstantiate(&hit->exec, graph, 0) == cudaSuccess;
+            if (graph) cudaGraphDestroy(graph);
+        }
+        if (!good) {
+            cudaGetLastError();
+            hit->exec = nullptr;
+            rt->replay_ok = false;
+            return launch_pass(g, batch, in, out, stream_v, nullptr);
+        }
+    }
+    const cudaError_t e = cudaGraphLaunch(hit->exec, stream);
+    if (e != cudaSuccess) return cuda_fail(g, "kernel launch", e);
+    return XENOS_OK;
+}
+
 xenos_status_t runtime_status(Graph &g, void *stream_v) {
     cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
     cudaError_t e = cudaStreamSynchronize(stream);
@@ -837,7 +911,7 @@ xenos_status_t runtime_run_builtin(Graph &g, int batch, const void *const *in, v
         if ((e = cudaMemsetAsync(static_cast<uint8_t *>(scratch) + g.status_off, 0, 256 + g.cnt_bytes, stream)) != cudaSuccess)
             st = cuda_fail(g, "status clear", e);
     }
-    if (st == XENOS_OK) st = runtime_run(g, batch, in, out, stream, nullptr);
+    if (st == XENOS_OK) st = launch_pass(g, batch, in, out, stream, nullptr);      // (never recorded: that would allocate)
     if (st == XENOS_OK) st = runtime_status(g, stream);
     return st;
 }
