@@ -33,7 +33,8 @@ namespace xk {
 constexpr int kCvEpiWarps = 8;
 constexpr int kCvThreads = 128 + 32 * kCvEpiWarps;
 constexpr int kCvMaxStages = 6;
-enum { CE_STORE = 0, CE_SKIP = 1, CE_VEC = 2, CE_GAP = 3, CE_SPLIT = 4 };
+enum { CE_STORE = 0, CE_SKIP = 1, CE_VEC = 2, CE_GAP = 3, CE_SPLIT = 4, CE_CLUSTER = 5 };
+constexpr int kCvMaxCluster = 8;
 
 // Exact division of n < 2^31 by a constant of the launch.
 struct FastDiv {
@@ -540,8 +541,82 @@ __device__ __forceinline__ bool conv_epilogue_split(const ConvParams &g, uint8_t
     return true;
 }
 
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t saddr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Reduction split over a thread-block cluster: the chunks of a tile are the CTAs of one cluster (rank = chunk).  Each CTA owns
+// an equal share of the tile's rows; every CTA sends its fp32 partial sums of a row to the row's owner through distributed
+// shared memory, and the owner adds the chunks in ascending order and stores.  The exchange buffer is [chunk][row of the
+// share][tile_n + 4] (the 4 words of padding spread a warp's rows over the banks); "arrived" counts the warps of all CTAs.
+// Measured for 8 chunks of 256 -> 256 channels, 14 x 14, batch 1: see the design doc's table; through global memory and
+// counters the exchange took 5 us (fence 0.7, partial sums 0.5, counter 0.9, reads and stores 2.7), as much as the product.
+__device__ __forceinline__ bool conv_epilogue_cluster(const ConvParams &g, uint8_t *sm, uint32_t bar, uint32_t tmem_base, uint32_t arrived) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, e = warp - 4, quarter = warp & 3, half = e >> 2;
+    const int row = quarter * 32 + lane, et = threadIdx.x - 128;
+    const uint32_t sbase = smem_u32(sm), bias_s = sbase + g.off_bias, buf = sbase + g.off_stage;
+    const ConvTile t = conv_tile(g, blockIdx.x);
+    const int n0 = t.nt * g.tile_n, m0 = t.mt * g.tile_rows;
+    const int live = min(kTileM, g.rows - m0), per = (live + g.ksplit - 1) / g.ksplit;
+    const uint32_t pitch = (uint32_t)(g.tile_n + 4) * 4u;
+    const bool ok = mbar_wait(bar + 8u * (2 * kCvMaxStages), 0u);
+    if (ok) {
+        tc_fence_after();
+        const int owner = row / per;
+        const uint32_t dst = cluster_addr(buf, (uint32_t)min(owner, g.ksplit - 1)) + (uint32_t)(t.ks * per + row - owner * per) * pitch;
+#pragma unroll 1
+        for (int j = half; j < g.nchunks; j += 2) {
+            float v[16];
+            tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + j * 16, v);
+            if (row < live)
+#pragma unroll
+                for (int q4 = 0; q4 < 16; q4 += 4)
+                    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(j * 16 + q4) * 4u), "f"(v[q4]), "f"(v[q4 + 1]),
+                                 "f"(v[q4 + 2]), "f"(v[q4 + 3]) : "memory");
+        }
+        tc_fence_before();
+    }
+    __syncwarp();
+    // one arrival per warp at every owner (also after a wait that gave up: nobody waits in vain for this CTA)
+    if (lane < g.ksplit)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr(arrived, (uint32_t)lane)) : "memory");
+    if (!ok) return false;
+    const int r0 = t.ks * per, mine = min(per, live - r0), c4n = g.tile_n >> 2;
+    bool seen = false;
+#pragma unroll 1
+    for (int i = 0; i < kSpinLimit && !seen; ++i) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0, %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done) : "r"(arrived), "r"(kSuspendHintNs) : "memory");
+        seen = done != 0;
+    }
+    if (!seen) return false;
+#pragma unroll 1
+    for (int idx = et; idx < mine * c4n; idx += 32 * kCvEpiWarps) {
+        const int rr = idx / c4n, c4 = idx - rr * c4n, nc = n0 + c4 * 4;
+        if (nc >= g.N) continue;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int s = 0; s < g.ksplit; ++s) {
+            const float4 x = ld_shared_f4(buf + (uint32_t)(s * per + rr) * pitch + (uint32_t)c4 * 16u);
+            a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+        }
+        conv_finish_store4(g, a, ld_shared_f4(bias_s + (uint32_t)nc * 4u), nc, (size_t)(m0 + r0 + rr));
+    }
+    return true;
+}
+
 template <int kEpi>
-__global__ void __launch_bounds__(kCvThreads, 1)
+__global__ void __launch_bounds__(kCvThreads, kEpi == CE_GAP ? 1 : 2)
 conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmS, const __grid_constant__ ConvParams g) {
     extern __shared__ uint8_t smem_raw[];
@@ -556,6 +631,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     auto acce_bar = [&](int b) { return bar + 8u * (2 * kCvMaxStages + 2 + b); };
     auto bres_bar = [&](int q) { return bar + 8u * (2 * kCvMaxStages + 4 + q); };                       // 4
     auto skip_bar = [&](int e, int b) { return bar + 8u * (2 * kCvMaxStages + 8 + 2 * e + b); };       // 16
+    const uint32_t arrived = skip_bar(0, 0);      // (a split has no shortcut boxes)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + g.off_bar + 8 * (2 * kCvMaxStages + 24));
     volatile int *fail_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);      // [0] give-up, [1], [2] agreement of a split / average
 
@@ -565,6 +641,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
         for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), kCvEpiWarps); }
         for (int q = 0; q < 4; ++q) mbar_init(bres_bar(q), 1);
         if (kEpi == CE_SKIP) for (int e = 0; e < 2 * kCvEpiWarps; ++e) mbar_init(skip_bar(0, e), 1);
+        if (kEpi == CE_CLUSTER) mbar_init(arrived, kCvEpiWarps * g.ksplit);
         fail_flag[0] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA0) : "memory");
@@ -580,6 +657,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     }
     tc_fence_before();
     __syncthreads();
+    if (kEpi == CE_CLUSTER) cluster_sync();      // every CTA's "arrived" barrier exists
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     bool ok = true;
@@ -759,12 +837,15 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                 warp_arrive(acce_bar(b), lane);
             }
         } else {
-            ok = kEpi == CE_GAP ? conv_epilogue_gap(g, sm, bar, tmem_base, fail_flag) : conv_epilogue_split(g, sm, bar, tmem_base, fail_flag);
+            ok = kEpi == CE_GAP ? conv_epilogue_gap(g, sm, bar, tmem_base, fail_flag)
+               : kEpi == CE_CLUSTER ? conv_epilogue_cluster(g, sm, bar, tmem_base, arrived)
+               : conv_epilogue_split(g, sm, bar, tmem_base, fail_flag);
         }
         if (!ok && lane == 0) atomicCAS(g.status, 0u, gave_up | (5u << 8));
     }
     tc_fence_before();
     __syncthreads();
+    if (kEpi == CE_CLUSTER) cluster_sync();      // (no CTA leaves while another may still write to its shared memory)
     if (warp == 3) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)g.tmem_cols) : "memory");

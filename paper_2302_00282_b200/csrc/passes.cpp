@@ -702,18 +702,27 @@ struct Lower {
     // the slower of the tensor pipe (max(48, tile_n / 2) cycles per K = 16 step) and the operand traffic from L2 (75
     // bytes per cycle and SM); a tile's epilogue overlaps the next tile's product; a split adds the exchange of the partial
     // sums.  The constants are measurements on B200 (see conv_tc.cuh).
-    double conv_cycles(const Launch &L, int tile_n, int n_tiles, int ksplit) const {
+    // Clusters of ks CTAs that fit the device at once, one CTA or two (half) per SM (queried on B200; clusters stay inside a
+    // GPC, so the larger ones leave SMs unused).
+    static int cluster_capacity(int ks, bool half) {
+        static const int one[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15}, two[9] = {0, 296, 148, 93, 71, 56, 45, 37, 33};
+        return half ? two[ks] : one[ks];
+    }
+    static int conv_smem_cap(bool half) { return half ? kClusterSmem : 227 * 1024; }
+    static constexpr int kClusterSmem = 112 * 1024;      // what two CTAs of an SM can have each
+    // Exchange buffer of a cluster's partial sums.
+    static int cluster_bytes(int rows, int tile_n, int ks) { return (int)align_up((size_t)ks * ceil_div(rows, ks) * (tile_n + 4) * 4, 1024); }
+    double conv_cycles(const Launch &L, int tile_n, int n_tiles, int ksplit, bool half) const {
         const double units = g.hw.sm_count;
-        const double tiles = (double)L.m_tiles * n_tiles * ksplit;
-        const double waves = std::ceil(tiles / units);
+        const double tiles = (double)L.m_tiles * n_tiles;
         const int kb = ceil_div(L.kblocks, ksplit);
         const double mma = 4.0 * std::max(48.0, tile_n / 2.0);
         const double load = (L.a_rows * 128.0 + tile_n * 128.0) / 75.0;
-        const double main = kb * std::max(mma, std::max(load, 150.0));
+        const double main = kb * std::max(mma, std::max(load, 300.0));
         const double epi = 400.0 + 5.0 * tile_n;
-        double t = waves * std::max(main, epi) + std::min(main, epi);
-        if (ksplit > 1) t += 2600.0 + L.a_rows * tile_n * 8.0 / 40.0;
-        return t;
+        if (ksplit == 1) return std::ceil(tiles / units) * std::max(main, epi) + std::min(main, epi);
+        const double shared = std::max(1.0, tiles * ksplit / units);      // CTAs of one SM share its pipes
+        return std::ceil(tiles / cluster_capacity(ksplit, half)) * (main * (half ? std::min(2.0, shared) : 1.0) + epi) + 1700.0 + L.a_rows * tile_n / 32.0;
     }
     // Widths are the equal cuts of the output channels (Section 4.2.1) down to 32 columns; the reduction is cut (Section
     // 4.2.2) only where that is modelled to be faster, into chunks of at least two K blocks that run at the same time.
@@ -725,20 +734,30 @@ struct Lower {
             const int tn = round_up(ceil_div(N16, nt), 16);
             if ((nt - 1) * tn >= N16) continue;                    // an empty last tile
             if (tn < 32 && nt > ceil_div(N16, 256)) break;
-            for (int ks : {1, 2, 3, 4, 6, 8, 12, 16}) {
-                if (ks > 1 && (!can_split || L.kblocks < 2 * ks || (long)L.m_tiles * nt * ks > g.hw.sm_count)) break;
-                const int per = ceil_div(L.kblocks, ks);
-                if (ks > 1 && ceil_div(L.kblocks, per) != ks) continue;
-                // (a fully connected layer of few rows is a pass over its weights: it always spreads over the units)
-                const double c = conv_cycles(L, tn, nt, ks) + (fc && ks == 1 && L.m_tiles == 1 && L.kblocks >= 4 ? 1e6 : 0);
-                if (best < 0 || c < best) { best = c; L.n_tiles = nt; L.tile_n = tn; ksplit = ks; }
-            }
+            for (int ks = 1; ks <= 8; ++ks)
+                for (int half = 0; half < 2; ++half) {
+                    const int per = ceil_div(L.kblocks, ks);
+                    if (ks == 1 && half) continue;
+                    if (ks > 1) {
+                        if (!can_split || L.kblocks < 2 * ks || ceil_div(L.kblocks, per) != ks) continue;
+                        const int ring = conv_smem_cap(half) - 1536 - (int)align_up((size_t)nt * tn * 4, 128) - cluster_bytes(L.a_rows, tn, ks);
+                        if (ring < std::min(4, std::max(3, per)) * (16384 + tn * 128)) continue;
+                        if ((long)L.m_tiles * nt > cluster_capacity(ks, half) || (fc && (long)L.m_tiles * nt * ks > g.hw.sm_count)) continue;
+                    }
+                    // (a fully connected layer of few rows is a pass over its weights: it always spreads over the units)
+                    const double c = conv_cycles(L, tn, nt, ks, half) + (fc && ks == 1 && L.m_tiles == 1 && L.kblocks >= 4 ? 1e6 : 0);
+                    if (best < 0 || c < best) { best = c; L.n_tiles = nt; L.tile_n = tn; ksplit = ks; L.half = half; }
+                }
         }
     }
     // Shared memory and epilogue shape of conv_tc_kernel.
     xenos_status_t layout_conv(Launch &L, const Tensor &ot) {
         const bool vec = L.out_dtype == XENOS_DTYPE_F32 || ot.c % 8;
-        L.cv_epi = L.epi == EPI_GAP ? 3 : L.ksplit > 1 ? 4 : vec ? 2 : L.skip >= 0 ? 1 : 0;
+        // (up to eight chunks are the CTAs of a cluster while the exchange buffer leaves room for the ring; other splits go
+        // through the workspace)
+        const int xbytes = cluster_bytes(std::min(128, g.max_batch * L.rows_per_image), L.tile_n, L.ksplit);
+        const bool cluster = L.ksplit > 1 && L.ksplit <= 8 && xbytes + 3 * (16384 + L.tile_n * 128) + L.npad * 4 + 2048 <= conv_smem_cap(L.half);
+        L.cv_epi = L.epi == EPI_GAP ? 3 : cluster ? 5 : L.ksplit > 1 ? 4 : vec ? 2 : L.skip >= 0 ? 1 : 0;
         if (L.cv_epi == 2 && L.skip >= 0) return fail(g, XENOS_E_UNSUPPORTED, "internal: shortcut on a vector result");
         int stg = 0;
         L.chunk = 16;
@@ -748,6 +767,8 @@ struct Lower {
             for (int c : {64, 32, 16})
                 if (L.tile_n % c == 0 && (L.tile_n / c) % 2 == 0 && !(c == 64 && L.tile_n > 160)) { L.chunk = c; break; }
             stg = 16 * L.chunk * 64;                 // two 32-row boxes for each of eight warps
+        } else if (L.cv_epi == 5) {
+            stg = xbytes;
         } else if (L.cv_epi == 3) {
             L.chunk = 32;
             stg = 2 * (128 * 33 + 128) * 4;
@@ -755,7 +776,10 @@ struct Lower {
         L.nchunks = ceil_div(L.tile_n, L.chunk);
         stg = (int)align_up((size_t)stg, 1024);
         const int bias = (int)align_up((size_t)L.npad * 4, 128);
-        const int room = std::min(g.hw.smem_bytes_per_cta, 227 * 1024) - 1024 - 512 - bias - stg;
+        // (a CTA with one tile takes half an SM when four stages fit there: the next kernel's CTAs can then set up beside it)
+        const bool half = (L.cv_epi == 5 && L.half) || (L.ksplit == 1 && (long)L.m_tiles * L.n_tiles <= g.hw.sm_count &&
+                                                        kClusterSmem - 1536 - bias - stg >= std::min(4, std::max(2, L.kblocks)) * (16384 + L.tile_n * 128));
+        const int room = std::min(g.hw.smem_bytes_per_cta, half ? kClusterSmem : 227 * 1024) - 1024 - 512 - bias - stg;
         const int bbytes = L.kblocks * L.tile_n * 128;
         // weights stay in shared memory when a CTA meets more than one tile of its channel tile and four operand stages
         // still fit beside them
@@ -1538,7 +1562,7 @@ xenos_status_t plan_workspace(Graph &g) {
     // arrival counters of the reduction-split launches sit behind the status words and are cleared with them
     g.cnt_bytes = 0; g.split_bytes = 0;
     for (Launch &L : g.launches)
-        if (L.kind == LK_GEMM && L.ksplit > 1) {
+        if (L.kind == LK_GEMM && L.ksplit > 1 && !(L.conv_tc && L.cv_epi == 5)) {
             L.split_cnt_off = off + g.cnt_bytes;
             g.cnt_bytes += align_up((size_t)L.m_tiles * L.n_tiles * 8, 16);      // [arrived, reduced] per tile
             g.split_bytes = std::max(g.split_bytes, (size_t)L.ksplit * g.max_batch * L.rows_per_image * L.npad * 4);

@@ -348,6 +348,7 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
             (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_SKIP>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_GAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(conv)", e);
     if (any_gemm)
@@ -378,15 +379,21 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
 // Programmatic dependent launch: the kernel may be scheduled while its predecessor in the stream drains, runs its set-up
 // and then waits (griddepcontrol.wait) before it touches the predecessor's results.
 template <class... P, class... A>
-static cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t stream, A &&...args) {
+static cudaError_t launch_pdl_cluster(void (*kernel)(P...), int grid, int block, int smem, int cluster, cudaStream_t stream, A &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = stream;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+template <class... P, class... A>
+static cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t stream, A &&...args) {
+    return launch_pdl_cluster(kernel, grid, block, smem, 1, stream, std::forward<A>(args)...);
 }
 
 static int ew_grid(long long total, int block, int sms) {
@@ -646,8 +653,8 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 const int lgrid = (int)std::min(p.total, limit), lblock = (int)xk::kCvThreads;
                 auto *k = L.cv_epi == xk::CE_STORE ? xk::conv_tc_kernel<xk::CE_STORE> : L.cv_epi == xk::CE_SKIP ? xk::conv_tc_kernel<xk::CE_SKIP>
                         : L.cv_epi == xk::CE_VEC ? xk::conv_tc_kernel<xk::CE_VEC> : L.cv_epi == xk::CE_GAP ? xk::conv_tc_kernel<xk::CE_GAP>
-                        : xk::conv_tc_kernel<xk::CE_SPLIT>;
-                cudaError_t le = launch_pdl(k, lgrid, lblock, L.smem_bytes, stream, maps->a0, maps->a1, rt->tmaps[li], maps->o, maps->s, p);
+                        : L.cv_epi == xk::CE_CLUSTER ? xk::conv_tc_kernel<xk::CE_CLUSTER> : xk::conv_tc_kernel<xk::CE_SPLIT>;
+                cudaError_t le = launch_pdl_cluster(k, L.cv_epi == xk::CE_CLUSTER ? p.total : lgrid, lblock, L.smem_bytes, L.cv_epi == xk::CE_CLUSTER ? L.ksplit : 1, stream, maps->a0, maps->a1, rt->tmaps[li], maps->o, maps->s, p);
                 if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
                 break;
             }
