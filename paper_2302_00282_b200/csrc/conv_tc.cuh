@@ -555,8 +555,8 @@ __device__ __forceinline__ void cluster_sync() {
 // an equal share of the tile's rows; every CTA sends its fp32 partial sums of a row to the row's owner through distributed
 // shared memory, and the owner adds the chunks in ascending order and stores.  The exchange buffer is [chunk][row of the
 // share][tile_n + 4] (the 4 words of padding spread a warp's rows over the banks); "arrived" counts the warps of all CTAs.
-// Measured for 8 chunks of 256 -> 256 channels, 14 x 14, batch 1: see the design doc's table; through global memory and
-// counters the exchange took 5 us (fence 0.7, partial sums 0.5, counter 0.9, reads and stores 2.7), as much as the product.
+// Measured at batch 1: through global memory and counters the exchange took 5 us (fence 0.7, partial sums 0.5, counter 0.9,
+// reads and stores 2.7), as much as the product; the 12 split launches of a batch-1 ResNet-18 gave back 16 of 131 us.
 __device__ __forceinline__ bool conv_epilogue_cluster(const ConvParams &g, uint8_t *sm, uint32_t bar, uint32_t tmem_base, uint32_t arrived) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, e = warp - 4, quarter = warp & 3, half = e >> 2;
     const int row = quarter * 32 + lane, et = threadIdx.x - 128;

@@ -145,6 +145,9 @@ struct Launch {
     int dw_groups = 0, dw_wpg_log2 = 0, dw_br = 1, dw_batch = 1, h_slots = 0, out_bufs = 1;      // ... their groups, a thread's block rows, halo slots, result boxes
     // convolution, product or fc in conv_tc_kernel: its epilogue kind, rows of an operand box, resident weights, column chunks
     int conv_tc = 0, half = 0, cv_epi = 0, a_rows = 128, b_resident = 0, b_group = 0, chunk = 0, nchunks = 0, off_b = 0;
+    // convolution of the image in stem_tc_kernel: elements a piece starts before its window, aligned loads, column blocks and
+    // their width in output columns, row slots, steps in flight, pieces per (slot, channel), staged pixel, chunk pairs
+    int stem_tc = 0, st_lead = 0, st_vec = 0, st_cbs = 1, st_cw = 0, st_slots = 0, st_qp = 0, st_pc = 0, st_pairs = 0;
     int n_acc = 1;                                                 // dw_tc_kernel: channel tiles of tile_n columns per CTA (2: both accumulators hold one tile)
     int pair = 0, a_slots = 0, b_slots = 0, off_b2 = 0;            // LK_GEMM2 with a 1x1 consumer: pair_tc_kernel and its rings
     // ---- two linked convolutions (LK_GEMM2): producer tile rh1 x rw1 = patch_rh x patch_rw, consumer tile rh2 x rw2

@@ -751,6 +751,93 @@ struct Lower {
         }
     }
     // Shared memory and epilogue shape of conv_tc_kernel.
+    // Convolution of an NCHW image in stem_tc_kernel: false when the shape is outside it (1 x 1 windows, more than 7 channels, a
+    // pool whose windows overlap by more than one row, rows too wide for the ring).
+    bool layout_stem(Launch &L, const Node &M, const Tensor &src, const Node *pooln, int N, const SplitRequest &rq) {
+        const int C = src.c, k = M.k, S = M.stride;
+        if (k < 2 || k > 8 || C > 7 || (rq.user && (rq.h > 1 || rq.w > 1 || rq.k > 1))) return false;
+        if (pooln && (pooln->k - pooln->stride > 1 || pooln->pad > pooln->stride || pooln->pad >= pooln->k)) return false;
+        L.n_tiles = rq.user && rq.outc > 0 ? rq.outc : ceil_div(N, 64);
+        L.tile_n = round_up(ceil_div(N, L.n_tiles), 16);
+        if (L.tile_n > 64 || (L.n_tiles - 1) * L.tile_n >= N) return false;
+        L.npad = L.n_tiles * L.tile_n;
+        // A piece may start before its window (the extra elements meet zero weights) where that makes the loads of two
+        // adjacent columns of a stride-2 window whole aligned groups of 4 elements; rows must then be multiples of a group, too.
+        L.st_lead = 0; L.st_vec = 0;
+        if (S == 2) {
+            const int lead = (4 - M.pad % 4) % 4;
+            if (k + lead <= 8) { L.st_lead = lead; L.st_vec = src.w % 4 == 0 ? 1 : 0; }
+        }
+        const int rows = pooln ? L.PP : L.P, cols = pooln ? L.PQ : L.Q;
+        L.st_pairs = k / 2 * C + (k % 2 ? (C + 1) / 2 : 0);
+        const int wbytes = L.st_pairs * 2 * L.tile_n * 16, pc = L.tile_n <= 16 ? 1 : L.tile_n <= 32 ? 2 : 3;
+        const int cap = std::min(g.hw.smem_bytes_per_cta, 227 * 1024) - 1024 - 512;
+        // (a producer warp makes at most 128 lanes' worth of a row: two columns each, or one for strides above 2)
+        const int most = S <= 2 ? 256 : 128;
+        auto fit = [&](int cbs) {
+            L.st_cbs = cbs;
+            L.st_cw = round_up(ceil_div(cols, cbs), 2);
+            // (columns of the convolution behind a block of the pool's columns; their first is rounded down to an even one)
+            const int width = std::min(L.Q, pooln ? (L.st_cw - 1) * pooln->stride + pooln->k + 1 : L.st_cw);
+            if (width > most) return false;
+            L.st_qp = round_up(width, 8);
+            const int row = C * L.st_qp * 16, stage = pooln ? 2 * width << (4 + pc) : 0;
+            const int base = wbytes + 2048 + 256 + (int)align_up((size_t)stage, 128);
+            for (int D = 6; D >= 2; --D) {
+                L.st_slots = (D - 1) * std::min(S, k) + k;
+                if ((L.st_slots + 1) * row + base > cap) continue;
+                L.hstages = D;
+                L.off_b = (int)align_up((size_t)(L.st_slots + 1) * row + 2048, 128);       // (a tile's last rows read past its pieces)
+                L.off_bias = L.off_b + wbytes;
+                L.off_stg = L.off_bias + 256;
+                L.off_bar = (int)align_up((size_t)(L.off_stg + stage), 128);
+                L.smem_bytes = L.off_bar + 512 + 1024;
+                return true;
+            }
+            return false;
+        };
+        int cbs = ceil_div(cols, most);
+        while (!fit(cbs)) {
+            if (ceil_div(cols, cbs) <= 8) return false;
+            ++cbs;
+        }
+        // few images: columns are cut until the rows of all blocks cover the units (a block of at least 32 columns)
+        while ((long)g.max_batch * rows * cbs * L.n_tiles * 2 <= g.hw.sm_count && ceil_div(L.Q, cbs * 2) >= 32 && fit(cbs * 2)) cbs *= 2;
+        if (!fit(cbs)) return false;
+        L.st_cbs = ceil_div(cols, L.st_cw);
+        L.stem_tc = 1; L.st_pc = pc;
+        L.m_tiles = pooln ? g.max_batch * L.tiles_y * L.tiles_x : g.max_batch * L.P * L.st_cbs * ceil_div(L.st_qp, 128);
+        L.stages = L.hstages;
+        L.grid = (int)std::min<long>((long)g.max_batch * rows * L.st_cbs, std::max(1, g.hw.sm_count / L.n_tiles)) * L.n_tiles;
+        L.block = 512;
+        L.acc_stride = L.tile_n <= 32 ? 32 : 64;
+        L.tmem_cols = 4 * L.acc_stride;
+        return true;
+    }
+    // Weights in the order of its products: [channel tile][pair][two chunks][output channel][8 elements of a window row].
+    void pack_stem(Launch &L, const Node &M, int C) {
+        const int k = M.k;
+        L.w_off = blob_reserve(g, (size_t)L.n_tiles * L.st_pairs * 2 * L.tile_n * 16);
+        L.b_off = blob_reserve(g, (size_t)L.npad * 4);
+        uint16_t *wp = reinterpret_cast<uint16_t *>(g.param_blob.data() + L.w_off);
+        float *bp = reinterpret_cast<float *>(g.param_blob.data() + L.b_off);
+        auto chunk = [&](int pair, int half, int c, int r) {
+            for (int o = 0; o < M.cout; ++o) {
+                const int nt = o / L.tile_n, n = o - nt * L.tile_n;
+                uint16_t *d = wp + ((((size_t)nt * L.st_pairs + pair) * 2 + half) * L.tile_n + n) * 8 + L.st_lead;
+                for (int s = 0; s < k; ++s) d[s] = f32_to_bf16_rne(M.w[(((size_t)o * C + c) * k + r) * k + s]);
+            }
+        };
+        int pair = 0;
+        for (int r = 0; r + 1 < k; r += 2)
+            for (int c = 0; c < C; ++c, ++pair) { chunk(pair, 0, c, r); chunk(pair, 1, c, r + 1); }
+        if (k % 2) {
+            for (int c = 0; c + 1 < C; c += 2, ++pair) { chunk(pair, 0, c, k - 1); chunk(pair, 1, c + 1, k - 1); }
+            if (C % 2) chunk(pair, 1, C - 1, k - 1);
+        }
+        for (int o = 0; o < M.cout; ++o) bp[o] = M.b[o];
+    }
+
     xenos_status_t layout_conv(Launch &L, const Tensor &ot) {
         const bool vec = L.out_dtype == XENOS_DTYPE_F32 || ot.c % 8;
         // (up to eight chunks are the CTAs of a cluster while the exchange buffer leaves room for the ring; other splits go
@@ -1002,6 +1089,15 @@ struct Lower {
             // The stem stages the tile's input patch in shared memory, so its tile is a patch too:
             // the pool patch when a pool is linked, else th x tw output pixels with the fewest tiles.
             if (gapn) return fail(g, XENOS_E_UNSUPPORTED, "a convolution on an NCHW image cannot be linked with a global average");
+            if (!addn && !catn && last->out >= 0 && !g.tensors[last->out].is_vec && g.tensors[last->out].c % 8 == 0 && layout_stem(L, M, src, pooln, N, ch.split)) {
+                L.out = last->out;
+                L.out_ctot = g.tensors[L.out].c; L.out_coff = 0;
+                pack_stem(L, M, src.c);
+                for (int ni : cover) L.flops += 2.0 * node_macs(g.nodes[ni]);
+                L.bytes = tbytes(L.in0) + tbytes(L.out) + (double)L.npad * L.st_pairs * 32 + 4.0 * L.npad;
+                push(L, ci);
+                return XENOS_OK;
+            }
             if (!pooln) {
                 L.map_mode = MAP_PATCH;
                 L.ni = 1;
@@ -1688,7 +1784,7 @@ void emit_plan_json(Graph &g) {
             jint(s, "patch_rw", L.patch_rw); jint(s, "tiles_y", L.tiles_y); jint(s, "tiles_x", L.tiles_x);
             jint(s, "stages", L.stages); jint(s, "tmem_cols", L.tmem_cols); jint(s, "acc_stride", L.acc_stride);
             jint(s, "ni", L.ni); jint(s, "step_y", L.step_y); jint(s, "step_x", L.step_x); jint(s, "off_y", L.off_y); jint(s, "off_x", L.off_x);
-            jint(s, "hstages", L.hstages); jint(s, "halo_h", L.halo_h); jint(s, "halo_w", L.halo_w); jint(s, "halo_cb", L.halo_cb);
+            jint(s, "hstages", L.hstages); jint(s, "stem_tc", L.stem_tc); jint(s, "halo_h", L.halo_h); jint(s, "halo_w", L.halo_w); jint(s, "halo_cb", L.halo_cb);
             jint(s, "halo_bytes", L.halo_bytes);
             jint(s, "ksplit", L.ksplit); jint(s, "kb_per", L.kb_per); jint(s, "a_tma", L.a_tma); jint(s, "fc_small", L.fc_small); jint(s, "dw_workers", L.dw_workers); jint(s, "dw_groups", L.dw_groups); jint(s, "dw_br", L.dw_br); jint(s, "chunk", L.chunk); jint(s, "out_bufs", L.out_bufs); jint(s, "b_slots", L.b_slots); jint(s, "n_acc", L.n_acc); jint(s, "gap_parts", L.gap_parts); jint(s, "conv_tc", L.conv_tc); jint(s, "b_resident", L.b_resident);
         }

@@ -15,6 +15,7 @@
 
 #include "chain2_tc.cuh"
 #include "conv_tc.cuh"
+#include "stem_tc.cuh"
 #include "dw_tc.cuh"
 #include "gemm_tc.cuh"
 #include "graph.hpp"
@@ -236,6 +237,18 @@ static DwKernel dw_kernel_of(int stride, int br) {
     if (stride == 1) return br == 4 ? xk::dw_tc_kernel<kEpi, 1, 4> : br == 2 ? xk::dw_tc_kernel<kEpi, 1, 2> : xk::dw_tc_kernel<kEpi, 1, 1>;
     return br == 4 ? xk::dw_tc_kernel<kEpi, 2, 4> : br == 2 ? xk::dw_tc_kernel<kEpi, 2, 2> : xk::dw_tc_kernel<kEpi, 2, 1>;
 }
+// Convolution of an image: how its rows are loaded, the image's type, with or without a pool.
+using StemKernel = void (*)(xk::StemParams);
+template <int kMode>
+static StemKernel stem_kernel_of(bool f32, bool pool) {
+    return f32 ? (pool ? xk::stem_tc_kernel<kMode, true, true> : xk::stem_tc_kernel<kMode, true, false>)
+               : (pool ? xk::stem_tc_kernel<kMode, false, true> : xk::stem_tc_kernel<kMode, false, false>);
+}
+static StemKernel stem_kernel(int mode, bool f32, bool pool) {
+    return mode == xk::SM_S1 ? stem_kernel_of<xk::SM_S1>(f32, pool) : mode == xk::SM_S2 ? stem_kernel_of<xk::SM_S2>(f32, pool)
+         : mode == xk::SM_S2X ? stem_kernel_of<xk::SM_S2X>(f32, pool) : stem_kernel_of<xk::SM_ANY>(f32, pool);
+}
+
 static DwKernel dw_kernel(int epi, int stride, int br) {
     return epi == xk::DE_STORE ? dw_kernel_of<xk::DE_STORE>(stride, br) : epi == xk::DE_GAP ? dw_kernel_of<xk::DE_GAP>(stride, br) : dw_kernel_of<xk::DE_SPLIT>(stride, br);
 }
@@ -309,7 +322,7 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
                 if (st != XENOS_OK) return st;
                 continue;
             }
-            if (L.kind != LK_GEMM) continue;
+            if (L.kind != LK_GEMM || L.stem_tc) continue;
             cuuint64_t dims[2] = {(cuuint64_t)L.kpad, (cuuint64_t)L.npad};
             cuuint64_t strides[1] = {(cuuint64_t)L.kpad * 2};
             cuuint32_t box[2] = {64u, (cuuint32_t)L.tile_n};
@@ -358,6 +371,9 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
                     if ((e = cudaFuncSetAttribute(dw_kernel(epi, stride, br), cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
                         return cuda_fail(g, "cudaFuncSetAttribute(dw)", e);
     if (any_gemm)
+        for (int i = 0; i < 16; ++i)
+            if ((e = cudaFuncSetAttribute(stem_kernel(i & 3, (i >> 2) & 1, i >> 3), cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
+                return cuda_fail(g, "cudaFuncSetAttribute(stem)", e);
         if ((e = cudaFuncSetAttribute(xk::fc_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(fc)", e);
     if (any_gemm2)
@@ -379,9 +395,9 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
 // Programmatic dependent launch: the kernel may be scheduled while its predecessor in the stream drains, runs its set-up
 // and then waits (griddepcontrol.wait) before it touches the predecessor's results.
 template <class... P, class... A>
-static cudaError_t launch_pdl_cluster(void (*kernel)(P...), int grid, int block, int smem, int cluster, cudaStream_t stream, A &&...args) {
+static cudaError_t launch_pdl_cluster(void (*kernel)(P...), dim3 grid, int block, int smem, int cluster, cudaStream_t stream, A &&...args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block);
+    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = stream;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -392,7 +408,7 @@ static cudaError_t launch_pdl_cluster(void (*kernel)(P...), int grid, int block,
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 template <class... P, class... A>
-static cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t stream, A &&...args) {
+static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, int block, int smem, cudaStream_t stream, A &&...args) {
     return launch_pdl_cluster(kernel, grid, block, smem, 1, stream, std::forward<A>(args)...);
 }
 
@@ -613,6 +629,29 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 xk::fc_small_kernel<<<grid, 256, (size_t)N * L.C * 2, stream>>>(
                     (const __nv_bfloat16 *)ptr(L.seg[0].tensor), (const __nv_bfloat16 *)(ws + L.w_off), (const float *)(ws + L.b_off), ptr(L.out), N, L.C,
                     L.kpad, L.K, L.act, L.out_dtype == XENOS_DTYPE_F32, L.out_ctot, L.out_coff);
+                break;
+            }
+            if (L.stem_tc) {
+                xk::StemParams p;
+                std::memset(&p, 0, sizeof p);
+                const bool pool = L.epi == EPI_POOL, f32 = L.seg[0].src_dtype == XENOS_DTYPE_F32;
+                p.src = ptr(L.in0); p.w = (const uint4 *)(ws + L.w_off); p.bias = (const float *)(ws + L.b_off); p.out = ptr(L.out); p.status = status;
+                p.rows = pool ? L.PP : L.P; p.cbs = L.st_cbs; p.cw = L.st_cw; p.units = N * p.cbs * p.rows;
+                p.d_rows = xk::make_fastdiv((uint32_t)p.rows); p.d_cbs = xk::make_fastdiv((uint32_t)p.cbs);
+                p.C = L.C; p.H = L.H; p.W = L.W; p.k = L.k; p.stride = L.stride; p.pad = L.pad; p.lead = L.st_lead;
+                p.P = L.P; p.Q = L.Q; p.N = L.K; p.tile_n = L.tile_n; p.npairs = L.st_pairs;
+                p.R = L.st_slots; p.D = L.hstages; p.nacc = 4; p.acc_stride = L.acc_stride; p.qp = L.st_qp;
+                p.pk = L.pool_k; p.ps = L.pool_stride; p.pp = L.pool_pad; p.PQ = L.PQ; p.pc_log2 = L.st_pc;
+                p.act = L.act; p.out_ctot = L.out_ctot; p.out_coff = L.out_coff;
+                p.idesc = make_idesc(L.tile_n);
+                p.off_w = L.off_b; p.off_bias = L.off_bias; p.off_stage = L.off_stg; p.stage_bytes = (L.off_bar - L.off_stg) / 2 & ~15; p.off_bar = L.off_bar;
+                p.launch_id = (int)li;
+                const int gx = std::min(p.units, std::max(1, sms / L.n_tiles));
+                // whole groups of elements where rows are made of them and the image is aligned; else element by element
+                const bool vec = L.st_vec && ((uintptr_t)p.src & 15u) == 0;
+                const int mode = L.stride == 2 ? (vec ? xk::SM_S2 : xk::SM_S2X) : L.stride == 1 ? xk::SM_S1 : xk::SM_ANY;
+                cudaError_t le = launch_pdl(stem_kernel(mode, f32, pool), dim3(gx, L.n_tiles), L.block, L.smem_bytes, stream, p);
+                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
                 break;
             }
             if (L.conv_tc) {
