@@ -251,11 +251,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Programmatic dependent launch: let the next kernel of the stream be scheduled early / wait until
-// the previous kernel's memory is complete and visible (no-ops without the launch attribute).
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
 // ---- row <-> pixel -----------------------------------------------------------------------------
@@ -579,11 +574,6 @@ __device__ __forceinline__ DwUnit make_dw_unit(const GemmParams &g, int pt, int 
 __device__ __forceinline__ uint32_t clamp_bf16x2(uint32_t v, uint32_t lo, uint32_t hi) {
     __nv_bfloat162 x = *reinterpret_cast<__nv_bfloat162 *>(&v);
     x = __hmin2(__hmax2(x, *reinterpret_cast<__nv_bfloat162 *>(&lo)), *reinterpret_cast<__nv_bfloat162 *>(&hi));
-    return *reinterpret_cast<uint32_t *>(&x);
-}
-
-__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
-    __nv_bfloat162 x = __hmax2(*reinterpret_cast<__nv_bfloat162 *>(&a), *reinterpret_cast<__nv_bfloat162 *>(&b));
     return *reinterpret_cast<uint32_t *>(&x);
 }
 

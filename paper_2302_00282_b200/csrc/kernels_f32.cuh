@@ -9,6 +9,11 @@
 
 namespace xk {
 
+// Programmatic dependent launch: let the next kernel of the stream be scheduled early / wait until
+// the previous kernel's memory is complete and visible (no-ops without the launch attribute).
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ float apply_act(float v, int act) {
     if (act >= 1) v = fmaxf(v, 0.0f);
     if (act == 2) v = fminf(v, 6.0f);

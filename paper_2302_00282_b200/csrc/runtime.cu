@@ -374,7 +374,8 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
         for (int i = 0; i < 16; ++i)
             if ((e = cudaFuncSetAttribute(stem_kernel(i & 3, (i >> 2) & 1, i >> 3), cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
                 return cuda_fail(g, "cudaFuncSetAttribute(stem)", e);
-        if ((e = cudaFuncSetAttribute(xk::fc_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess)
+        if ((e = cudaFuncSetAttribute(xk::fc_small_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(xk::fc_small_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess)
             return cuda_fail(g, "cudaFuncSetAttribute(fc)", e);
     if (any_gemm2)
         if ((e = cudaFuncSetAttribute(xk::pair_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
@@ -515,13 +516,23 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
         }
         case LK_POOL: {
             long long total = (long long)N * L.P * L.Q * (L.C / 8);
-            xk::pool_kernel<<<ew_grid(total, 256, sms), 256, 0, stream>>>(
-                (const __nv_bfloat16 *)ptr(L.in0), (__nv_bfloat16 *)ptr(L.out), N, L.C, L.H, L.W, L.P, L.Q, L.pool_k, L.pool_stride, L.pool_pad, L.pool_kind);
+            const bool small = L.pool_kind == 0 && L.pool_k <= 3 && total < (1ll << 31);
+            // four outputs a thread where that still fills the device
+            const int rows = total >= 4ll * 1024 * sms ? 4 : 1, bands = (L.P + rows - 1) / rows;
+            const int items = (int)(small ? (long long)N * bands * L.Q * (L.C / 8) : 0);
+            const __nv_bfloat16 *x = (const __nv_bfloat16 *)ptr(L.in0);
+            __nv_bfloat16 *y = (__nv_bfloat16 *)ptr(L.out);
+            cudaError_t le = small ? launch_pdl(rows == 4 ? xk::maxpool_kernel<4> : xk::maxpool_kernel<1>, (items + 255) / 256, 256, 0, stream, x, y, items, L.C / 8,
+                                                L.H, L.W, L.P, L.Q, bands, L.pool_k, L.pool_stride, L.pool_pad)
+                                   : launch_pdl(xk::pool_kernel, ew_grid(total, 256, sms), 256, 0, stream, x, y, N, L.C, L.H, L.W, L.P, L.Q, L.pool_k,
+                                                L.pool_stride, L.pool_pad, L.pool_kind);
+            if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
         }
         case LK_GAP: {
-            int total = N * (L.C / 8);
-            xk::gap_kernel<<<(total + 127) / 128, 128, 0, stream>>>((const __nv_bfloat16 *)ptr(L.in0), ptr(L.out), N, L.C, L.H * L.W, L.out_dtype == XENOS_DTYPE_F32);
+            cudaError_t le = launch_pdl(xk::gap_kernel, dim3((L.C + 63) / 64, N), 256, 0, stream, (const __nv_bfloat16 *)ptr(L.in0), ptr(L.out), L.C, L.H * L.W,
+                                        L.out_dtype == XENOS_DTYPE_F32);
+            if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
         }
         case LK_ADD: {
@@ -626,9 +637,10 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
         case LK_GEMM: {
             if (L.fc_small) {
                 const int grid = std::min(sms, (L.K + 7) / 8);
-                xk::fc_small_kernel<<<grid, 256, (size_t)N * L.C * 2, stream>>>(
+                cudaError_t le = launch_pdl(N == 1 ? xk::fc_small_kernel<1> : xk::fc_small_kernel<8>, grid, 256, N * L.C * 2, stream,
                     (const __nv_bfloat16 *)ptr(L.seg[0].tensor), (const __nv_bfloat16 *)(ws + L.w_off), (const float *)(ws + L.b_off), ptr(L.out), N, L.C,
                     L.kpad, L.K, L.act, L.out_dtype == XENOS_DTYPE_F32, L.out_ctot, L.out_coff);
+                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
                 break;
             }
             if (L.stem_tc) {
