@@ -462,7 +462,7 @@ dw_tc_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CU
 #pragma unroll 1
                         for (int item = wt; item < per; item += 32 * kDwWorkers) {
                             const int c = item & 31, tri = item >> 5, sl = tri & 3, img = tri >> 2, n = t.n0 + img, nc = n0 + (p0 + sl) * 32 + c;
-                            if (p0 + sl >= nchunks || n >= g.batch || nc >= g.N) continue;
+                            if ((p0 + sl) * 32 + c >= cols || n >= g.batch || nc >= g.N) continue;
                             float acc = 0.0f;
                             for (int pa = 0; pa < parts; ++pa) acc += parts_mem[((tri * parts + pa) << 5) + c];
                             acc /= (float)g.gap_rpi;

@@ -1,0 +1,148 @@
+"""Every kernel of the fast paths at the sizes where it can go wrong: edges of tiles, remainders, the smallest and the
+largest of its range.  The oracle and the tolerances are those of the parity tests."""
+import numpy as np
+import pytest
+
+import oracle as xo
+from oracle import interp
+from xenos_workloads import graphs
+from xenos_workloads.graphs import GraphSpec
+
+from gpu_util import GpuGraph, rel_err_fp32
+from test_gpu_parity import FP32_TOL, check_bf16
+
+pytestmark = pytest.mark.gpu
+
+
+def _spec(shape, build, precision="bf16"):
+    g = GraphSpec("unit", shape, precision=precision) if precision == "fp32" else GraphSpec("unit", shape)
+    build(g)
+    return g
+
+
+# operand boxes of 16, 32 and 64 channels (several taps to a stage), strides and frames beyond the image, one output pixel,
+# row counts around one 128-row tile, one tile per column width, resident weights with many tiles per CTA
+@pytest.mark.parametrize("cin,h,w,cout,k,st,pad,batch,resident", [
+    (8, 5, 5, 8, 3, 1, 1, 1, None), (16, 9, 17, 24, 5, 2, 2, 2, None), (32, 13, 6, 40, 3, 2, 1, 3, None), (40, 7, 7, 16, 3, 1, 0, 2, None),
+    (72, 11, 5, 264, 3, 3, 2, 1, None), (64, 8, 16, 64, 1, 1, 0, 1, None), (64, 3, 43, 48, 1, 1, 0, 1, None), (128, 2, 2, 32, 2, 2, 0, 1, None),
+    (24, 9, 9, 520, 1, 2, 0, 2, None), (64, 56, 56, 64, 3, 1, 1, 8, 1), (16, 55, 55, 16, 1, 1, 0, 12, 1)])
+def test_convolution_tiles(cin, h, w, cout, k, st, pad, batch, resident):
+    spec = _spec((cin, h, w), lambda g: g.cbr("c", "input", cout, k, st, pad))
+    _, _, gg = check_bf16(f"conv_tiles{(cin, h, w, cout, k, st, pad)}", spec, batch, in_mode="bf16_nhwc")
+    L = gg.g.plan()["launches"][0]
+    assert L["conv_tc"] == 1 and (resident is None or L["b_resident"] == resident)
+
+
+# the chunks of a reduction as the CTAs of a cluster (2 to 8) and through the workspace (more); fewer rows than chunks, a tile
+# whose rows do not divide among them, several column tiles
+@pytest.mark.parametrize("cin,hw,cout,k,parts_k,batch", [(128, 1, 16, 1, 2, 3), (256, 3, 64, 3, 4, 1), (320, 5, 72, 1, 5, 2), (448, 12, 200, 1, 7, 2),
+                                                         (512, 6, 264, 1, 8, 4), (256, 6, 64, 3, 9, 3), (256, 7, 48, 3, 36, 1)])
+def test_reduction_split_over_clusters(cin, hw, cout, k, parts_k, batch):
+    spec = _spec((cin, hw, hw), lambda g: g.cbr("c", "input", cout, k, 1, k // 2))
+    _, _, gg = check_bf16(f"cluster_split{(cin, hw, cout, k, parts_k)}", spec, batch, in_mode="bf16_nhwc", splits=[("c", dict(parts_k=parts_k))])
+    assert gg.g.plan()["launches"][0]["ksplit"] == parts_k
+
+
+# middle tiles of 8 to 256 channels, one row to many tiles, output blocks that end inside 128 columns, with and without shortcut
+@pytest.mark.parametrize("cin,h,w,k,cmid,cout,add,batch", [(64, 1, 1, 1, 8, 8, False, 1), (64, 8, 16, 3, 64, 64, True, 1), (128, 3, 43, 1, 256, 136, False, 2),
+                                                           (192, 5, 27, 3, 192, 192, True, 3), (64, 40, 40, 3, 40, 392, False, 13)])
+def test_two_convolutions_with_a_1x1_consumer(cin, h, w, k, cmid, cout, add, batch):
+    def build(g):
+        y = g.cbr("c1", "input", cmid, k, 1, k // 2)
+        y = g.cbr("c2", y, cout, 1, act=None if add else "relu6")
+        if add:
+            g.act("relu", g.add("add", y, "input"), "relu")
+    _, _, gg = check_bf16(f"pair{(cin, h, w, k, cmid, cout, add)}", _spec((cin, h, w), build), batch, in_mode="bf16_nhwc",
+                          links=[["c1", "c2"] + (["add"] if add else [])])
+    assert gg.g.launch_count() == 1
+
+
+# both strides, maps smaller than a tile and much wider, channel counts that end inside an 8-channel piece's K block, one and
+# many tiles per CTA, the global average of one and of many images per tile
+@pytest.mark.parametrize("c,h,w,cout,st,gap,batch", [(8, 1, 1, 8, 1, False, 1), (24, 3, 5, 40, 2, False, 2), (16, 79, 79, 32, 1, False, 3), (72, 17, 66, 136, 2, False, 2),
+                                                     (256, 9, 130, 264, 1, False, 1), (32, 112, 112, 64, 1, False, 4), (512, 10, 10, 512, 1, False, 2),
+                                                     (40, 5, 5, 48, 1, True, 7), (128, 11, 11, 264, 2, True, 3), (1024, 7, 7, 1024, 1, True, 1)])
+def test_depthwise_pointwise_tiles(c, h, w, cout, st, gap, batch):
+    def build(g):
+        y = g.cbr("pw", g.cbr("dw", "input", c, 3, st, 1, groups=c, act="relu6"), cout, 1, act="relu6")
+        if gap:
+            g.gap("gap", y)
+    _, _, gg = check_bf16(f"dw_pw{(c, h, w, cout, st, gap)}", _spec((c, h, w), build), batch, in_mode="bf16_nhwc")
+    assert gg.g.launch_count() == 1
+
+
+# 1 to 7 channels, windows of 2 to 8, strides 1, 2 (rows of whole groups of four elements and not) and 3, several column blocks,
+# output channels that end inside a tile and in a second one; pools that overlap by one row, that do not, and over wide images
+@pytest.mark.parametrize("cin,h,w,cout,k,st,pad,pool,batch", [
+    (1, 2, 2, 8, 2, 1, 0, None, 1), (3, 19, 300, 24, 3, 1, 1, None, 2), (2, 21, 45, 72, 4, 2, 1, None, 3), (7, 16, 40, 16, 8, 3, 2, None, 2),
+    (3, 40, 520, 64, 7, 2, 3, None, 1), (3, 33, 36, 200, 5, 2, 2, None, 20), (3, 61, 64, 64, 7, 2, 3, (3, 2, 1), 9), (4, 30, 37, 40, 3, 1, 1, (2, 2, 0), 2),
+    (3, 25, 1100, 64, 3, 2, 0, (3, 2, 0), 1), (5, 28, 28, 8, 6, 2, 2, (3, 3, 1), 3)])
+@pytest.mark.parametrize("in_mode", ["f32_nchw", "bf16_nchw"])
+def test_image_convolution(cin, h, w, cout, k, st, pad, pool, batch, in_mode):
+    def build(g):
+        y = g.cbr("stem", "input", cout, k, st, pad)
+        if pool:
+            g.pool("mp", y, "maxpool", *pool)
+    links = [["stem", "mp"]] if pool else None
+    if not pool and k == 3 and cout <= 64 and batch <= 8:
+        batch = 9          # (smaller batches of a 3 x 3 window run on the CUDA cores)
+    _, _, gg = check_bf16(f"stem{(cin, h, w, cout, k, st, pad, pool)}{in_mode}", _spec((cin, h, w), build), batch, in_mode=in_mode, links=links)
+    assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
+
+
+# one output row per thread and four, bands that end inside the map, windows of 1 to 3; averages of one row and of more rows than
+# a CTA's lane groups, channels that end inside a 64-channel block
+@pytest.mark.parametrize("c,h,w,k,st,pad,batch", [(8, 1, 1, 3, 2, 1, 1), (24, 9, 14, 2, 2, 0, 3), (64, 113, 111, 3, 2, 0, 26), (128, 58, 57, 3, 1, 1, 12), (16, 40, 40, 1, 3, 0, 2)])
+def test_max_pool_and_average(c, h, w, k, st, pad, batch):
+    spec = _spec((c, h, w), lambda g: g.pool("mp", "input", "maxpool", k, st, pad))
+    check_bf16(f"maxpool{(c, h, w, k, st, pad)}", spec, batch, in_mode="bf16_nhwc", images=[0, batch - 1])
+    spec = _spec((c, min(h, 40), min(w, 40)), lambda g: g.gap("ap", "input"))
+    check_bf16(f"average{(c, h, w)}", spec, batch, in_mode="bf16_nhwc", images=[0, batch - 1])
+
+
+# both register tiles, weights in shared memory and not, pools of 2 and 3 (maximum and average), strides, ragged edges
+@pytest.mark.parametrize("cin,hw,cmid,cout,k,st,pool,batch", [(1, 5, 1, 3, 3, 1, ("maxpool", 2, 2, 0), 1), (16, 33, 32, 24, 3, 1, ("maxpool", 3, 2, 0), 2), (48, 40, 64, 64, 3, 1, ("avgpool", 2, 2, 0), 9),
+                                                              (8, 30, 20, 13, 5, 2, ("avgpool", 3, 3, 0), 5), (200, 12, 96, 100, 3, 1, ("maxpool", 2, 2, 0), 20)])
+def test_fp32_chain_tiles(cin, hw, cmid, cout, k, st, pool, batch):
+    def build(g):
+        g.pool("mp", g.cbr("c1", g.cbr("c3", "input", cmid, k, st, k // 2), cout, 1), *pool)
+    spec = _spec((cin, hw, hw), build, "fp32")
+    P, x = graphs.make_params(spec), graphs.make_input(spec, batch)
+    gg = GpuGraph(spec, P, batch)
+    y = gg.run(x)
+    assert gg.g.launch_count() == 1 and not np.isnan(y).any()
+    assert rel_err_fp32(y, interp.run_graph(spec, P, x)) <= FP32_TOL
+
+
+# the recorded form of a pass: repeated calls, images that change in place, other buffers and batches in turn (more than are
+# kept), a call inside the caller's own capture
+@pytest.mark.parametrize("name,kw", [("mobilenet_v1", dict(hw=64, width=0.25, classes=24)), ("resnet18", dict(hw=64, base=16, classes=10))])
+def test_repeated_passes(name, kw):
+    import torch
+    spec = getattr(graphs, name)(**kw)
+    x = graphs.make_input(spec, 6)
+    gg = GpuGraph(spec, graphs.make_params(spec), 3)
+    want = {b: gg.run(x[:b]) for b in (1, 2, 3)}
+    other = gg.run(x[3:6])
+    xin = gg.upload(x[:3])
+    for turn in range(3):
+        for b in (3, 1, 2):
+            for _ in range(3):
+                out = [gg.alloc_out(b) for _ in range(4)]
+                for o in out + out:
+                    gg.g.run(b, [xin.data_ptr()], [o.data_ptr()], gg.stream)
+                assert all(np.array_equal(o.float().cpu().numpy(), want[b]) for o in out), (turn, b)
+    out = gg.alloc_out(3)
+    for src, ref in ((x[:3], want[3]), (x[3:6], other), (x[:3], want[3])):
+        xin.copy_(gg.upload(src))
+        gg.g.run(3, [xin.data_ptr()], [out.data_ptr()], gg.stream)
+        assert np.array_equal(out.float().cpu().numpy(), ref)
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        gg.g.run(3, [xin.data_ptr()], [out.data_ptr()], side.cuda_stream)
+    out.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(out.float().cpu().numpy(), want[3])
+    gg.g.status(gg.stream)
