@@ -862,7 +862,7 @@ struct Lower {
             stg = xbytes;
         } else if (L.cv_epi == 3) {
             L.chunk = 32;
-            stg = 2 * (128 * 33 + 128) * 4;
+            stg = 2 * 4352 * 4;
         }
         L.nchunks = ceil_div(L.tile_n, L.chunk);
         stg = (int)align_up((size_t)stg, 1024);
