@@ -35,6 +35,7 @@ constexpr int kCvThreads = 128 + 32 * kCvEpiWarps;
 constexpr int kCvMaxStages = 6;
 enum { CE_STORE = 0, CE_SKIP = 1, CE_VEC = 2, CE_GAP = 3, CE_SPLIT = 4, CE_CLUSTER = 5 };
 constexpr int kCvMaxCluster = 8;
+constexpr int kMaxSkipSlots = 4;         // shortcut / result boxes per epilogue warp
 constexpr int kGapFloats = 4352;         // column sums of an average, per half of the epilogue
 
 // Exact division of n < 2^31 by a constant of the launch.
@@ -71,6 +72,7 @@ struct ConvParams {
     int kblocks, stages, stage_bytes, b_resident, b_group;
     int acc_stride, tmem_cols;
     int chunk, nchunks, box_bytes; // epilogue: columns per chunk, chunks per tile, bytes of one 32-row staging box
+    int s_slots;                   // boxes per epilogue warp
     int act, act2, out_ctot, out_f32;
     uint32_t idesc;
     int off_b, off_stage, off_bias, off_bar;
@@ -657,9 +659,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     auto accf_bar = [&](int b) { return bar + 8u * (2 * kCvMaxStages + b); };
     auto acce_bar = [&](int b) { return bar + 8u * (2 * kCvMaxStages + 2 + b); };
     auto bres_bar = [&](int q) { return bar + 8u * (2 * kCvMaxStages + 4 + q); };                       // 4
-    auto skip_bar = [&](int e, int b) { return bar + 8u * (2 * kCvMaxStages + 8 + 2 * e + b); };       // 16
+    auto skip_bar = [&](int e, int b) { return bar + 8u * (2 * kCvMaxStages + 8 + kMaxSkipSlots * e + b); };
     const uint32_t arrived = skip_bar(0, 0);      // (a split has no shortcut boxes)
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + g.off_bar + 8 * (2 * kCvMaxStages + 24));
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + g.off_bar + 8 * (2 * kCvMaxStages + 8 + kMaxSkipSlots * kCvEpiWarps));
     volatile int *fail_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);      // [0] give-up, [1], [2] agreement of a split / average
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -667,7 +669,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
         for (int s = 0; s < g.stages; ++s) { mbar_init(full_bar(s), g.b_resident ? 1u : 2u); mbar_init(empty_bar(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), kCvEpiWarps); }
         for (int q = 0; q < 4; ++q) mbar_init(bres_bar(q), 1);
-        if (kEpi == CE_SKIP) for (int e = 0; e < 2 * kCvEpiWarps; ++e) mbar_init(skip_bar(0, e), 1);
+        if (kEpi == CE_SKIP) for (int e = 0; e < kMaxSkipSlots * kCvEpiWarps; ++e) mbar_init(skip_bar(0, e), 1);
         if (kEpi == CE_CLUSTER) mbar_init(arrived, kCvEpiWarps * g.ksplit);
         fail_flag[0] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -757,16 +759,27 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
         if (kEpi == CE_STORE || kEpi == CE_SKIP) {
             const int last_act = (kEpi == CE_SKIP) ? g.act2 : g.act;
             const uint32_t plo = last_act >= 1 ? 0u : 0xff80ff80u, phi = last_act == 2 ? 0x40c040c0u : 0x7f807f80u;
-            const uint32_t stage0 = sbase + g.off_stage + (uint32_t)(2 * e) * g.box_bytes;
-            int i = 0, cnt = 0;      // tiles; boxes this warp has stored
-            if (kEpi == CE_SKIP && (int)blockIdx.x < g.total && half < g.nchunks) {
-                const ConvTile t = conv_tile(g, blockIdx.x);
-                if (elect_one()) {
-                    mbar_arrive_expect_tx(skip_bar(e, 0), (uint32_t)g.box_bytes);
-                    tma_load_2d(stage0, &tmS, t.nt * g.tile_n + half * g.chunk, t.mt * g.tile_rows + quarter * 32, skip_bar(e, 0));
+            const uint32_t stage0 = sbase + g.off_stage + (uint32_t)(g.s_slots * e) * g.box_bytes;
+            const int depth = in_reg(g.s_slots);
+            int i = 0, slot = 0;
+            // Shortcut boxes are asked for s_slots - 1 ahead of their use: with one ahead every box cost a warp the whole latency
+            // of the load.  (ati, aj): the next box to ask for.
+            uint32_t sph = 0;
+            int ati = half < g.nchunks ? (int)blockIdx.x : g.total, aj = half;
+            auto ask_skip = [&](int to) {
+                const ConvTile u = conv_tile(g, ati);
+                mbar_arrive_expect_tx(skip_bar(e, to), (uint32_t)g.box_bytes);
+                tma_load_2d(stage0 + (uint32_t)to * g.box_bytes, &tmS, u.nt * g.tile_n + aj * g.chunk, u.mt * g.tile_rows + quarter * 32, skip_bar(e, to));
+            };
+            auto advance = [&]() {
+                aj += 2;
+                if (aj >= g.nchunks) { aj = half; ati += (int)gridDim.x; }
+            };
+            if (kEpi == CE_SKIP)
+                for (int d = 0; d + 1 < depth && ati < g.total; ++d, advance()) {
+                    if (elect_one()) ask_skip(d);
+                    __syncwarp();
                 }
-                __syncwarp();
-            }
 #pragma unroll 1
             for (int ti = blockIdx.x; ti < g.total && ok; ti += gridDim.x, ++i) {
                 const ConvTile t = conv_tile(g, ti);
@@ -775,15 +788,15 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                 tc_fence_after();
                 const uint32_t t_acc = t_warp + b * g.acc_stride;
 #pragma unroll 1
-                for (int j = half; j < g.nchunks; j += 2, ++cnt) {
-                    const uint32_t buf = stage0 + (uint32_t)(cnt & 1) * g.box_bytes;
+                for (int j = half; j < g.nchunks; j += 2) {
+                    const uint32_t buf = stage0 + (uint32_t)slot * g.box_bytes;
                     const int x = t.nt * g.tile_n + j * g.chunk;
                     const uint32_t sb = bias_s + (uint32_t)x * 4u;
                     if (kEpi == CE_STORE) {
                         if (elect_one()) bulk_wait_read<1>();      // the store before last has left this box
                         __syncwarp();
                     } else {
-                        ok = mbar_wait(skip_bar(e, cnt & 1), (cnt >> 1) & 1);
+                        ok = mbar_wait(skip_bar(e, slot), sph);
                         if (!ok) break;
                     }
 #pragma unroll 1
@@ -816,23 +829,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                     __syncwarp();
                     if (elect_one()) { tma_store_2d(&tmO, buf, x, y); bulk_commit(); }
                     __syncwarp();
-                    if (kEpi == CE_SKIP) {
-                        // request the next shortcut box (this tile's next chunk or the next tile's first) into the other
-                        // buffer, once the store before this one has left it
-                        int jn = j + 2, tn = ti;
-                        if (jn >= g.nchunks) { jn = half; tn = ti + (int)gridDim.x; }
-                        if (tn < g.total) {
-                            const ConvTile u = conv_tile(g, tn);
-                            if (elect_one()) {
-                                bulk_wait_read<1>();
-                                const uint32_t nb = skip_bar(e, (cnt + 1) & 1);
-                                mbar_arrive_expect_tx(nb, (uint32_t)g.box_bytes);
-                                tma_load_2d(stage0 + (uint32_t)((cnt + 1) & 1) * g.box_bytes, &tmS, u.nt * g.tile_n + jn * g.chunk,
-                                            u.mt * g.tile_rows + quarter * 32, nb);
-                            }
-                            __syncwarp();
-                        }
+                    // (into the box before this one, once that one's store has left it)
+                    if (kEpi == CE_SKIP && ati < g.total) {
+                        if (elect_one()) { bulk_wait_read<1>(); ask_skip(slot ? slot - 1 : depth - 1); }
+                        __syncwarp();
+                        advance();
                     }
+                    if (++slot == depth) { slot = 0; sph ^= 1u; }
                 }
                 if (half >= g.nchunks && ok) warp_arrive(acce_bar(b), lane);      // a warp without a chunk in so narrow a tile
             }

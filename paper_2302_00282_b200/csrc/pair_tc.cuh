@@ -31,6 +31,7 @@ struct PairParams {
     FastDiv d_rpi, d_q;
     int rows, tiles, n1pad, n1_slots, kblocks2, n2_blocks, npad2;
     int a_slots, b_slots, resident, dbl;      // dbl: two first accumulators
+    int s_slots;                    // staging boxes per epilogue warp
     int act1, act2, act3;
     uint32_t idesc1, idesc2;
     int off_b, off_mid, off_stage, off_bias, off_bar;
@@ -90,8 +91,8 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t a_full = bar, b_full = bar + 8u * 2 * kPairMaxSlots, d_bar = bar + 8u * 4 * kPairMaxSlots;
     // d_bar: first accumulator full [2] / empty [2], second full [2] / empty [2], middle full, middle empty, resident weights
     const uint32_t d1f = d_bar, d1e = d_bar + 16u, d2f = d_bar + 32u, d2e = d_bar + 48u, midf = d_bar + 64u, mide = d_bar + 72u, bres = d_bar + 80u;
-    const uint32_t skip0 = d_bar + 96u;                                           // 2 per epilogue warp
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + g.off_bar + 8 * (4 * kPairMaxSlots + 12 + 16));
+    const uint32_t skip0 = d_bar + 96u;                                           // kMaxSkipSlots per epilogue warp
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + g.off_bar + 8 * (4 * kPairMaxSlots + 12 + kMaxSkipSlots * kCvEpiWarps));
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0 && elect_one()) {
@@ -104,7 +105,7 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             mbar_init(d2f + 8u * b, 1); mbar_init(d2e + 8u * b, kCvEpiWarps);
         }
         mbar_init(midf, kCvEpiWarps); mbar_init(mide, 1); mbar_init(bres, 1);
-        for (int e = 0; e < 2 * kCvEpiWarps; ++e) mbar_init(skip0 + 8u * e, 1);
+        for (int e = 0; e < kMaxSkipSlots * kCvEpiWarps; ++e) mbar_init(skip0 + 8u * e, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB1) : "memory");
@@ -265,7 +266,7 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int e = warp - 4, quarter = warp & 3, half = e >> 2, row = quarter * 32 + lane;
         const uint32_t t_warp = tmem_base + ((uint32_t)(quarter * 32) << 16);
         const uint32_t bias1 = sbase + g.off_bias, bias2 = bias1 + (uint32_t)g.n1pad * 4u;
-        const uint32_t mid = sbase + g.off_mid, stage0 = sbase + g.off_stage + (uint32_t)(2 * e) * 2048u;
+        const uint32_t mid = sbase + g.off_mid, stage0 = sbase + g.off_stage + (uint32_t)(g.s_slots * e) * 2048u;
         const uint32_t lo1 = g.act1 >= 1 ? 0u : 0xff80ff80u, hi1 = g.act1 == 2 ? 0x40c040c0u : 0x7f807f80u;
         const int last_act = kSkip ? g.act3 : g.act2;
         const uint32_t lo2 = last_act >= 1 ? 0u : 0xff80ff80u, hi2 = last_act == 2 ? 0x40c040c0u : 0x7f807f80u;
@@ -280,14 +281,25 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 t[2 * q + 1] = __fadd2_rn(make_float2(v[4 * q + 2], v[4 * q + 3]), make_float2(bz.z, bz.w));
             }
         };
-        auto ask_skip = [&](int cnt, int t, int c, int j) {      // shortcut box of chunk j of channel block c of tile t
-            const uint32_t sb = skip0 + 8u * (2 * e + (cnt & 1));
+        // Shortcut boxes are asked for s_slots - 1 ahead of their use: with one box of 2 KB ahead every box cost a warp the whole
+        // latency of the load (3.5 TB/s of traffic at best).  (at, ac, aj): the next box to ask for.
+        const int depth = in_reg(g.s_slots), step_c = n2;
+        int at = blockIdx.x, ac = 0, aj = 0;
+        auto ask_skip = [&](int slot) {
+            const uint32_t sb = skip0 + 8u * (kMaxSkipSlots * e + slot);
             mbar_arrive_expect_tx(sb, 2048u);
-            tma_load_2d(stage0 + (uint32_t)(cnt & 1) * 2048u, &tmS, c * 128 + (half * 2 + j) * 32, t * kTileM + quarter * 32, sb);
+            tma_load_2d(stage0 + (uint32_t)slot * 2048u, &tmS, ac * 128 + (half * 2 + aj) * 32, at * kTileM + quarter * 32, sb);
         };
-        int i = 0, c2 = 0, cnt = 0;
-        if (kSkip && (int)blockIdx.x < tiles && elect_one()) ask_skip(0, blockIdx.x, 0, 0);
-        __syncwarp();
+        auto advance = [&]() {
+            if (++aj == 2) { aj = 0; if (++ac == step_c) { ac = 0; at += step; } }
+        };
+        int i = 0, c2 = 0, slot = 0;
+        uint32_t sph = 0;
+        if (kSkip)
+            for (int d = 0; d + 1 < depth && at < tiles; ++d, advance()) {
+                if (elect_one()) ask_skip(d);
+                __syncwarp();
+            }
 #pragma unroll 1
         for (int t = blockIdx.x; t < tiles && ok; t += step, ++i) {
             // middle: first accumulator -> operand layout of the second product
@@ -324,11 +336,11 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (!ok) break;
                 tc_fence_after();
 #pragma unroll 1
-                for (int j = 0; j < 2; ++j, ++cnt) {
-                    const uint32_t buf = stage0 + (uint32_t)(cnt & 1) * 2048u;
+                for (int j = 0; j < 2; ++j) {
+                    const uint32_t buf = stage0 + (uint32_t)slot * 2048u;
                     const int col = (half * 2 + j) * 32;
                     if (kSkip) {
-                        ok = mbar_wait(skip0 + 8u * (2 * e + (cnt & 1)), (cnt >> 1) & 1);
+                        ok = mbar_wait(skip0 + 8u * (kMaxSkipSlots * e + slot), sph);
                         if (!ok) break;
                     } else {
                         if (elect_one()) bulk_wait_read<1>();
@@ -365,13 +377,11 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     if (elect_one()) {
                         tma_store_2d(&tmO, buf, c * 128 + col, t * kTileM + quarter * 32);
                         bulk_commit();
-                        if (kSkip) {
-                            // the next shortcut box goes to the other buffer, once the store before this one has left it
-                            int jn = j + 1, cn = c, tn = t;
-                            if (jn == 2) { jn = 0; if (++cn == n2) { cn = 0; tn += step; } }
-                            if (tn < tiles) { bulk_wait_read<1>(); ask_skip(cnt + 1, tn, cn, jn); }
-                        }
+                        // the next shortcut box goes where the box before this one was, once that one's store has left it
+                        if (kSkip && at < tiles) { bulk_wait_read<1>(); ask_skip(slot ? slot - 1 : depth - 1); }
                     }
+                    if (kSkip && at < tiles) advance();
+                    if (++slot == depth) { slot = 0; sph ^= 1u; }
                     __syncwarp();
                 }
             }

@@ -342,7 +342,7 @@ static bool try_match(const LinkCtx &cx, int a, Allowed allowed, Chain &out, boo
             // with the average cannot take part in a reduction split, and at batch 1 the 72 K blocks of ResNet-18's last
             // convolution then run one after the other on 16 units, 38 us against 14 + 6 us as two kernels)
             const long gap_tiles = (long)((g.max_batch * cx.rows(b) + 127) / 128) * ((A.cout + 31) / 32);
-            const bool serial_k = by_model && (long)A.k * A.k * A.cin >= 16 * 64 && gap_tiles * 2 <= g.hw.sm_count;
+            const bool serial_k = by_model && (long)A.k * A.k * A.cin >= 16 * 64 && gap_tiles <= g.hw.sm_count;
             if (c >= 0 && allowed(c) && g.nodes[c].kind == NK_GAP && cx.rows(b) <= 128 && !serial_k) {
                 out.nodes.push_back(c);
                 out.pattern += " -> ZPooling (global average)";
@@ -857,7 +857,8 @@ struct Lower {
             // (at tile_n = 256 the 64-column boxes would take the fourth stage of the ring)
             for (int c : {64, 32, 16})
                 if (L.tile_n % c == 0 && (L.tile_n / c) % 2 == 0 && !(c == 64 && L.tile_n > 160)) { L.chunk = c; break; }
-            stg = 16 * L.chunk * 64;                 // two 32-row boxes for each of eight warps
+            if (L.cv_epi == 1) L.s_slots = 4;
+            stg = 8 * L.s_slots * L.chunk * 64;      // 32-row boxes of eight warps
         } else if (L.cv_epi == 5) {
             stg = xbytes;
         } else if (L.cv_epi == 3) {
@@ -1404,10 +1405,12 @@ struct Lower {
             L.pair = 1;
             L.m_tiles = ceil_div(g.max_batch * L.rows_per_image, 128);
             L.tile_n = 128; L.n_tiles = ceil_div(N2, 128); L.npad = L.n_tiles * 128;
-            const int mid = (L.n1pad / 64) * 16384, stg = 16 * 2048, bias = (int)align_up((size_t)(L.n1pad + L.npad) * 4, 128);
-            const int room = cap - 512 - mid - stg - bias;
+            const int mid = (L.n1pad / 64) * 16384, bias = (int)align_up((size_t)(L.n1pad + L.npad) * 4, 128);
+            if (L.skip >= 0) L.s_slots = 3;      // (a fourth box each takes operand slots: 256 against 276 us, 64 channels, 128 x 128, batch 64; 295 with two)
+            const int stg = 8 * L.s_slots * 2048;
+            const int room = cap - 1024 - mid - stg - bias;
             const int weights = L.kblocks * L.n1pad * 128 + L.kblocks2 * L.n_tiles * 16384;
-            L.b_resident = room - weights >= 4 * 16384;
+            L.b_resident = room - weights >= 3 * 16384;
             const int slots = (room - (L.b_resident ? weights : 0)) / 16384;
             L.a_slots = L.b_resident ? std::min(8, slots) : slots * 2 / 5;
             L.b_slots = L.b_resident ? 0 : std::min(8, slots - L.a_slots);
@@ -1418,7 +1421,7 @@ struct Lower {
             L.off_stg = L.off_mid + mid;
             L.off_bias = L.off_stg + stg;
             L.off_bar = L.off_bias + bias;
-            L.smem_bytes = L.off_bar + 512 + 1024;
+            L.smem_bytes = L.off_bar + 1024 + 1024;
             L.stages = L.a_slots;
             L.a_rows = 128;
             L.block = 384;

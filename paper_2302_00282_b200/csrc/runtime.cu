@@ -587,7 +587,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 p.rows = N * L.rows_per_image; p.tiles = (p.rows + 127) / 128;
                 p.d_rpi = xk::make_fastdiv((uint32_t)L.rows_per_image); p.d_q = xk::make_fastdiv((uint32_t)L.Q);
                 p.n1pad = L.n1pad; p.n1_slots = (L.n1pad + 127) / 128; p.kblocks2 = L.kblocks2; p.n2_blocks = L.n_tiles; p.npad2 = L.npad;
-                p.a_slots = L.a_slots; p.b_slots = L.b_slots; p.resident = L.b_resident; p.dbl = L.n1pad <= 128;
+                p.a_slots = L.a_slots; p.b_slots = L.b_slots; p.s_slots = L.s_slots; p.resident = L.b_resident; p.dbl = L.n1pad <= 128;
                 // (without a shortcut the two last clamps are one)
                 p.act1 = L.act; p.act2 = L.skip >= 0 ? L.act2 : std::max(L.act2, L.act3); p.act3 = L.act3;
                 p.idesc1 = make_idesc(std::min(128, L.n1pad)); p.idesc2 = make_idesc(128);
@@ -679,7 +679,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 p.total = mt * L.n_tiles * L.ksplit; p.tile_n = L.tile_n; p.npad = L.npad; p.N = L.K;
                 p.kblocks = L.kblocks; p.stages = L.stages; p.stage_bytes = L.stage_bytes; p.b_resident = L.b_resident; p.b_group = L.b_group;
                 p.acc_stride = L.acc_stride; p.tmem_cols = L.tmem_cols;
-                p.chunk = L.chunk; p.nchunks = L.nchunks; p.box_bytes = L.chunk * 64;
+                p.chunk = L.chunk; p.nchunks = L.nchunks; p.box_bytes = L.chunk * 64; p.s_slots = L.s_slots;
                 // (two clamps in a row with no shortcut between them are one: none < ReLU < ReLU6)
                 p.act = L.skip >= 0 ? L.act : std::max(L.act, L.act2); p.act2 = L.skip >= 0 ? L.act2 : 0; p.out_ctot = L.out_ctot; p.out_f32 = L.out_dtype == XENOS_DTYPE_F32;
                 p.idesc = make_idesc(L.tile_n);
