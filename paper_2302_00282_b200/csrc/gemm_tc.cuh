@@ -1,25 +1,19 @@
-// Linked-chain implicit GEMM on the 5th-generation tensor cores (sm_100a), persistent form.
+// Implicit GEMM on the 5th-generation tensor cores (sm_100a), persistent form, for the operands that the copy engine cannot
+// lay out: windows of an image outside stem_tc_kernel's range, and convolutions with a linked max pool, whose tiles are the
+// pool's patches.  (Also the tensor-core and barrier primitives that the other kernels share.)
 //
-// One CTA per SM walks over the tiles of a chain (tile = 128 output pixels x tile_n <= 256 output
-// channels: the operator split of Section 4.2 of the Xenos paper, output channels first, then
-// rows / columns), so that tensor-memory allocation, barrier set-up and descriptor fetches are
-// paid once and the stages of neighbouring tiles overlap:
-//   warp 0        : TMA producer - weight tiles (128-byte swizzle) and, for linked depthwise
-//                   chains, the input halo tile of the depthwise stage (4-D box, zero fill = padding)
-//   warp 1        : one lane issues tcgen05.mma (bf16 x bf16 -> fp32) into one of two
-//                   tensor-memory accumulators
-//   warps 2..9    : produce the activation operand straight into shared memory in the layout the
-//                   tensor core reads (K-major, 128-byte swizzle) - the paper's "write in the
-//                   order the next operator reads" (Section 4.1)
+// One CTA per SM walks over tiles of 128 output pixels x tile_n <= 256 output channels:
+//   warp 0        : TMA producer - weight tiles (128-byte swizzle) and the image patch of a stem (4-D box, zero fill = padding)
+//   warp 1        : one lane issues tcgen05.mma (bf16 x bf16 -> fp32) into one of two tensor-memory accumulators
+//   warps 2..9    : produce the activation operand straight into shared memory in the layout the tensor core reads (K-major,
+//                   128-byte swizzle) - the paper's "write in the order the next operator reads" (Section 4.1)
 //   warps 10..13  : epilogue of the previous tile, overlapped with the production of the next
 // The activation operand of one 64-wide K block comes from one of
 //   gather : a k x k / strided / padded window of an NHWC bf16 tensor (16-byte cp.async, zero fill)
 //   stem   : a k x k window of a small-channel NCHW image (scalar loads, converted to bf16)
-//   dw     : a depthwise 3x3 + bias + activation computed from the halo tile in shared memory
-// and a second gather segment can append the K blocks of a shortcut 1x1 convolution, so the
-// residual sum of a shortcut connection happens in the accumulator.
-// Epilogues: bias, activation, identity-shortcut add, then a store at a channel offset (concat
-// needs no kernel), a max pool over the tile's patch, or a global average.
+// and a second gather segment can append the K blocks of a shortcut 1x1 convolution, so the residual sum of a shortcut
+// connection happens in the accumulator.  Epilogues: bias, activation, identity-shortcut add, then a store at a channel offset
+// (concat needs no kernel), or a max pool over the tile's patch.
 //
 // Every wait on an mbarrier is bounded; on expiry the role records XENOS_E_TIMEOUT in the status
 // word and leaves through the common exit (tensor memory is always released).
@@ -34,9 +28,8 @@
 
 namespace xk {
 
-enum { GA_NONE = 0, GA_GATHER = 1, GA_STEM = 2, GA_DW = 3 };
-enum { GE_STORE = 0, GE_GAP = 1, GE_POOL = 2 };
-enum { GM_FLAT = 0, GM_PATCH = 1 };
+enum { GA_NONE = 0, GA_GATHER = 1, GA_STEM = 2 };
+enum { GE_STORE = 0, GE_POOL = 2 };
 
 constexpr int kTileM = 128;
 constexpr int kTileK = 64;
@@ -56,8 +49,7 @@ constexpr unsigned kSuspendHintNs = 16000;       // a waiting thread sleeps in h
 
 struct GemmSeg {
     const void *src;
-    const float *dw_w, *dw_b;
-    int mode, C, H, W, k, stride, pad, kelems, kblocks, src_f32, dw_act;
+    int mode, C, H, W, k, stride, pad, kelems, kblocks, src_f32;
 };
 
 struct GemmParams {
@@ -66,38 +58,18 @@ struct GemmParams {
     const __nv_bfloat16 *skip;
     void *out;
     unsigned int *status;
-    int batch, P, Q, rpi;
-    int map_mode, tile_rows;
-    // PATCH tiles: ni images x rh x rw positions of the conv output, origin (ty*step_y - off_y, tx*step_x - off_x)
+    int batch, P, Q;
+    // tiles: ni images x rh x rw positions of the conv output, origin (ty*step_y - off_y, tx*step_x - off_x)
     int ni, rh, rw, tiles_y, tiles_x, step_y, step_x, off_y, off_x;
     int pool_k, pool_stride, PP, PQ, pth, ptw;     // max-pool epilogue: pth x ptw pool outputs per tile
-    int gap_imgs, gap_area, gap_rpi;               // global-average epilogue: whole images per tile (area rows each, rpi of them real)
     int kblocks, stages, tile_n, n_tiles, m_tiles, N;
     int acc_stride, tmem_cols;                     // two accumulators, acc_stride columns apart
-    int hstages, halo_bytes, halo_stride, halo_h, halo_w, halo_cb;   // halo ring (depthwise input tile / stem image patch)
+    int hstages, halo_bytes, halo_stride, halo_h, halo_w;   // ring of image patches
     int stem_tma, stem_align;                       // stem: patch by TMA; x origin alignment in elements
-    // Activation operand by TMA where a K block of it is a box of the NHWC tensor (stride 1, channels a multiple of
-    // 64): 1 = the tile's 128 rows of the [pixels][C] matrix (1x1 convolution, fc), 2 = the tile's rh x rw patch
-    // shifted by the tap (k x k; out-of-range coordinates read zeros, which is the padding).  The copy engine
-    // writes the 128-byte-swizzled operand layout itself and the producer warps have nothing to do.
-    int a_tma, a_box_bytes, a_cpb;                  // a_cpb: 64-channel blocks per tap
     int off_halo, off_stg, off_dww, off_bias, off_bar;   // shared-memory offsets from the 1024-aligned base
     int act, act2, epi, out_ctot, out_coff, out_f32, skip_ctot;
     uint32_t idesc;
-    // reduction split (Section 4.2.2: the C / R / S split, which needs an additional reduction): the K blocks are cut
-    // into ksplit chunks of kb_per blocks; n_tiles counts (channel tile, chunk) pairs, chunk fastest; partial sums go to
-    // split_part [chunk][output pixel][split_ld] as fp32; when all chunks of a tile have arrived (split_cnt), each
-    // chunk's CTA adds the chunks, in ascending order, for its share of the tile's rows
-    int ksplit, kb_per, split_ld;
-    long long split_stride;
-    float *split_part;
-    unsigned int *split_cnt;
     int launch_id;                                  // position of this launch in the plan, reported with a give-up
-    int n_acc;                                      // dwpw_kernel: channel tiles per CTA (2: one 512-column tile in both accumulators)
-    // global average of images with more than 128 pixels (1x1 convolution, rows by TMA): an image is cut into gap_parts
-    // tiles of 128 rows; a tile leaves its column sums in split_part [image][part][split_ld], and the tile that arrives
-    // last at the image's counter (split_cnt) adds the parts in ascending order and stores the mean
-    int gap_parts;
 };
 
 // Status word of a wait that gave up: the code, the role that waited (1 TMA, 2 MMA, 3 producer, 4 producer helping
@@ -150,13 +122,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int lane) {
     int ok = 1;
     if (lane == 0) ok = mbar_wait(bar, parity) ? 1 : 0;
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    return ok != 0;
-}
-// Two barriers, one poller, one broadcast.
-__device__ __forceinline__ bool mbar_wait2_warp(uint32_t bar_a, uint32_t par_a, uint32_t bar_b, uint32_t par_b, int lane) {
-    int ok = 1;
-    if (lane == 0) ok = (mbar_wait(bar_a, par_a) && mbar_wait(bar_b, par_b)) ? 1 : 0;
     ok = __shfl_sync(0xffffffffu, ok, 0);
     return ok != 0;
 }
@@ -272,76 +237,44 @@ struct TileWalk {
     __device__ __forceinline__ void init(const GemmParams &g) {
         ti = (int)blockIdx.x; mt = ti / g.n_tiles; nt = ti - mt * g.n_tiles;
         d_mt = (int)gridDim.x / g.n_tiles; d_nt = (int)gridDim.x - d_mt * g.n_tiles;
-        grp = ty = tx = d_grp = d_ty = d_tx = 0;
-        if (g.map_mode == GM_PATCH) {
-            const int per = g.tiles_y * g.tiles_x;
-            grp = mt / per;
-            int t = mt - grp * per;
-            ty = t / g.tiles_x; tx = t - ty * g.tiles_x;
-            d_grp = d_mt / per;
-            t = d_mt - d_grp * per;
-            d_ty = t / g.tiles_x; d_tx = t - d_ty * g.tiles_x;
-        }
+        const int per = g.tiles_y * g.tiles_x;
+        grp = mt / per;
+        int t = mt - grp * per;
+        ty = t / g.tiles_x; tx = t - ty * g.tiles_x;
+        d_grp = d_mt / per;
+        t = d_mt - d_grp * per;
+        d_ty = t / g.tiles_x; d_tx = t - d_ty * g.tiles_x;
     }
     __device__ __forceinline__ void next(const GemmParams &g) {
         ti += (int)gridDim.x; mt += d_mt; nt += d_nt;
         int carry = 0;
         if (nt >= g.n_tiles) { nt -= g.n_tiles; ++mt; carry = 1; }
-        if (g.map_mode == GM_PATCH) {
-            tx += d_tx + carry;
-            if (tx >= g.tiles_x) { tx -= g.tiles_x; ++ty; }
-            ty += d_ty;
-            if (ty >= g.tiles_y) { ty -= g.tiles_y; ++grp; }
-            grp += d_grp;
-        }
+        tx += d_tx + carry;
+        if (tx >= g.tiles_x) { tx -= g.tiles_x; ++ty; }
+        ty += d_ty;
+        if (ty >= g.tiles_y) { ty -= g.tiles_y; ++grp; }
+        grp += d_grp;
     }
 };
-
-// (channel tile, K chunk) of a tile: n_tiles counts pairs when the reduction is split.
-struct TileK { int nt, kb0, kb1, ks; };
-template <int kSplit>
-__device__ __forceinline__ TileK tile_k(const GemmParams &g, int ntv) {
-    TileK t;
-    t.nt = ntv; t.ks = 0; t.kb0 = 0; t.kb1 = g.kblocks;
-    if (kSplit && g.ksplit > 1) {
-        t.nt = ntv / g.ksplit; t.ks = ntv - t.nt * g.ksplit;
-        t.kb0 = t.ks * g.kb_per; t.kb1 = min(g.kblocks, t.kb0 + g.kb_per);
-    }
-    return t;
-}
 
 // Position of tile row r inside a patch tile: fixed for a thread over the whole kernel.
 struct RowLocal { int img, dy, dx; };
 
 __device__ __forceinline__ RowLocal row_local(const GemmParams &g, int r) {
     RowLocal l;
-    l.img = 0; l.dy = 0; l.dx = 0;
-    if (g.map_mode == GM_PATCH) {
-        const int area = g.rh * g.rw;
-        l.img = r / area;
-        const int rem = r - l.img * area;
-        l.dy = rem / g.rw; l.dx = rem - l.dy * g.rw;
-    }
+    const int area = g.rh * g.rw;
+    l.img = r / area;
+    const int rem = r - l.img * area;
+    l.dy = rem / g.rw; l.dx = rem - l.dy * g.rw;
     return l;
 }
 
 __device__ __forceinline__ RowPos map_row(const GemmParams &g, const TileWalk &w, const RowLocal &l, int r) {
     RowPos o;
-    o.valid = 0; o.n = 0; o.p = 0; o.q = 0;
-    if (g.map_mode == GM_FLAT) {
-        const unsigned m = (unsigned)w.mt * (unsigned)g.tile_rows + (unsigned)r;     // < 2^31 rows by construction
-        if (r < g.tile_rows && m < (unsigned)g.batch * (unsigned)g.rpi) {
-            o.n = (int)(m / (unsigned)g.rpi);
-            const int rem = (int)(m - (unsigned)o.n * (unsigned)g.rpi);
-            o.p = rem / g.Q; o.q = rem - o.p * g.Q;
-            o.valid = 1;
-        }
-    } else {
-        o.n = w.grp * g.ni + l.img;
-        o.p = w.ty * g.step_y - g.off_y + l.dy;
-        o.q = w.tx * g.step_x - g.off_x + l.dx;
-        o.valid = (l.img < g.ni) && o.n < g.batch && o.p >= 0 && o.p < g.P && o.q >= 0 && o.q < g.Q;
-    }
+    o.n = w.grp * g.ni + l.img;
+    o.p = w.ty * g.step_y - g.off_y + l.dy;
+    o.q = w.tx * g.step_x - g.off_x + l.dx;
+    o.valid = (l.img < g.ni) && o.n < g.batch && o.p >= 0 && o.p < g.P && o.q >= 0 && o.q < g.Q;
     return o;
 }
 
@@ -540,114 +473,10 @@ __device__ __forceinline__ void produce_stem_direct(const GemmSeg &sg, int kb_lo
     }
 }
 
-// depthwise 3x3 + bias + activation from the halo tile in shared memory ([image][y][x][cb channels],
-// dense bf16), rounded to bf16 and stored in the consumer's operand layout.
-// A thread owns a BR x 4 block of output pixels for FOUR channels: it walks the block's input window
-// once with 8-byte loads (every input value is read once per block and feeds up to 3 * BR outputs)
-// and keeps the 36 tap weights in registers.  A 64-channel K block has 16 channel quads, so the 256
-// producer threads cover 16 blocks of 2 x 4 pixels; with 32 or fewer channels per K block they
-// cover 32 blocks of 1 x 4.
-struct DwUnit {
-    int q;          // channel quad inside the K block
-    int base;       // byte offset of the window origin in the halo tile (channel offset included)
-    int row0;       // tile row of the block's top-left output pixel
-    int nrows;      // live output rows of the block (the tile may end inside it)
-    int live;
-};
-
-// The unit of producer thread pt: (pixel block, channel quad) of the tile's depthwise stage.
-__device__ __forceinline__ DwUnit make_dw_unit(const GemmParams &g, int pt, int dw_quads, int dw_br) {
-    DwUnit du;
-    du.q = pt & (dw_quads - 1);
-    const int blk = pt / dw_quads;               // (image, block row, block column)
-    const int upr = g.rw >> 2, upi = ((g.rh + dw_br - 1) / dw_br) * upr;
-    const int img = blk / upi, rem = blk - img * upi;
-    const int uy = rem / upr, ux = rem - uy * upr;
-    const int S = g.seg[0].stride;
-    du.live = img < g.ni && du.q * 4 < g.halo_cb;
-    du.base = ((img * g.halo_h + dw_br * uy * S) * g.halo_w + 4 * ux * S) * g.halo_cb * 2 + du.q * 8;
-    du.row0 = img * g.rh * g.rw + dw_br * uy * g.rw + 4 * ux;
-    du.nrows = min(dw_br, max(0, g.rh - dw_br * uy));
-    return du;
-}
-
 __device__ __forceinline__ uint32_t clamp_bf16x2(uint32_t v, uint32_t lo, uint32_t hi) {
     __nv_bfloat162 x = *reinterpret_cast<__nv_bfloat162 *>(&v);
     x = __hmin2(__hmax2(x, *reinterpret_cast<__nv_bfloat162 *>(&lo)), *reinterpret_cast<__nv_bfloat162 *>(&hi));
     return *reinterpret_cast<uint32_t *>(&x);
-}
-
-template <int S, int BR>
-__device__ __forceinline__ void produce_dw(const GemmSeg &sg, const GemmParams &g, int kb_local, uint32_t halo, uint32_t dww,
-                                           const DwUnit &u, uint32_t a_base) {
-    if (!u.live) return;
-    const int c0 = kb_local * kTileK + u.q * 4;
-    const uint32_t half = (uint32_t)(u.q & 1) * 8u;      // which 8 bytes of the 16-byte chunk
-    const int j = u.q >> 1;
-    if (c0 >= sg.C) {
-        // K padding inside the block: zeros, so that the zero weights there never meet a NaN
-        for (int a = 0; a < u.nrows; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int r = u.row0 + a * g.rw + b;
-                asm volatile("st.shared.v2.b32 [%0], {%1, %1};" ::"r"(a_chunk_addr(a_base, r, j) + half), "r"(0u) : "memory");
-            }
-        return;
-    }
-    // tap weights [9][C] and the bias [C] were staged in shared memory when the CTA started
-    float2 w[9][2];
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-        const float4 wv = ld_shared_f4(dww + (uint32_t)(t * sg.C + c0) * 4u);
-        w[t][0] = make_float2(wv.x, wv.y); w[t][1] = make_float2(wv.z, wv.w);
-    }
-    float2 acc[BR][4][2];
-    {
-        const float4 bv = ld_shared_f4(dww + (uint32_t)(9 * sg.C + c0) * 4u);
-#pragma unroll
-        for (int a = 0; a < BR; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) { acc[a][b][0] = make_float2(bv.x, bv.y); acc[a][b][1] = make_float2(bv.z, bv.w); }
-    }
-    const uint32_t hb = halo + u.base;
-    const int cbytes = g.halo_cb * 2;
-#pragma unroll
-    for (int iy = 0; iy < (BR - 1) * S + 3; ++iy) {
-#pragma unroll
-        for (int ci = 0; ci < 3 * S + 3; ++ci) {
-            uint32_t r0, r1;
-            asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(hb + (uint32_t)((iy * g.halo_w + ci) * cbytes)));
-            const float2 x0 = make_float2(__uint_as_float(r0 << 16), __uint_as_float(r0 & 0xffff0000u));
-            const float2 x1 = make_float2(__uint_as_float(r1 << 16), __uint_as_float(r1 & 0xffff0000u));
-#pragma unroll
-            for (int ry = 0; ry < 3; ++ry) {
-                if ((iy - ry) % S != 0 || iy - ry < 0 || (iy - ry) / S >= BR) continue;      // resolved at compile time
-                const int a = (iy - ry) / S;
-#pragma unroll
-                for (int sx = 0; sx < 3; ++sx) {
-                    if ((ci - sx) % S != 0 || ci - sx < 0 || (ci - sx) / S >= 4) continue;
-                    const int b = (ci - sx) / S;
-                    acc[a][b][0] = __ffma2_rn(x0, w[ry * 3 + sx][0], acc[a][b][0]);
-                    acc[a][b][1] = __ffma2_rn(x1, w[ry * 3 + sx][1], acc[a][b][1]);
-                }
-            }
-        }
-    }
-    // round to bf16, then clamp: the bounds 0 and 6 are bf16 values and rounding is monotonic, so
-    // this equals clamping first
-    const uint32_t lo = sg.dw_act >= 1 ? 0u : 0xff80ff80u;              // 0 | -inf, as bf16 pairs
-    const uint32_t hi = sg.dw_act == 2 ? 0x40c040c0u : 0x7f807f80u;     // 6 | +inf
-#pragma unroll
-    for (int a = 0; a < BR; ++a) {
-        if (a >= u.nrows) break;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int r = u.row0 + a * g.rw + b;
-            const uint32_t p0 = clamp_bf16x2(pack2(acc[a][b][0].x, acc[a][b][0].y), lo, hi);
-            const uint32_t p1 = clamp_bf16x2(pack2(acc[a][b][1].x, acc[a][b][1].y), lo, hi);
-            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a_chunk_addr(a_base, r, j) + half), "r"(p0), "r"(p1) : "memory");
-        }
-    }
 }
 
 // The common store epilogue (bias, one activation as a clamp, bf16) for the 16-column chunks
@@ -684,33 +513,6 @@ __device__ __forceinline__ void store_chunks(const GemmParams &g, uint32_t t_lan
                 if (nc + 16 <= g.N) *reinterpret_cast<uint4 *>(o + 8) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
             }
         }
-    }
-}
-
-// Four adjacent columns of one output pixel: bias, activation, identity-shortcut add, second activation, store.
-// (nc is a multiple of 4 and channel counts are multiples of 8, so the four columns are inside the tensor or, for
-// fp32 vector outputs, checked one by one.)
-__device__ __forceinline__ void finish_store4(const GemmParams &g, float4 a, const float4 bz, int nc, size_t pix) {
-    const float lo1 = act_lo(g.act), hi1 = act_hi(g.act), lo2 = act_lo(g.act2), hi2 = act_hi(g.act2);
-    float v[4] = {a.x + bz.x, a.y + bz.y, a.z + bz.z, a.w + bz.w};
-#pragma unroll
-    for (int c = 0; c < 4; ++c) v[c] = fminf(fmaxf(v[c], lo1), hi1);
-    if (g.skip) {
-        const uint2 sk = __ldg(reinterpret_cast<const uint2 *>(g.skip + pix * g.skip_ctot + nc));
-        v[0] += __uint_as_float(sk.x << 16); v[1] += __uint_as_float(sk.x & 0xffff0000u);
-        v[2] += __uint_as_float(sk.y << 16); v[3] += __uint_as_float(sk.y & 0xffff0000u);
-    }
-    if (g.act2) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = fminf(fmaxf(v[c], lo2), hi2);
-    }
-    if (g.out_f32) {
-        float *o = reinterpret_cast<float *>(g.out) + pix * g.out_ctot + g.out_coff + nc;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) if (nc + c < g.N) o[c] = v[c];
-    } else {
-        __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(g.out) + pix * g.out_ctot + g.out_coff + nc;
-        *reinterpret_cast<uint2 *>(o) = make_uint2(pack2(v[0], v[1]), pack2(v[2], v[3]));
     }
 }
 
@@ -770,9 +572,6 @@ __global__ void wait_expiry_probe_kernel(unsigned int *status, int polls) {
 }
 
 // ---- the kernel --------------------------------------------------------------------------------
-// kSplit = 1: the instance that also carries the reduction-split path (launches with ksplit > 1 use it; the
-// common instance is compiled without that code).
-template <int kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmH, const GemmParams g) {
     extern __shared__ uint8_t smem_raw[];
@@ -799,23 +598,18 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int total_tiles = g.m_tiles * g.n_tiles;
-    const bool dw_mode = g.seg[0].mode == GA_DW;
     // gather stages complete through cp.async arrivals (one per thread); the others through one
     // arrival per producer warp
-    const bool tma_a = g.a_tma != 0;
     const bool async_gather = g.seg[0].mode == GA_GATHER;
-    // depthwise: the producer threads are (pixel block, channel quad of the K block) pairs
-    const int dw_quads = g.halo_cb > 32 ? 16 : 8;
-    const int dw_br = g.halo_cb > 32 ? 2 : 1;       // block rows
     // On a CTA's last tile the producer warps take two thirds of the columns of a plain store epilogue.
-    const bool help_last = g.epi == GE_STORE && !g.skip && !g.act2 && !g.out_f32 && g.tile_n >= 96 && g.ksplit <= 1;
+    const bool help_last = g.epi == GE_STORE && !g.skip && !g.act2 && !g.out_f32 && g.tile_n >= 96;
     const int help_per = (((g.tile_n / 16) + 2) / 3 + 1) & ~1;      // 16-column chunks per sharing warp, even
 
     if (threadIdx.x == 0) {
         // arrivals on a stage's "full" barrier: the TMA lane plus the producers of that stage (every
         // thread for cp.async gathers, every warp otherwise)
         const uint32_t prod_warps = kProducerThreads / 32;
-        const uint32_t full_count = tma_a ? 1u : (async_gather ? kProducerThreads : prod_warps) + 1;
+        const uint32_t full_count = (async_gather ? kProducerThreads : prod_warps) + 1;
         for (int s = 0; s < g.stages; ++s) { mbar_init(full_bar(s), full_count); mbar_init(empty_bar(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), kEpilogueThreads / 32); }
         for (int s = 0; s < g.hstages; ++s) { mbar_init(hfull_bar(s), 1); mbar_init(hempty_bar(s), prod_warps); }
@@ -823,7 +617,7 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
         *fail_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
-        if (dw_mode || g.stem_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmH) : "memory");
+        if (g.stem_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmH) : "memory");
     }
     if (warp == 0) {
         // The TMA lane needs the barriers only: warp 0 signals that they exist and goes straight to its
@@ -834,14 +628,6 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"((uint32_t)g.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (dw_mode && threadIdx.x >= 64 && threadIdx.x < 64 + kProducerThreads) {
-        // depthwise tap weights [9][C] followed by the bias [C], fp32, once per CTA
-        const int C = g.seg[0].C;
-        float4 *dst = reinterpret_cast<float4 *>(sm + g.off_dww);
-        const float4 *w4 = reinterpret_cast<const float4 *>(g.seg[0].dw_w), *b4 = reinterpret_cast<const float4 *>(g.seg[0].dw_b);
-        for (int i = threadIdx.x - 64; i < 9 * C / 4; i += kProducerThreads) dst[i] = __ldg(w4 + i);
-        for (int i = threadIdx.x - 64; i < C / 4; i += kProducerThreads) dst[9 * C / 4 + i] = __ldg(b4 + i);
     }
     if (g.stem_tma && threadIdx.x >= 64 && threadIdx.x < 64 + kProducerThreads) {
         const int C = g.seg[0].C, k = g.seg[0].k;
@@ -872,13 +658,13 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
     if (warp != 1) pdl_wait();
 
     if (warp == 0) {
-        // ---- TMA: weight tiles, and the depthwise halo tiles ----
+        // ---- TMA: weight tiles and the image patches of a stem ----
         if (lane == 0) {
             TileWalk w;
             w.init(g);
             Ring st = {0, 0u}, hr = {0, 0u};
             for (; w.ti < total_tiles && ok; w.next(g)) {
-                // input origin of the tile's patch (depthwise halo / stem image patch)
+                // input origin of the tile's image patch
                 const int hn = w.grp * g.ni;
                 const int hy = (w.ty * g.step_y - g.off_y) * g.seg[0].stride - g.seg[0].pad;
                 const int hx = (w.tx * g.step_x - g.off_x) * g.seg[0].stride - g.seg[0].pad;
@@ -891,28 +677,11 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
                     tma_load_4d(sbase + g.off_halo + hr.s * g.halo_stride, &tmH, hx & ~(g.stem_align - 1), hy, 0, hn, hfull_bar(hr.s));
                     hr.next(g.hstages);
                 }
-                const TileK tk = tile_k<kSplit>(g, w.nt);
-                for (int kb = tk.kb0; kb < tk.kb1 && ok; ++kb) {
-                    if (dw_mode) {
-                        ok = mbar_wait(hempty_bar(hr.s), hr.ph ^ 1u);
-                        if (!ok) break;
-                        mbar_arrive_expect_tx(hfull_bar(hr.s), (uint32_t)g.halo_bytes);
-                        tma_load_4d(sbase + g.off_halo + hr.s * g.halo_stride, &tmH, kb * kTileK, hx, hy, hn, hfull_bar(hr.s));
-                        hr.next(g.hstages);
-                    }
+                for (int kb = 0; kb < g.kblocks && ok; ++kb) {
                     ok = mbar_wait(empty_bar(st.s), st.ph ^ 1u);
                     if (!ok) break;
-                    mbar_arrive_expect_tx(full_bar(st.s), (uint32_t)g.tile_n * 128u + (tma_a ? (uint32_t)g.a_box_bytes : 0u));
-                    if (g.a_tma == 1) {
-                        const int arow = (kSplit && g.gap_parts > 1) ? (w.mt / g.gap_parts) * g.gap_rpi + (w.mt % g.gap_parts) * kTileM : w.mt * g.tile_rows;
-                        tma_load_2d(sbase + st.s * stage_bytes, &tmH, kb * kTileK, arow, full_bar(st.s));
-                    } else if (g.a_tma == 2) {
-                        const int tap = kb / g.a_cpb, cb = kb - tap * g.a_cpb;
-                        const int tr = tap / g.seg[0].k, ts = tap - tr * g.seg[0].k;
-                        tma_load_4d(sbase + st.s * stage_bytes, &tmH, cb * kTileK, w.tx * g.step_x - g.off_x + ts - g.seg[0].pad,
-                                    w.ty * g.step_y - g.off_y + tr - g.seg[0].pad, hn, full_bar(st.s));
-                    }
-                    tma_load_2d(sbase + st.s * stage_bytes + kABytes, &tmB, kb * kTileK, tk.nt * g.tile_n, full_bar(st.s));
+                    mbar_arrive_expect_tx(full_bar(st.s), (uint32_t)g.tile_n * 128u);
+                    tma_load_2d(sbase + st.s * stage_bytes + kABytes, &tmB, kb * kTileK, w.nt * g.tile_n, full_bar(st.s));
                     st.next(g.stages);
                 }
             }
@@ -929,8 +698,7 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + b * g.acc_stride;
-                const TileK tk = tile_k<kSplit>(g, kSplit ? ti % g.n_tiles : 0);
-                for (int kb = tk.kb0; kb < tk.kb1 && ok; ++kb) {
+                for (int kb = 0; kb < g.kblocks && ok; ++kb) {
                     const int s = st.s;
                     ok = mbar_wait(full_bar(s), st.ph);
                     if (!ok) break;
@@ -943,7 +711,7 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
 #pragma unroll
                     for (int k4 = 0; k4 < kTileK / 16; ++k4)
                         umma_bf16(d_tmem, umma_desc_sw128(a + k4 * 32), umma_desc_sw128(bb + k4 * 32), g.idesc,
-                                  (kb > tk.kb0 || k4 > 0) ? 1u : 0u);
+                                  (kb > 0 || k4 > 0) ? 1u : 0u);
                     umma_commit(empty_bar(s));
                 }
                 if (ok) {
@@ -957,24 +725,6 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
         // ---- activation operand ----
         const int pt = threadIdx.x - 64;                 // 0..255
         const int grow = pt & 127, gpart = pt >> 7;      // gather / stem mapping
-        DwUnit du;
-        du.q = 0; du.base = 0; du.row0 = 0; du.nrows = 0; du.live = 0;
-        int zero_from = 8;                               // chunks >= zero_from of every row are K padding
-        if (dw_mode) {
-            zero_from = g.halo_cb >> 3;
-            du = make_dw_unit(g, pt, dw_quads, dw_br);
-        }
-        // K-padding chunks of a depthwise stage are only ever written with zeros: when no other
-        // producer shares the ring they are cleared once, here, instead of with every K block
-        const bool zero_once = dw_mode && g.seg[1].mode == GA_NONE;
-        if (zero_once && zero_from < 8) {
-            const int nz = 8 - zero_from;
-            for (int idx = pt; idx < g.stages * kTileM * nz; idx += kProducerThreads) {
-                const int sr = idx / nz, jj = zero_from + idx - sr * nz, s = sr / kTileM, row = sr - s * kTileM;
-                st_shared16(a_chunk_addr(sbase + s * stage_bytes, row, jj), make_uint4(0u, 0u, 0u, 0u));
-            }
-            fence_proxy_async();      // ordered before every later arrival of this thread
-        }
         const RowLocal rl = row_local(g, grow);
         TileWalk w;
         w.init(g);
@@ -1012,46 +762,14 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
                 if (ok) warp_arrive(hempty_bar(shs), lane);      // the image patch has been read
             }
         }
-        if (dw_mode) {
-            // ---- depthwise stage of a linked chain: every K block comes from a halo tile ----
-            const uint32_t dww = sbase + g.off_dww;
-            const GemmSeg &sg = g.seg[0];
-            for (; w.ti < total_tiles && ok; w.next(g)) {
-                const TileK tk = tile_k<kSplit>(g, w.nt);
-                for (int kb = tk.kb0; kb < tk.kb1 && ok; ++kb) {
-                    const int s = st.s, hs = hr.s;
-                    ok = mbar_wait2_warp(empty_bar(s), st.ph ^ 1u, hfull_bar(hs), hr.ph, lane);
-                    if (!ok) break;
-                    st.next(g.stages); hr.next(g.hstages);
-                    const uint32_t a_base = sbase + s * stage_bytes, halo = sbase + g.off_halo + hs * g.halo_stride;
-                    if (dw_br == 2) {
-                        if (sg.stride == 1) produce_dw<1, 2>(sg, g, kb, halo, dww, du, a_base);
-                        else produce_dw<2, 2>(sg, g, kb, halo, dww, du, a_base);
-                    } else {
-                        if (sg.stride == 1) produce_dw<1, 1>(sg, g, kb, halo, dww, du, a_base);
-                        else produce_dw<2, 1>(sg, g, kb, halo, dww, du, a_base);
-                    }
-                    // K padding: chunks the block's channels do not reach must be zero, not stale
-                    if (!zero_once)
-                        for (int idx = pt; idx < kTileM * (8 - zero_from); idx += kProducerThreads) {
-                            const int row = idx / (8 - zero_from), jj = zero_from + idx - row * (8 - zero_from);
-                            st_shared16(a_chunk_addr(a_base, row, jj), make_uint4(0u, 0u, 0u, 0u));
-                        }
-                    fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) { mbar_arrive(full_bar(s)); mbar_arrive(hempty_bar(hs)); }     // stage filled, halo tile read
-                }
-            }
-        }
         // ---- general form: gathers (one or two K segments), direct stem loads ----
         const int grow0 = pt >> 3, gj = pt & 7;          // gather mapping: rows grow0 + 32 i, chunk gj
         RowLocal grl[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) grl[i] = row_local(g, grow0 + 32 * i);
-        for (; !g.stem_tma && !dw_mode && !tma_a && w.ti < total_tiles && ok; w.next(g)) {
+        for (; !g.stem_tma && w.ti < total_tiles && ok; w.next(g)) {
             RowPos rp;
             rp.valid = 0; rp.n = 0; rp.p = 0; rp.q = 0;
-            const TileK tk = tile_k<kSplit>(g, w.nt);
             if (g.seg[0].mode == GA_STEM) rp = map_row(g, w, rl, grow);
             GatherRow gr0[4], gr1[4];
             GatherState gs0 = {0, 0, 0}, gs1 = {0, 0, 0};
@@ -1062,14 +780,10 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
                     gr0[i] = gather_row(g.seg[0], r4);
                     gr1[i] = gather_row(g.seg[1], r4);       // (unused without a second segment)
                 }
-                if (gj + 8 * tk.kb0) gather_advance(gs0, gj + 8 * tk.kb0, g.seg[0].C >> 3, g.seg[0].k);
-                if (g.seg[1].mode == GA_GATHER) {
-                    // (a chunk of a split reduction may begin inside the second segment)
-                    const int adv = gj + 8 * max(0, tk.kb0 - g.seg[0].kblocks);
-                    if (adv) gather_advance(gs1, adv, g.seg[1].C >> 3, g.seg[1].k);
-                }
+                if (gj) gather_advance(gs0, gj, g.seg[0].C >> 3, g.seg[0].k);
+                if (g.seg[1].mode == GA_GATHER && gj) gather_advance(gs1, gj, g.seg[1].C >> 3, g.seg[1].k);
             }
-            for (int kb = tk.kb0; kb < tk.kb1 && ok; ++kb) {
+            for (int kb = 0; kb < g.kblocks && ok; ++kb) {
                 const int s = st.s;
                 const uint32_t sph = st.ph;
                 st.next(g.stages);
@@ -1125,12 +839,11 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
         const int row = quarter * 32 + lane;
         const int et = threadIdx.x - (64 + kProducerThreads);      // 0..127
         const uint32_t stg = sbase + g.off_stg;
-        float *stgf = reinterpret_cast<float *>(sm + g.off_stg);
         const int pool_pitch = g.tile_n * 2 + 16;
         const int nchunks = g.tile_n / 16;
         const float lo1 = act_lo(g.act), hi1 = act_hi(g.act), lo2 = act_lo(g.act2), hi2 = act_hi(g.act2);
         // the common epilogue (bias, one activation, bf16 store or pool) runs on packed pairs
-        const bool fast = !g.skip && !g.act2 && !g.out_f32 && g.epi != GE_GAP;
+        const bool fast = !g.skip && !g.act2 && !g.out_f32;
         const uint32_t plo = g.act >= 1 ? 0u : 0xff80ff80u, phi = g.act == 2 ? 0x40c040c0u : 0x7f807f80u;
         // 32-byte stores need a 32-byte aligned row start and column offset
         const bool wide_ok = ((reinterpret_cast<uintptr_t>(g.out) | (uintptr_t)(g.out_ctot * 2) | (uintptr_t)(g.out_coff * 2)) & 31u) == 0;
@@ -1139,9 +852,7 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
         w.init(g);
         int i = 0, bias_nt = -1, bias_buf = 0;
         for (; w.ti < total_tiles; w.next(g), ++i) {
-            const TileK tk = tile_k<kSplit>(g, w.nt);
-            const int mt = w.mt, nt = tk.nt;
-            const int b = i & 1;
+            const int nt = w.nt, b = i & 1;
             // the bias slice of this channel tile goes to shared memory when the channel tile changes
             // (two buffers: a warp is at most one tile ahead of the others)
             const bool new_bias = nt != bias_nt;
@@ -1151,10 +862,7 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
                     *reinterpret_cast<float4 *>(sm + g.off_bias + bias_buf * 1024 + et * 16) = __ldg(reinterpret_cast<const float4 *>(g.bias + nt * g.tile_n) + et);
             }
             const uint32_t sbias = sbase + g.off_bias + bias_buf * 1024;
-            RowPos rq = map_row(g, w, rl, row);
-            const bool gparts = kSplit && g.gap_parts > 1;
-            const int gp_img = gparts ? mt / g.gap_parts : 0, gp_t = gparts ? mt - gp_img * g.gap_parts : 0;
-            if (gparts) rq.valid = gp_t * kTileM + row < g.gap_rpi;      // rows of this image inside this tile
+            const RowPos rq = map_row(g, w, rl, row);
             const int n0 = nt * g.tile_n;
             const size_t pix = ((size_t)rq.n * g.P + rq.p) * g.Q + rq.q;
             // The four epilogue warps share named barriers (bias slice, pool and average staging), so they
@@ -1165,70 +873,6 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
             if (*fail_flag) { ok = false; break; }
             tc_fence_after();
             const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * g.acc_stride;
-            if (kSplit && g.ksplit > 1) {
-                // ---- reduction split: park this chunk's fp32 partial sums
-                float *part = g.split_part + (size_t)tk.ks * g.split_stride + pix * g.split_ld + n0;
-                for (int cbase = 0; cbase < nchunks; cbase += 2) {
-                    float vv[32];
-                    const int nsub = (cbase + 1 < nchunks) ? 2 : 1;
-                    if (nsub == 2) tmem_ld32(t_lane + cbase * 16, vv); else tmem_ld16(t_lane + cbase * 16, vv);
-                    if (cbase + nsub >= nchunks) {
-                        tc_fence_before();
-                        warp_arrive(acce_bar(b), lane);
-                    }
-                    if (rq.valid)
-#pragma unroll
-                        for (int q4 = 0; q4 < 32; q4 += 4)
-                            if (q4 < nsub * 16) __stcg(reinterpret_cast<float4 *>(part + cbase * 16 + q4), make_float4(vv[q4], vv[q4 + 1], vv[q4 + 2], vv[q4 + 3]));
-                }
-                // Every chunk's CTA then adds the partial sums of ITS share of the tile's rows, chunks in ascending order
-                // (a fixed order: the result does not depend on which CTA arrives when): the reduction's traffic
-                // is spread over the CTAs that made the partial sums, and every load is a coalesced 16 bytes.
-                __threadfence();
-                epi_bar();
-                unsigned int *cnt = g.split_cnt + 2 * ((size_t)mt * (g.n_tiles / g.ksplit) + nt);      // [arrived, reduced]
-                if (et == 0) {
-                    atomicAdd(cnt, 1u);
-                    int seen = 0;
-                    // the other chunks of this tile are consecutive tiles of the walk: they run on other units now, or
-                    // on units that are finishing an earlier tile (a wait never points at a later tile, so waits cannot
-                    // form a cycle); bounded like every other wait
-                    for (int spin = 0; spin < (1 << 22); ++spin) {
-                        if (*reinterpret_cast<volatile unsigned int *>(cnt) >= (unsigned int)g.ksplit) { seen = 1; break; }
-                        __nanosleep(64);
-                    }
-                    fail_flag[1] = seen;
-                    if (!seen) *fail_flag = 1;
-                }
-                epi_bar();
-                if (!fail_flag[1]) { ok = false; break; }
-                __threadfence();
-                {
-                    const int rows_per = (kTileM + g.ksplit - 1) / g.ksplit;
-                    const int r0 = tk.ks * rows_per, r1 = min(kTileM, r0 + rows_per);
-                    const int c4n = g.tile_n >> 2;
-                    for (int idx = et; idx < (r1 - r0) * c4n; idx += kEpilogueThreads) {
-                        const int rr = r0 + idx / c4n, c4 = idx - (rr - r0) * c4n;
-                        const RowPos rp = map_row(g, w, row_local(g, rr), rr);
-                        const int nc = n0 + c4 * 4;
-                        if (!rp.valid || nc >= g.N) continue;
-                        const size_t px = ((size_t)rp.n * g.P + rp.p) * g.Q + rp.q;
-                        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-                        for (int sp = 0; sp < g.ksplit; ++sp) {
-                            const float4 x4 = __ldcg(reinterpret_cast<const float4 *>(g.split_part + (size_t)sp * g.split_stride + px * g.split_ld + nc));
-                            a.x += x4.x; a.y += x4.y; a.z += x4.z; a.w += x4.w;
-                        }
-                        finish_store4(g, a, ld_shared_f4(sbias + (uint32_t)(c4 * 16)), nc, px);
-                    }
-                }
-                epi_bar();
-                if (et == 0) {
-                    __threadfence();
-                    const unsigned int old = atomicAdd(cnt + 1, 1u);
-                    if (old == (unsigned int)(g.ksplit - 1)) { cnt[0] = 0u; cnt[1] = 0u; }      // all have read: ready for the next run
-                }
-                continue;
-            }
             // (on the CTA's last tile the producer warps store the columns behind help_per)
             const int nchunks_own = (help_last && w.ti + (int)gridDim.x >= total_tiles) ? min(nchunks, help_per) : nchunks;
             for (int cbase = 0; cbase < nchunks_own; cbase += 2) {
@@ -1281,7 +925,7 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
                         continue;
                     }
                     if (g.epi == GE_STORE) { finish_store16(g, v, sbias, ch, nc, rq, pix); continue; }
-                    // (pool and global-average tiles: bias, activation, [identity shortcut, activation], values kept)
+                    // (pool tiles: bias, activation, [identity shortcut, activation], values kept)
 #pragma unroll
                     for (int q4 = 0; q4 < 16; q4 += 4) {
                         const float4 bz = ld_shared_f4(sbias + (uint32_t)(ch * 16 + q4) * 4u);
@@ -1309,78 +953,7 @@ gemm_chain_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant
                         st_shared16(stg + row * pool_pitch + ch * 32, pack8(lo));
                         st_shared16(stg + row * pool_pitch + ch * 32 + 16, pack8(hi));
                     }
-                    // (global average: the activated values stay in vv for the reduction below)
                 }
-                if (g.epi == GE_GAP) {
-                    // global average of up to 32 columns through shared memory: every thread parks its
-                    // row, then (image, column, part) items sum the rows r = part, part + parts, ... in
-                    // ascending order and the parts are added in ascending order: a fixed order
-                    const int ncols = nsub * 16, nc0 = n0 + cbase * 16;
-                    const int per = g.gap_imgs * 32;
-                    const int parts = per >= 128 ? 1 : (per >= 64 ? 2 : 4);
-                    float *part = stgf + kTileM * 33;
-                    epi_bar();          // the previous slab's readers are done
-#pragma unroll
-                    for (int c = 0; c < 32; ++c)
-                        if (c < ncols) stgf[row * 33 + c] = rq.valid ? vv[c] : 0.0f;
-                    epi_bar();
-                    for (int item = et; item < per * parts; item += kEpilogueThreads) {
-                        const int c = item & 31, rest = item >> 5;
-                        const int img = rest / parts, pa = rest - img * parts;
-                        float acc = 0.0f;
-                        if (c < ncols)
-                            for (int r = pa; r < g.gap_area; r += parts) acc += stgf[(img * g.gap_area + r) * 33 + c];
-                        if (parts > 1) { part[item] = acc; continue; }
-                        const int n = mt * g.gap_imgs + img;
-                        if (c >= ncols || n >= g.batch || nc0 + c >= g.N) continue;
-                        acc /= (float)g.gap_rpi;
-                        const size_t oi = (size_t)n * g.out_ctot + g.out_coff + nc0 + c;
-                        if (g.out_f32) reinterpret_cast<float *>(g.out)[oi] = acc;
-                        else reinterpret_cast<__nv_bfloat16 *>(g.out)[oi] = __float2bfloat16_rn(acc);
-                    }
-                    if (parts > 1) {
-                        epi_bar();
-                        for (int item = et; item < per; item += kEpilogueThreads) {
-                            const int c = item & 31, img = item >> 5;
-                            const int n = gparts ? gp_img : mt * g.gap_imgs + img;
-                            if (c >= ncols || n >= g.batch || nc0 + c >= g.N) continue;
-                            float acc = 0.0f;
-                            for (int pa = 0; pa < parts; ++pa) acc += part[((img * parts + pa) << 5) + c];
-                            if (gparts) {
-                                // this tile's share of the image's column sum
-                                __stcg(g.split_part + ((size_t)gp_img * g.gap_parts + gp_t) * g.split_ld + nc0 + c, acc);
-                                continue;
-                            }
-                            acc /= (float)g.gap_rpi;
-                            const size_t oi = (size_t)n * g.out_ctot + g.out_coff + nc0 + c;
-                            if (g.out_f32) reinterpret_cast<float *>(g.out)[oi] = acc;
-                            else reinterpret_cast<__nv_bfloat16 *>(g.out)[oi] = __float2bfloat16_rn(acc);
-                        }
-                    }
-                }
-            }
-            if (gparts) {
-                // the image's tiles meet at its counter; the one that arrives last adds the parts in ascending order
-                __threadfence();
-                epi_bar();
-                unsigned int *cnt = g.split_cnt + 2 * ((size_t)gp_img * g.n_tiles + nt);
-                if (et == 0) fail_flag[1] = atomicAdd(cnt, 1u) == (unsigned int)(g.gap_parts - 1) ? 1 : 0;
-                epi_bar();
-                if (fail_flag[1]) {
-                    __threadfence();
-                    for (int col = et; col < g.tile_n; col += kEpilogueThreads) {
-                        const int nc = n0 + col;
-                        if (nc >= g.N || gp_img >= g.batch) continue;
-                        float acc = 0.0f;
-                        for (int t = 0; t < g.gap_parts; ++t) acc += __ldcg(g.split_part + ((size_t)gp_img * g.gap_parts + t) * g.split_ld + nc);
-                        acc /= (float)g.gap_rpi;
-                        const size_t oi = (size_t)gp_img * g.out_ctot + g.out_coff + nc;
-                        if (g.out_f32) reinterpret_cast<float *>(g.out)[oi] = acc;
-                        else reinterpret_cast<__nv_bfloat16 *>(g.out)[oi] = __float2bfloat16_rn(acc);
-                    }
-                    if (et == 0) *cnt = 0u;      // ready for the next run
-                }
-                epi_bar();      // (fail_flag[1] is read before the next tile rewrites it)
             }
             if (g.epi == GE_POOL) {
                 epi_bar();

@@ -249,6 +249,23 @@ static StemKernel stem_kernel(int mode, bool f32, bool pool) {
          : mode == xk::SM_S2X ? stem_kernel_of<xk::SM_S2X>(f32, pool) : stem_kernel_of<xk::SM_ANY>(f32, pool);
 }
 
+// Whole groups of elements where rows are made of them and the image is aligned; else element by element.
+static StemKernel stem_kernel(const Launch &L, bool aligned) {
+    const int mode = L.stride == 2 ? (L.st_vec && aligned ? xk::SM_S2 : xk::SM_S2X) : L.stride == 1 ? xk::SM_S1 : xk::SM_ANY;
+    return stem_kernel(mode, L.seg[0].src_dtype == XENOS_DTYPE_F32, L.epi == EPI_POOL);
+}
+
+static auto *conv_kernel(const Launch &L) {
+    return L.cv_epi == xk::CE_STORE ? xk::conv_tc_kernel<xk::CE_STORE> : L.cv_epi == xk::CE_SKIP ? xk::conv_tc_kernel<xk::CE_SKIP>
+         : L.cv_epi == xk::CE_VEC ? xk::conv_tc_kernel<xk::CE_VEC> : L.cv_epi == xk::CE_GAP ? xk::conv_tc_kernel<xk::CE_GAP>
+         : L.cv_epi == xk::CE_CLUSTER ? xk::conv_tc_kernel<xk::CE_CLUSTER> : xk::conv_tc_kernel<xk::CE_SPLIT>;
+}
+
+static auto *f32_chain_kernel(const Launch &L) {
+    return L.f32_big ? (L.f32_ws ? xk::f32_chain_kernel<8, 4, true> : xk::f32_chain_kernel<8, 4, false>)
+                     : (L.f32_ws ? xk::f32_chain_kernel<2, 1, true> : xk::f32_chain_kernel<2, 1, false>);
+}
+
 static DwKernel dw_kernel(int epi, int stride, int br) {
     return epi == xk::DE_STORE ? dw_kernel_of<xk::DE_STORE>(stride, br) : epi == xk::DE_GAP ? dw_kernel_of<xk::DE_GAP>(stride, br) : dw_kernel_of<xk::DE_SPLIT>(stride, br);
 }
@@ -283,9 +300,8 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
     // TMA descriptors of the packed weight matrices
     bool any_gemm = false;
     int max_gemm_smem = 0, max_chain_smem = 0;
-    bool any_gemm2 = false;
     for (const Launch &L : g.launches) {
-        if (L.kind == LK_GEMM2) { any_gemm = any_gemm2 = true; max_gemm_smem = std::max(max_gemm_smem, L.smem_bytes); }
+        if (L.kind == LK_GEMM2) { any_gemm = true; max_gemm_smem = std::max(max_gemm_smem, L.smem_bytes); }
         if (L.kind == LK_GEMM) { any_gemm = true; max_gemm_smem = std::max(max_gemm_smem, L.smem_bytes); }
         if (L.kind == LK_F32_CONV_CONV_POOL) max_chain_smem = std::max(max_chain_smem, L.smem_bytes);
     }
@@ -352,44 +368,23 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
     const int optin = (int)prop.sharedMemPerBlockOptin;
     if (max_gemm_smem > optin || max_chain_smem > optin)
         return fail(g, XENOS_E_CUDA, "a kernel of this plan needs more shared memory than the device offers");
-    if (any_gemm)
-        if ((e = cudaFuncSetAttribute(xk::gemm_chain_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::gemm_chain_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
-            return cuda_fail(g, "cudaFuncSetAttribute(gemm)", e);
-    if (any_gemm)
-        if ((e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_SKIP>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_GAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::conv_tc_kernel<xk::CE_SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
-            return cuda_fail(g, "cudaFuncSetAttribute(conv)", e);
-    if (any_gemm)
-        for (int epi = 0; epi < 3; ++epi)
-            for (int stride = 1; stride <= 2; ++stride)
-                for (int br : {1, 2, 4})
-                    if ((e = cudaFuncSetAttribute(dw_kernel(epi, stride, br), cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
-                        return cuda_fail(g, "cudaFuncSetAttribute(dw)", e);
-    if (any_gemm)
-        for (int i = 0; i < 16; ++i)
-            if ((e = cudaFuncSetAttribute(stem_kernel(i & 3, (i >> 2) & 1, i >> 3), cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
-                return cuda_fail(g, "cudaFuncSetAttribute(stem)", e);
-        if ((e = cudaFuncSetAttribute(xk::fc_small_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::fc_small_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess)
-            return cuda_fail(g, "cudaFuncSetAttribute(fc)", e);
-    if (any_gemm2)
-        if ((e = cudaFuncSetAttribute(xk::pair_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::pair_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
-            return cuda_fail(g, "cudaFuncSetAttribute(pair)", e);
-    if (any_gemm2)
-        if ((e = cudaFuncSetAttribute(xk::chain2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
-            return cuda_fail(g, "cudaFuncSetAttribute(chain2)", e);
-    if (max_chain_smem > 0)
-        if ((e = cudaFuncSetAttribute(xk::f32_chain_kernel<8, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::f32_chain_kernel<8, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::f32_chain_kernel<2, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(xk::f32_chain_kernel<2, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
-            return cuda_fail(g, "cudaFuncSetAttribute(f32 chain)", e);
+    // (only for the kernels that this graph launches: the first mention of a kernel loads its code)
+    auto opt_in = [&](auto *kernel) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    };
+    e = cudaSuccess;
+    for (const Launch &L : g.launches) {
+        if (L.kind == LK_F32_CONV_CONV_POOL) opt_in(f32_chain_kernel(L));
+        else if (L.kind == LK_GEMM2 && L.pair) opt_in(L.skip >= 0 ? xk::pair_tc_kernel<true> : xk::pair_tc_kernel<false>);
+        else if (L.kind == LK_GEMM2) opt_in(xk::chain2_kernel);
+        else if (L.kind != LK_GEMM) continue;
+        else if (L.fc_small) { opt_in(xk::fc_small_kernel<1>); opt_in(xk::fc_small_kernel<8>); }
+        else if (L.stem_tc) { opt_in(stem_kernel(L, true)); opt_in(stem_kernel(L, false)); }
+        else if (L.conv_tc) opt_in(conv_kernel(L));
+        else if (L.seg[0].mode == AM_DW) opt_in(dw_kernel(L.cv_epi, L.seg[0].stride, L.dw_br));
+        else opt_in(xk::gemm_chain_kernel);
+    }
+    if (e != cudaSuccess) return cuda_fail(g, "cudaFuncSetAttribute", e);
     return XENOS_OK;
 }
 
@@ -491,9 +486,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
             // a CTA keeps its weights and walks over tiles when there are more tiles than resident CTAs
             const int occ = std::max(1, std::min(2048 / L.block, (228 * 1024) / (L.smem_bytes + 1024)));
             const int grid = (int)std::min<long long>((long long)N * L.grid, (long long)sms * occ);
-            auto *k = L.f32_big ? (L.f32_ws ? xk::f32_chain_kernel<8, 4, true> : xk::f32_chain_kernel<8, 4, false>)
-                                : (L.f32_ws ? xk::f32_chain_kernel<2, 1, true> : xk::f32_chain_kernel<2, 1, false>);
-            cudaError_t le = launch_pdl(k, grid, L.block, L.smem_bytes, stream, p);
+            cudaError_t le = launch_pdl(f32_chain_kernel(L), grid, L.block, L.smem_bytes, stream, p);
             if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
         }
@@ -646,7 +639,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
             if (L.stem_tc) {
                 xk::StemParams p;
                 std::memset(&p, 0, sizeof p);
-                const bool pool = L.epi == EPI_POOL, f32 = L.seg[0].src_dtype == XENOS_DTYPE_F32;
+                const bool pool = L.epi == EPI_POOL;
                 p.src = ptr(L.in0); p.w = (const uint4 *)(ws + L.w_off); p.bias = (const float *)(ws + L.b_off); p.out = ptr(L.out); p.status = status;
                 p.rows = pool ? L.PP : L.P; p.cbs = L.st_cbs; p.cw = L.st_cw; p.units = N * p.cbs * p.rows;
                 p.d_rows = xk::make_fastdiv((uint32_t)p.rows); p.d_cbs = xk::make_fastdiv((uint32_t)p.cbs);
@@ -659,10 +652,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 p.off_w = L.off_b; p.off_bias = L.off_bias; p.off_stage = L.off_stg; p.stage_bytes = (L.off_bar - L.off_stg) / 2 & ~15; p.off_bar = L.off_bar;
                 p.launch_id = (int)li;
                 const int gx = std::min(p.units, std::max(1, sms / L.n_tiles));
-                // whole groups of elements where rows are made of them and the image is aligned; else element by element
-                const bool vec = L.st_vec && ((uintptr_t)p.src & 15u) == 0;
-                const int mode = L.stride == 2 ? (vec ? xk::SM_S2 : xk::SM_S2X) : L.stride == 1 ? xk::SM_S1 : xk::SM_ANY;
-                cudaError_t le = launch_pdl(stem_kernel(mode, f32, pool), dim3(gx, L.n_tiles), L.block, L.smem_bytes, stream, p);
+                cudaError_t le = launch_pdl(stem_kernel(L, ((uintptr_t)p.src & 15u) == 0), dim3(gx, L.n_tiles), L.block, L.smem_bytes, stream, p);
                 if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
                 break;
             }
@@ -702,10 +692,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 int limit = sms;
                 if (L.b_resident) limit = std::max(1, sms / L.n_tiles) * L.n_tiles;
                 const int lgrid = (int)std::min(p.total, limit), lblock = (int)xk::kCvThreads;
-                auto *k = L.cv_epi == xk::CE_STORE ? xk::conv_tc_kernel<xk::CE_STORE> : L.cv_epi == xk::CE_SKIP ? xk::conv_tc_kernel<xk::CE_SKIP>
-                        : L.cv_epi == xk::CE_VEC ? xk::conv_tc_kernel<xk::CE_VEC> : L.cv_epi == xk::CE_GAP ? xk::conv_tc_kernel<xk::CE_GAP>
-                        : L.cv_epi == xk::CE_CLUSTER ? xk::conv_tc_kernel<xk::CE_CLUSTER> : xk::conv_tc_kernel<xk::CE_SPLIT>;
-                cudaError_t le = launch_pdl_cluster(k, L.cv_epi == xk::CE_CLUSTER ? p.total : lgrid, lblock, L.smem_bytes, L.cv_epi == xk::CE_CLUSTER ? L.ksplit : 1, stream, maps->a0, maps->a1, rt->tmaps[li], maps->o, maps->s, p);
+                cudaError_t le = launch_pdl_cluster(conv_kernel(L), L.cv_epi == xk::CE_CLUSTER ? p.total : lgrid, lblock, L.smem_bytes, L.cv_epi == xk::CE_CLUSTER ? L.ksplit : 1, stream, maps->a0, maps->a1, rt->tmaps[li], maps->o, maps->s, p);
                 if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
                 break;
             }
@@ -755,39 +742,27 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 const ASeg &a = L.seg[s];
                 xk::GemmSeg &d = p.seg[s];
                 d.mode = a.mode; d.src = ptr(a.tensor); d.C = a.C; d.H = a.H; d.W = a.W; d.k = a.k; d.stride = a.stride; d.pad = a.pad;
-                d.kelems = a.kelems; d.kblocks = a.kblocks; d.src_f32 = a.src_dtype == XENOS_DTYPE_F32; d.dw_act = a.dw_act;
-                d.dw_w = (const float *)(ws + a.dw_w_off); d.dw_b = (const float *)(ws + a.dw_b_off);
+                d.kelems = a.kelems; d.kblocks = a.kblocks; d.src_f32 = a.src_dtype == XENOS_DTYPE_F32;
             }
             p.bias = (const float *)(ws + L.b_off);
             p.skip = (const __nv_bfloat16 *)ptr(L.skip);
             p.skip_ctot = L.skip >= 0 ? g.tensors[L.skip].c : 0;
             p.out = ptr(L.out); p.status = status;
-            p.batch = N; p.P = L.P; p.Q = L.Q; p.rpi = L.rows_per_image;
-            p.map_mode = L.map_mode; p.tile_rows = L.tile_rows;
+            p.batch = N; p.P = L.P; p.Q = L.Q;
             p.ni = L.ni; p.rh = L.patch_rh; p.rw = L.patch_rw; p.tiles_y = L.tiles_y; p.tiles_x = L.tiles_x;
             p.step_y = L.step_y; p.step_x = L.step_x; p.off_y = L.off_y; p.off_x = L.off_x;
             p.pool_k = L.pool_k; p.pool_stride = L.pool_stride; p.PP = L.PP; p.PQ = L.PQ; p.pth = L.patch_th; p.ptw = L.patch_tw;
-            p.gap_imgs = L.gap_imgs; p.gap_area = L.gap_area; p.gap_rpi = L.gap_rpi;
-            p.kblocks = L.kblocks; p.stages = L.stages; p.tile_n = L.tile_n; p.n_tiles = L.n_tiles * L.ksplit; p.N = L.K;
-            p.ksplit = L.ksplit; p.kb_per = L.kb_per; p.split_ld = L.npad;
-            p.split_stride = (long long)N * L.rows_per_image * L.npad;
-            p.split_part = reinterpret_cast<float *>(ws + g.split_off);
-            p.split_cnt = reinterpret_cast<unsigned int *>(ws + L.split_cnt_off);
+            p.kblocks = L.kblocks; p.stages = L.stages; p.tile_n = L.tile_n; p.n_tiles = L.n_tiles; p.N = L.K;
             p.acc_stride = L.acc_stride; p.tmem_cols = L.tmem_cols;
             p.hstages = L.hstages; p.halo_bytes = L.halo_bytes; p.halo_stride = L.halo_stride;
-            p.halo_h = L.halo_h; p.halo_w = L.halo_w; p.halo_cb = L.halo_cb;
+            p.halo_h = L.halo_h; p.halo_w = L.halo_w;
             p.stem_tma = L.stem_tma; p.stem_align = L.stem_align;
             p.off_halo = L.off_halo; p.off_stg = L.off_stg; p.off_dww = L.off_dww; p.off_bias = L.off_bias; p.off_bar = L.off_bar;
-            p.n_acc = L.n_acc; p.gap_parts = L.gap_parts;
             p.act = L.act; p.act2 = L.act2; p.epi = L.epi; p.out_ctot = L.out_ctot; p.out_coff = L.out_coff;
             p.out_f32 = L.out_dtype == XENOS_DTYPE_F32;
             p.idesc = make_idesc(L.tile_n);
             p.launch_id = (int)li;
-            if (L.map_mode == MAP_PATCH) p.m_tiles = ((N + L.ni - 1) / L.ni) * L.tiles_y * L.tiles_x;
-            else if (L.epi == EPI_GAP) p.m_tiles = L.gap_parts > 1 ? N * L.gap_parts : (N + L.imgs_per_tile - 1) / L.imgs_per_tile;
-            else p.m_tiles = (int)(((long long)N * L.rows_per_image + 127) / 128);
-            // the halo tensor map of a linked depthwise stage points at the stage's input; when that
-            // is a caller buffer its address is only known now
+            p.m_tiles = ((N + L.ni - 1) / L.ni) * L.tiles_y * L.tiles_x;
             const CUtensorMap *tmh = &rt->tmaps[li];
             CUtensorMap tmh_now;
             if (L.stem_tma) {
@@ -800,9 +775,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 }
             }
             const int lgrid = std::min(p.m_tiles * p.n_tiles, sms), lblock = L.block;
-            cudaError_t le;
-            if (L.ksplit > 1 || L.gap_parts > 1) le = launch_pdl(xk::gemm_chain_kernel<1>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
-            else le = launch_pdl(xk::gemm_chain_kernel<0>, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
+            cudaError_t le = launch_pdl(xk::gemm_chain_kernel, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
             if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
         }
