@@ -208,7 +208,8 @@ XENOS_API xenos_status_t xenos_graph_bind(xenos_graph_t *g, void *workspace_dev,
  * inputs_dev / outputs_dev: HOST arrays of DEVICE pointers in declaration order; every
  * pointer must be 16-byte aligned (XENOS_E_INVALID otherwise: the kernels use 16-byte
  * vector accesses and TMA).  Asynchronous; does not synchronise.  Launch errors are returned, device-side status is
- * read with xenos_graph_status. */
+ * read with xenos_graph_status.  A pass that repeats (same batch, same buffers) is recorded as a CUDA graph and replayed,
+ * up to eight recordings per binding; inside a capture of the caller's the launches are captured as they are. */
 XENOS_API xenos_status_t xenos_graph_run(xenos_graph_t *g, int32_t batch,
                                          const void *const *inputs_dev, void *const *outputs_dev,
                                          void *cuda_stream);
