@@ -905,6 +905,7 @@ struct Lower {
         auto window = [&](int br) { return (int)align_up((size_t)L.ni * window_h(br) * L.halo_w * L.halo_cb * 2, 128); };
         const int rgrid = g.hw.sm_count / L.n_tiles * L.n_tiles;
         L.cv_epi = L.epi == EPI_GAP ? 1 : L.ksplit > 1 ? 2 : 0;
+        const bool batched = L.cv_epi == 0 && L.n_acc == 1 && !one;
         auto staging = [&](int chunk, int bufs) {
             if (L.cv_epi == 2) return 0;
             if (L.cv_epi == 1) {
@@ -922,21 +923,28 @@ struct Lower {
             for (int w = 0; w <= 4; ++w) {
                 if ((32 << w) < units) continue;
                 const int groups = 16 >> w;
+                // tiles of a batch: at least one item for every group, an accumulator pair each, no more than a CTA has
+                const int nb_most = batched ? std::max(1, std::min({g.hw.tmem_columns / (2 * L.acc_stride), 4, (int)((tiles + g.hw.sm_count - 1) / g.hw.sm_count)})) : 1;
+                const int nb_least = std::min(nb_most, batched ? ceil_div(groups, L.kblocks) : 1);
                 for (int res = 1; res >= 0; --res)
                     for (int chunk : {64, 32, 16})
+                      for (int nb = nb_least; nb <= nb_most; ++nb)
                         for (int bufs = 2; bufs >= 1; --bufs) {
-                            if (L.cv_epi == 0 && (cols % chunk || (chunk > 16 && cols / chunk < 4))) continue;
+                            if (L.cv_epi == 0 && cols % chunk) continue;
                             if (L.cv_epi != 0 && (chunk != (L.cv_epi == 1 ? 32 : 16) || bufs == 2)) continue;
                             if (res && (one || L.ksplit > 1 || rgrid == 0)) continue;
                             const int a_min = std::max(2, groups), h_min = std::max(2, groups), b_min = res ? 0 : 2;
                             const int ops = a_min * 16384 + (res ? L.kblocks * bslot : b_min * bslot), st = staging(chunk, bufs);
                             const int need = (one ? std::max(ops, st) : ops + st) + h_min * hstride;
                             if (a_min > 8 || h_min > 8 || need > room) continue;
-                            const double t = std::max((1 << w) * issue / 4.0, (300.0 + 2.2 * issue) / groups) +
-                                             (res ? 0.0 : 20.0) + (chunk == 16 ? 15.0 : 0.0) + (bufs == 1 ? 10.0 : 0.0);
+                            // The workers' time per tile: the stencils, then their group's boxes, which cost some 1100 cycles and
+                            // 14 a column (measured, barriers and store hand-over included), so that four groups with one 64-column
+                            // box each of four tiles beat four 16-column boxes of every tile.
+                            const double t = L.kblocks * (std::max((1 << w) * issue / 4.0, (300.0 + 2.2 * issue) / groups) + (res ? 0.0 : 20.0) + (bufs == 1 ? 10.0 : 0.0)) +
+                                             (L.cv_epi == 0 ? (double)ceil_div(nb * ceil_div(cols, chunk), 4) / nb * (1100.0 + 14.0 * chunk) : 0.0);
                             if (best >= 0 && t >= best) continue;
                             best = t;
-                            L.chunk = chunk;
+                            L.chunk = chunk; L.dw_batch = nb;
                             L.dw_br = br; L.dw_wpg_log2 = w; L.dw_groups = groups; L.b_resident = res; L.out_bufs = bufs;
                             L.a_slots = a_min; L.h_slots = h_min; L.b_slots = b_min;
                         }
@@ -969,10 +977,6 @@ struct Lower {
         L.dw_workers = 16;
         L.grid = (int)std::min<long>(tiles, L.b_resident ? rgrid : g.hw.sm_count);
         L.block = 64 + 32 * 16;
-        // tiles of a batch: enough items for every group, an accumulator pair each
-        L.dw_batch = 1;
-        if (L.cv_epi == 0 && L.n_acc == 1 && !one)
-            L.dw_batch = std::max(1, std::min(std::min(ceil_div(groups, L.kblocks), g.hw.tmem_columns / (2 * L.acc_stride)), 4));
         L.tmem_cols = 32;
         while (L.tmem_cols < (L.n_acc == 2 ? 2 : 2 * L.dw_batch) * L.acc_stride) L.tmem_cols *= 2;
         return XENOS_OK;
@@ -1790,7 +1794,7 @@ void emit_plan_json(Graph &g) {
             jint(s, "ni", L.ni); jint(s, "step_y", L.step_y); jint(s, "step_x", L.step_x); jint(s, "off_y", L.off_y); jint(s, "off_x", L.off_x);
             jint(s, "hstages", L.hstages); jint(s, "stem_tc", L.stem_tc); jint(s, "halo_h", L.halo_h); jint(s, "halo_w", L.halo_w); jint(s, "halo_cb", L.halo_cb);
             jint(s, "halo_bytes", L.halo_bytes);
-            jint(s, "ksplit", L.ksplit); jint(s, "kb_per", L.kb_per); jint(s, "a_tma", L.a_tma); jint(s, "fc_small", L.fc_small); jint(s, "dw_workers", L.dw_workers); jint(s, "dw_groups", L.dw_groups); jint(s, "dw_br", L.dw_br); jint(s, "chunk", L.chunk); jint(s, "out_bufs", L.out_bufs); jint(s, "b_slots", L.b_slots); jint(s, "n_acc", L.n_acc); jint(s, "gap_parts", L.gap_parts); jint(s, "conv_tc", L.conv_tc); jint(s, "b_resident", L.b_resident);
+            jint(s, "ksplit", L.ksplit); jint(s, "kb_per", L.kb_per); jint(s, "a_tma", L.a_tma); jint(s, "fc_small", L.fc_small); jint(s, "dw_workers", L.dw_workers); jint(s, "dw_groups", L.dw_groups); jint(s, "dw_br", L.dw_br); jint(s, "dw_batch", L.dw_batch); jint(s, "chunk", L.chunk); jint(s, "out_bufs", L.out_bufs); jint(s, "b_slots", L.b_slots); jint(s, "n_acc", L.n_acc); jint(s, "gap_parts", L.gap_parts); jint(s, "conv_tc", L.conv_tc); jint(s, "b_resident", L.b_resident);
         }
         if (L.kind == LK_GEMM2) {
             jint(s, "k2", L.k2); jint(s, "cmid", L.Cmid); jint(s, "n1pad", L.n1pad); jint(s, "kblocks", L.kblocks); jint(s, "kblocks2", L.kblocks2);
