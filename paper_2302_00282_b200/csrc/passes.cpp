@@ -788,7 +788,7 @@ struct Lower {
                 L.st_slots = (D - 1) * std::min(S, k) + k;
                 if ((L.st_slots + 1) * row + base > cap) continue;
                 L.hstages = D;
-                L.off_b = (int)align_up((size_t)(L.st_slots + 1) * row + 2048, 128);       // (a tile's last rows read past its pieces)
+                L.off_b = (int)align_up((size_t)(L.st_slots + 1) * row + 2048, 128);       // (zeros of one chunk; a tile's last rows read past its pieces)
                 L.off_bias = L.off_b + wbytes;
                 L.off_stg = L.off_bias + 256;
                 L.off_bar = (int)align_up((size_t)(L.off_stg + stage), 128);
@@ -834,7 +834,7 @@ struct Lower {
             for (int c = 0; c < C; ++c, ++pair) { chunk(pair, 0, c, r); chunk(pair, 1, c, r + 1); }
         if (k % 2) {
             for (int c = 0; c + 1 < C; c += 2, ++pair) { chunk(pair, 0, c, k - 1); chunk(pair, 1, c + 1, k - 1); }
-            if (C % 2) chunk(pair, 1, C - 1, k - 1);
+            if (C % 2) chunk(pair, 0, C - 1, k - 1);      // (its second chunk meets zeros)
         }
         for (int o = 0; o < M.cout; ++o) bp[o] = M.b[o];
     }

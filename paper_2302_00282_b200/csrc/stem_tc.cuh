@@ -6,7 +6,9 @@
 // (image row, channel, q); with no swizzle the tensor core addresses 8-row groups and K chunks by two free strides, so every
 // window row of every output row reads the same pieces in place: an im2col operand would be 3.5 times the shared-memory
 // stores for a 7 x 7 window of stride 2.  Products (K = 16, two chunks each) pair two window rows of a channel; the last row
-// of an odd window pairs two channels, and a last single chunk is paired with a row or channel that meets zero weights.
+// of an odd window pairs two channels, and a last single chunk is paired with zeros kept behind the ring.
+// A piece holds zeros outside its window: those elements meet zero weights, but an infinity or a NaN times zero would reach
+// columns whose window does not hold it (the zeros cost the producers 1 us of ResNet-18's 255 at batch 32).
 //
 // A CTA walks down a column block of the image: image rows enter a ring of row slots (slot R repeats slot 0, so that a pair
 // of rows is contiguous wherever the ring wraps), one step per convolution row.
@@ -135,9 +137,10 @@ __device__ __forceinline__ void stem_load(uint32_t (&raw)[4][StemForm<kMode, kF3
 }
 
 // ... and from there to the ring: dst is this lane's first piece, again the distance of a repetition (0: none), left the lanes'
-// worth of the row from this lane on.
+// worth of the row from this lane on, in_window the elements of a piece that belong to its window.
 template <int kMode, bool kF32>
-__device__ __forceinline__ void stem_store(const uint32_t (&raw)[4][StemForm<kMode, kF32>::words], uint32_t dst, uint32_t again, int left, int passes, int lane) {
+__device__ __forceinline__ void stem_store(const uint32_t (&raw)[4][StemForm<kMode, kF32>::words], uint32_t dst, uint32_t again, int left, int passes, int lane,
+                                           const uint4 &in_window) {
     using F = StemForm<kMode, kF32>;
     // eight lanes store 128 bytes apart in pairs: every second group of four lanes stores its second piece first, so that the
     // eight pieces of a store meet eight different groups of banks
@@ -155,15 +158,18 @@ __device__ __forceinline__ void stem_store(const uint32_t (&raw)[4][StemForm<kMo
             else w[j] = r[2 * j % F::words] | (r[(2 * j + 1) % F::words] << 16);
         }
         const uint32_t step = (uint32_t)(32 * F::run * 16 * i);
-        const uint4 a = make_uint4(w[0], w[1], w[2], w[3]);
+        auto piece = [&](uint32_t x, uint32_t y, uint32_t z, uint32_t u) {
+            return make_uint4(x & in_window.x, y & in_window.y, z & in_window.z, u & in_window.w);
+        };
+        const uint4 a = piece(w[0], w[1], w[2], w[3]);
         if (32 * i < left) {
             if (F::run == 1) {
                 st_shared16(dst + step, a);
                 if (again) st_shared16(dst + again + step, a);
             } else {
-                const uint4 b = F::S == 2 ? make_uint4(w[1], w[2], w[3], w[4])
-                                          : make_uint4(__funnelshift_r(w[0], w[1], 16), __funnelshift_r(w[1], w[2], 16),
-                                                       __funnelshift_r(w[2], w[3], 16), __funnelshift_r(w[3], w[4], 16));
+                const uint4 b = F::S == 2 ? piece(w[1], w[2], w[3], w[4])
+                                          : piece(__funnelshift_r(w[0], w[1], 16), __funnelshift_r(w[1], w[2], 16),
+                                                  __funnelshift_r(w[2], w[3], 16), __funnelshift_r(w[3], w[4], 16));
                 const uint4 x = f ? b : a, y = f ? a : b;
                 st_shared16(d0 + step, x);
                 st_shared16(d1 + step, y);
@@ -186,6 +192,11 @@ __device__ __forceinline__ bool stem_produce(const StemParams &g, uint32_t sbase
     if (j0 >= rstep) j0 = k;                              // a warp without rows only keeps the steps' counts
     const uint32_t slot_bytes = in_reg((uint32_t)(g.qp * C * 16)), ring = in_reg(sbase + (uint32_t)((c * g.qp + F::run * lane) * 16)), wrap = (uint32_t)R * slot_bytes;
     const uint32_t pitch = in_reg((uint32_t)(W * es));
+    auto both = [&](int j) {                              // which of elements j, j + 1 of a piece the window takes
+        const uint32_t x = (unsigned)(j - g.lead) < (unsigned)k, y = (unsigned)(j + 1 - g.lead) < (unsigned)k;
+        return in_reg(x * 0xffffu | y * 0xffff0000u);
+    };
+    const uint4 in_window = make_uint4(both(0), both(2), both(4), both(6));
     uint32_t raw[4][F::words];
     int t = 0, sl = 0, slot = 0;                          // step, its barrier, ring slot of its window row 0
     uint32_t ph = 0;
@@ -218,7 +229,7 @@ __device__ __forceinline__ bool stem_produce(const StemParams &g, uint32_t sbase
                 if (have) {
                     int s = slot + d;
                     if (s >= R) s -= R;
-                    stem_store<kMode, kF32>(raw, ring + (uint32_t)s * slot_bytes, s == 0 ? wrap : 0u, left, passes, lane);
+                    stem_store<kMode, kF32>(raw, ring + (uint32_t)s * slot_bytes, s == 0 ? wrap : 0u, left, passes, lane, in_window);
                     d += rstep;
                 }
                 if (d >= k) {
@@ -294,10 +305,9 @@ __device__ __forceinline__ bool stem_mma(const StemParams &g, uint32_t sbase, ui
 #pragma unroll 1
                     for (int c = 1; c < C; c += 2, al += 2 * cp16) mma(al);
                     if (C & 1) {
-                        // the last channel's chunk behind the row above it, which meets zero weights
-                        int s1 = s - 1;
-                        if (s1 < 0) s1 += R;
-                        mma((ring16 + (uint32_t)s1 * rp16 + (uint32_t)(C - 1) * cp16 + (uint32_t)seg * 128u) | (rp16 << 16));
+                        // the last channel's chunk before the zeros behind the ring
+                        const uint32_t last = ring16 + (uint32_t)s * rp16 + (uint32_t)(C - 1) * cp16 + (uint32_t)seg * 128u;
+                        mma(last | ((ring16 + (uint32_t)(R + 1) * rp16 - last) << 16));
                     }
                 }
                 umma_commit(accf + 8u * a);
@@ -312,28 +322,20 @@ __device__ __forceinline__ bool stem_mma(const StemParams &g, uint32_t sbase, ui
     return true;
 }
 
-// 16 columns of an accumulator: bias, activation, bf16 pairs.  The conversion itself clamps at zero.
-template <bool kRelu>
-__device__ __forceinline__ uint32_t stem_cvt(float a, float b) {
-    uint32_t r;
-    if (kRelu) asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
-    else asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
-    return r;
-}
+// 16 columns of an accumulator: bias, bf16 pairs, activation.  (Maximum with zero, not the conversion's own clamp, which keeps
+// a NaN: max(x, 0) is 0 there, as in every other kernel.)
 __device__ __forceinline__ void stem_pack(const float *v, const float2 (&bias)[8], int act, uint32_t (&o)[8]) {
     float2 x[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) x[i] = __fadd2_rn(make_float2(v[2 * i], v[2 * i + 1]), bias[i]);
-    if (act) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] = stem_cvt<true>(x[i].x, x[i].y);
-    } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] = stem_cvt<false>(x[i].x, x[i].y);
-    }
+    for (int i = 0; i < 8; ++i) o[i] = pack2(x[i].x, x[i].y);
     if (act == 2) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) o[i] = clamp_bf16x2(o[i], 0u, 0x40c040c0u);
+    } else if (act) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i] = max_bf16x2(o[i], 0u);
     }
 }
 __device__ __forceinline__ void stem_bias(uint32_t at, float2 (&b)[8]) {
@@ -531,6 +533,8 @@ stem_tc_kernel(const __grid_constant__ StemParams g) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     } else {
+        // (zeros of one chunk, 128 pieces, behind the ring)
+        if (threadIdx.x < 128) st_shared16(sbase + (uint32_t)((g.R + 1) * g.qp * g.C * 16) + threadIdx.x * 16u, make_uint4(0u, 0u, 0u, 0u));
         if ((int)threadIdx.x < g.tile_n) reinterpret_cast<float *>(sm + g.off_bias)[threadIdx.x] = __ldg(g.bias + blockIdx.y * g.tile_n + threadIdx.x);
     }
     tc_fence_before();

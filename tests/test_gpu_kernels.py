@@ -9,7 +9,7 @@ from xenos_workloads import graphs
 from xenos_workloads.graphs import GraphSpec
 
 from gpu_util import GpuGraph, rel_err_fp32
-from test_gpu_parity import FP32_TOL, check_bf16
+from test_gpu_parity import BF16_TOL, FP32_TOL, check_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -88,6 +88,33 @@ def test_image_convolution(cin, h, w, cout, k, st, pad, pool, batch, in_mode):
         batch = 9          # (smaller batches of a 3 x 3 window run on the CUDA cores)
     _, _, gg = check_bf16(f"stem{(cin, h, w, cout, k, st, pad, pool)}{in_mode}", _spec((cin, h, w), build), batch, in_mode=in_mode, links=links)
     assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
+
+
+# Pixels that are infinite or no number reach exactly the outputs whose window holds them, as they are: windows shorter than the
+# eight elements the operand is made of, aligned (lead elements before the window) and not, odd and even window rows and channels
+@pytest.mark.parametrize("cin,h,w,cout,k,st,pad,act,pool,batch", [
+    (3, 24, 32, 24, 3, 1, 1, "relu", None, 9), (3, 33, 36, 72, 3, 2, 1, None, None, 9), (3, 40, 50, 64, 7, 2, 3, "relu6", None, 2), (3, 40, 48, 64, 7, 2, 3, "relu", (3, 2, 1), 2),
+    (1, 17, 20, 8, 2, 1, 0, None, None, 2), (2, 21, 45, 16, 4, 2, 1, "relu", (2, 2, 0), 2), (4, 25, 28, 24, 5, 3, 2, "relu", None, 2), (5, 19, 24, 16, 8, 1, 3, "relu6", None, 2)])
+@pytest.mark.parametrize("in_mode", ["f32_nchw", "bf16_nchw"])
+def test_image_convolution_of_non_finite_pixels(cin, h, w, cout, k, st, pad, act, pool, batch, in_mode):
+    def build(g):
+        y = g.cbr("stem", "input", cout, k, st, pad, act=act)
+        if pool:
+            g.pool("mp", y, "maxpool", *pool)
+    spec = _spec((cin, h, w), build)
+    P, x = graphs.make_params(spec), xo.round_bf16(graphs.make_input(spec, batch))
+    rng = np.random.default_rng(1)
+    for n in range(batch):
+        for v in (np.nan, np.inf, -np.inf):
+            x[n, rng.integers(cin), rng.integers(h), rng.integers(w)] = v
+    gg = GpuGraph(spec, P, batch, in_mode=in_mode, links=[["stem", "mp"]] if pool else None)
+    assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
+    y, o = gg.run(x), interp.run_graph(spec, P, x)
+    assert act == "relu6" or not np.isfinite(o).all()
+    for special in (np.isnan, np.isposinf, np.isneginf):
+        assert np.array_equal(special(y), special(o)), special.__name__
+    fine = np.isfinite(o)
+    assert np.abs(y[fine] - o[fine]).max() <= BF16_TOL * np.abs(o[fine]).max()
 
 
 # one output row per thread and four, bands that end inside the map, windows of 1 to 3; averages of one row and of more rows than
