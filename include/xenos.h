@@ -200,7 +200,8 @@ XENOS_API xenos_status_t xenos_graph_compile(xenos_graph_t *g, int32_t max_batch
 
 /* Attach a caller-owned DEVICE workspace (256-byte aligned, >= workspace_bytes) and upload
  * the packed weights into it on `cuda_stream` (a cudaStream_t; NULL = default stream).
- * The workspace must stay valid and unshared until destroy or the next bind. */
+ * The workspace must stay valid and unshared until destroy or the next bind.  The pass for max_batch images is recorded as a
+ * CUDA graph, which later runs use with their own buffers. */
 XENOS_API xenos_status_t xenos_graph_bind(xenos_graph_t *g, void *workspace_dev, size_t bytes,
                                           void *cuda_stream);
 
@@ -208,8 +209,10 @@ XENOS_API xenos_status_t xenos_graph_bind(xenos_graph_t *g, void *workspace_dev,
  * inputs_dev / outputs_dev: HOST arrays of DEVICE pointers in declaration order; every
  * pointer must be 16-byte aligned (XENOS_E_INVALID otherwise: the kernels use 16-byte
  * vector accesses and TMA).  Asynchronous; does not synchronise.  Launch errors are returned, device-side status is
- * read with xenos_graph_status.  A pass that repeats (same batch, same buffers) is recorded as a CUDA graph and replayed,
- * up to eight recordings per binding; inside a capture of the caller's the launches are captured as they are. */
+ * read with xenos_graph_status.  A pass of several kernels runs as the CUDA graph that xenos_graph_bind recorded, pointed at
+ * this call's buffers; a batch other than that of the pass before may be launched kernel by kernel, and inside a capture of
+ * the caller's the kernels are captured as they are.  Several host threads may enqueue passes of one binding as long as the
+ * passes follow one another on the device. */
 XENOS_API xenos_status_t xenos_graph_run(xenos_graph_t *g, int32_t batch,
                                          const void *const *inputs_dev, void *const *outputs_dev,
                                          void *cuda_stream);

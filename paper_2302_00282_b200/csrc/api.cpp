@@ -309,7 +309,7 @@ xenos_status_t xenos_graph_bind(xenos_graph_t *gp, void *workspace_dev, size_t b
     if (!workspace_dev) return fail(g, XENOS_E_WORKSPACE, "bind: workspace is NULL");
     if (bytes < g.workspace_bytes) return fail(g, XENOS_E_WORKSPACE, "bind: workspace too small");
     if (((uintptr_t)workspace_dev & 255u) != 0) return fail(g, XENOS_E_WORKSPACE, "bind: workspace must be 256-byte aligned");
-    xenos_status_t st = runtime_bind(g, workspace_dev, bytes, cuda_stream);
+    xenos_status_t st = runtime_bind(g, workspace_dev, cuda_stream, true);
     if (st == XENOS_OK) g.state = ST_BOUND;
     return st;
     XENOS_GUARD_END(gp)
@@ -336,7 +336,7 @@ xenos_status_t xenos_graph_profile(xenos_graph_t *gp, int32_t batch, const void 
     if (xenos_status_t st = check_run_args(g, "profile", batch, inputs_dev, outputs_dev)) return st;
     if (!ms_per_launch) return fail(g, XENOS_E_INVALID, "profile: NULL pointer");
     if (n_launches != (int32_t)g.launches.size()) return fail(g, XENOS_E_INVALID, "profile: n_launches must equal xenos_graph_launch_count");
-    return runtime_run(g, batch, inputs_dev, outputs_dev, cuda_stream, ms_per_launch);
+    return runtime_profile(g, batch, inputs_dev, outputs_dev, cuda_stream, ms_per_launch);
     XENOS_GUARD_END(gp)
 }
 

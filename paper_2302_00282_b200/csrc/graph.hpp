@@ -236,9 +236,9 @@ xenos_status_t search_splits(Graph &g, int max_batch, int precision, void *ws, s
 void save_graph(const Graph &g, std::vector<uint8_t> &out);
 xenos_status_t load_graph(Graph &g, const uint8_t *buf, size_t bytes, bool *compiled);
 // runtime.cu
-xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream);
-xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *const *out, void *stream,
-                           float *ms_per_launch = nullptr);
+xenos_status_t runtime_bind(Graph &g, void *ws, void *stream, bool record);
+xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *const *out, void *stream);
+xenos_status_t runtime_profile(Graph &g, int batch, const void *const *in, void *const *out, void *stream, float *ms_per_launch);
 xenos_status_t runtime_status(Graph &g, void *stream);
 xenos_status_t runtime_selftest_wait_expiry(Graph &g, void *stream);
 void runtime_free(Graph &g);

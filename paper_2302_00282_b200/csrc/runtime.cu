@@ -27,22 +27,17 @@ namespace xenos {
 
 struct ConvMaps { CUtensorMap a0, a1, o, s; };      // operand segments, result, shortcut of a conv_tc_kernel launch
 
-// One recorded pass: the launches of a graph for one batch size and one set of caller buffers, replayed as a CUDA graph.
-struct Replay {
-    std::vector<const void *> key;      // batch, inputs, outputs
-    cudaGraphExec_t exec = nullptr;     // null: seen once, not recorded
-    uint64_t used = 0;
-};
-constexpr size_t kReplays = 8;          // passes remembered per binding; the least recently used one makes room
-
 struct Runtime {
-    std::vector<Replay> replays;
-    cudaStream_t record_stream = nullptr;      // records replays (never runs anything)
-    uint64_t tick = 0;
-    bool replay_ok = true;              // cleared when recording fails: passes are then launched one kernel at a time
+    // The pass as a CUDA graph (null: launches go to the stream one by one), its kernel nodes in launch order, the batch whose
+    // grids they hold and the batch of the last call.
+    cudaGraphExec_t exec = nullptr;
+    cudaGraph_t graph = nullptr;        // what exec was made of: its nodes name those of exec
+    std::vector<cudaGraphNode_t> nodes;
+    int exec_batch = 0, last_batch = 0;
+    std::mutex exec_mutex;              // a call points the nodes at its buffers and launches them
     ~Runtime() {
-        for (Replay &r : replays) if (r.exec) cudaGraphExecDestroy(r.exec);
-        if (record_stream) cudaStreamDestroy(record_stream);
+        if (exec) cudaGraphExecDestroy(exec);
+        if (graph) cudaGraphDestroy(graph);
     }
     int device = -1;
     int sm_count = 0;
@@ -164,6 +159,13 @@ static bool conv_has_external(const Graph &g, const Launch &L) {
     return external(L.seg[0].tensor) || (L.seg[1].mode != AM_NONE && external(L.seg[1].tensor)) || external(L.out) || external(L.skip);
 }
 
+// Whether a launch reads or writes a buffer that the caller names at run time.
+static bool touches_caller(const Graph &g, const Launch &L) {
+    auto external = [&](int t) { return t >= 0 && (g.tensors[t].input_slot >= 0 || g.tensors[t].output_slot >= 0); };
+    return external(L.in0) || external(L.in1) || external(L.in2) || external(L.out) || external(L.skip) ||
+           (L.seg[0].mode != AM_NONE && external(L.seg[0].tensor)) || (L.seg[1].mode != AM_NONE && external(L.seg[1].tensor));
+}
+
 static xk::ConvSegment conv_segment(const Launch &L, const ASeg &a) {
     xk::ConvSegment s;
     std::memset(&s, 0, sizeof s);
@@ -270,13 +272,76 @@ static DwKernel dw_kernel(int epi, int stride, int br) {
     return epi == xk::DE_STORE ? dw_kernel_of<xk::DE_STORE>(stride, br) : epi == xk::DE_GAP ? dw_kernel_of<xk::DE_GAP>(stride, br) : dw_kernel_of<xk::DE_SPLIT>(stride, br);
 }
 
+// Where launch_pass hands its kernels: to a stream, to the node of a recorded pass that holds the launch, or nowhere (the
+// kernels of a graph are only made ready to run).
+struct Issue {
+    enum Mode { LAUNCH, POINT, READY } mode = LAUNCH;
+    cudaStream_t stream = nullptr;
+    Runtime *rt = nullptr;
+    bool external_only = false;         // POINT: only launches that read or write the caller's buffers
+    int optin = 0;                      // READY: shared memory a block may ask for
+    size_t li = 0;                      // the launch at hand
+
+    // Programmatic dependent launch: the kernel may be scheduled while its predecessor in the stream drains, runs its set-up
+    // and then waits (griddepcontrol.wait) before it touches the predecessor's results.
+    template <class... P, class... A>
+    cudaError_t pdl(void (*kernel)(P...), dim3 grid, int block, int smem, A &&...args) const {
+        return put(kernel, grid, dim3((unsigned)block), smem, 1, true, std::forward<A>(args)...);
+    }
+    template <class... P, class... A>
+    cudaError_t pdl_cluster(void (*kernel)(P...), dim3 grid, int block, int smem, int cluster, A &&...args) const {
+        return put(kernel, grid, dim3((unsigned)block), smem, cluster, true, std::forward<A>(args)...);
+    }
+    template <class... P, class... A>
+    cudaError_t plain(void (*kernel)(P...), dim3 grid, dim3 block, int smem, A &&...args) const {
+        return put(kernel, grid, block, smem, 1, false, std::forward<A>(args)...);
+    }
+
+private:
+    template <class... P, class... A>
+    cudaError_t put(void (*kernel)(P...), dim3 grid, dim3 block, int smem, int cluster, bool programmatic, A &&...args) const {
+        return [&](P... exact) {
+            void *argv[] = {&exact...};
+            return issue(reinterpret_cast<const void *>(kernel), grid, block, smem, cluster, programmatic, argv);
+        }(std::forward<A>(args)...);
+    }
+    cudaError_t issue(const void *kernel, dim3 grid, dim3 block, int smem, int cluster, bool programmatic, void **argv) const {
+        if (mode == READY) {
+            // the first mention of a kernel loads its code.  The opt-in limit is a per-function, per-device setting shared by
+            // every graph in the process: always the device's maximum, so that binding one graph never lowers it for another.
+            cudaFuncAttributes at;
+            return smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) : cudaFuncGetAttributes(&at, kernel);
+        }
+        if (mode == POINT) {
+            cudaKernelNodeParams p = {};
+            p.func = const_cast<void *>(kernel); p.gridDim = grid; p.blockDim = block; p.sharedMemBytes = (unsigned)smem; p.kernelParams = argv;
+            return cudaGraphExecKernelNodeSetParams(rt->exec, rt->nodes[li], &p);
+        }
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid; cfg.blockDim = block;
+        cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = stream;
+        cudaLaunchAttribute at[2];
+        unsigned n = 0;
+        if (programmatic) {
+            at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at[n++].val.programmaticStreamSerializationAllowed = 1;
+        }
+        if (cluster > 1) {
+            at[n].id = cudaLaunchAttributeClusterDimension;
+            at[n].val.clusterDim.x = (unsigned)cluster; at[n].val.clusterDim.y = 1; at[n++].val.clusterDim.z = 1;
+        }
+        cfg.attrs = at; cfg.numAttrs = n;
+        return cudaLaunchKernelExC(&cfg, kernel, argv);
+    }
+};
+
 void runtime_free(Graph &g) {
     delete static_cast<Runtime *>(g.rt);
     g.rt = nullptr;
 }
 
-xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
-    (void)bytes;
+// Uploads the parameters and encodes the maps of what lies in the workspace.
+static xenos_status_t attach(Graph &g, void *ws, void *stream_v) {
     cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
@@ -363,49 +428,10 @@ xenos_status_t runtime_bind(Graph &g, void *ws, size_t bytes, void *stream_v) {
             }
         }
     }
-    // The opt-in limit is a per-function, per-device setting shared by every graph in the process:
-    // always raise it to the device maximum so that binding one graph never lowers it for another.
     const int optin = (int)prop.sharedMemPerBlockOptin;
     if (max_gemm_smem > optin || max_chain_smem > optin)
         return fail(g, XENOS_E_CUDA, "a kernel of this plan needs more shared memory than the device offers");
-    // (only for the kernels that this graph launches: the first mention of a kernel loads its code)
-    auto opt_in = [&](auto *kernel) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-    };
-    e = cudaSuccess;
-    for (const Launch &L : g.launches) {
-        if (L.kind == LK_F32_CONV_CONV_POOL) opt_in(f32_chain_kernel(L));
-        else if (L.kind == LK_GEMM2 && L.pair) opt_in(L.skip >= 0 ? xk::pair_tc_kernel<true> : xk::pair_tc_kernel<false>);
-        else if (L.kind == LK_GEMM2) opt_in(xk::chain2_kernel);
-        else if (L.kind != LK_GEMM) continue;
-        else if (L.fc_small) { opt_in(xk::fc_small_kernel<1>); opt_in(xk::fc_small_kernel<8>); }
-        else if (L.stem_tc) { opt_in(stem_kernel(L, true)); opt_in(stem_kernel(L, false)); }
-        else if (L.conv_tc) opt_in(conv_kernel(L));
-        else if (L.seg[0].mode == AM_DW) opt_in(dw_kernel(L.cv_epi, L.seg[0].stride, L.dw_br));
-        else opt_in(xk::gemm_chain_kernel);
-    }
-    if (e != cudaSuccess) return cuda_fail(g, "cudaFuncSetAttribute", e);
     return XENOS_OK;
-}
-
-// Programmatic dependent launch: the kernel may be scheduled while its predecessor in the stream drains, runs its set-up
-// and then waits (griddepcontrol.wait) before it touches the predecessor's results.
-template <class... P, class... A>
-static cudaError_t launch_pdl_cluster(void (*kernel)(P...), dim3 grid, int block, int smem, int cluster, cudaStream_t stream, A &&...args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = stream;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = (unsigned)cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
-}
-template <class... P, class... A>
-static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, int block, int smem, cudaStream_t stream, A &&...args) {
-    return launch_pdl_cluster(kernel, grid, block, smem, 1, stream, std::forward<A>(args)...);
 }
 
 static int ew_grid(long long total, int block, int sms) {
@@ -416,10 +442,10 @@ static int ew_grid(long long total, int block, int sms) {
     return (int)b;
 }
 
-static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, void *const *out, void *stream_v,
-                                  float *ms_per_launch) {
+// The kernels of one pass, in order; each(li) is called behind launch li.
+template <class Each>
+static xenos_status_t issue_pass(Graph &g, int batch, const void *const *in, void *const *out, Issue to, Each each) {
     Runtime *rt = static_cast<Runtime *>(g.rt);
-    cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
     uint8_t *ws = static_cast<uint8_t *>(g.ws);
     unsigned int *status = reinterpret_cast<unsigned int *>(ws + g.status_off);
     auto ptr = [&](int t) -> void * {
@@ -430,48 +456,44 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
         return ws + g.place[t].off;
     };
     const int sms = rt->sm_count;
-    std::vector<cudaEvent_t> ev;
-    if (ms_per_launch) {
-        ev.resize(g.launches.size() + 1);
-        for (auto &e : ev)
-            if (cudaEventCreate(&e) != cudaSuccess) return fail(g, XENOS_E_CUDA, "cudaEventCreate failed");
-        cudaEventRecord(ev[0], stream);
-    }
     for (size_t li = 0; li < g.launches.size(); ++li) {
         const Launch &L = g.launches[li];
         const int N = batch;
+        if (to.external_only && !touches_caller(g, L)) continue;
+        to.li = li;
+        cudaError_t le = cudaSuccess;
         switch (L.kind) {
         case LK_F32_CONV: {
             long long total = (long long)N * L.K * L.P * L.Q;
-            xk::f32_conv_kernel<<<ew_grid(total, 256, sms), 256, 0, stream>>>(
+            le = to.plain(xk::f32_conv_kernel, ew_grid(total, 256, sms), 256, 0,
                 (const float *)ptr(L.in0), (const float *)(ws + L.w_off), (const float *)(ws + L.b_off), (float *)ptr(L.out),
                 N, L.C, L.H, L.W, L.K, L.P, L.Q, L.k, L.stride, L.pad, L.groups, L.act);
             break;
         }
         case LK_F32_POOL: {
             long long total = (long long)N * L.C * L.P * L.Q;
-            xk::f32_pool_kernel<<<ew_grid(total, 256, sms), 256, 0, stream>>>(
+            le = to.plain(xk::f32_pool_kernel, ew_grid(total, 256, sms), 256, 0,
                 (const float *)ptr(L.in0), (float *)ptr(L.out), N, L.C, L.H, L.W, L.P, L.Q, L.pool_k, L.pool_stride, L.pool_pad, L.pool_kind);
             break;
         }
         case LK_F32_GAP: {
             long long warps = (long long)N * L.C;
-            xk::f32_gap_kernel<<<(int)((warps * 32 + 255) / 256), 256, 0, stream>>>((const float *)ptr(L.in0), (float *)ptr(L.out), N * L.C, L.H * L.W);
+            le = to.plain(xk::f32_gap_kernel, (int)((warps * 32 + 255) / 256), 256, 0, (const float *)ptr(L.in0), (float *)ptr(L.out), N * L.C, L.H * L.W);
             break;
         }
         case LK_F32_ADD: {
             const Tensor &t = g.tensors[L.out];
             long long total = (long long)N * (t.is_vec ? t.c : t.c * t.h * t.w);
-            xk::f32_add_kernel<<<ew_grid(total, 256, sms), 256, 0, stream>>>((const float *)ptr(L.in0), (const float *)ptr(L.in1), (float *)ptr(L.out), total, L.act);
+            le = to.plain(xk::f32_add_kernel, ew_grid(total, 256, sms), 256, 0, (const float *)ptr(L.in0), (const float *)ptr(L.in1), (float *)ptr(L.out), total, L.act);
             break;
         }
         case LK_F32_CONCAT_PART: {
             long long total = (long long)N * L.C * L.H * L.W;
-            xk::f32_concat_part_kernel<<<ew_grid(total, 256, sms), 256, 0, stream>>>((const float *)ptr(L.in0), (float *)ptr(L.out), N, L.C, L.H * L.W, L.out_ctot, L.out_coff);
+            le = to.plain(xk::f32_concat_part_kernel, ew_grid(total, 256, sms), 256, 0, (const float *)ptr(L.in0), (float *)ptr(L.out), N, L.C, L.H * L.W, L.out_ctot, L.out_coff);
             break;
         }
         case LK_F32_FC:
-            xk::f32_fc_kernel<<<(N * L.K + 255) / 256, 256, 0, stream>>>((const float *)ptr(L.in0), (const float *)(ws + L.w_off), (const float *)(ws + L.b_off), (float *)ptr(L.out), N, L.C, L.K, L.act);
+            le = to.plain(xk::f32_fc_kernel, (N * L.K + 255) / 256, 256, 0, (const float *)ptr(L.in0), (const float *)(ws + L.w_off), (const float *)(ws + L.b_off), (float *)ptr(L.out), N, L.C, L.K, L.act);
             break;
         case LK_F32_CONV_CONV_POOL: {
             xk::F32ChainParams p;
@@ -486,23 +508,22 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
             // a CTA keeps its weights and walks over tiles when there are more tiles than resident CTAs
             const int occ = std::max(1, std::min(2048 / L.block, (228 * 1024) / (L.smem_bytes + 1024)));
             const int grid = (int)std::min<long long>((long long)N * L.grid, (long long)sms * occ);
-            cudaError_t le = launch_pdl(f32_chain_kernel(L), grid, L.block, L.smem_bytes, stream, p);
-            if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+            le = to.pdl(f32_chain_kernel(L), grid, L.block, L.smem_bytes, p);
             break;
         }
         case LK_STEM3X3: {
             const int grid = N * L.grid;
             if (L.seg[0].src_dtype == XENOS_DTYPE_F32)
-                xk::stem3x3_kernel<float><<<grid, 256, (size_t)L.smem_bytes, stream>>>((const float *)ptr(L.in0), (const float *)(ws + L.w_off), (const float *)(ws + L.b_off),
+                le = to.plain(xk::stem3x3_kernel<float>, grid, 256, L.smem_bytes, (const float *)ptr(L.in0), (const float *)(ws + L.w_off), (const float *)(ws + L.b_off),
                     (__nv_bfloat16 *)ptr(L.out), N, L.C, L.H, L.W, L.K, L.P, L.Q, L.stride, L.pad, L.act);
             else
-                xk::stem3x3_kernel<__nv_bfloat16><<<grid, 256, (size_t)L.smem_bytes, stream>>>((const __nv_bfloat16 *)ptr(L.in0), (const float *)(ws + L.w_off), (const float *)(ws + L.b_off),
+                le = to.plain(xk::stem3x3_kernel<__nv_bfloat16>, grid, 256, L.smem_bytes, (const __nv_bfloat16 *)ptr(L.in0), (const float *)(ws + L.w_off), (const float *)(ws + L.b_off),
                     (__nv_bfloat16 *)ptr(L.out), N, L.C, L.H, L.W, L.K, L.P, L.Q, L.stride, L.pad, L.act);
             break;
         }
         case LK_DW: {
             long long total = (long long)N * L.P * L.Q * (L.C / 8);
-            xk::dw3x3_kernel<<<ew_grid(total, 256, sms), 256, 0, stream>>>(
+            le = to.plain(xk::dw3x3_kernel, ew_grid(total, 256, sms), 256, 0,
                 (const __nv_bfloat16 *)ptr(L.in0), (const float *)(ws + L.w_off), (const float *)(ws + L.b_off),
                 (__nv_bfloat16 *)ptr(L.out), N, L.C, L.H, L.W, L.P, L.Q, L.stride, L.pad, L.act);
             break;
@@ -515,60 +536,58 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
             const int items = (int)(small ? (long long)N * bands * L.Q * (L.C / 8) : 0);
             const __nv_bfloat16 *x = (const __nv_bfloat16 *)ptr(L.in0);
             __nv_bfloat16 *y = (__nv_bfloat16 *)ptr(L.out);
-            cudaError_t le = small ? launch_pdl(rows == 4 ? xk::maxpool_kernel<4> : xk::maxpool_kernel<1>, (items + 255) / 256, 256, 0, stream, x, y, items, L.C / 8,
+            le = small ? to.pdl(rows == 4 ? xk::maxpool_kernel<4> : xk::maxpool_kernel<1>, (items + 255) / 256, 256, 0, x, y, items, L.C / 8,
                                                 L.H, L.W, L.P, L.Q, bands, L.pool_k, L.pool_stride, L.pool_pad)
-                                   : launch_pdl(xk::pool_kernel, ew_grid(total, 256, sms), 256, 0, stream, x, y, N, L.C, L.H, L.W, L.P, L.Q, L.pool_k,
+                                   : to.pdl(xk::pool_kernel, ew_grid(total, 256, sms), 256, 0, x, y, N, L.C, L.H, L.W, L.P, L.Q, L.pool_k,
                                                 L.pool_stride, L.pool_pad, L.pool_kind);
-            if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
         }
         case LK_GAP: {
-            cudaError_t le = launch_pdl(xk::gap_kernel, dim3((L.C + 63) / 64, N), 256, 0, stream, (const __nv_bfloat16 *)ptr(L.in0), ptr(L.out), L.C, L.H * L.W,
+            le = to.pdl(xk::gap_kernel, dim3((L.C + 63) / 64, N), 256, 0, (const __nv_bfloat16 *)ptr(L.in0), ptr(L.out), L.C, L.H * L.W,
                                         L.out_dtype == XENOS_DTYPE_F32);
-            if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
             break;
         }
         case LK_ADD: {
             const Tensor &t = g.tensors[L.out];
             long long n8 = (long long)N * (t.is_vec ? t.c : t.c * t.h * t.w) / 8;
-            xk::add_kernel<<<ew_grid(n8, 256, sms), 256, 0, stream>>>((const __nv_bfloat16 *)ptr(L.in0), (const __nv_bfloat16 *)ptr(L.in1), (__nv_bfloat16 *)ptr(L.out), n8, L.act);
+            le = to.plain(xk::add_kernel, ew_grid(n8, 256, sms), 256, 0, (const __nv_bfloat16 *)ptr(L.in0), (const __nv_bfloat16 *)ptr(L.in1), (__nv_bfloat16 *)ptr(L.out), n8, L.act);
             break;
         }
         case LK_CONCAT_PART: {
             long long pixels = (long long)N * L.H * L.W;
-            xk::concat_part_kernel<<<ew_grid(pixels * (L.C / 8), 256, sms), 256, 0, stream>>>((const __nv_bfloat16 *)ptr(L.in0), (__nv_bfloat16 *)ptr(L.out), pixels, L.C, L.out_ctot, L.out_coff);
+            le = to.plain(xk::concat_part_kernel, ew_grid(pixels * (L.C / 8), 256, sms), 256, 0, (const __nv_bfloat16 *)ptr(L.in0), (__nv_bfloat16 *)ptr(L.out), pixels, L.C, L.out_ctot, L.out_coff);
             break;
         }
         case LK_MULMAC: {
             const Tensor &t = g.tensors[L.out];
             long long n8 = (long long)N * (t.is_vec ? t.c : t.c * t.h * t.w) / 8;
-            xk::mulmac_kernel<<<ew_grid(n8, 256, sms), 256, 0, stream>>>((const __nv_bfloat16 *)ptr(L.in0), (const __nv_bfloat16 *)ptr(L.in1),
+            le = to.plain(xk::mulmac_kernel, ew_grid(n8, 256, sms), 256, 0, (const __nv_bfloat16 *)ptr(L.in0), (const __nv_bfloat16 *)ptr(L.in1),
                                                                          (const __nv_bfloat16 *)ptr(L.in2), (__nv_bfloat16 *)ptr(L.out), n8);
             break;
         }
         case LK_F32_MULMAC: {
             const Tensor &t = g.tensors[L.out];
             long long total = (long long)N * (t.is_vec ? t.c : t.c * t.h * t.w);
-            xk::f32_mulmac_kernel<<<ew_grid(total, 256, sms), 256, 0, stream>>>((const float *)ptr(L.in0), (const float *)ptr(L.in1),
+            le = to.plain(xk::f32_mulmac_kernel, ew_grid(total, 256, sms), 256, 0, (const float *)ptr(L.in0), (const float *)ptr(L.in1),
                                                                                 (const float *)ptr(L.in2), (float *)ptr(L.out), total);
             break;
         }
         case LK_TRANSPOSE:      // NHWC: per image [H rows][C columns] -> [C][H]
-            xk::transpose_kernel<__nv_bfloat16><<<dim3((L.C + 31) / 32, (L.H + 31) / 32, N), dim3(32, 8), 0, stream>>>(
+            le = to.plain(xk::transpose_kernel<__nv_bfloat16>, dim3((L.C + 31) / 32, (L.H + 31) / 32, N), dim3(32, 8), 0,
                 (const __nv_bfloat16 *)ptr(L.in0), (__nv_bfloat16 *)ptr(L.out), L.H, L.C);
             break;
         case LK_F32_TRANSPOSE:  // NCHW: per image [C][H] -> [H][C]
-            xk::transpose_kernel<float><<<dim3((L.H + 31) / 32, (L.C + 31) / 32, N), dim3(32, 8), 0, stream>>>(
+            le = to.plain(xk::transpose_kernel<float>, dim3((L.H + 31) / 32, (L.C + 31) / 32, N), dim3(32, 8), 0,
                 (const float *)ptr(L.in0), (float *)ptr(L.out), L.C, L.H);
             break;
         case LK_SLICE: {
             long long pixels = (long long)N * L.H * L.W;
-            xk::slice_kernel<<<ew_grid(pixels * (L.K / 8), 256, sms), 256, 0, stream>>>((const __nv_bfloat16 *)ptr(L.in0), (__nv_bfloat16 *)ptr(L.out), pixels, L.K, L.C, L.out_coff);
+            le = to.plain(xk::slice_kernel, ew_grid(pixels * (L.K / 8), 256, sms), 256, 0, (const __nv_bfloat16 *)ptr(L.in0), (__nv_bfloat16 *)ptr(L.out), pixels, L.K, L.C, L.out_coff);
             break;
         }
         case LK_F32_SLICE: {
             long long total = (long long)N * L.K * L.H * L.W;
-            xk::f32_slice_kernel<<<ew_grid(total, 256, sms), 256, 0, stream>>>((const float *)ptr(L.in0), (float *)ptr(L.out), N, L.K, L.H * L.W, L.C, L.out_coff);
+            le = to.plain(xk::f32_slice_kernel, ew_grid(total, 256, sms), 256, 0, (const float *)ptr(L.in0), (float *)ptr(L.out), N, L.K, L.H * L.W, L.C, L.out_coff);
             break;
         }
         case LK_GEMM2: {
@@ -595,8 +614,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                     maps = &now;
                 }
                 const int lgrid = (int)std::min(p.tiles, sms), lblock = (int)xk::kCvThreads;
-                cudaError_t le = launch_pdl(L.skip >= 0 ? xk::pair_tc_kernel<true> : xk::pair_tc_kernel<false>, lgrid, lblock, L.smem_bytes, stream, maps->a0, rt->tmaps[li], rt->tmaps2[li], maps->o, maps->s, p);
-                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+                le = to.pdl(L.skip >= 0 ? xk::pair_tc_kernel<true> : xk::pair_tc_kernel<false>, lgrid, lblock, L.smem_bytes, maps->a0, rt->tmaps[li], rt->tmaps2[li], maps->o, maps->s, p);
                 break;
             }
             xk::Chain2Params p;
@@ -623,17 +641,15 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 tma = &tma_now;
             }
             const int lgrid = (int)std::min(p.m_tiles, sms), lblock = (int)xk::kC2Threads;
-            cudaError_t le = launch_pdl(xk::chain2_kernel, lgrid, lblock, L.smem_bytes, stream, *tma, rt->tmaps[li], rt->tmaps2[li], p);
-            if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+            le = to.pdl(xk::chain2_kernel, lgrid, lblock, L.smem_bytes, *tma, rt->tmaps[li], rt->tmaps2[li], p);
             break;
         }
         case LK_GEMM: {
             if (L.fc_small) {
                 const int grid = std::min(sms, (L.K + 7) / 8);
-                cudaError_t le = launch_pdl(N == 1 ? xk::fc_small_kernel<1> : xk::fc_small_kernel<8>, grid, 256, N * L.C * 2, stream,
+                le = to.pdl(N == 1 ? xk::fc_small_kernel<1> : xk::fc_small_kernel<8>, grid, 256, N * L.C * 2,
                     (const __nv_bfloat16 *)ptr(L.seg[0].tensor), (const __nv_bfloat16 *)(ws + L.w_off), (const float *)(ws + L.b_off), ptr(L.out), N, L.C,
                     L.kpad, L.K, L.act, L.out_dtype == XENOS_DTYPE_F32, L.out_ctot, L.out_coff);
-                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
                 break;
             }
             if (L.stem_tc) {
@@ -652,8 +668,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 p.off_w = L.off_b; p.off_bias = L.off_bias; p.off_stage = L.off_stg; p.stage_bytes = (L.off_bar - L.off_stg) / 2 & ~15; p.off_bar = L.off_bar;
                 p.launch_id = (int)li;
                 const int gx = std::min(p.units, std::max(1, sms / L.n_tiles));
-                cudaError_t le = launch_pdl(stem_kernel(L, ((uintptr_t)p.src & 15u) == 0), dim3(gx, L.n_tiles), L.block, L.smem_bytes, stream, p);
-                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+                le = to.pdl(stem_kernel(L, ((uintptr_t)p.src & 15u) == 0), dim3(gx, L.n_tiles), L.block, L.smem_bytes, p);
                 break;
             }
             if (L.conv_tc) {
@@ -692,8 +707,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 int limit = sms;
                 if (L.b_resident) limit = std::max(1, sms / L.n_tiles) * L.n_tiles;
                 const int lgrid = (int)std::min(p.total, limit), lblock = (int)xk::kCvThreads;
-                cudaError_t le = launch_pdl_cluster(conv_kernel(L), L.cv_epi == xk::CE_CLUSTER ? p.total : lgrid, lblock, L.smem_bytes, L.cv_epi == xk::CE_CLUSTER ? L.ksplit : 1, stream, maps->a0, maps->a1, rt->tmaps[li], maps->o, maps->s, p);
-                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+                le = to.pdl_cluster(conv_kernel(L), L.cv_epi == xk::CE_CLUSTER ? p.total : lgrid, lblock, L.smem_bytes, L.cv_epi == xk::CE_CLUSTER ? L.ksplit : 1, maps->a0, maps->a1, rt->tmaps[li], maps->o, maps->s, p);
                 break;
             }
             if (L.seg[0].mode == AM_DW) {
@@ -732,8 +746,7 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 }
                 const int limit = L.b_resident ? std::max(1, sms / L.n_tiles) * L.n_tiles : sms;
                 auto *k = dw_kernel(L.cv_epi, a.stride, L.dw_br);
-                cudaError_t le = launch_pdl(k, std::min(p.total, limit), L.block, L.smem_bytes, stream, maps->a0, rt->tmaps[li], maps->o, p);
-                if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+                le = to.pdl(k, std::min(p.total, limit), L.block, L.smem_bytes, maps->a0, rt->tmaps[li], maps->o, p);
                 break;
             }
             xk::GemmParams p;
@@ -775,83 +788,151 @@ static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, vo
                 }
             }
             const int lgrid = std::min(p.m_tiles * p.n_tiles, sms), lblock = L.block;
-            cudaError_t le = launch_pdl(xk::gemm_chain_kernel, lgrid, lblock, L.smem_bytes, stream, rt->tmaps[li], *tmh, p);
-            if (le != cudaSuccess) return cuda_fail(g, "kernel launch", le);
+            le = to.pdl(xk::gemm_chain_kernel, lgrid, lblock, L.smem_bytes, rt->tmaps[li], *tmh, p);
             break;
         }
         default:
             return fail(g, XENOS_E_UNSUPPORTED, "internal: launch record without a kernel");
         }
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_fail(g, "kernel launch", e);
-        if (ms_per_launch) cudaEventRecord(ev[li + 1], stream);
-    }
-    if (ms_per_launch) {
-        cudaError_t e = cudaStreamSynchronize(stream);
-        for (size_t li = 0; li < g.launches.size(); ++li) {
-            ms_per_launch[li] = 0.0f;
-            if (e == cudaSuccess) cudaEventElapsedTime(&ms_per_launch[li], ev[li], ev[li + 1]);
+        if (le != cudaSuccess) {
+            cudaGetLastError();
+            return cuda_fail(g, "kernel launch", le);
         }
-        for (auto &x : ev) cudaEventDestroy(x);
-        if (e != cudaSuccess) return cuda_fail(g, "profile synchronize", e);
+        const xenos_status_t st = each(li);
+        if (st != XENOS_OK) return st;
     }
     return XENOS_OK;
 }
 
-// A pass of several launches that comes again with the same batch and buffers is recorded on its second call and from then
-// on replayed as one CUDA graph (programmatic dependencies between the kernels included).  Single launches cost the host 2.3
-// to 4.5 us each, more than many of these kernels run on a small batch; a replay costs one call.  Passes whose buffers
-// change from call to call, passes inside a caller's own stream capture and single launches go to the stream directly (a
-// graph of one kernel takes 2.5 us longer than the kernel).
-xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *const *out, void *stream_v, float *ms_per_launch) {
+static xenos_status_t launch_pass(Graph &g, int batch, const void *const *in, void *const *out, void *stream_v) {
+    Issue to;
+    to.stream = static_cast<cudaStream_t>(stream_v);
+    return issue_pass(g, batch, in, out, to, [](size_t) -> xenos_status_t { return XENOS_OK; });
+}
+
+xenos_status_t runtime_profile(Graph &g, int batch, const void *const *in, void *const *out, void *stream_v, float *ms_per_launch) {
+    struct Events {
+        std::vector<cudaEvent_t> v;
+        ~Events() { for (cudaEvent_t e : v) cudaEventDestroy(e); }
+    } ev;
+    Issue to;
+    to.stream = static_cast<cudaStream_t>(stream_v);
+    for (size_t i = 0; i <= g.launches.size(); ++i) {
+        cudaEvent_t e;
+        if (cudaEventCreate(&e) != cudaSuccess) return fail(g, XENOS_E_CUDA, "cudaEventCreate failed");
+        ev.v.push_back(e);
+    }
+    cudaEventRecord(ev.v[0], to.stream);
+    const xenos_status_t st = issue_pass(g, batch, in, out, to, [&](size_t li) -> xenos_status_t {
+        cudaEventRecord(ev.v[li + 1], to.stream);
+        return XENOS_OK;
+    });
+    if (st != XENOS_OK) return st;
+    const cudaError_t e = cudaStreamSynchronize(to.stream);
+    if (e != cudaSuccess) return cuda_fail(g, "profile synchronize", e);
+    for (size_t li = 0; li < g.launches.size(); ++li) {
+        ms_per_launch[li] = 0.0f;
+        cudaEventElapsedTime(&ms_per_launch[li], ev.v[li], ev.v[li + 1]);
+    }
+    return XENOS_OK;
+}
+
+// Records the pass: a graph's launches for max_batch images, as they follow one another in a stream (programmatic dependencies
+// included), with the workspace in the place of the caller's buffers.  Nothing runs.
+static xenos_status_t record_pass(Graph &g, const std::vector<void *> &in, const std::vector<void *> &out, cudaStream_t stream) {
+    Runtime *rt = static_cast<Runtime *>(g.rt);
+    struct Scope {
+        cudaStream_t stream = nullptr;
+        cudaGraph_t graph = nullptr;
+        ~Scope() {
+            if (graph) cudaGraphDestroy(graph);
+            if (stream) cudaStreamDestroy(stream);
+        }
+    } sc;
+    std::vector<cudaGraphNode_t> nodes(g.launches.size(), nullptr);
+    cudaError_t e = cudaStreamCreateWithFlags(&sc.stream, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return cuda_fail(g, "cudaStreamCreateWithFlags", e);
+    if ((e = cudaStreamBeginCapture(sc.stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return cuda_fail(g, "cudaStreamBeginCapture", e);
+    Issue to;
+    to.stream = sc.stream;
+    const xenos_status_t st = issue_pass(g, g.max_batch, in.data(), out.data(), to, [&](size_t li) -> xenos_status_t {
+        // the launch's node is what a next one would depend on
+        cudaStreamCaptureStatus cap;
+        const cudaGraphNode_t *last = nullptr;
+        const cudaGraphEdgeData *edges = nullptr;
+        size_t n = 0;
+        const cudaError_t e = cudaStreamGetCaptureInfo_v3(sc.stream, &cap, nullptr, nullptr, &last, &edges, &n);
+        if (e != cudaSuccess || cap != cudaStreamCaptureStatusActive || n != 1) return cuda_fail(g, "cudaStreamGetCaptureInfo", e);
+        nodes[li] = last[0];
+        return XENOS_OK;
+    });
+    e = cudaStreamEndCapture(sc.stream, &sc.graph);
+    if (st != XENOS_OK) return st;
+    if (e != cudaSuccess) return cuda_fail(g, "cudaStreamEndCapture", e);
+    cudaGraphExec_t exec = nullptr;
+    if ((e = cudaGraphInstantiate(&exec, sc.graph, 0)) != cudaSuccess) return cuda_fail(g, "cudaGraphInstantiate", e);
+    // (else the first pass would wait for it: 147 us instead of 109 for the first pass of SqueezeNet at batch 1)
+    if ((e = cudaGraphUpload(exec, stream)) != cudaSuccess) {
+        cudaGraphExecDestroy(exec);
+        return cuda_fail(g, "cudaGraphUpload", e);
+    }
+    rt->exec = exec;
+    std::swap(rt->graph, sc.graph);
+    rt->nodes.swap(nodes);
+    rt->exec_batch = g.max_batch;
+    return XENOS_OK;
+}
+
+xenos_status_t runtime_bind(Graph &g, void *ws, void *stream_v, bool record) {
+    xenos_status_t st = attach(g, ws, stream_v);
+    if (st != XENOS_OK) return st;
+    Issue to;
+    to.mode = Issue::READY;
+    cudaError_t e = cudaDeviceGetAttribute(&to.optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, static_cast<Runtime *>(g.rt)->device);
+    if (e != cudaSuccess) return cuda_fail(g, "cudaDeviceGetAttribute", e);
+    // (any aligned address does for buffers that only a run names; some kernels have a form of their own for one image)
+    const std::vector<void *> in(g.inputs.size(), ws), out(g.outputs.size(), ws);
+    for (int batch : {g.max_batch, 1}) {
+        st = issue_pass(g, batch, in.data(), out.data(), to, [](size_t) -> xenos_status_t { return XENOS_OK; });
+        if (st != XENOS_OK) return st;
+    }
+    if (record && g.launches.size() > 1 && record_pass(g, in, out, static_cast<cudaStream_t>(stream_v)) != XENOS_OK) cudaGetLastError();      // (launched one by one then)
+    return XENOS_OK;
+}
+
+// A pass of several launches runs as the CUDA graph that the binding recorded, the nodes that meet the caller's buffers pointed
+// at them on every call (1 us): single launches cost the host 2.3 to 4.5 us each, more than many of these kernels run on a small
+// batch, and leave gaps between kernels that follow at once in the graph.  MobileNet at batch 1, other buffers on every call:
+// 98.3 us a pass and 4.4 us of the host, 104.1 and 86.6 in single launches.
+// Another batch than the recorded one is launched one by one; when it comes a second time in a row, all nodes are set to it
+// behind that launch (1.7 us each: before the launch a pass alone would wait 25 us for them).  Passes inside a caller's own
+// stream capture and single launches go to the stream directly (a graph of one kernel takes 2.5 us longer than the kernel).
+xenos_status_t runtime_run(Graph &g, int batch, const void *const *in, void *const *out, void *stream_v) {
     Runtime *rt = static_cast<Runtime *>(g.rt);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
-    if (ms_per_launch || !rt->replay_ok || g.launches.size() < 2) return launch_pass(g, batch, in, out, stream_v, ms_per_launch);
+    if (!rt->exec) return launch_pass(g, batch, in, out, stream_v);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
-        return launch_pass(g, batch, in, out, stream_v, nullptr);
+        return launch_pass(g, batch, in, out, stream_v);
     }
-    const size_t ni = g.inputs.size(), no = g.outputs.size();
-    auto same = [&](const Replay &r) {
-        if (r.key[0] != (const void *)(uintptr_t)batch) return false;
-        for (size_t i = 0; i < ni; ++i) if (r.key[1 + i] != in[i]) return false;
-        for (size_t i = 0; i < no; ++i) if (r.key[1 + ni + i] != out[i]) return false;
-        return true;
+    std::lock_guard<std::mutex> lock(rt->exec_mutex);
+    auto point = [&](bool external_only) {
+        Issue to;
+        to.mode = Issue::POINT; to.rt = rt; to.external_only = external_only;
+        rt->exec_batch = 0;             // (until every node has been set)
+        const xenos_status_t st = issue_pass(g, batch, in, out, to, [](size_t) -> xenos_status_t { return XENOS_OK; });
+        if (st == XENOS_OK) rt->exec_batch = batch;
+        return st;
     };
-    Replay *hit = nullptr;
-    for (Replay &r : rt->replays) if (same(r)) { hit = &r; break; }
-    if (!hit) {
-        // first call with these buffers: remember it (in the slot of the least recently used pass), launch directly
-        if (rt->replays.size() < kReplays) rt->replays.emplace_back();
-        hit = &rt->replays[0];
-        for (Replay &r : rt->replays) if (r.used < hit->used) hit = &r;
-        if (hit->exec) { cudaGraphExecDestroy(hit->exec); hit->exec = nullptr; }
-        hit->key.assign(1, (const void *)(uintptr_t)batch);
-        hit->key.insert(hit->key.end(), in, in + ni);
-        for (size_t i = 0; i < no; ++i) hit->key.push_back(out[i]);
-        hit->used = ++rt->tick;
-        return launch_pass(g, batch, in, out, stream_v, nullptr);
+    const bool again = batch == rt->last_batch;
+    rt->last_batch = batch;
+    if (batch != rt->exec_batch) {
+        const xenos_status_t st = launch_pass(g, batch, in, out, stream_v);
+        return st == XENOS_OK && again ? point(false) : st;
     }
-    hit->used = ++rt->tick;
-    if (!hit->exec) {
-        cudaGraph_t graph = nullptr;
-        bool good = rt->record_stream || cudaStreamCreateWithFlags(&rt->record_stream, cudaStreamNonBlocking) == cudaSuccess;
-        good = good && cudaStreamBeginCapture(rt->record_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        if (good) {
-            const xenos_status_t st = launch_pass(g, batch, in, out, rt->record_stream, nullptr);
-            good = cudaStreamEndCapture(rt->record_stream, &graph) == cudaSuccess && st == XENOS_OK && graph;
-            good = good && cudaGraphInstantiate(&hit->exec, graph, 0) == cudaSuccess;
-            if (graph) cudaGraphDestroy(graph);
-        }
-        if (!good) {
-            cudaGetLastError();
-            hit->exec = nullptr;
-            rt->replay_ok = false;
-            return launch_pass(g, batch, in, out, stream_v, nullptr);
-        }
-    }
-    const cudaError_t e = cudaGraphLaunch(hit->exec, stream);
+    if (xenos_status_t st = point(true)) return st;
+    const cudaError_t e = cudaGraphLaunch(rt->exec, stream);
     if (e != cudaSuccess) return cuda_fail(g, "kernel launch", e);
     return XENOS_OK;
 }
@@ -934,7 +1015,7 @@ xenos_status_t runtime_run_builtin(Graph &g, int batch, const void *const *in, v
     if (!rb || rb->device != dev || g_builtin_owner[dev] != g.serial) {
         // the array holds nothing or another graph's data: upload parameters, clear status, encode maps
         g_builtin_owner[dev] = 0;
-        st = runtime_bind(g, scratch, kBuiltinScratchBytes, stream);
+        st = runtime_bind(g, scratch, stream, false);      // (never recorded: that would allocate)
         g_builtin_owner[dev] = st == XENOS_OK ? g.serial : 0;
     } else {
         g.ws = scratch;
@@ -942,7 +1023,7 @@ xenos_status_t runtime_run_builtin(Graph &g, int batch, const void *const *in, v
         if ((e = cudaMemsetAsync(static_cast<uint8_t *>(scratch) + g.status_off, 0, 256 + g.cnt_bytes, stream)) != cudaSuccess)
             st = cuda_fail(g, "status clear", e);
     }
-    if (st == XENOS_OK) st = launch_pass(g, batch, in, out, stream, nullptr);      // (never recorded: that would allocate)
+    if (st == XENOS_OK) st = launch_pass(g, batch, in, out, stream);
     if (st == XENOS_OK) st = runtime_status(g, stream);
     return st;
 }

@@ -95,10 +95,10 @@ xenos_status_t search_splits(Graph &g, int max_batch, int precision, void *ws, s
         if (trial.workspace_bytes > ws_bytes)
             return fail(g, XENOS_E_WORKSPACE, "search: a trial plan needs " + std::to_string(trial.workspace_bytes) + " workspace bytes");
         if ((int)trial.chains.size() != nc) return fail(g, XENOS_E_INVALID, "internal: chains changed between trials");
-        st = runtime_bind(trial, ws, ws_bytes, stream);
+        st = runtime_bind(trial, ws, stream, false);
         std::vector<float> per(trial.launches.size()), acc(trial.launches.size(), 0.0f);
         for (int r = 0; r <= repeats && st == XENOS_OK; ++r) {      // the first run warms up
-            st = runtime_run(trial, max_batch, in, out, stream, per.data());
+            st = runtime_profile(trial, max_batch, in, out, stream, per.data());
             if (r > 0) for (size_t i = 0; i < per.size(); ++i) acc[i] += per[i];
         }
         if (st == XENOS_OK) st = runtime_status(trial, stream);

@@ -1,5 +1,10 @@
 """Every kernel of the fast paths at the sizes where it can go wrong: edges of tiles, remainders, the smallest and the
 largest of its range.  The oracle and the tolerances are those of the parity tests."""
+import os
+import subprocess
+import sys
+import threading
+
 import numpy as np
 import pytest
 
@@ -172,4 +177,65 @@ def test_repeated_passes(name, kw):
     graph.replay()
     torch.cuda.synchronize()
     assert np.array_equal(out.float().cpu().numpy(), want[3])
+    gg.g.status(gg.stream)
+
+
+# Buffers that no call has seen before cost the host what repeated ones do, and no run reserves device memory (in a process of its
+# own: what a library holds stays reserved until the process ends).  In single launches a pass of this graph takes the host some
+# twenty times as long as the one call of its recorded form; the bound lies between.
+def test_new_buffers_cost_what_repeated_ones_do():
+    child = """
+import statistics, sys, time
+import torch
+from gpu_util import GpuGraph
+from xenos_workloads import graphs
+spec = graphs.mobilenet_v1(hw=64, width=0.25, classes=24)
+gg = GpuGraph(spec, graphs.make_params(spec), 3)
+xin = [gg.upload(graphs.make_input(spec, 3)) for _ in range(40)]
+out = [gg.alloc_out(3) for _ in range(40)]
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+def host_us(i, b):
+    torch.cuda.synchronize()
+    t = time.perf_counter()
+    gg.g.run(b, [xin[i].data_ptr()], [out[i].data_ptr()], gg.stream)
+    return (time.perf_counter() - t) * 1e6
+new = statistics.median(host_us(i, 3) for i in range(40))
+old = statistics.median(host_us(0, 3) for _ in range(40))
+for b in (1, 2, 2, 2, 3, 3):
+    host_us(0, b)
+torch.cuda.synchronize()
+taken = free - torch.cuda.mem_get_info()[0]
+print(new, old, taken)
+sys.exit(0 if new <= 3 * old and taken == 0 else 1)
+"""
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(here), here]))
+    r = subprocess.run([sys.executable, "-c", child], env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+# two host threads enqueue passes of one binding on one stream, each with buffers of its own
+def test_passes_from_two_threads():
+    import torch
+    spec = graphs.mobilenet_v1(hw=64, width=0.25, classes=24)
+    x = graphs.make_input(spec, 6)
+    gg = GpuGraph(spec, graphs.make_params(spec), 3)
+    want = [gg.run(x[:3]), gg.run(x[3:5])]
+    xin = [gg.upload(x[:3]), gg.upload(x[3:5])]
+    wrong = []
+
+    def work(i, batch):
+        for _ in range(100):
+            out = gg.alloc_out(batch)
+            gg.g.run(batch, [xin[i].data_ptr()], [out.data_ptr()], gg.stream)
+            if not np.array_equal(out.cpu().numpy(), want[i]):
+                wrong.append(i)
+    threads = [threading.Thread(target=work, args=a) for a in ((0, 3), (1, 2))]
+    torch.cuda.synchronize()
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
     gg.g.status(gg.stream)
