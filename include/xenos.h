@@ -201,7 +201,8 @@ XENOS_API xenos_status_t xenos_graph_compile(xenos_graph_t *g, int32_t max_batch
 /* Attach a caller-owned DEVICE workspace (256-byte aligned, >= workspace_bytes) and upload
  * the packed weights into it on `cuda_stream` (a cudaStream_t; NULL = default stream).
  * The workspace must stay valid and unshared until destroy or the next bind.  The pass for max_batch images is recorded as a
- * CUDA graph, which later runs use with their own buffers. */
+ * CUDA graph, which later runs use with their own buffers.  When that fails (the driver has no memory left for it) the call
+ * succeeds all the same, runs launch their kernels one by one, and xenos_last_error says why until the next call on g. */
 XENOS_API xenos_status_t xenos_graph_bind(xenos_graph_t *g, void *workspace_dev, size_t bytes,
                                           void *cuda_stream);
 
@@ -297,7 +298,8 @@ XENOS_API xenos_status_t xenos_graph_launch_count(const xenos_graph_t *g, int32_
 
 XENOS_API xenos_status_t xenos_graph_destroy(xenos_graph_t *g);
 
-/* Message of the last failing call on g (never NULL; valid until the next call on g).
+/* Message of the last failing call on g, or of a binding without a recorded pass (never NULL; valid until the next call on
+ * g).
  * With g == NULL: message of the last failing xenos_graph_create on this thread. */
 XENOS_API const char *xenos_last_error(const xenos_graph_t *g);
 

@@ -896,7 +896,10 @@ xenos_status_t runtime_bind(Graph &g, void *ws, void *stream_v, bool record) {
         st = issue_pass(g, batch, in.data(), out.data(), to, [](size_t) -> xenos_status_t { return XENOS_OK; });
         if (st != XENOS_OK) return st;
     }
-    if (record && g.launches.size() > 1 && record_pass(g, in, out, static_cast<cudaStream_t>(stream_v)) != XENOS_OK) cudaGetLastError();      // (launched one by one then)
+    if (record && g.launches.size() > 1 && record_pass(g, in, out, static_cast<cudaStream_t>(stream_v)) != XENOS_OK) {
+        cudaGetLastError();             // (not a reason to refuse the binding: the kernels are launched one by one then)
+        g.err = "bind: passes run kernel by kernel, recording them failed: " + g.err;
+    }
     return XENOS_OK;
 }
 
