@@ -16,8 +16,11 @@
  *  - HOST pointers: every pointer inside xenos_op_desc_t, xenos_hw_info_t, id arrays, the
  *    JSON buffer.  They are read during the call only; the caller keeps ownership.
  *  - DEVICE pointers: the workspace given to xenos_graph_bind and the input / output
- *    arrays given to xenos_graph_run.  The library never allocates or frees device memory;
- *    the caller (typically PyTorch) owns all of it and owns the stream.
+ *    arrays given to xenos_graph_run.  The caller (typically PyTorch) owns all of it and owns
+ *    the stream; the library never allocates or frees device memory for tensors, parameters
+ *    or scratch.  What the CUDA driver itself keeps for loaded kernels and for the recorded
+ *    pass of a binding is reserved by xenos_graph_bind (2 MB for the first recording of a
+ *    process), never by xenos_graph_run; xenos_graph_run_builtin_scratch records nothing.
  *  - There is no CPU fallback: xenos_graph_bind / xenos_graph_run fail with XENOS_E_CUDA
  *    when no sm_100 device is usable.
  *  - State machine: create -> add_input / add_op / mark_output -> (link)* -> (split)* ->

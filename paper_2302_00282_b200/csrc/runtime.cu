@@ -1,6 +1,6 @@
 // CUDA runtime of the library: uploads the packed parameters into the caller's workspace,
 // encodes the TMA descriptors, and enqueues one kernel per launch record on the caller's stream.
-// Allocates no device memory.  (Section 3 of the Xenos paper: the runtime executes the optimised
+// Allocates no device memory of its own (the driver keeps some for the pass that a binding records).  (Section 3 of the Xenos paper: the runtime executes the optimised
 // model on the parallel units on top of the operator library.)
 #include <cuda.h>
 #include <cudaTypedefs.h>
