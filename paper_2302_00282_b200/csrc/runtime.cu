@@ -41,6 +41,7 @@ struct Runtime {
     }
     int device = -1;
     int sm_count = 0;
+    int optin = 0;                      // shared memory a block may ask for
     std::vector<CUtensorMap> tmaps;     // one per launch record (used by gemm launches only)
     std::vector<CUtensorMap> hmaps;     // halo maps of linked depthwise stages / activation operand maps
     std::vector<CUtensorMap> tmaps2;    // second weight matrix of two linked convolutions
@@ -346,14 +347,19 @@ static xenos_status_t attach(Graph &g, void *ws, void *stream_v) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(g, "no CUDA device (this library has no CPU fallback)", e);
-    cudaDeviceProp prop;
-    if ((e = cudaGetDeviceProperties(&prop, dev)) != cudaSuccess) return cuda_fail(g, "cudaGetDeviceProperties", e);
-    if (prop.major != 10) return fail(g, XENOS_E_CUDA, "device is not sm_100 (B200); the kernels are built for sm_100a only");
+    // (single attributes: the whole property record takes 2.8 ms, several times the rest of a binding)
+    int major = 0, sms = 0, optin = 0;
+    if ((e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
+        return cuda_fail(g, "cudaDeviceGetAttribute", e);
+    if (major != 10) return fail(g, XENOS_E_CUDA, "device is not sm_100 (B200); the kernels are built for sm_100a only");
     runtime_free(g);
     Runtime *rt = new Runtime();
     g.rt = rt;
     rt->device = dev;
-    rt->sm_count = prop.multiProcessorCount;
+    rt->sm_count = sms;
+    rt->optin = optin;
     // parameters -> workspace, status words cleared
     if (!g.param_blob.empty())
         if ((e = cudaMemcpyAsync(ws, g.param_blob.data(), g.param_blob.size(), cudaMemcpyHostToDevice, stream)) != cudaSuccess)
@@ -428,7 +434,6 @@ static xenos_status_t attach(Graph &g, void *ws, void *stream_v) {
             }
         }
     }
-    const int optin = (int)prop.sharedMemPerBlockOptin;
     if (max_gemm_smem > optin || max_chain_smem > optin)
         return fail(g, XENOS_E_CUDA, "a kernel of this plan needs more shared memory than the device offers");
     return XENOS_OK;
@@ -888,8 +893,7 @@ xenos_status_t runtime_bind(Graph &g, void *ws, void *stream_v, bool record) {
     if (st != XENOS_OK) return st;
     Issue to;
     to.mode = Issue::READY;
-    cudaError_t e = cudaDeviceGetAttribute(&to.optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, static_cast<Runtime *>(g.rt)->device);
-    if (e != cudaSuccess) return cuda_fail(g, "cudaDeviceGetAttribute", e);
+    to.optin = static_cast<Runtime *>(g.rt)->optin;
     // (any aligned address does for buffers that only a run names; some kernels have a form of their own for one image)
     const std::vector<void *> in(g.inputs.size(), ws), out(g.outputs.size(), ws);
     for (int batch : {g.max_batch, 1}) {

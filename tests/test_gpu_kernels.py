@@ -239,3 +239,18 @@ def test_passes_from_two_threads():
         t.join()
     assert not wrong
     gg.g.status(gg.stream)
+
+
+# A binding is an upload, some maps and the recording of a pass: 0.33 ms for a small graph (a device's whole property record alone
+# takes 2.8 ms)
+def test_binding_is_quick():
+    import statistics
+    import time
+    spec = graphs.mobilenet_v1(hw=64, width=0.25, classes=24)
+    gg = GpuGraph(spec, graphs.make_params(spec), 1)
+
+    def once():
+        t = time.perf_counter()
+        gg.g.bind(gg.ws.data_ptr(), gg.ws.numel(), gg.stream)
+        return time.perf_counter() - t
+    assert statistics.median(once() for _ in range(21)) < 2e-3
