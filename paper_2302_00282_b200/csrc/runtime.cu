@@ -252,9 +252,9 @@ static StemKernel stem_kernel(int mode, bool f32, bool pool) {
          : mode == xk::SM_S2X ? stem_kernel_of<xk::SM_S2X>(f32, pool) : stem_kernel_of<xk::SM_ANY>(f32, pool);
 }
 
-// Whole groups of elements where rows are made of them and the image is aligned; else element by element.
-static StemKernel stem_kernel(const Launch &L, bool aligned) {
-    const int mode = L.stride == 2 ? (L.st_vec && aligned ? xk::SM_S2 : xk::SM_S2X) : L.stride == 1 ? xk::SM_S1 : xk::SM_ANY;
+// Whole groups of elements where rows are made of them (images are 16-byte aligned); else element by element.
+static StemKernel stem_kernel(const Launch &L) {
+    const int mode = L.stride == 2 ? (L.st_vec ? xk::SM_S2 : xk::SM_S2X) : L.stride == 1 ? xk::SM_S1 : xk::SM_ANY;
     return stem_kernel(mode, L.seg[0].src_dtype == XENOS_DTYPE_F32, L.epi == EPI_POOL);
 }
 
@@ -673,7 +673,7 @@ static xenos_status_t issue_pass(Graph &g, int batch, const void *const *in, voi
                 p.off_w = L.off_b; p.off_bias = L.off_bias; p.off_stage = L.off_stg; p.stage_bytes = (L.off_bar - L.off_stg) / 2 & ~15; p.off_bar = L.off_bar;
                 p.launch_id = (int)li;
                 const int gx = std::min(p.units, std::max(1, sms / L.n_tiles));
-                le = to.pdl(stem_kernel(L, ((uintptr_t)p.src & 15u) == 0), dim3(gx, L.n_tiles), L.block, L.smem_bytes, p);
+                le = to.pdl(stem_kernel(L), dim3(gx, L.n_tiles), L.block, L.smem_bytes, p);
                 break;
             }
             if (L.conv_tc) {
@@ -785,12 +785,9 @@ static xenos_status_t issue_pass(Graph &g, int batch, const void *const *in, voi
             CUtensorMap tmh_now;
             if (L.stem_tma) {
                 // the image is a caller buffer: encode its patch map now
-                if (((uintptr_t)ptr(L.seg[0].tensor) & 15u) != 0) p.stem_tma = 0;      // unaligned image: direct loads
-                else {
-                    xenos_status_t st = encode_stem_map(g, rt, L, ptr(L.seg[0].tensor), N, &tmh_now);
-                    if (st != XENOS_OK) return st;
-                    tmh = &tmh_now;
-                }
+                xenos_status_t st = encode_stem_map(g, rt, L, ptr(L.seg[0].tensor), N, &tmh_now);
+                if (st != XENOS_OK) return st;
+                tmh = &tmh_now;
             }
             const int lgrid = std::min(p.m_tiles * p.n_tiles, sms), lblock = L.block;
             le = to.pdl(xk::gemm_chain_kernel, lgrid, lblock, L.smem_bytes, rt->tmaps[li], *tmh, p);
