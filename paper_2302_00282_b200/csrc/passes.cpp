@@ -699,20 +699,21 @@ struct Lower {
     // Packs the [npad][kpad] bf16 weight matrix of an implicit GEMM: row n = output channel,
     // K order = (tap r*k+s, input channel c) per segment, each segment padded to 64.
     // ---- tiles of conv_tc_kernel ------------------------------------------------------------------------------------
-    // Modelled cycles of a plan with tile_n columns and ksplit chunks on `units` SMs.  Per 64-wide K block a CTA waits for
-    // the slower of the tensor pipe (max(48, tile_n / 2) cycles per K = 16 step) and the operand traffic from L2 (75
-    // bytes per cycle and SM); a tile's epilogue overlaps the next tile's product; a split adds the exchange of the partial
-    // sums.  The constants are measurements on B200 (see conv_tc.cuh).
-    // Clusters of ks CTAs that fit the device at once, one CTA or two (half) per SM (queried on B200; clusters stay inside a
-    // GPC, so the larger ones leave SMs unused).
-    static int cluster_capacity(int ks, bool half) {
+    // Clusters of ks CTAs that fit the units of the hardware description at once, one CTA or two (half) per unit.  The table is
+    // what the 148 SMs of a B200 answer (clusters stay inside a GPC, so the larger ones leave SMs unused); other unit counts get
+    // their share of it.
+    int cluster_capacity(int ks, bool half) const {
         static const int one[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15}, two[9] = {0, 296, 148, 93, 71, 56, 45, 37, 33};
-        return half ? two[ks] : one[ks];
+        return (int)((long)(half ? two[ks] : one[ks]) * g.hw.sm_count / 148);
     }
     static int conv_smem_cap(bool half) { return half ? kClusterSmem : 227 * 1024; }
     static constexpr int kClusterSmem = 112 * 1024;      // what two CTAs of an SM can have each
     // Exchange buffer of a cluster's partial sums.
     static int cluster_bytes(int rows, int tile_n, int ks) { return (int)align_up((size_t)ks * ceil_div(rows, ks) * (tile_n + 4) * 4, 1024); }
+    // Modelled cycles of a plan with tile_n columns and ksplit chunks on `units` SMs.  Per 64-wide K block a CTA waits for
+    // the slower of the tensor pipe (max(48, tile_n / 2) cycles per K = 16 step) and the operand traffic from L2 (75
+    // bytes per cycle and SM); a tile's epilogue overlaps the next tile's product; a split adds the exchange of the partial
+    // sums.  The constants are measurements on B200 (see conv_tc.cuh).
     double conv_cycles(const Launch &L, int tile_n, int n_tiles, int ksplit, bool half) const {
         const double units = g.hw.sm_count;
         const double tiles = (double)L.m_tiles * n_tiles;

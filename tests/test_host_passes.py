@@ -314,6 +314,18 @@ def _unit(build, cin, hw):
     return g
 
 
+@pytest.mark.parametrize("sms", [1, 8, 16, 32, 64, 148])
+@pytest.mark.parametrize("cin,hw,cout,k", [(512, 7, 512, 3), (256, 14, 256, 3), (128, 28, 128, 3), (2048, 7, 512, 1)])
+def test_automatic_reduction_split_fits_the_described_units(cin, hw, cout, k, sms):
+    """The chunks of a reduction that the planner cuts by itself run at the same time: at most two CTAs per unit of the hardware
+    description."""
+    spec = _unit(lambda g: g.cbr("c", "input", cout, k, 1, k // 2), cin, hw)
+    for batch in (1, 4):
+        g, _ = compiled(spec, batch, hw=xb.HwInfo(sms, 227 * 1024, 512, 126 << 20), nhwc=True)
+        L = g.plan()["launches"][0]
+        assert L["ksplit"] == 1 or L["m_tiles"] * L["n_tiles"] * L["ksplit"] <= 2 * sms
+
+
 @pytest.mark.parametrize("parts_k", [2, 3, 4, 6, 9, 18, 36])
 def test_reduction_split_is_an_ascending_exact_cover_of_the_k_blocks(parts_k):
     """Section 4.2.2: the reduction (C, R, S) is cut last and needs an additional reduction.  Here: chunks of
