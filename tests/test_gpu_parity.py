@@ -555,6 +555,19 @@ def test_split_search_keeps_the_fastest_measured_scheme_bf16():
     assert abs_err_scaled(y, o) <= BF16_TOL and abs_err_scaled(y, y_plain) <= 2.0 ** -7
 
 
+def test_split_search_cuts_the_reduction_of_a_block_with_a_shortcut_convolution():
+    def build(g):
+        x = g.cbr("c1", "input", 128, 3, 2, 1)
+        x = g.cbr("c2", x, 128, 3, 1, 1, act=None)
+        s = g.cbr("proj", "input", 128, 1, 2, 0, act=None)
+        g.act("out", g.add("add", x, s), "relu")
+    spec = _one(build, 64, 12)
+    report, plan, y, y_plain, o = _searched(spec, 1, "bf16_nhwc")
+    tail = [c for c in report["chains"] if plan["launches"][plan["chains"][c["id"]]["launches"][0]]["a1"] != "none"]
+    assert len(tail) == 1 and any(k["label"].startswith("k ") for k in tail[0]["candidates"])
+    assert abs_err_scaled(y, o) <= BF16_TOL and abs_err_scaled(y, y_plain) <= 2.0 ** -7
+
+
 def test_split_search_on_the_fp32_chain():
     spec = graphs.single_chain()
     report, plan, y, y_plain, o = _searched(spec, 1, "f32_nchw")
