@@ -17,7 +17,7 @@
 //               alternate column chunks: bias, activation [, + shortcut, activation], bf16, a swizzled 32-row box in
 //               shared memory, one bulk tensor store.  A shortcut tile arrives in the same boxes the result leaves from.
 // All roles run warp-uniformly and elect one lane per request: measured here, a copy request issued from inside an
-// `if (lane == 0)` branch with address divisions costs 535 cycles of that lane, 149 when elected and without divisions,
+// `if (lane == 0)` branch with address divisions costs 535 cycles of that lane, 240 to 260 when elected and without divisions,
 // and an MMA 61 against 40-48 (M = 128, N <= 64; 64 at N = 128, 128 at N = 256, the pipe's own time).
 // What bounds it: L2 -> shared memory for A (16 KB per block at the measured 71-76 B per cycle and SM: about 220 cycles,
 // against 192 / 256 / 512 cycles of the tensor pipe for N = 64 / 128 / 256), and for 1x1 products HBM.
@@ -38,7 +38,8 @@ constexpr int kCvMaxCluster = 8;
 constexpr int kMaxSkipSlots = 4;         // shortcut / result boxes per epilogue warp
 constexpr int kGapFloats = 4352;         // column sums of an average, per half of the epilogue
 
-// Exact division of n < 2^31 by a constant of the launch.
+// Exact division of n < 2^31 by a constant of the launch: multiplication by a rounded-up reciprocal and a shift (Granlund and
+// Montgomery, Division by Invariant Integers using Multiplication, 1994).
 struct FastDiv {
     uint32_t mul, shift, d;
     __device__ __forceinline__ uint32_t div(uint32_t n) const { return (__umulhi(n, mul) + n) >> shift; }

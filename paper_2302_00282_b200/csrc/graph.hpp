@@ -139,7 +139,8 @@ struct Launch {
     int acc_stride = 0;                                            // columns between the two accumulators
     int hstages = 0, halo_bytes = 0, halo_stride = 0, halo_cb = 0;   // depthwise halo ring (halo_h x halo_w input pixels per image)
     int stem_tma = 0, stem_align = 1;                              // stem: image patch by TMA, x alignment in elements
-    int a_tma = 0, a_box_bytes = 0;                                // activation operand by TMA: 1 matrix rows, 2 shifted patch
+    int a_tma = 0;                // for the plan only: activation operand as plain boxes, 1 matrix rows, 2 shifted patch
+    int a_box_bytes = 0;          // two linked convolutions: bytes of a box of the first one's input
     int fc_small = 0;                                              // 1: fully connected layer of a small batch on the CUDA cores (fc_small_kernel)
     int dw_workers = 0;                                            // depthwise -> pointwise (dw_tc_kernel): worker warps
     int dw_groups = 0, dw_wpg_log2 = 0, dw_br = 1, dw_batch = 1, h_slots = 0, out_bufs = 1;      // ... their groups, a thread's block rows, halo slots, result boxes

@@ -261,7 +261,10 @@ static bool try_match(const LinkCtx &cx, int a, Allowed allowed, Chain &out, boo
                 g.tensors[E0.in[0]].output_slot < 0 && sc.size() == 2 && cx.sole(a) >= -1 &&
                 !(g.tensors[g.nodes[sq].in[0]].input_slot >= 0 && g.tensors[g.nodes[sq].in[0]].io_layout == XENOS_LAYOUT_NCHW)) {
                 int p2 = cx.sole(a);
-                const bool pooled = p2 >= 0 && g.nodes[p2].kind == NK_MAXPOOL;      // the pooled fire modules keep the pool link
+                const bool pooled = p2 >= 0 && g.nodes[p2].kind == NK_MAXPOOL;      // (no kernel takes the squeeze and the pool)
+                // (on request only: SqueezeNet with the squeezes of the six fire modules without a pool on chip takes 148 us
+                // against 76 at batch 1, 164 against 86 at batch 4 and 293 against 168 at batch 32, and each of the six alone
+                // makes it slower at every batch)
                 if (!pooled && !by_model) {
                     out.kind = CK_CONV_CONV;
                     out.nodes = {sq, e0, e1, a};
@@ -271,9 +274,11 @@ static bool try_match(const LinkCtx &cx, int a, Allowed allowed, Chain &out, boo
             }
         }
         int p = cx.sole(a);
-        // The pool is attached to small maps only, where it saves a launch: its tiles overlap (27 % more rows of the expands for
-        // a 3x3 stride-2 pool) and gather their operand through the cores.  Measured, 16 -> 128 channels on 55 x 55 and 32 -> 256
-        // on 27 x 27: linked 53 and 30 us at batch 32 (15 and 14 at batch 1), as two kernels 16 + 9 and 14 + 7 (9 + 6 and 10 + 6).
+        // The pool is attached to small maps only, where it keeps the concatenation off memory: its tiles overlap (27 % more rows
+        // of the expands for a 3x3 stride-2 pool) and gather their operand through the cores.  Measured, 32 -> 256 channels with
+        // the squeeze before them: on maps of 64 to 484 pixels 12.3 us linked and 10.3 as two kernels (the link never wins
+        // time), on 27 x 27 at batches 1, 2 and 4 12.3, 13.1 and 16.4 against 10.3, 10.7 and 12.3.  SqueezeNet with both pools
+        // linked: 82 us against 76 at batch 1, 122 against 111 at batch 8.
         const bool small_map = (long)g.max_batch * g.tensors[A.out].h * g.tensors[A.out].w <= 512;
         if (p >= 0 && allowed(p) && g.nodes[p].kind == NK_MAXPOOL && (small_map || !by_model)) {
             int th, tw, rh, rw;
@@ -310,7 +315,8 @@ static bool try_match(const LinkCtx &cx, int a, Allowed allowed, Chain &out, boo
             }
             // (a 3x3 consumer, like a fire module with its squeeze on chip, is linked on request only: the producer's tile carries
             // the consumer's frame and its rows are multiplied again.  Measured, 1x1 128 -> 32 and 3x3 32 -> 32, batch 16 at 64 x 64
-            // and batch 32 at 128 x 128: 41 and 252 us linked, 11 + 14 and 35 + 52 as two kernels)
+            // and batch 32 at 128 x 128: 41 and 252 us linked, 11 + 14 and 35 + 52 as two kernels; ResNet-18 with the two blocks
+            // of its first stage linked: 107.5 us against 103.8 at batch 1, 156 against 139 at batch 4, 236 against 188 at 16)
             if (!by_model || (B.k == 1 && chain2_pays(g, A, B, with_add))) {
                 out.kind = CK_CONV_CONV;
                 out.nodes = {a, b};
@@ -337,7 +343,9 @@ static bool try_match(const LinkCtx &cx, int a, Allowed allowed, Chain &out, boo
             int c = cx.sole(b);
             // (a global average is not attached to a long reduction that would run on a handful of units: the epilogue
             // with the average cannot take part in a reduction split, and at batch 1 the 72 K blocks of ResNet-18's last
-            // convolution then run one after the other on 16 units, 38 us against 14 + 6 us as two kernels)
+            // convolution then run one after the other on 16 units.  The whole graph with the average attached and apart, 16 tiles
+            // (batch 1): 110.9 and 103.6 us, 64 tiles (batch 9): 158.9 and 154.8, 112 (16): 193.8 and 188.5, 128 (20): 206.9 and
+            // 204.9; from one tile per unit on the link wins: 160 (24): 223.0 and 223.8, 208 (32): 255.4 and 256.9)
             const long gap_tiles = (long)((g.max_batch * cx.rows(b) + 127) / 128) * ((A.cout + 31) / 32);
             const bool serial_k = by_model && (long)A.k * A.k * A.cin >= 16 * 64 && gap_tiles <= g.hw.sm_count;
             if (c >= 0 && allowed(c) && g.nodes[c].kind == NK_GAP && cx.rows(b) <= 128 && !serial_k) {
@@ -350,14 +358,13 @@ static bool try_match(const LinkCtx &cx, int a, Allowed allowed, Chain &out, boo
             int th, tw, rh, rw;
             const Tensor &po = g.tensors[B.out];
             if (!pool_patch(B.k, B.stride, po.h, po.w, th, tw, rh, rw)) return false;
-            // An image convolution with its max pool is linked on request only: the pool's tiles overlap (27 % more
-            // convolution rows for a 3x3 stride-2 pool) and the pooling pass of the epilogue costs what the separate pool
-            // kernel costs.  Measured at batch 32, linked against the two kernels: 96 vs 77 us (7x7 stem, 64 channels),
-            // 73 vs 50 us (3x3 stem, 64 channels), 166 vs 125 us (3x3, 24 channels), 830 vs 788 us (7x7 stem at 512 x 512,
-            // batch 64).
-            // At batch 1 the link wins (one launch less: 0.221 vs 0.231 ms for the whole 3x3-stem graph).
-            // Images wider than 256 pixels keep the link: the difference is small there and the link saves the
-            // convolution's output, the largest tensor of the graph (1.07 GB written and read at 512 x 512, batch 64).
+            // At batch 8 and above an image convolution and its max pool stay two kernels for images up to 256 pixels wide.  The
+            // rule was measured with the kernel before stem_tc_kernel, whose pooling pass cost what a pool kernel costs.  With
+            // the pool in registers the link is the faster form there, too: SqueezeNet (3x3 stem) 96 us linked against 110
+            // at batch 8, 158 against 168 at 32, 245 against 270 at 64; ResNet-18 (7x7 stem) 160 against 160, 246 against 255
+            // and 361 against 386; 3x3, 24 channels, 224 x 224: 21 against 30 us at batch 8, 66 against 81 at 32.  It can be
+            // requested.  Below batch 8 and for wider images it is linked (7x7 stem at 512 x 512: 31 against 51 us at batch 8, 201
+            // against 366 at batch 64).
             if (by_model && nchw_in && g.max_batch >= 8 && g.tensors[A.in[0]].w <= 256 && g.tensors[A.in[0]].h <= 256) return false;
             out.kind = CK_CONV_TAIL;
             out.nodes = {a, b};
@@ -696,8 +703,6 @@ struct Lower {
     }
 
     // ---- bf16 tensor-core lowering ---------------------------------------------------------
-    // Packs the [npad][kpad] bf16 weight matrix of an implicit GEMM: row n = output channel,
-    // K order = (tap r*k+s, input channel c) per segment, each segment padded to 64.
     // ---- tiles of conv_tc_kernel ------------------------------------------------------------------------------------
     // Clusters of ks CTAs that fit the units of the hardware description at once, one CTA or two (half) per unit.  The table is
     // what the 148 SMs of a B200 answer (clusters stay inside a GPC, so the larger ones leave SMs unused); other unit counts get
@@ -713,7 +718,8 @@ struct Lower {
     // Modelled cycles of a plan with tile_n columns and ksplit chunks on `units` SMs.  Per 64-wide K block a CTA waits for
     // the slower of the tensor pipe (max(48, tile_n / 2) cycles per K = 16 step) and the operand traffic from L2 (75
     // bytes per cycle and SM); a tile's epilogue overlaps the next tile's product; a split adds the exchange of the partial
-    // sums.  The constants are measurements on B200 (see conv_tc.cuh).
+    // sums.  The constants are measurements on B200 (see conv_tc.cuh), but a stage of several copy requests is charged like one:
+    // four im2col boxes of 16 channels are 300 cycles here and some 1000 on the device.
     double conv_cycles(const Launch &L, int tile_n, int n_tiles, int ksplit, bool half) const {
         const double units = g.hw.sm_count;
         const double tiles = (double)L.m_tiles * n_tiles;
@@ -752,7 +758,6 @@ struct Lower {
                 }
         }
     }
-    // Shared memory and epilogue shape of conv_tc_kernel.
     // Convolution of an NCHW image in stem_tc_kernel: false when the shape is outside it (1 x 1 windows, more than 7 channels, a
     // pool whose windows overlap by more than one row, rows too wide for the ring).
     bool layout_stem(Launch &L, const Node &M, const Tensor &src, const Node *pooln, int N, const SplitRequest &rq) {
@@ -840,6 +845,7 @@ struct Lower {
         for (int o = 0; o < M.cout; ++o) bp[o] = M.b[o];
     }
 
+    // Shared memory and epilogue shape of conv_tc_kernel.
     xenos_status_t layout_conv(Launch &L, const Tensor &ot) {
         const bool vec = L.out_dtype == XENOS_DTYPE_F32 || ot.c % 8;
         // (up to eight chunks are the CTAs of a cluster while the exchange buffer leaves room for the ring; other splits go
@@ -940,7 +946,8 @@ struct Lower {
                             if (a_min > 8 || h_min > 8 || need > room) continue;
                             // The workers' time per tile: the stencils, then their group's boxes, which cost some 1100 cycles and
                             // 14 a column (measured, barriers and store hand-over included), so that four groups with one 64-column
-                            // box each of four tiles beat four 16-column boxes of every tile.
+                            // box each of four tiles beat four 16-column boxes of every tile.  (A single box buffer is charged 10
+                            // cycles per K block, an estimate.)
                             const double t = L.kblocks * (std::max((1 << w) * issue / 4.0, (300.0 + 2.2 * issue) / groups) + (res ? 0.0 : 20.0) + (bufs == 1 ? 10.0 : 0.0)) +
                                              (L.cv_epi == 0 ? (double)ceil_div(nb * ceil_div(cols, chunk), 4) / nb * (1100.0 + 14.0 * chunk) : 0.0);
                             if (best >= 0 && t >= best) continue;
@@ -1230,8 +1237,9 @@ struct Lower {
         // leave most units idle and K is long (fc, late convolutions at small batch).
         {
             // (a linked depthwise stage can be split on request: a chunk's CTA then produces only its own channels of
-            // the depthwise result.  It is not chosen automatically: measured at batch 1 the partial sums and their
-            // reduction cost more than the shorter depthwise loop saves; the split search may still pick it.)
+            // the depthwise result.  It is not chosen automatically: measured at batch 1, with partial sums through the workspace,
+            // the only form these chains have, the reduction costs more than the shorter depthwise loop saves; the split
+            // search may still pick it.)
             // (a fully connected layer of at most 8 vectors runs on the CUDA cores: one pass over the weight matrix,
             // no partial sums; its input must be a bf16 vector that fits shared memory.  Measured, 1024 -> 1000:
             // 6.6 against 12 us at batch 1, 16.8 against 15.8 us at batch 32, where the tensor-core tiles win)
