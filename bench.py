@@ -329,18 +329,17 @@ def main():
             acc += np.array(ms)
     acc /= reps
     peaks = measured_peaks()
-    by_kind = {}
+    by_kernel = {}
     for L, ms in zip(plan["launches"], acc):
-        d = by_kind.setdefault(L["kind"], dict(ms=0.0, bytes=0.0, flops=0.0, launches=0))
+        d = by_kernel.setdefault(L["kernel"], dict(ms=0.0, bytes=0.0, flops=0.0, launches=0))
         d["ms"] += float(ms); d["bytes"] += L["bytes"]; d["flops"] += L["flops"]; d["launches"] += 1
-    dom = max(by_kind, key=lambda k: by_kind[k]["ms"])
-    dk = by_kind[dom]
+    dom = max(by_kernel, key=lambda k: by_kernel[k]["ms"])
+    dk = by_kernel[dom]
     t_mem = dk["bytes"] / (peaks["hbm_gbs"] * 1e9)
     t_tc = dk["flops"] / (peaks["bf16_tflops"] * 1e12)
     # In-stream duration of the dominant kernel's launches: the timed step minus the other kernels' share of it
-    # (shares from the serialised per-launch times; when the step runs one kernel only, as the linked tensor-core
-    # graphs do, this is the timed step itself).
-    all_ms = sum(d["ms"] for d in by_kind.values())
+    # (shares from the serialised per-launch times).
+    all_ms = sum(d["ms"] for d in by_kernel.values())
     step_ms = total_ms / args.steps
     dom_ms_in_stream = step_ms * dk["ms"] / all_ms
     if t_tc > t_mem and not fp32:

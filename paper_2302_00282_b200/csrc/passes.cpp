@@ -1748,6 +1748,19 @@ static void jarr(std::string &s, const char *k, const std::vector<int> &v, bool 
     s += "]"; if (comma) s += ",";
 }
 
+// The kernel a launch runs (a pool of windows up to 3 runs maxpool_kernel when its items fit 31 bits).
+static std::string kernel_of(const Launch &L) {
+    if (L.kind == LK_GEMM)
+        return L.fc_small ? "fc_small_kernel" : L.stem_tc ? "stem_tc_kernel" : L.conv_tc ? "conv_tc_kernel" : L.seg[0].mode == AM_DW ? "dw_tc_kernel" : "gemm_chain_kernel";
+    if (L.kind == LK_GEMM2) return L.pair ? "pair_tc_kernel" : "chain2_kernel";
+    if (L.kind == LK_POOL) return L.pool_kind == 0 && L.pool_k <= 3 ? "maxpool_kernel" : "pool_kernel";
+    static const char *k[] = {"?", "gemm_chain_kernel", "dw3x3_kernel", "pool_kernel", "gap_kernel", "add_kernel", "concat_part_kernel", "mulmac_kernel",
+                              "transpose_kernel", "slice_kernel", "f32_conv_kernel", "f32_pool_kernel", "f32_gap_kernel", "f32_add_kernel",
+                              "f32_concat_part_kernel", "f32_fc_kernel", "f32_chain_kernel", "f32_mulmac_kernel", "transpose_kernel", "f32_slice_kernel",
+                              "chain2_kernel", "stem3x3_kernel"};
+    return k[L.kind];
+}
+
 void emit_plan_json(Graph &g) {
     static const char *nk[] = {"?", "conv", "dwconv", "fc", "maxpool", "avgpool", "gap", "add", "concat", "mul", "mac", "transpose", "split"};
     static const char *ck[] = {"single", "conv_conv_pool", "dw_pw", "conv_tail", "expand_concat", "matmul_matmul", "conv_conv"};
@@ -1790,7 +1803,7 @@ void emit_plan_json(Graph &g) {
         const Launch &L = g.launches[i];
         if (i) s += ",";
         s += "{";
-        jint(s, "id", (long long)i); jstr(s, "kind", lk[L.kind]); jint(s, "chain", L.chain); jarr(s, "nodes", L.nodes);
+        jint(s, "id", (long long)i); jstr(s, "kind", lk[L.kind]); jstr(s, "kernel", kernel_of(L)); jint(s, "chain", L.chain); jarr(s, "nodes", L.nodes);
         jint(s, "in0", L.in0); jint(s, "in1", L.in1); jint(s, "in2", L.in2); jint(s, "skip", L.skip); jint(s, "out", L.out);
         jint(s, "out_coff", L.out_coff); jint(s, "out_ctot", L.out_ctot);
         jint(s, "C", L.C); jint(s, "H", L.H); jint(s, "W", L.W); jint(s, "K", L.K); jint(s, "P", L.P); jint(s, "Q", L.Q);

@@ -588,3 +588,14 @@ def test_image_convolution_and_max_pool_link_by_measured_cost():
     pl = compiled(graphs.resnet50_stress(), 8, linked=False)[0].plan()
     stem = pl["launches"][0]
     assert stem["a0"] == "stem" and (stem["patch_rw"] - 1) * 2 + 18 <= 256 and stem["hstages"] >= 2      # hstages: patches by TMA
+
+
+def test_plan_names_the_kernel_of_every_launch():
+    """A step of one graph runs several kernels; whoever adds launches up by kernel reads the name from the plan."""
+    def kernels(spec, batch, **kw):
+        return [l["kernel"] for l in compiled(spec, batch, **kw)[0].plan()["launches"]]
+    assert kernels(graphs.mobilenet_v1(), 32) == ["stem_tc_kernel"] + ["dw_tc_kernel"] * 13 + ["conv_tc_kernel"]
+    assert kernels(graphs.mobilenet_v1(), 1) == ["stem3x3_kernel"] + ["dw_tc_kernel"] * 13 + ["fc_small_kernel"]
+    assert kernels(graphs.single_chain(), 1) == ["f32_chain_kernel"]
+    assert kernels(graphs.single_chain(), 1, linked=False) == ["f32_conv_kernel", "f32_conv_kernel", "f32_pool_kernel"]
+    assert set(kernels(graphs.resnet50_stress(), 8)) == {"stem_tc_kernel", "conv_tc_kernel", "pair_tc_kernel"}
