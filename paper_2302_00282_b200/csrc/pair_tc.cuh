@@ -13,8 +13,10 @@
 // second product's blocks follow the first one's without a gap.  Where both weight matrices fit beside four A slots (64
 // middle channels) they are loaded once per CTA.  With at most 128 middle channels accumulator 1 exists twice and GEMM 1 of
 // the next tile is issued before GEMM 2 of this one, which waits for the middle epilogue.
-// Bound: HBM (input + shortcut + output of a tile, 144 / 288 / 576 KB for 64 / 128 / 256 middle channels) while the L2 ->
-// shared-memory stream of weights (0 / 426 / 1700 KB a tile) stays below it; at 256 middle channels both are equal.
+// A tile moves 144 / 288 / 576 KB of input, shortcut and output for 64 / 128 / 256 middle channels through HBM and 0 / 426 /
+// 1700 KB of weights from L2.  Reached, 512 x 512 images, batch 64: 260 / 183 / 161 us a launch, 0.71 and 0.51 of the HBM rate
+// and 0.51 of the tensor rate (counters at batch 8: tensor pipe 14 to 18 %, DRAM 6 to 29 %, issue slots 19 to 27 %): no unit is
+// full.  At 256 middle channels first product, middle and second product of a tile follow one another.
 // One thread per role issues all requests; every wait is bounded.
 #pragma once
 

@@ -146,8 +146,8 @@ def test_fp32_chain_tiles(cin, hw, cmid, cout, k, st, pool, batch):
     assert rel_err_fp32(y, interp.run_graph(spec, P, x)) <= FP32_TOL
 
 
-# the recorded form of a pass: repeated calls, images that change in place, other buffers and batches in turn (more than are
-# kept), a call inside the caller's own capture
+# the recorded form of a pass: repeated calls, images that change in place, other buffers and batches in turn, a call inside the
+# caller's own capture
 @pytest.mark.parametrize("name,kw", [("mobilenet_v1", dict(hw=64, width=0.25, classes=24)), ("resnet18", dict(hw=64, base=16, classes=10))])
 def test_repeated_passes(name, kw):
     import torch
