@@ -874,7 +874,8 @@ static xenos_status_t record_pass(Graph &g, const std::vector<void *> &in, const
     cudaGraphExec_t exec = nullptr;
     if ((e = cudaGraphInstantiate(&exec, sc.graph, 0)) != cudaSuccess) return cuda_fail(g, "cudaGraphInstantiate", e);
     // (else the first pass would wait for it: 147 us instead of 109 for the first pass of SqueezeNet at batch 1)
-    if ((e = cudaGraphUpload(exec, stream)) != cudaSuccess) {
+    // (a run in another stream need not be ordered behind it: it is waited for here)
+    if ((e = cudaGraphUpload(exec, stream)) != cudaSuccess || (e = cudaStreamSynchronize(stream)) != cudaSuccess) {
         cudaGraphExecDestroy(exec);
         return cuda_fail(g, "cudaGraphUpload", e);
     }

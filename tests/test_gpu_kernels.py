@@ -254,3 +254,22 @@ def test_binding_is_quick():
         gg.g.bind(gg.ws.data_ptr(), gg.ws.numel(), gg.stream)
         return time.perf_counter() - t
     assert statistics.median(once() for _ in range(21)) < 2e-3
+
+
+# a pass in another stream than the binding's, right behind it; the graph destroyed while its pass is on the way
+def test_passes_in_another_stream():
+    import torch
+    spec = graphs.mobilenet_v1(hw=64, width=0.25, classes=24)
+    P, x = graphs.make_params(spec), graphs.make_input(spec, 2)
+    gg = GpuGraph(spec, P, 2)
+    want, xin = gg.run(x), gg.upload(x)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(5):
+        g2 = GpuGraph(spec, P, 2)
+        out = g2.alloc_out(2)
+        side.wait_stream(torch.cuda.current_stream())
+        g2.g.run(2, [xin.data_ptr()], [out.data_ptr()], side.cuda_stream)
+        g2.g.destroy()
+        side.synchronize()
+        assert np.array_equal(out.cpu().numpy(), want)
