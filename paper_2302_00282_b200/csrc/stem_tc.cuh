@@ -418,7 +418,9 @@ __device__ __forceinline__ bool stem_epilogue_pool(const StemParams &g, uint32_t
     StemEpi s;
     s.init(g, bar, tmem_base);
     const uint32_t bias_at = sbase + (uint32_t)g.off_bias + (uint32_t)s.ch0 * 64u;
-    constexpr uint32_t kNone = 0xff80ff80u;
+    // (a maximum that starts at zero is ReLU's, too)
+    const uint32_t none = in_reg(s.act ? 0u : 0xff80ff80u);
+    const int act = s.act == 1 ? 0 : s.act;
     const uint32_t pc = in_reg((uint32_t)g.pc_log2), m = (1u << pc) - 1u;
     const int cc = (int)(threadIdx.x & m), pk = in_reg(g.pk), ps = in_reg(g.ps), pp = in_reg(g.pp), qlast = g.Q - 1;
     __nv_bfloat16 *out = reinterpret_cast<__nv_bfloat16 *>(g.out) + g.out_coff + s.n0 + cc * 8;
@@ -431,7 +433,7 @@ __device__ __forceinline__ bool stem_epilogue_pool(const StemParams &g, uint32_t
         int prow = r.row;                            // the row whose maximum is being formed
         uint32_t cur[2][2][8];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) cur[i >> 4][(i >> 3) & 1][i & 7] = kNone;
+        for (int i = 0; i < 32; ++i) cur[i >> 4][(i >> 3) & 1][i & 7] = none;
 #pragma unroll 1
         for (int p = r.p0; p < r.p1; ++p) {
             const int w0 = prow * ps - pp;
@@ -455,7 +457,7 @@ __device__ __forceinline__ bool stem_epilogue_pool(const StemParams &g, uint32_t
                     float2 bias[8];
                     uint32_t o[8];
                     stem_bias(bias_at + (uint32_t)j * 64u, bias);
-                    stem_pack(v, bias, s.act, o);
+                    stem_pack(v, bias, act, o);
                     uint32_t(&c)[8] = cur[j];
                     if (within) {
 #pragma unroll
@@ -468,7 +470,7 @@ __device__ __forceinline__ bool stem_epilogue_pool(const StemParams &g, uint32_t
                             st_shared16(at + (((c2 + 1) ^ x) << 4), make_uint4(c[4], c[5], c[6], c[7]));
                         }
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) c[i] = again ? o[i] : kNone;
+                        for (int i = 0; i < 8; ++i) c[i] = again ? max_bf16x2(o[i], none) : none;
                     }
                 }
             };
