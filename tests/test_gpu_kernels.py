@@ -273,3 +273,14 @@ def test_passes_in_another_stream():
         g2.g.destroy()
         side.synchronize()
         assert np.array_equal(out.cpu().numpy(), want)
+
+
+# one image and several run kernels of their own, both with more shared memory than a launch gets without asking
+def test_wide_fully_connected_layer_of_one_image_and_of_two():
+    spec = _spec((32768, 1, 1), lambda g: g.fc("fc", g.gap("flat", "input"), 16))
+    P, x = graphs.make_params(spec), xo.round_bf16(graphs.make_input(spec, 2))
+    gg = GpuGraph(spec, P, 2, in_mode="bf16_nhwc")
+    assert [l["kernel"] for l in gg.g.plan()["launches"]] == ["gap_kernel", "fc_small_kernel"]
+    o = interp.run_graph(spec, P, x)
+    for batch in (2, 1, 1, 1, 2):
+        assert np.abs(gg.run(x[:batch]) - o[:batch]).max() <= BF16_TOL * np.abs(o).max()
