@@ -132,15 +132,19 @@ __device__ __forceinline__ int conv_row0(const ConvParams &g, int mt) {
 __device__ __forceinline__ int in_reg(int x) { asm volatile("" : "+r"(x)); return x; }
 __device__ __forceinline__ uint32_t in_reg(uint32_t x) { asm volatile("" : "+r"(x)); return x; }
 
-// The ring as its issuing thread sees it: slot, phase, and the addresses of the slot's barrier and data.
+// The ring as its issuing thread sees it: slot, phase, and the addresses of the slot's barrier and data.  Barriers
+// are asked as little and as early as possible (see mbar_test): a filling thread knows that the first `fresh` slots are free,
+// a multiplying thread asks for the next slot before it multiplies this one (ready).
 struct ConvRing {
-    int s, n, step;
-    uint32_t ph, fb, data, fb0, data0;
+    int s, n, step, fresh;
+    uint32_t ph, fb, data, fb0, data0, ready;
     __device__ __forceinline__ void init(const ConvParams &g, uint32_t sbase, uint32_t bar) {
-        s = 0; n = in_reg(g.stages); step = in_reg(g.stage_bytes); ph = 0;
+        s = 0; n = in_reg(g.stages); step = in_reg(g.stage_bytes); ph = 0; ready = 0; fresh = n;
         fb = fb0 = bar; data = data0 = sbase;
     }
     __device__ __forceinline__ uint32_t empty() const { return fb + 8u * kCvMaxStages; }
+    __device__ __forceinline__ bool room() { return --fresh >= 0 || mbar_wait(empty(), ph ^ 1u); }
+    __device__ __forceinline__ bool full() const { return ready || mbar_wait(fb, ph); }
     __device__ __forceinline__ void next() {
         ++s; fb += 8u; data += (uint32_t)step;
         if (s == n) { s = 0; ph ^= 1u; fb = fb0; data = data0; }
@@ -156,7 +160,7 @@ __device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorM
     if (!sg.im2col && sg.per_stage == 1) {
 #pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
-            if (!mbar_wait(st.empty(), st.ph ^ 1u)) return false;
+            if (!st.room()) return false;
             mbar_arrive_expect_tx(st.fb, box);
             tma_load_2d(st.data, tm, kb * kTileK, m0, st.fb);
             st.next();
@@ -174,7 +178,7 @@ __device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorM
         }
 #pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
-            if (!mbar_wait(st.empty(), st.ph ^ 1u)) return false;
+            if (!st.room()) return false;
             mbar_arrive_expect_tx(st.fb, box);
             tma_load_im2col(st.data, tm, c, w0, h0, n, st.fb, s, r);
             st.next();
@@ -190,7 +194,7 @@ __device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorM
 #pragma unroll 1
     for (int kb = kb0; kb < kb1; ++kb) {
         const int nb = min(per, taps - tap);
-        if (!mbar_wait(st.empty(), st.ph ^ 1u)) return false;
+        if (!st.room()) return false;
         mbar_arrive_expect_tx(st.fb, box * nb);
 #pragma unroll 1
         for (int b = 0; b < nb; ++b) {
@@ -219,8 +223,8 @@ template <int kSeg, bool kRes>
 __device__ __forceinline__ bool conv_mma(const ConvParams &g, ConvRing &st, uint32_t bar, int kb0, int kb1, int kb_off, uint32_t d_tmem, uint32_t acc,
                                          int &bseen, uint32_t b_res) {
     const ConvSegment &sg = g.seg[kSeg];
-    constexpr uint64_t b_hi = (uint64_t)(64u | (1u << 14) | (2u << 29)) << 32;      // 128-byte swizzle, 1024-byte groups
-    const uint64_t a_hi = (uint64_t)in_reg(sg.desc_hi) << 32;
+    constexpr uint32_t b_hi = 64u | (1u << 14) | (2u << 29);      // 128-byte swizzle, 1024-byte groups
+    const uint32_t a_hi = in_reg(sg.desc_hi);
     const uint32_t idesc = in_reg(g.idesc), tile16 = in_reg((uint32_t)g.tile_n * 8u);
     const int per = in_reg(sg.per_stage);
     if (kRes && bseen < 4)
@@ -235,25 +239,15 @@ __device__ __forceinline__ bool conv_mma(const ConvParams &g, ConvRing &st, uint
         int cb = kb0 ? kb0 % cblocks : 0;
 #pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
-            const uint32_t a4 = 0x10000u | (st.data >> 4);      // (shared addresses are below 2^18)
+            const uint32_t a4 = 0x10000u | (st.data >> 4), used = st.empty();      // (shared addresses are below 2^18)
             if (!kRes) b4 = a4 + (kABytes >> 4);
             int steps = 4;
             if (++cb == cblocks) { cb = 0; steps = last; }
-            if (!mbar_wait(st.fb, st.ph)) return false;
-            tc_fence_after();
-            umma_bf16(d_tmem, a_hi | a4, b_hi | b4, idesc, acc);
-            if (steps == 4) {
-                umma_bf16_acc(d_tmem, a_hi | (a4 + 2), b_hi | (b4 + 2), idesc);
-                umma_bf16_acc(d_tmem, a_hi | (a4 + 4), b_hi | (b4 + 4), idesc);
-                umma_bf16_acc(d_tmem, a_hi | (a4 + 6), b_hi | (b4 + 6), idesc);
-            } else {
-#pragma unroll 1
-                for (int x = 1; x < steps; ++x) umma_bf16_acc(d_tmem, a_hi | (a4 + 2 * x), b_hi | (b4 + 2 * x), idesc);
-            }
-            umma_commit(st.empty());
+            if (!st.full()) return false;
+            st.next();
+            st.ready = umma_block(d_tmem, a_hi, a4, 2u, 4u, 6u, b_hi, b4, idesc, acc, steps, used, st.fb, st.ph);
             acc = 1u;
             if (kRes) b4 += tile16;
-            st.next();
         }
     } else {
         // descriptor advance per K = 16 step, in 16-byte units: a box holds one step (16 channels) or two (32)
@@ -263,20 +257,15 @@ __device__ __forceinline__ bool conv_mma(const ConvParams &g, ConvRing &st, uint
         int left = sg.taps - kb0 * per;
 #pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
-            const uint32_t a4 = 0x10000u | (st.data >> 4);
+            const uint32_t a4 = 0x10000u | (st.data >> 4), used = st.empty();
             if (!kRes) b4 = a4 + (kABytes >> 4);
             const int steps = min(per, left) * spb;
             left -= per;
-            if (!mbar_wait(st.fb, st.ph)) return false;
-            tc_fence_after();
-            umma_bf16(d_tmem, a_hi | a4, b_hi | b4, idesc, acc);
-            if (steps > 1) umma_bf16_acc(d_tmem, a_hi | (a4 + s1), b_hi | (b4 + 2), idesc);
-            if (steps > 2) umma_bf16_acc(d_tmem, a_hi | (a4 + s2), b_hi | (b4 + 4), idesc);
-            if (steps > 3) umma_bf16_acc(d_tmem, a_hi | (a4 + s1 + s2), b_hi | (b4 + 6), idesc);
-            umma_commit(st.empty());
+            if (!st.full()) return false;
+            st.next();
+            st.ready = umma_block(d_tmem, a_hi, a4, s1, s2, s1 + s2, b_hi, b4, idesc, acc, steps, used, st.fb, st.ph);
             acc = 1u;
             if (kRes) b4 += tile16;
-            st.next();
         }
     }
     return true;
@@ -292,7 +281,7 @@ __device__ __forceinline__ bool conv_mma_loop(const ConvParams &g, uint32_t sbas
     for (int ti = blockIdx.x; ti < total; ti += gridDim.x, ++i) {
         const int b = i & 1;
         const ConvTile t = conv_tile(g, ti);
-        if (!mbar_wait(accf + 8u * (2 + b), ((i >> 1) & 1) ^ 1u)) return false;      // the epilogue has drained this accumulator
+        if (i > 1 && !mbar_wait(accf + 8u * (2 + b), ((i >> 1) & 1) ^ 1u)) return false;      // the epilogue has drained this accumulator
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + b * acc_stride;
         if (t.kb0 < k0 && !conv_mma<0, kRes>(g, st, bar, t.kb0, min(t.kb1, k0), 0, d_tmem, 0u, bseen, b_res)) return false;
@@ -655,8 +644,6 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     const uint32_t sbase = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (sbase - raw);
     const uint32_t bar = sbase + g.off_bar;
-    auto full_bar = [&](int s) { return bar + 8u * s; };
-    auto empty_bar = [&](int s) { return bar + 8u * (kCvMaxStages + s); };
     auto accf_bar = [&](int b) { return bar + 8u * (2 * kCvMaxStages + b); };
     auto acce_bar = [&](int b) { return bar + 8u * (2 * kCvMaxStages + 2 + b); };
     auto bres_bar = [&](int q) { return bar + 8u * (2 * kCvMaxStages + 4 + q); };                       // 4
@@ -666,16 +653,15 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     volatile int *fail_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);      // [0] give-up, [1], [2] agreement of a split / average
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0 && elect_one()) {
-        for (int s = 0; s < g.stages; ++s) { mbar_init(full_bar(s), g.b_resident ? 1u : 2u); mbar_init(empty_bar(s), 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(accf_bar(b), 1); mbar_init(acce_bar(b), kCvEpiWarps); }
-        for (int q = 0; q < 4; ++q) mbar_init(bres_bar(q), 1);
-        if (kEpi == CE_SKIP) for (int e = 0; e < kMaxSkipSlots * kCvEpiWarps; ++e) mbar_init(skip_bar(0, e), 1);
-        if (kEpi == CE_CLUSTER) mbar_init(arrived, kCvEpiWarps * g.ksplit);
-        fail_flag[0] = 0;
+    if (warp == 0) {
+        // (a lane per barrier: one thread takes half a microsecond for all of them)
+        constexpr int acce = 2 * kCvMaxStages + 2, first_skip = 2 * kCvMaxStages + 8, n_bars = kEpi == CE_SKIP ? first_skip + kMaxSkipSlots * kCvEpiWarps : first_skip + 1;
+        for (int i = lane; i < n_bars; i += 32)
+            mbar_init(bar + 8u * i, i < kCvMaxStages ? (g.b_resident ? 1u : 2u) : i == acce || i == acce + 1 ? kCvEpiWarps : kEpi == CE_CLUSTER && i == first_skip ? kCvEpiWarps * g.ksplit : 1u);
+        if (lane == 0) fail_flag[0] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA0) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
+        if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA0) : "memory");
+        if (lane == 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
     }
     if (warp == 3) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"((uint32_t)g.tmem_cols) : "memory");
@@ -696,16 +682,17 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     if (warp == 0) {
         // ---- A operand ----
         if (elect_one()) {
-            pdl_wait();
             ConvRing st;
             st.init(g, sbase, bar);
             const int k0 = in_reg(g.seg[0].kblocks), total = in_reg(g.total);
+            bool waited = false;
 #pragma unroll 1
             for (int ti = blockIdx.x; ti < total && ok; ti += gridDim.x) {
                 const ConvTile t = conv_tile(g, ti);
                 const int m0 = conv_row0(g, t.mt);
                 const int n = (int)g.d_rpi.div((uint32_t)m0), rem = m0 - n * (int)g.d_rpi.d;
                 const int p = (int)g.d_q.div((uint32_t)rem), q = rem - p * (int)g.d_q.d;
+                if (!waited) { pdl_wait(); waited = true; }      // (behind the first tile's divisions)
                 if (t.kb0 < k0) ok = conv_load_a<0>(g, &tmA0, st, t.kb0, min(t.kb1, k0), m0, n, p, q);
                 if (ok && t.kb1 > k0) ok = conv_load_a<1>(g, &tmA1, st, max(t.kb0 - k0, 0), t.kb1 - k0, m0, n, p, q);
             }
@@ -740,7 +727,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                     const int row = t.nt * tile_n;
 #pragma unroll 1
                     for (int kb = t.kb0; kb < t.kb1; ++kb) {
-                        ok = mbar_wait(st.empty(), st.ph ^ 1u);
+                        ok = st.room();
                         if (!ok) break;
                         mbar_arrive_expect_tx(st.fb, bytes);
                         tma_load_2d(st.data + kABytes, &tmB, kb * kTileK, row, st.fb);

@@ -2,13 +2,12 @@
 // the pointwise product reads and never leaves the SM), with a store, global-average or reduction-split epilogue.
 //
 // A CTA walks over tiles of ni images x rh x rw <= 128 output pixels (rw a multiple of 4) x n_acc * tile_n channels.
-//   warp 0     copies the tile's input window of each 64-channel block (zero fill = padding) into the halo ring and the
-//              weight blocks into theirs (or once, when a CTA meets several tiles and they fit: b_resident).  Weights are
-//              constants: the first ones are requested before the wait for the predecessor kernel
+//   warp 0     copies the tile's input window of each 64-channel block (zero fill = padding) into the halo ring
 //   warp 1     tensor memory; tcgen05.mma: depthwise block x weight block -> accumulator
 //   warps 2-17 workers: the stencils of the next batch of tiles, then the epilogues of this one (all of them do both, so that
 //              neither half of the CTA idles in chains with one tile per CTA).  nothing of the stencil stays in registers across an
 //              epilogue: spilled values were reloaded from L2, since the shared memory leaves no L1 to speak of
+//   warp 18    copies the weight blocks into their ring (or once, when a CTA meets several tiles and they fit: b_resident)
 // The workers form G groups; a (tile, channel block) item is the work of one group, items are dealt in turn (a batch has at least one item per group: with one
 // channel block per tile several tiles form a batch, each with its own accumulator pair), and a group's
 // slots of the rings are its own (ring sizes are multiples of G: a group meets every phase of its slots' barriers).  A
@@ -24,7 +23,7 @@
 namespace xk {
 
 constexpr int kDwWorkers = 16;
-constexpr int kDwThreads = 64 + 32 * kDwWorkers;
+constexpr int kDwThreads = 96 + 32 * kDwWorkers;
 constexpr int kDwMaxSlots = 8;
 enum { DE_STORE = 0, DE_GAP = 1, DE_SPLIT = 2 };
 
@@ -38,6 +37,7 @@ struct DwParams {
     int total, kblocks, last_steps, tile_n, n_acc, N, kb_per;
     int groups, wpg_log2, pairs;              // worker groups, log2(warps per group), lanes (channel pairs) per block
     int batch_tiles, n_bufs;                  // tiles per batch; accumulator buffers (2 per tile of a batch; 1 when a tile takes all columns)
+    int a_stride;                             // distance of operand slots: tiles of few rows have short ones (see layout_dw)
     int a_slots, b_slots, h_slots, b_resident, halo_bytes, halo_stride, halo_h, halo_w, halo_cb;
     int acc_stride, tmem_cols;
     int chunk, nchunks, box_bytes, out_bufs;
@@ -75,7 +75,11 @@ __device__ __forceinline__ DwTile dw_tile(const DwParams &g, int ti) {
 
 // A worker thread's unit of a tile: BR x 4 pixels of a channel pair; the lanes of a warp take the pairs of one block of pixels
 // (of two blocks when a channel block has at most 32 channels).
-struct DwWork { int q, base, row0, nrows, live; };
+// a_row, a_step: where its first pixel's row of the operand block starts and how far the next block row is; a_piece: its
+// channel pair in that row (K-major, 128-byte swizzle: bits 4..6 of an address are xor-ed with the row's low bits; rows start on
+// multiples of four, so pixel b of a block row has piece ^ (b << 4), and an odd block row of an odd number of fours the other 64)
+struct DwWork { int q, base, nrows, live; uint32_t a_row, a_step, a_piece; };
+__device__ __forceinline__ uint32_t dw_flip(const DwWork &u) { return (u.a_step >> 3) & 64u; }
 
 // The tap weights and bias of a thread's two channels.
 struct DwTaps { float2 w[9], b; };
@@ -89,14 +93,15 @@ __device__ __forceinline__ void dw_load_taps(DwTaps &t, uint32_t dww, int C, int
     for (int i = 0; i < 9; ++i) t.w[i] = ld_shared_f2(dww + (uint32_t)(i * C + c0) * 4u);
     t.b = ld_shared_f2(dww + (uint32_t)(9 * C + c0) * 4u);
 }
-// Where row r's channel pair q sits in the K-major swizzled operand block.
-__device__ __forceinline__ uint32_t dw_a_addr(uint32_t a_base, int r, int q) { return a_base + r * 128 + ((((q >> 2) ^ (r & 7)) << 4) | ((q & 3) << 2)); }
 
 // Depthwise 3x3 + bias + activation of one unit, rounded to bf16 and stored in the operand layout.  Every input pair is read
 // once per unit (one 128-byte row per warp and read) and feeds up to 9 results.
-template <int S, int BR>
-__device__ __forceinline__ void dw_stencil(const DwTaps &t, const DwWork &u, uint32_t halo, uint32_t a_base, int row_bytes, int cbytes, int rw,
+// kCB: channels of a window block where they are known at compile time (the loads of a row are then one address and
+// immediate offsets), 0 otherwise.
+template <int S, int BR, int kCB>
+__device__ __forceinline__ void dw_stencil(const DwTaps &t, const DwWork &u, uint32_t halo, uint32_t a_base, int row_bytes, int cb,
                                            uint32_t lo, uint32_t hi) {
+    const int cbytes = kCB ? 2 * kCB : 2 * cb;
     float2 acc[BR][4];
 #pragma unroll
     for (int a = 0; a < BR; ++a)
@@ -105,11 +110,10 @@ __device__ __forceinline__ void dw_stencil(const DwTaps &t, const DwWork &u, uin
     uint32_t rowp = halo + u.base;
 #pragma unroll
     for (int iy = 0; iy < (BR - 1) * S + 3; ++iy, rowp += row_bytes) {
-        uint32_t p = rowp;
 #pragma unroll
-        for (int ci = 0; ci < 3 * S + 3; ++ci, p += cbytes) {
+        for (int ci = 0; ci < 3 * S + 3; ++ci) {
             uint32_t v;
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(p));
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(rowp + ci * cbytes));
             const float2 x = make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 #pragma unroll
             for (int ry = 0; ry < 3; ++ry) {
@@ -123,12 +127,14 @@ __device__ __forceinline__ void dw_stencil(const DwTaps &t, const DwWork &u, uin
         }
     }
     // (rounding, then clamping: the bounds 0 and 6 are bf16 values and rounding is monotonic)
+    uint32_t row = a_base + u.a_row, piece = u.a_piece;
+    asm volatile("" : "+r"(piece));      // (the addresses are made here, not kept through the sums)
 #pragma unroll
-    for (int a = 0; a < BR; ++a) {
+    for (int a = 0; a < BR; ++a, row += u.a_step, piece ^= dw_flip(u)) {
         if (a >= u.nrows) break;
 #pragma unroll
         for (int b = 0; b < 4; ++b)
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(dw_a_addr(a_base, u.row0 + a * rw + b, u.q)), "r"(clamp_bf16x2(pack2(acc[a][b].x, acc[a][b].y), lo, hi)) : "memory");
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(row + b * 128 + (piece ^ (b << 4))), "r"(clamp_bf16x2(pack2(acc[a][b].x, acc[a][b].y), lo, hi)) : "memory");
     }
 }
 // Output pixel of tile row r, -1 when the row lies outside the map or the batch.
@@ -141,7 +147,7 @@ __device__ __forceinline__ long long dw_pixel(const DwParams &g, const DwTile &t
 
 // kS, kBR: stride and block rows of the stencil (an instance carries one stencil: instruction fetch is what a launch with one
 // tile per CTA spends most of its time on)
-template <int kEpi, int kS, int kBR>
+template <int kEpi, int kS, int kBR, int kCB>
 __global__ void __launch_bounds__(kDwThreads, 1)
 dw_tc_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmO,
              const __grid_constant__ DwParams g) {
@@ -158,15 +164,17 @@ dw_tc_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CU
     volatile int *fail_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0 && elect_one()) {
-        const uint32_t wpg = 1u << g.wpg_log2;
-        for (int s = 0; s < g.a_slots; ++s) { mbar_init(a_full + 8u * s, wpg); mbar_init(a_full + kEmpty + 8u * s, 1); }
-        for (int s = 0; s < g.b_slots; ++s) { mbar_init(b_full + 8u * s, 1); mbar_init(b_full + kEmpty + 8u * s, 1); }
-        for (int s = 0; s < g.h_slots; ++s) { mbar_init(h_full + 8u * s, 1); mbar_init(h_full + kEmpty + 8u * s, wpg); }
-        for (int b = 0; b < g.n_bufs; ++b) { mbar_init(accf + 8u * b, 1); mbar_init(acce + 8u * b, kEpi == DE_STORE ? 4u * g.nchunks : kDwWorkers); }
-        mbar_init(bres, 1); mbar_init(dww_bar, 1);
-        fail_flag[0] = 0;
+    if (warp == 0) {
+        // (a lane per barrier: a_full, empty, b_full, empty, h_full, empty, accf, acce of 8 each, bres, dww_bar)
+        for (int i = lane; i < 8 * kDwMaxSlots + 2; i += 32) {
+            const int kind = i / kDwMaxSlots;
+            mbar_init(bar + 8u * i, kind == 0 || kind == 5 ? 1u << g.wpg_log2 : kind == 7 ? (kEpi == DE_STORE ? 4u * g.nchunks : kDwWorkers) : 1u);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        __syncwarp();
+    }
+    if (warp == 0 && elect_one()) {
+        fail_flag[0] = 0;
         // depthwise taps [9][C] and bias [C]: constants, awaited by the workers before their first stencil
         const uint32_t C = (uint32_t)g.C;
         mbar_arrive_expect_tx(dww_bar, 40u * C);
@@ -195,105 +203,124 @@ dw_tc_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CU
 
     if (warp == 0) {
         if (elect_one()) {
-            // ---- input windows and weights ----
-            PairRing rh = {0, in_reg(g.h_slots), 0u}, rb = {0, in_reg(g.b_slots), 0u};
+            // ---- input windows (those of the first tile that find a fresh slot are asked for by the worker groups) ----
+            PairRing rh = {0, in_reg(g.h_slots), 0u, 0u};
             const int total = in_reg(g.total), step = gridDim.x, stride = in_reg(g.stride), pad = in_reg(g.pad), hstride = in_reg(g.halo_stride);
-            const int tile_n = in_reg(g.tile_n), n_acc = in_reg(g.n_acc), cols = tile_n * n_acc;
-            const uint32_t hbytes = in_reg((uint32_t)g.halo_bytes), dst0 = sbase + g.off_halo, part = (uint32_t)tile_n * 128u, bytes = part * n_acc, b0 = sbase + g.off_b;
-            const bool stream = !g.b_resident;
-            int tb = blockIdx.x;             // the weight blocks run ahead of the windows: their own tile and K block
-            DwTile wb = dw_tile(g, tb);
-            int kb_b = wb.kb0;
-            auto weights = [&]() {
-                const uint32_t fb = b_full + 8u * rb.s;
-                if (!mbar_wait(fb + kEmpty, rb.ph ^ 1u)) return false;
-                mbar_arrive_expect_tx(fb, bytes);
-#pragma unroll 1
-                for (int h = 0; h < n_acc; ++h) tma_load_2d(b0 + rb.s * bytes + h * part, &tmB, kb_b * kTileK, wb.nt * cols + h * tile_n, fb);
-                rb.next();
-                if (++kb_b == wb.kb1) {
-                    tb += step;
-                    wb = dw_tile(g, tb);
-                    kb_b = wb.kb0;
-                }
-                return true;
-            };
-            if (!stream) {
-                mbar_arrive_expect_tx(bres, bytes * g.kblocks);
-#pragma unroll 1
-                for (int kb = 0; kb < g.kblocks; ++kb)
-#pragma unroll 1
-                    for (int h = 0; h < n_acc; ++h) tma_load_2d(b0 + kb * bytes + h * part, &tmB, kb * kTileK, wb.nt * cols + h * tile_n, bres);
-            } else {
-#pragma unroll 1
-                for (int i = 0; i < g.b_slots && tb < total && ok; ++i) ok = weights();
-            }
+            const uint32_t hbytes = in_reg((uint32_t)g.halo_bytes), dst0 = sbase + g.off_halo;
             pdl_wait();
-            int wi = 0;
+            bool first = true;
+            int fresh = rh.n;      // slots that nothing has been put in yet: no need to ask for room
 #pragma unroll 1
             for (int ti = blockIdx.x; ti < total && ok; ti += step) {
                 const DwTile t = dw_tile(g, ti);
                 const int hy = t.y0 * stride - pad, hx = t.x0 * stride - pad;
+                int kb = t.kb0;
+                if (first) {
+                    first = false;
+                    const int n = min(rh.n, t.kb1 - t.kb0);
+                    kb += n;
+                    fresh -= n;
+                    rh.s = n;
+                    if (n == rh.n) { rh.s = 0; rh.ph = 1u; }
+                }
 #pragma unroll 1
-                for (int kb = t.kb0; kb < t.kb1; ++kb) {
+                for (; kb < t.kb1; ++kb) {
                     const uint32_t fb = h_full + 8u * rh.s;
-                    ok = mbar_wait(fb + kEmpty, rh.ph ^ 1u);
+                    ok = --fresh >= 0 || mbar_wait(fb + kEmpty, rh.ph ^ 1u);
                     if (!ok) break;
                     mbar_arrive_expect_tx(fb, hbytes);
                     tma_load_4d(dst0 + rh.s * hstride, &tmH, kb * kTileK, hx, hy, t.n0, fb);
                     rh.next();
-                    // (one weight block per window from the h_slots-th on: its slot is then about to be free, so this thread does
-                    // not wait for it while windows are due)
-                    if (stream && tb < total && ++wi > rh.n) ok = ok && weights();
                 }
             }
-            while (stream && ok && tb < total) ok = weights();
+            if (!ok) atomicCAS(g.status, 0u, gave_up | (1u << 8));
+        }
+    } else if (warp == kDwThreads / 32 - 1) {
+        if (elect_one()) {
+            // ---- weights: constants, so nothing here waits for the predecessor kernel.  A slot holds one block of tile_n columns ----
+            const int total = in_reg(g.total), step = gridDim.x, tile_n = in_reg(g.tile_n), n_acc = in_reg(g.n_acc), cols = tile_n * n_acc;
+            const uint32_t part = (uint32_t)tile_n * 128u, b0 = sbase + g.off_b;
+            if (g.b_resident) {
+                const int nt = dw_tile(g, blockIdx.x).nt;
+                mbar_arrive_expect_tx(bres, part * n_acc * g.kblocks);
+#pragma unroll 1
+                for (int kb = 0; kb < g.kblocks; ++kb)
+#pragma unroll 1
+                    for (int h = 0; h < n_acc; ++h) tma_load_2d(b0 + (kb * n_acc + h) * part, &tmB, kb * kTileK, nt * cols + h * tile_n, bres);
+            } else {
+                PairRing rb = {0, in_reg(g.b_slots), 0u, 0u};
+                int fresh = rb.n;
+#pragma unroll 1
+                for (int ti = blockIdx.x; ti < total && ok; ti += step) {
+                    const DwTile t = dw_tile(g, ti);
+#pragma unroll 1
+                    for (int kb = t.kb0; kb < t.kb1 && ok; ++kb)
+#pragma unroll 1
+                        for (int h = 0; h < n_acc; ++h) {
+                            const uint32_t fb = b_full + 8u * rb.s;
+                            ok = --fresh >= 0 || mbar_wait(fb + kEmpty, rb.ph ^ 1u);
+                            if (!ok) break;
+                            mbar_arrive_expect_tx(fb, part);
+                            tma_load_2d(b0 + rb.s * part, &tmB, kb * kTileK, t.nt * cols + h * tile_n, fb);
+                            rb.next();
+                        }
+                }
+            }
             if (!ok) atomicCAS(g.status, 0u, gave_up | (1u << 8));
         }
     } else if (warp == 1) {
         if (elect_one()) {
             // ---- MMA ----
-            PairRing ra = {0, in_reg(g.a_slots), 0u}, rb = {0, in_reg(g.b_slots), 0u};
-            const int total = in_reg(g.total), step = gridDim.x, kblocks = in_reg(g.kblocks), last = in_reg(g.last_steps), n_acc = in_reg(g.n_acc), resident = in_reg(g.b_resident);
+            PairRing ra = {0, in_reg(g.a_slots), 0u, 0u}, rb = {0, in_reg(g.b_slots), 0u, 0u};
+            const int total = in_reg(g.total), step = gridDim.x, kblocks = in_reg(g.kblocks), last = in_reg(g.last_steps), n_acc = in_reg(g.n_acc), resident = in_reg(g.b_resident), a_stride = in_reg(g.a_stride);
             const uint32_t idesc = in_reg(g.idesc), part = (uint32_t)in_reg(g.tile_n) * 128u, bytes = part * n_acc, b0 = sbase + g.off_b, acc_stride = in_reg((uint32_t)g.acc_stride);
-            constexpr uint64_t hi = (uint64_t)(64u | (1u << 14) | (2u << 29)) << 32;
-            PairRing rc = {0, in_reg(g.n_bufs), 0u};      // accumulators
+            constexpr uint32_t hi = 64u | (1u << 14) | (2u << 29);
+            PairRing rc = {0, in_reg(g.n_bufs), 0u, 0u};      // accumulators
+            int fresh = rc.n;
             if (resident) ok = mbar_wait(bres, 0u);
+            const uint32_t a_last = a_full + 8u * (uint32_t)(ra.n - 1), a_step = (uint32_t)a_stride >> 4, a0 = 0x10000u | (sbase >> 4), b_step = bytes >> 4, w0 = 0x10000u | (b0 >> 4);
+            uint32_t af = a_full, a4 = a0, ready = 0u;      // the operand slot at hand: its barrier, its address, what is known of it
 #pragma unroll 1
             for (int ti = blockIdx.x; ti < total && ok; ti += step) {
-                const DwTile t = dw_tile(g, ti);
+                int kb0 = 0, kb1 = kblocks;
+                if (kEpi == DE_SPLIT) { const DwTile t = dw_tile(g, ti); kb0 = t.kb0; kb1 = t.kb1; }
                 const int b = rc.s;
-                ok = mbar_wait(acce + 8u * b, rc.ph ^ 1u);
+                ok = --fresh >= 0 || mbar_wait(acce + 8u * b, rc.ph ^ 1u);
                 if (!ok) break;
                 rc.next();
                 tc_fence_after();
                 const uint32_t d = tmem_base + b * acc_stride;
-                uint32_t acc = 0u;
+                uint32_t acc = 0u, b4 = w0 + kb0 * b_step;
+                // (few instructions and no branches in here: a lone thread needs some eight cycles for each)
 #pragma unroll 1
-                for (int kb = t.kb0; kb < t.kb1; ++kb) {
+                for (int kb = kb0; kb < kb1; ++kb) {
                     const int steps = kb == kblocks - 1 ? last : 4;
-                    uint32_t bb = b0 + kb * bytes;
-                    if (!resident) {
-                        ok = mbar_wait(b_full + 8u * rb.s, rb.ph);
+                    if (!ready) {
+                        ok = mbar_wait(af, ra.ph);
                         if (!ok) break;
-                        bb = b0 + rb.s * bytes;
                     }
-                    ok = mbar_wait(a_full + 8u * ra.s, ra.ph);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t a4 = 0x10000u | ((sbase + ra.s * kABytes) >> 4);
+                    const uint32_t now = a4, used = af + kEmpty;
+                    const bool wrap = af == a_last;
+                    af = wrap ? a_full : af + 8u;
+                    a4 = wrap ? a0 : a4 + a_step;
+                    ra.ph ^= wrap ? 1u : 0u;
+                    if (resident) {
+                        ready = umma_block(d, hi, now, 2u, 4u, 6u, hi, b4, idesc, acc, steps, used, af, ra.ph);
+                        b4 += b_step;
+                    } else {
+                        ready = 0u;
 #pragma unroll 1
-                    for (int h = 0; h < n_acc; ++h) {
-                        const uint32_t b4 = 0x10000u | ((bb + h * part) >> 4), dh = d + h * acc_stride;
-                        umma_bf16(dh, hi | a4, hi | b4, idesc, acc);
-                        if (steps > 1) umma_bf16_acc(dh, hi | (a4 + 2), hi | (b4 + 2), idesc);
-                        if (steps > 2) umma_bf16_acc(dh, hi | (a4 + 4), hi | (b4 + 4), idesc);
-                        if (steps > 3) umma_bf16_acc(dh, hi | (a4 + 6), hi | (b4 + 6), idesc);
+                        for (int h = 0; h < n_acc; ++h) {
+                            ok = rb.ready || mbar_wait(b_full + 8u * rb.s, rb.ph);
+                            if (!ok) break;
+                            const uint32_t bs = 0x10000u | ((b0 + rb.s * part) >> 4), b_used = b_full + kEmpty + 8u * rb.s;
+                            rb.next();
+                            rb.ready = umma_block(d + h * acc_stride, hi, now, 2u, 4u, 6u, hi, bs, idesc, acc, steps, b_used, b_full + 8u * rb.s, rb.ph);
+                        }
+                        if (!ok) break;
+                        umma_commit(used);
                     }
-                    umma_commit(a_full + kEmpty + 8u * ra.s);
-                    if (!resident) { umma_commit(b_full + kEmpty + 8u * rb.s); rb.next(); }
                     acc = 1u;
-                    ra.next();
                 }
                 if (ok) umma_commit(accf + 8u * b);
             }
@@ -304,7 +331,7 @@ dw_tc_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CU
         const int wk = warp - 2, wt = threadIdx.x - 64, wpg_log2 = in_reg(g.wpg_log2), groups = in_reg(g.groups);
         const int grp = wk >> wpg_log2, pt = wt - (grp << (wpg_log2 + 5));      // group; thread inside the group
         const int pairs = in_reg(g.pairs), cb = in_reg(g.halo_cb), rw = in_reg(g.rw), kblocks = in_reg(g.kblocks);
-        const int row_bytes = in_reg(g.halo_w * g.halo_cb * 2), C = in_reg(g.C);
+        const int row_bytes = in_reg(g.halo_w * g.halo_cb * 2), C = in_reg(g.C), a_stride = in_reg(g.a_stride);
         DwWork u;
         {
             u.q = pt & (pairs - 1);
@@ -312,64 +339,90 @@ dw_tc_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CU
             const int img = blk / upi, rem = blk - img * upi, uy = rem / upr, ux = rem - uy * upr;
             u.live = img < g.ni && u.q * 2 < ((cb + 15) & ~15);
             u.base = ((img * g.halo_h + kBR * uy * kS) * g.halo_w + 4 * ux * kS) * cb * 2 + u.q * 4;
-            u.row0 = img * g.rh * g.rw + kBR * uy * g.rw + 4 * ux;
+            const int row0 = img * g.rh * g.rw + kBR * uy * g.rw + 4 * ux;      // (a multiple of 4)
+            u.a_row = (uint32_t)row0 * 128u; u.a_step = in_reg((uint32_t)g.rw * 128u);
+            u.a_piece = ((((uint32_t)(u.q >> 2) ^ (row0 & 4))) << 4) | ((u.q & 3) << 2);
             u.nrows = min(kBR, max(0, g.rh - kBR * uy));
         }
         const uint32_t dlo = g.dw_act >= 1 ? 0u : 0xff80ff80u, dhi = g.dw_act == 2 ? 0x40c040c0u : 0x7f807f80u;
         const uint32_t plo = g.act >= 1 ? 0u : 0xff80ff80u, phi = g.act == 2 ? 0x40c040c0u : 0x7f807f80u;
         const uint32_t dww = sbase + g.off_dww, halo0 = sbase + g.off_halo;
         const int a_per = in_reg(g.a_slots) / groups, h_per = in_reg(g.h_slots) / groups, hstride = in_reg(g.halo_stride);
-        PairRing ra = {0, a_per, 0u}, rh = {0, h_per, 0u};      // this group's slots: grp + groups * s
+        PairRing ra = {0, a_per, 0u, 0u}, rh = {0, h_per, 0u, 0u};      // this group's slots: grp + groups * s
+        int fresh = a_per;
         int base = 0;      // items before the tile at hand, modulo groups
-        ok = mbar_wait(dww_bar, 0u);
-        auto stencil = [&](const DwTile &t) {
+        if ((wk & ((1 << wpg_log2) - 1)) == 0) {
+            // The first tile's windows, asked for by one warp per group (its own slots): a request is some 250 to 400 cycles of the
+            // thread that makes it, so one thread brought the last of eight windows 2800 cycles after the first.
+            const DwTile t = dw_tile(g, blockIdx.x);
+            const int hy = t.y0 * kS - g.pad, hx = t.x0 * kS - g.pad, n = min(g.h_slots, t.kb1 - t.kb0);
+            pdl_wait();
+            if (elect_one())
 #pragma unroll 1
-            for (int kb = t.kb0 + ((grp - base) & (groups - 1)); kb < t.kb1; kb += groups) {
+                for (int i = grp; i < n; i += groups) {
+                    mbar_arrive_expect_tx(h_full + 8u * i, (uint32_t)g.halo_bytes);
+                    tma_load_4d(halo0 + i * hstride, &tmH, (t.kb0 + i) * kTileK, hx, hy, t.n0, h_full + 8u * i);
+                }
+            __syncwarp();
+        }
+        ok = mbar_wait(dww_bar, 0u);
+        auto stencil = [&](int kb0, int kb1) {
+#pragma unroll 1
+            for (int kb = kb0 + ((grp - base) & (groups - 1)); kb < kb1; kb += groups) {
                 const int as = grp + groups * ra.s, hs = grp + groups * rh.s;
-                ok = ok && mbar_wait(a_full + kEmpty + 8u * as, ra.ph ^ 1u) && mbar_wait(h_full + 8u * hs, rh.ph);
+                // (both barriers are asked at once; the first round's operand slots are free)
+                const uint32_t got = --fresh >= 0 ? 1u : mbar_test(a_full + kEmpty + 8u * as, ra.ph ^ 1u), win = mbar_test(h_full + 8u * hs, rh.ph);
+                ok = ok && (got || mbar_wait(a_full + kEmpty + 8u * as, ra.ph ^ 1u)) && (win || mbar_wait(h_full + 8u * hs, rh.ph));
                 if (!ok) return;
                 const int c0 = kb * kTileK + u.q * 2;
-                const uint32_t halo = halo0 + hs * hstride, a_base = sbase + as * kABytes;
+                const uint32_t halo = halo0 + hs * hstride, a_base = sbase + as * a_stride;
                 if (u.live && c0 < C) {
                     DwTaps taps;
                     dw_load_taps(taps, dww, C, c0);
-                    dw_stencil<kS, kBR>(taps, u, halo, a_base, row_bytes, cb * 2, rw, dlo, dhi);
+                    dw_stencil<kS, kBR, kCB>(taps, u, halo, a_base, row_bytes, cb, dlo, dhi);
                 } else if (u.live && c0 < ((C + 15) & ~15)) {
                     // the last K = 16 step reads up to 8 channels beyond C: zeros (their weights are zeros too)
 #pragma unroll 1
                     for (int x = 0; x < u.nrows * 4; ++x)
-                        asm volatile("st.shared.b32 [%0], %1;" ::"r"(dw_a_addr(a_base, u.row0 + (x >> 2) * rw + (x & 3), u.q)), "r"(0u) : "memory");
+                        asm volatile("st.shared.b32 [%0], %1;" ::"r"(a_base + u.a_row + (x >> 2) * u.a_step + (((x & 4) ? dw_flip(u) : 0u) ^ u.a_piece ^ (uint32_t)((x & 3) << 4)) + (x & 3) * 128u), "r"(0u) : "memory");
                 }
                 fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) { mbar_arrive(a_full + 8u * as); mbar_arrive(h_full + kEmpty + 8u * hs); }
                 ra.next(); rh.next();
             }
-            base = (base + t.kb1 - t.kb0) & (groups - 1);
+            base = (base + kb1 - kb0) & (groups - 1);
         };
         const int total = in_reg(g.total), step = gridDim.x, nb = in_reg(g.batch_tiles);
         const int quarter = warp & 3, cgroup = wk >> 2, row = quarter * 32 + lane;      // accumulator lanes; which column chunks
         const uint32_t bias_s = sbase + g.off_bias, t_warp = tmem_base + ((uint32_t)(quarter * 32) << 16);
         const int chunk = in_reg(g.chunk), nchunks = in_reg(g.nchunks), cols = g.n_acc * g.tile_n;
-        PairRing rc = {0, in_reg(g.n_bufs), 0u};      // accumulators
+        PairRing rc = {0, in_reg(g.n_bufs), 0u, 0u};      // accumulators
         int ts = blockIdx.x, te = -1, cnt = 0;
         // the stencils of the next batch of tiles, then the epilogues of this one (one copy of either)
 #pragma unroll 1
         for (;;) {
 #pragma unroll 1
-            for (int j = 0, tj = ts; j < nb && tj < total; ++j, tj += step) stencil(dw_tile(g, tj));
+            for (int j = 0, tj = ts; j < nb && tj < total; ++j, tj += step) {
+                if (kEpi == DE_SPLIT) { const DwTile t = dw_tile(g, tj); stencil(t.kb0, t.kb1); }
+                else stencil(0, kblocks);
+            }
             if (te >= 0) {
 #pragma unroll 1
               for (int j = 0, tj = te, unit = 0; j < nb && tj < total; ++j, tj += step) {
-                const DwTile t = dw_tile(g, tj);
+                const DwTile t = dw_tile(g, tj);      // (a store needs all of it in one thread only)
                 const int b = rc.s, n0 = t.nt * cols;
                 const uint32_t ph = rc.ph, t_acc = t_warp + b * g.acc_stride;
                 rc.next();
                 if (kEpi == DE_STORE) {
+                    // this thread's row of a result box and the swizzle of its 16-byte pieces (box_piece), made anew per tile
+                    int r = row;
+                    asm volatile("" : "+r"(r));
+                    const bool live_rows = quarter * 32 < g.tile_rows;
+                    const uint32_t box_row = (uint32_t)(r * chunk * 2), box_xor = chunk == 64 ? (r & 7u) << 4 : chunk == 32 ? ((r >> 1) & 3u) << 4 : ((r >> 2) & 1u) << 4;
                     // (tile, column chunk) pairs are dealt to the four column groups in turn
 #pragma unroll 1
-                    for (int c = 0; c < nchunks; ++c, ++unit) {
-                        if ((unit & 3) != cgroup) continue;
+                    for (int c = (cgroup - unit) & 3; c < nchunks; c += 4) {
                         const uint32_t buf = sbase + g.off_stage + (uint32_t)(cgroup * g.out_bufs + (g.out_bufs == 2 ? (cnt & 1) : 0)) * g.box_bytes;
                         // (the group's warps meet twice per box: all know whether to go on, and the box is free)
                         ok = ok && mbar_wait(accf + 8u * b, ph);
@@ -381,8 +434,10 @@ dw_tc_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CU
                         asm volatile("bar.sync %0, 128;" ::"r"(2 + cgroup) : "memory");
                         if (fail_flag[0]) { ok = false; break; }
                         tc_fence_after();
+                        // (a quarter of the accumulator's lanes behind the tile's rows has nothing to store)
+                        if (!live_rows) warp_arrive(acce + 8u * b, lane);
 #pragma unroll 1
-                        for (int c0 = 0; c0 < chunk; c0 += 32) {
+                        for (int c0 = 0; live_rows && c0 < chunk; c0 += 32) {
                             const bool wide = chunk - c0 >= 32;
                             float v[32];
                             if (wide) tmem_ld32(t_acc + c * chunk + c0, v); else tmem_ld16(t_acc + c * chunk + c0, v);
@@ -399,9 +454,9 @@ dw_tc_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CU
                                     pk[q4 / 2] = clamp_bf16x2(pack2(t0.x, t0.y), plo, phi);
                                     pk[q4 / 2 + 1] = clamp_bf16x2(pack2(t1.x, t1.y), plo, phi);
                                 }
-                                const int piece = (c0 >> 3) + 2 * h;
-                                st_shared16(buf + box_piece(chunk, row, piece), make_uint4(pk[0], pk[1], pk[2], pk[3]));
-                                st_shared16(buf + box_piece(chunk, row, piece + 1), make_uint4(pk[4], pk[5], pk[6], pk[7]));
+                                const uint32_t piece = (uint32_t)(c0 * 2 + 32 * h);      // bytes in front of it, before the swizzle
+                                st_shared16(buf + box_row + (piece ^ box_xor), make_uint4(pk[0], pk[1], pk[2], pk[3]));
+                                st_shared16(buf + box_row + ((piece + 16u) ^ box_xor), make_uint4(pk[4], pk[5], pk[6], pk[7]));
                             }
                         }
                         fence_proxy_async();
@@ -415,6 +470,7 @@ dw_tc_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CU
                         }
                         ++cnt;
                     }
+                    unit += nchunks;
                     if (!ok) break;
                     continue;
                 }

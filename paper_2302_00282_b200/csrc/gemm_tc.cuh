@@ -90,19 +90,21 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// Bounded wait for the phase with the given parity: one plain test, then at most `limit` polls that each
-// sleep in hardware up to `hint_ns`.  Returns false when it gave up.
+// Whether the phase with the given parity is complete.  The answer takes some 190 cycles however long ago that was (a wait that
+// finds its phase complete costs 240, four MMAs of N = 64 with their commit 190; measured): a multiplying thread asks for the
+// next block before it issues this one (umma_block), and nobody asks for ring slots that nothing has been put in yet.
+__device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done;
+}
+// Bounded wait for the phase with the given parity: at most `limit` polls that each sleep in hardware up to `hint_ns` (a poll
+// that finds the phase complete takes 205 cycles, a plain test 190; a test in front only lengthens the waits that do wait).  Returns false when it gave up.
 __device__ __forceinline__ bool mbar_wait_limited(uint32_t bar, uint32_t parity, int limit, uint32_t hint_ns) {
-    {
-        // most waits find their phase complete: a plain test is cheaper than a suspending wait
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-        if (done) return true;
-    }
 #pragma unroll 1
     for (int i = 0; i < limit; ++i) {
         uint32_t done;
@@ -184,6 +186,36 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t da, uint64_t
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
+}
+// (tcgen05.fence::after_thread_sync takes 200 cycles in a CTA of 19 warps.  It orders this thread's products behind other
+// threads' tensor-memory reads and belongs behind the wait for an accumulator; operands in shared memory need their full
+// barrier and, where threads wrote them, the writers' proxy fence.)
+// The products of one K block, their commit to a barrier, and the state of the next block's barrier, which is asked for first
+// and looked at last: its answer arrives while the products are issued (235 cycles a block of N = 64 instead of 430 with a test
+// in front, 510 with two).  One to four K = 16 steps (the first always), at offsets a1, a2, a3 of the activation operand and 2,
+// 4, 6 of the weights, in 16-byte units; hi: the upper halves of the descriptors.
+__device__ __forceinline__ uint32_t umma_block(uint32_t d_tmem, uint32_t a_hi, uint32_t a_lo, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b_hi, uint32_t b_lo,
+                                               uint32_t idesc, uint32_t acc, int steps, uint32_t commit, uint32_t next, uint32_t next_ph) {
+    uint32_t ready;
+    asm volatile(
+        "{\n\t.reg .pred p, q, s1, s2, s3;\n\t.reg .b64 da, db;\n\t.reg .b32 x, y;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 q, [%12], %13;\n\t"
+        "setp.ne.b32 p, %9, 0;\n\tsetp.gt.s32 s1, %10, 1;\n\tsetp.gt.s32 s2, %10, 2;\n\tsetp.gt.s32 s3, %10, 3;\n\t"
+        "mov.b64 da, {%3, %2};\n\tmov.b64 db, {%8, %7};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%1], da, db, %14, p;\n\t"
+        "setp.eq.u32 p, 0, 0;\n\t"
+        "add.u32 x, %3, %4;\n\tadd.u32 y, %8, 2;\n\tmov.b64 da, {x, %2};\n\tmov.b64 db, {y, %7};\n\t"
+        "@s1 tcgen05.mma.cta_group::1.kind::f16 [%1], da, db, %14, p;\n\t"
+        "add.u32 x, %3, %5;\n\tadd.u32 y, %8, 4;\n\tmov.b64 da, {x, %2};\n\tmov.b64 db, {y, %7};\n\t"
+        "@s2 tcgen05.mma.cta_group::1.kind::f16 [%1], da, db, %14, p;\n\t"
+        "add.u32 x, %3, %6;\n\tadd.u32 y, %8, 6;\n\tmov.b64 da, {x, %2};\n\tmov.b64 db, {y, %7};\n\t"
+        "@s3 tcgen05.mma.cta_group::1.kind::f16 [%1], da, db, %14, p;\n\t"
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%11];\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(ready)
+        : "r"(d_tmem), "r"(a_hi), "r"(a_lo), "r"(a1), "r"(a2), "r"(a3), "r"(b_hi), "r"(b_lo), "r"(acc), "r"(steps), "r"(commit), "r"(next), "r"(next_ph),
+          "r"(idesc) : "memory");
+    return ready;
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");

@@ -150,7 +150,7 @@ struct Launch {
     // their width in output columns, row slots, steps in flight, pieces per (slot, channel), staged pixel, chunk pairs
     int stem_tc = 0, st_lead = 0, st_vec = 0, st_cbs = 1, st_cw = 0, st_slots = 0, st_qp = 0, st_pc = 0, st_pairs = 0;
     int n_acc = 1;                                                 // dw_tc_kernel: channel tiles of tile_n columns per CTA (2: both accumulators hold one tile)
-    int pair = 0, a_slots = 0, b_slots = 0, off_b2 = 0, s_slots = 2;            // LK_GEMM2 with a 1x1 consumer: pair_tc_kernel and its rings
+    int pair = 0, a_stride = 0, a_slots = 0, b_slots = 0, off_b2 = 0, s_slots = 2;            // LK_GEMM2 with a 1x1 consumer: pair_tc_kernel and its rings
     // ---- two linked convolutions (LK_GEMM2): producer tile rh1 x rw1 = patch_rh x patch_rw, consumer tile rh2 x rw2
     int k2 = 1, kblocks2 = 0, n1pad = 0, halo2 = 0, rh2 = 0, rw2 = 0, act3 = 0, off_mid = 0, stage_bytes = 0;
     int off_halo = 0, off_stg = 0, off_dww = 0, off_bias = 0, off_bar = 0;                    // shared-memory layout

@@ -42,7 +42,7 @@ struct PairParams {
 
 struct PairRing {
     int s, n;
-    uint32_t ph;
+    uint32_t ph, ready;      // ready: as in ConvRing
     __device__ __forceinline__ void next() { if (++s == n) { s = 0; ph ^= 1u; } }
 };
 
@@ -50,31 +50,31 @@ struct PairRing {
 __device__ __forceinline__ bool pair_gemm1(const PairParams &g, PairRing &ra, PairRing &rb, uint32_t sbase, uint32_t a_full, uint32_t b_full, uint32_t d1) {
     const uint32_t idesc = in_reg(g.idesc1);
     const int n = in_reg(g.seg.kblocks), slots = in_reg(g.n1_slots), resident = in_reg(g.resident), n1pad = in_reg(g.n1pad);
-    constexpr uint64_t hi = (uint64_t)(64u | (1u << 14) | (2u << 29)) << 32;
+    constexpr uint32_t hi = 64u | (1u << 14) | (2u << 29);
     const uint32_t b0 = sbase + g.off_b;
     uint32_t acc = 0u;
 #pragma unroll 1
     for (int kb = 0; kb < n; ++kb) {
-        if (!mbar_wait(a_full + 8u * ra.s, ra.ph)) return false;
-        const uint32_t a4 = 0x10000u | ((sbase + ra.s * kABytes) >> 4);
+        if (!ra.ready && !mbar_wait(a_full + 8u * ra.s, ra.ph)) return false;
+        const uint32_t a4 = 0x10000u | ((sbase + ra.s * kABytes) >> 4), a_used = a_full + 8u * (kPairMaxSlots + ra.s);
+        ra.next();
+        ra.ready = 0u;
 #pragma unroll 1
         for (int h = 0; h < slots; ++h) {
-            uint32_t b4;
+            uint32_t b4, b_used = 0u;
             if (resident) b4 = 0x10000u | ((b0 + kb * n1pad * 128) >> 4);
             else {
-                if (!mbar_wait(b_full + 8u * rb.s, rb.ph)) return false;
+                if (!rb.ready && !mbar_wait(b_full + 8u * rb.s, rb.ph)) return false;
                 b4 = 0x10000u | ((b0 + rb.s * kABytes) >> 4);
+                b_used = b_full + 8u * (kPairMaxSlots + rb.s);
+                rb.next();
             }
-            tc_fence_after();
             const uint32_t d = d1 + h * 128;
-            umma_bf16(d, hi | a4, hi | b4, idesc, acc);
-            umma_bf16_acc(d, hi | (a4 + 2), hi | (b4 + 2), idesc);
-            umma_bf16_acc(d, hi | (a4 + 4), hi | (b4 + 4), idesc);
-            umma_bf16_acc(d, hi | (a4 + 6), hi | (b4 + 6), idesc);
-            if (!resident) { umma_commit(b_full + 8u * (kPairMaxSlots + rb.s)); rb.next(); }
+            // (resident weights: one block per activation slot, whose successor is asked for; else the next weight slot)
+            if (resident) ra.ready = umma_block(d, hi, a4, 2u, 4u, 6u, hi, b4, idesc, acc, 4, a_used, a_full + 8u * ra.s, ra.ph);
+            else rb.ready = umma_block(d, hi, a4, 2u, 4u, 6u, hi, b4, idesc, acc, 4, b_used, b_full + 8u * rb.s, rb.ph);
         }
-        umma_commit(a_full + 8u * (kPairMaxSlots + ra.s));
-        ra.next();
+        if (!resident) umma_commit(a_used);
         acc = 1u;
     }
     return true;
@@ -97,20 +97,16 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + g.off_bar + 8 * (4 * kPairMaxSlots + 12 + kMaxSkipSlots * kCvEpiWarps));
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0 && elect_one()) {
-        for (int s = 0; s < kPairMaxSlots; ++s) {
-            mbar_init(a_full + 8u * s, 1); mbar_init(a_full + 8u * (kPairMaxSlots + s), 1);
-            mbar_init(b_full + 8u * s, 1); mbar_init(b_full + 8u * (kPairMaxSlots + s), 1);
+    if (warp == 0) {
+        // (a lane per barrier; d1e, d2e and midf count the epilogue warps)
+        constexpr int d0 = 4 * kPairMaxSlots, n_bars = d0 + 12 + kMaxSkipSlots * kCvEpiWarps;
+        for (int i = lane; i < n_bars; i += 32) {
+            const int d = i - d0;
+            mbar_init(bar + 8u * i, d == 2 || d == 3 || (d >= 6 && d <= 8) ? kCvEpiWarps : 1);
         }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(d1f + 8u * b, 1); mbar_init(d1e + 8u * b, kCvEpiWarps);
-            mbar_init(d2f + 8u * b, 1); mbar_init(d2e + 8u * b, kCvEpiWarps);
-        }
-        mbar_init(midf, kCvEpiWarps); mbar_init(mide, 1); mbar_init(bres, 1);
-        for (int e = 0; e < kMaxSkipSlots * kCvEpiWarps; ++e) mbar_init(skip0 + 8u * e, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB1) : "memory");
+        if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
+        if (lane == 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB1) : "memory");
     }
     if (warp == 3) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
@@ -132,7 +128,8 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (elect_one()) {
             // ---- A: im2col boxes of the first convolution ----
             pdl_wait();
-            PairRing ra = {0, in_reg(g.a_slots), 0u};
+            PairRing ra = {0, in_reg(g.a_slots), 0u, 0u};
+            int fresh = ra.n;      // slots that nothing has been put in yet
             const int tiles = in_reg(g.tiles), n_kb = in_reg(g.seg.kblocks), cend = in_reg(g.seg.cblocks * kTileK), k = in_reg(g.seg.k);
 #pragma unroll 1
             for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
@@ -145,7 +142,7 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
                 for (int kb = 0; kb < n_kb; ++kb) {
                     const uint32_t fb = a_full + 8u * ra.s;
-                    ok = mbar_wait(fb + 8u * kPairMaxSlots, ra.ph ^ 1u);
+                    ok = --fresh >= 0 || mbar_wait(fb + 8u * kPairMaxSlots, ra.ph ^ 1u);
                     if (!ok) break;
                     mbar_arrive_expect_tx(fb, kABytes);
                     if (im2col) tma_load_im2col(sbase + ra.s * kABytes, &tmA, c, w0, h0, n, fb, s, r);
@@ -171,7 +168,8 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
                     for (int kb = 0; kb < kb2n; ++kb) tma_load_2d(b0 + n_kb * n1pad * 128 + (c * kb2n + kb) * kABytes, &tmB2, kb * kTileK, c * 128, bres);
             } else {
-                PairRing rb = {0, in_reg(g.b_slots), 0u};
+                PairRing rb = {0, in_reg(g.b_slots), 0u, 0u};
+                int fresh = rb.n;
                 const uint32_t bytes1 = (uint32_t)min(n1pad, 128) * 128u;
                 auto first = [&]() {
 #pragma unroll 1
@@ -179,7 +177,7 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
                         for (int h = 0; h < slots; ++h) {
                             const uint32_t fb = b_full + 8u * rb.s;
-                            ok = mbar_wait(fb + 8u * kPairMaxSlots, rb.ph ^ 1u);
+                            ok = --fresh >= 0 || mbar_wait(fb + 8u * kPairMaxSlots, rb.ph ^ 1u);
                             if (!ok) break;
                             mbar_arrive_expect_tx(fb, bytes1);
                             tma_load_2d(b0 + rb.s * kABytes, &tmB1, kb * kTileK, h * 128, fb);
@@ -192,7 +190,7 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
                         for (int kb = 0; kb < kb2n; ++kb) {
                             const uint32_t fb = b_full + 8u * rb.s;
-                            ok = mbar_wait(fb + 8u * kPairMaxSlots, rb.ph ^ 1u);
+                            ok = --fresh >= 0 || mbar_wait(fb + 8u * kPairMaxSlots, rb.ph ^ 1u);
                             if (!ok) break;
                             mbar_arrive_expect_tx(fb, kABytes);
                             tma_load_2d(b0 + rb.s * kABytes, &tmB2, kb * kTileK, c * 128, fb);
@@ -212,10 +210,10 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     } else if (warp == 1) {
         if (elect_one()) {
             // ---- MMA ----
-            PairRing ra = {0, in_reg(g.a_slots), 0u}, rb = {0, in_reg(g.b_slots), 0u};
+            PairRing ra = {0, in_reg(g.a_slots), 0u, 0u}, rb = {0, in_reg(g.b_slots), 0u, 0u};
             const int tiles = in_reg(g.tiles), step = gridDim.x, kb2n = in_reg(g.kblocks2), n2 = in_reg(g.n2_blocks), resident = in_reg(g.resident), dbl = in_reg(g.dbl);
             const uint32_t idesc2 = in_reg(g.idesc2), mid = sbase + g.off_mid, b0 = sbase + g.off_b, b2 = b0 + g.seg.kblocks * g.n1pad * 128;
-            constexpr uint64_t hi = (uint64_t)(64u | (1u << 14) | (2u << 29)) << 32;
+            constexpr uint32_t hi = 64u | (1u << 14) | (2u << 29);
             int i1 = 0, c2 = 0;      // first products issued; second-accumulator uses
             auto first = [&]() {
                 const int b = dbl ? i1 & 1 : 0, use = dbl ? i1 >> 1 : i1;
@@ -238,23 +236,29 @@ pair_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     const int b = c2 & 1;
                     ok = mbar_wait(d2e + 8u * b, ((c2 >> 1) & 1) ^ 1u);
                     if (!ok) break;
+                    tc_fence_after();
                     const uint32_t d = tmem_base + 256 + b * 128;
 #pragma unroll 1
                     for (int kb = 0; kb < kb2n; ++kb) {
                         const uint32_t a4 = 0x10000u | ((mid + kb * kABytes) >> 4);
-                        uint32_t b4;
+                        uint32_t b4, b_used = 0u;
                         if (resident) b4 = 0x10000u | ((b2 + (c * kb2n + kb) * kABytes) >> 4);
                         else {
-                            ok = mbar_wait(b_full + 8u * rb.s, rb.ph);
+                            ok = rb.ready || mbar_wait(b_full + 8u * rb.s, rb.ph);
                             if (!ok) break;
                             b4 = 0x10000u | ((b0 + rb.s * kABytes) >> 4);
+                            b_used = b_full + 8u * (kPairMaxSlots + rb.s);
+                            rb.next();
                         }
-                        tc_fence_after();
-                        umma_bf16(d, hi | a4, hi | b4, idesc2, kb > 0 ? 1u : 0u);
-                        umma_bf16_acc(d, hi | (a4 + 2), hi | (b4 + 2), idesc2);
-                        umma_bf16_acc(d, hi | (a4 + 4), hi | (b4 + 4), idesc2);
-                        umma_bf16_acc(d, hi | (a4 + 6), hi | (b4 + 6), idesc2);
-                        if (!resident) { umma_commit(b_full + 8u * (kPairMaxSlots + rb.s)); rb.next(); }
+                        // (resident weights have no slot to give back)
+                        if (!resident) rb.ready = umma_block(d, hi, a4, 2u, 4u, 6u, hi, b4, idesc2, kb > 0 ? 1u : 0u, 4, b_used, b_full + 8u * rb.s, rb.ph);
+                        else {
+                            const uint64_t h64 = (uint64_t)hi << 32;
+                            umma_bf16(d, h64 | a4, h64 | b4, idesc2, kb > 0 ? 1u : 0u);
+                            umma_bf16_acc(d, h64 | (a4 + 2), h64 | (b4 + 2), idesc2);
+                            umma_bf16_acc(d, h64 | (a4 + 4), h64 | (b4 + 4), idesc2);
+                            umma_bf16_acc(d, h64 | (a4 + 6), h64 | (b4 + 6), idesc2);
+                        }
                     }
                     if (ok) umma_commit(d2f + 8u * b);
                 }

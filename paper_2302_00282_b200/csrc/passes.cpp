@@ -906,7 +906,11 @@ struct Lower {
         const bool one = tiles <= g.hw.sm_count;                  // a CTA's only tile: results leave through the operand ring
         const int dww = (int)align_up((size_t)40 * C, 1024), bias = (int)align_up((size_t)L.npad * 4, 128);
         const int room = std::min(g.hw.smem_bytes_per_cta, 227 * 1024) - 2048 - 512 - dww - bias;
-        const int bslot = cols * 128;
+        // A slot of the operand ring holds the tile's rows, in whole groups of eight; a product reads 128 rows from its start and
+        // what the rows behind the tile's own give is not stored.  `ops_end`: the reads of the last slot stay inside the allocation.
+        L.a_stride = ceil_div(L.tile_rows, 8) * 1024;
+        auto ops_end = [&](int a_slots, int b_bytes) { return std::max(a_slots * L.a_stride + b_bytes, (a_slots - 1) * L.a_stride + 16384); };
+        const int bslot = L.tile_n * 128, bblk = L.n_acc * bslot;      // a slot of the weight ring; the weights of a K block
         // (the window covers whole blocks of br rows)
         auto window_h = [&](int br) { return (round_up(L.patch_rh, br) - 1) * s0.stride + 3; };
         auto window = [&](int br) { return (int)align_up((size_t)L.ni * window_h(br) * L.halo_w * L.halo_cb * 2, 128); };
@@ -939,9 +943,9 @@ struct Lower {
                         for (int bufs = 2; bufs >= 1; --bufs) {
                             if (L.cv_epi == 0 && cols % chunk) continue;
                             if (L.cv_epi != 0 && (chunk != (L.cv_epi == 1 ? 32 : 16) || bufs == 2)) continue;
-                            if (res && (one || L.ksplit > 1 || rgrid == 0)) continue;
-                            const int a_min = std::max(2, groups), h_min = std::max(2, groups), b_min = res ? 0 : 2;
-                            const int ops = a_min * 16384 + (res ? L.kblocks * bslot : b_min * bslot), st = staging(chunk, bufs);
+                            if (res && (L.ksplit > 1 || L.n_acc > 1 || rgrid == 0)) continue;
+                            const int a_min = std::max(2, groups), h_min = std::max(2, groups), b_min = res ? 0 : 1 + L.n_acc;
+                            const int ops = ops_end(a_min, res ? L.kblocks * bblk : b_min * bslot), st = staging(chunk, bufs);
                             const int need = (one ? std::max(ops, st) : ops + st) + h_min * hstride;
                             if (a_min > 8 || h_min > 8 || need > room) continue;
                             // The workers' time per tile: the stencils, then their group's boxes, which cost some 1100 cycles and
@@ -964,17 +968,18 @@ struct Lower {
         L.halo_bytes = L.ni * L.halo_h * L.halo_w * L.halo_cb * 2;
         L.halo_stride = hstride;
         auto used = [&]() {
-            const int ops = L.a_slots * 16384 + (L.b_resident ? L.kblocks * bslot : L.b_slots * bslot);
+            const int ops = ops_end(L.a_slots, L.b_resident ? L.kblocks * bblk : L.b_slots * bslot);
             return (one ? std::max(ops, st) : ops + st) + L.h_slots * hstride;
         };
         // deeper rings with what is left: windows first (they come from the predecessor's tensor), then weights, then operands
         auto grow = [&](int &slots, int by, int most) { while (slots + by <= most) { slots += by; if (used() > room) { slots -= by; break; } } };
         grow(L.h_slots, groups, std::min(8, 2 * std::max(2, groups)));
-        if (!L.b_resident) grow(L.b_slots, 1, std::min(4, std::max(2, L.kblocks)));
-        grow(L.a_slots, groups, std::min(8, 2 * std::max(2, groups)));
+        // (a CTA with one tile asks for all of its weights while the predecessor drains, where they fit)
+        if (!L.b_resident) grow(L.b_slots, 1, std::min(one ? 8 : 4, std::max(2, L.n_acc * L.kblocks)));
+        grow(L.a_slots, groups, std::min(8, one ? L.kblocks : 2 * std::max(2, groups)));
         L.nchunks = ceil_div(cols, L.chunk);
-        L.off_b = L.a_slots * 16384;
-        const int ops = L.off_b + (L.b_resident ? L.kblocks * bslot : L.b_slots * bslot);
+        L.off_b = L.a_slots * L.a_stride;
+        const int ops = ops_end(L.a_slots, L.b_resident ? L.kblocks * bblk : L.b_slots * bslot);
         L.off_stg = one ? 0 : ops;
         L.off_halo = (int)align_up((size_t)(one ? std::max(ops, st) : ops + st), 1024);
         L.off_dww = (int)align_up((size_t)L.off_halo + (size_t)L.h_slots * hstride, 128);
@@ -984,7 +989,7 @@ struct Lower {
         L.stages = std::min(6, L.a_slots); L.hstages = L.h_slots;
         L.dw_workers = 16;
         L.grid = (int)std::min<long>(tiles, L.b_resident ? rgrid : g.hw.sm_count);
-        L.block = 64 + 32 * 16;
+        L.block = 96 + 32 * 16;
         L.tmem_cols = 32;
         while (L.tmem_cols < (L.n_acc == 2 ? 2 : 2 * L.dw_batch) * L.acc_stride) L.tmem_cols *= 2;
         return XENOS_OK;

@@ -235,10 +235,10 @@ static xenos_status_t encode_stem_map(const Graph &g, Runtime *rt, const Launch 
 }
 
 typedef void (*DwKernel)(CUtensorMap, CUtensorMap, CUtensorMap, xk::DwParams);
-template <int kEpi>
+template <int kEpi, int kCB>
 static DwKernel dw_kernel_of(int stride, int br) {
-    if (stride == 1) return br == 4 ? xk::dw_tc_kernel<kEpi, 1, 4> : br == 2 ? xk::dw_tc_kernel<kEpi, 1, 2> : xk::dw_tc_kernel<kEpi, 1, 1>;
-    return br == 4 ? xk::dw_tc_kernel<kEpi, 2, 4> : br == 2 ? xk::dw_tc_kernel<kEpi, 2, 2> : xk::dw_tc_kernel<kEpi, 2, 1>;
+    if (stride == 1) return br == 4 ? xk::dw_tc_kernel<kEpi, 1, 4, kCB> : br == 2 ? xk::dw_tc_kernel<kEpi, 1, 2, kCB> : xk::dw_tc_kernel<kEpi, 1, 1, kCB>;
+    return br == 4 ? xk::dw_tc_kernel<kEpi, 2, 4, kCB> : br == 2 ? xk::dw_tc_kernel<kEpi, 2, 2, kCB> : xk::dw_tc_kernel<kEpi, 2, 1, kCB>;
 }
 // Convolution of an image: how its rows are loaded, the image's type, with or without a pool.
 using StemKernel = void (*)(xk::StemParams);
@@ -269,8 +269,10 @@ static auto *f32_chain_kernel(const Launch &L) {
                      : (L.f32_ws ? xk::f32_chain_kernel<2, 1, true> : xk::f32_chain_kernel<2, 1, false>);
 }
 
-static DwKernel dw_kernel(int epi, int stride, int br) {
-    return epi == xk::DE_STORE ? dw_kernel_of<xk::DE_STORE>(stride, br) : epi == xk::DE_GAP ? dw_kernel_of<xk::DE_GAP>(stride, br) : dw_kernel_of<xk::DE_SPLIT>(stride, br);
+static DwKernel dw_kernel(int epi, int stride, int br, int cb) {
+    if (epi == xk::DE_STORE)
+        return cb == 64 ? dw_kernel_of<xk::DE_STORE, 64>(stride, br) : cb == 32 ? dw_kernel_of<xk::DE_STORE, 32>(stride, br) : dw_kernel_of<xk::DE_STORE, 0>(stride, br);
+    return epi == xk::DE_GAP ? dw_kernel_of<xk::DE_GAP, 0>(stride, br) : dw_kernel_of<xk::DE_SPLIT, 0>(stride, br);
 }
 
 // Where launch_pass hands its kernels: to a stream, to the node of a recorded pass that holds the launch, or nowhere (the
@@ -730,7 +732,7 @@ static xenos_status_t issue_pass(Graph &g, int batch, const void *const *in, voi
                 p.kb_per = L.ksplit > 1 ? L.kb_per : L.kblocks;
                 p.groups = L.dw_groups; p.wpg_log2 = L.dw_wpg_log2; p.pairs = L.halo_cb > 32 ? 32 : 16;
                 p.batch_tiles = L.dw_batch; p.n_bufs = L.n_acc == 2 ? 1 : 2 * L.dw_batch;
-                p.a_slots = L.a_slots; p.b_slots = L.b_slots; p.h_slots = L.h_slots; p.b_resident = L.b_resident;
+                p.a_stride = L.a_stride; p.a_slots = L.a_slots; p.b_slots = L.b_slots; p.h_slots = L.h_slots; p.b_resident = L.b_resident;
                 p.halo_bytes = L.halo_bytes; p.halo_stride = L.halo_stride; p.halo_h = L.halo_h; p.halo_w = L.halo_w; p.halo_cb = L.halo_cb;
                 p.acc_stride = L.acc_stride; p.tmem_cols = L.tmem_cols;
                 p.chunk = L.chunk; p.nchunks = L.nchunks; p.box_bytes = 128 * L.chunk * 2; p.out_bufs = L.out_bufs;
@@ -750,7 +752,7 @@ static xenos_status_t issue_pass(Graph &g, int batch, const void *const *in, voi
                     maps = &now;
                 }
                 const int limit = L.b_resident ? std::max(1, sms / L.n_tiles) * L.n_tiles : sms;
-                auto *k = dw_kernel(L.cv_epi, a.stride, L.dw_br);
+                auto *k = dw_kernel(L.cv_epi, a.stride, L.dw_br, L.halo_cb);
                 le = to.pdl(k, std::min(p.total, limit), L.block, L.smem_bytes, maps->a0, rt->tmaps[li], maps->o, p);
                 break;
             }
