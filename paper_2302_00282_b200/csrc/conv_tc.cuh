@@ -6,7 +6,7 @@
 //
 // A CTA walks over tiles of 128 consecutive output pixels (numbered image, row, column: a tile may span rows and images,
 // so no row of the MMA is padding except in the last tile) x tile_n <= 256 channels (Section 4.2.1's split).
-//   warp 0      A operand: one box per 64-channel block and tap.  A 1x1 stride-1 product reads rows of the [pixels][C]
+//   warp 0      A operand (with warp 3 where a block takes several boxes): one box per 64-channel block and tap.  A 1x1 stride-1 product reads rows of the [pixels][C]
 //               matrix; every other window is fetched in the copy engine's im2col form, which walks the output pixels
 //               with the convolution's stride and fills padding with zeros.  No thread computes an address per element.
 //   warp 1      tcgen05.mma into one of two tensor-memory accumulators
@@ -133,17 +133,15 @@ __device__ __forceinline__ int in_reg(int x) { asm volatile("" : "+r"(x)); retur
 __device__ __forceinline__ uint32_t in_reg(uint32_t x) { asm volatile("" : "+r"(x)); return x; }
 
 // The ring as its issuing thread sees it: slot, phase, and the addresses of the slot's barrier and data.  Barriers
-// are asked as little and as early as possible (see mbar_test): a filling thread knows that the first `fresh` slots are free,
-// a multiplying thread asks for the next slot before it multiplies this one (ready).
+// are asked as little and as early as possible (see mbar_test): `ready` is what is known of the slot at hand.
 struct ConvRing {
-    int s, n, step, fresh;
+    int s, n, step;
     uint32_t ph, fb, data, fb0, data0, ready;
     __device__ __forceinline__ void init(const ConvParams &g, uint32_t sbase, uint32_t bar) {
-        s = 0; n = in_reg(g.stages); step = in_reg(g.stage_bytes); ph = 0; ready = 0; fresh = n;
+        s = 0; n = in_reg(g.stages); step = in_reg(g.stage_bytes); ph = 0; ready = 0;
         fb = fb0 = bar; data = data0 = sbase;
     }
     __device__ __forceinline__ uint32_t empty() const { return fb + 8u * kCvMaxStages; }
-    __device__ __forceinline__ bool room() { return --fresh >= 0 || mbar_wait(empty(), ph ^ 1u); }
     __device__ __forceinline__ bool full() const { return ready || mbar_wait(fb, ph); }
     __device__ __forceinline__ void next() {
         ++s; fb += 8u; data += (uint32_t)step;
@@ -151,20 +149,45 @@ struct ConvRing {
     }
 };
 
+// A filling thread's view of the ring: every turn-th slot.  Two threads bring the activation operand where a stage takes several
+// boxes (16 or 32 channels: some 180 cycles a box, 720 a stage); else one does (it gets a 64-channel block in 250, as often as
+// the products ask for one, and a second thread's look at the barriers costs more than it brings: ResNet-18 at batch 32 250 us
+// against 248; SqueezeNet, whose expands have such stages, 162 with two threads against 165).
+struct ConvFill {
+    int s, n, turn, skip;              // skip: blocks of the next stretch before this thread's first one
+    uint32_t ph, fresh, fb, data, step, back;
+    __device__ __forceinline__ void init(const ConvParams &g, uint32_t sbase, uint32_t bar, int which) {
+        turn = in_reg(g.seg[0].per_stage > 1 ? 2 : 1);
+        s = skip = which; n = in_reg(g.stages); ph = 0u; fresh = 1u;
+        step = in_reg((uint32_t)g.stage_bytes); back = (uint32_t)n * step;
+        fb = bar + 8u * which; data = sbase + step * which;
+    }
+    // (nothing has been put into the slots of the first round yet: no need to ask for room)
+    __device__ __forceinline__ bool room() const { return fresh || mbar_wait(fb + 8u * kCvMaxStages, ph ^ 1u); }
+    __device__ __forceinline__ void next() {
+        s += turn; fb += 8u * turn; data += (uint32_t)turn * step;
+        const bool wrap = s >= n;
+        s -= wrap ? n : 0; fb -= wrap ? 8u * (uint32_t)n : 0u; data -= wrap ? back : 0u;
+        ph ^= wrap ? 1u : 0u; fresh = wrap ? 0u : fresh;
+    }
+};
+
 // One thread's copies of a segment's K blocks [kb0, kb1) of a tile.  kSeg is a compile-time index: fields of g.seg[i] with a
 // run-time i are indexed constant loads.
 template <int kSeg>
-__device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorMap *tm, ConvRing &st, int kb0, int kb1, int m0, int n, int p, int q) {
+__device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorMap *tm, ConvFill &st, int kb0, int kb1, int m0, int n, int p, int q) {
     const ConvSegment &sg = g.seg[kSeg];
     const uint32_t box = in_reg(sg.box_bytes);
+    int kb = kb0 + st.skip;
     if (!sg.im2col && sg.per_stage == 1) {
 #pragma unroll 1
-        for (int kb = kb0; kb < kb1; ++kb) {
+        for (; kb < kb1; kb += st.turn) {
             if (!st.room()) return false;
             mbar_arrive_expect_tx(st.fb, box);
             tma_load_2d(st.data, tm, kb * kTileK, m0, st.fb);
             st.next();
         }
+        st.skip = kb - kb1;
         return true;
     }
     const int h0 = p * sg.stride + sg.low, w0 = q * sg.stride + sg.low;
@@ -172,27 +195,38 @@ __device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorM
     if (sg.per_stage == 1) {
         const int cend = in_reg(sg.cblocks * kTileK);
         int c = 0, r = 0, s = 0;
+        auto advance = [&]() {
+            c += kTileK;
+            const bool tap = c == cend;
+            c = tap ? 0 : c;
+            s += tap ? 1 : 0;
+            const bool row = s == k;
+            s = row ? 0 : s;
+            r += row ? 1 : 0;
+        };
         if (kb0) {
             const int tap = kb0 / sg.cblocks;
             c = (kb0 - tap * sg.cblocks) * kTileK; r = tap / k; s = tap - r * k;
         }
+        if (st.skip) advance();
 #pragma unroll 1
-        for (int kb = kb0; kb < kb1; ++kb) {
+        for (; kb < kb1; kb += st.turn) {
             if (!st.room()) return false;
             mbar_arrive_expect_tx(st.fb, box);
             tma_load_im2col(st.data, tm, c, w0, h0, n, st.fb, s, r);
             st.next();
-            c += kTileK;
-            if (c == cend) { c = 0; if (++s == k) { s = 0; ++r; } }
+            advance();
+            if (st.turn == 2) advance();
         }
+        st.skip = kb - kb1;
         return true;
     }
     // several taps of 16 or 32 channels share a stage
     const int per = in_reg(sg.per_stage), taps = in_reg(sg.taps);
     const uint32_t stride = in_reg(sg.box_stride);
-    int tap = kb0 * per, r = tap / k, s = tap - r * k;
+    int tap = kb * per, r = tap / k, s = tap - r * k;
 #pragma unroll 1
-    for (int kb = kb0; kb < kb1; ++kb) {
+    for (; kb < kb1; kb += st.turn) {
         const int nb = min(per, taps - tap);
         if (!st.room()) return false;
         mbar_arrive_expect_tx(st.fb, box * nb);
@@ -202,9 +236,12 @@ __device__ __forceinline__ bool conv_load_a(const ConvParams &g, const CUtensorM
             else tma_load_2d(st.data + b * stride, tm, 0, m0, st.fb);
             if (++s == k) { s = 0; ++r; }
         }
-        tap += nb;
+        tap += st.turn * per;
+        s += (st.turn - 1) * per;
+        while (s >= k) { s -= k; ++r; }
         st.next();
     }
+    st.skip = kb - kb1;
     return true;
 }
 
@@ -679,11 +716,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     bool ok = true;
 
     const unsigned gave_up = kStatusTimeout | (((unsigned)g.launch_id & 0xfffu) << 12);
-    if (warp == 0) {
+    if (warp == 0 || (warp == 3 && g.seg[0].per_stage > 1)) {
         // ---- A operand ----
         if (elect_one()) {
-            ConvRing st;
-            st.init(g, sbase, bar);
+            ConvFill st;
+            st.init(g, sbase, bar, warp ? 1 : 0);
             const int k0 = in_reg(g.seg[0].kblocks), total = in_reg(g.total);
             bool waited = false;
 #pragma unroll 1
@@ -721,13 +758,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                 ConvRing st;
                 st.init(g, sbase, bar);
                 const int total = in_reg(g.total);
+                int fresh = st.n;      // slots that nothing has been put in yet
 #pragma unroll 1
                 for (int ti = blockIdx.x; ti < total && ok; ti += gridDim.x) {
                     const ConvTile t = conv_tile(g, ti);
                     const int row = t.nt * tile_n;
 #pragma unroll 1
                     for (int kb = t.kb0; kb < t.kb1; ++kb) {
-                        ok = st.room();
+                        ok = --fresh >= 0 || mbar_wait(st.empty(), st.ph ^ 1u);
                         if (!ok) break;
                         mbar_arrive_expect_tx(st.fb, bytes);
                         tma_load_2d(st.data + kABytes, &tmB, kb * kTileK, row, st.fb);
