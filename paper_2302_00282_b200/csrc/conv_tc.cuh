@@ -500,13 +500,16 @@ __device__ __forceinline__ bool conv_epilogue_gap(const ConvParams &g, uint8_t *
 
 // Four adjacent columns of one output pixel behind a split reduction: bias, activation, identity shortcut, second
 // activation, store.
-__device__ __forceinline__ void conv_finish_store4(const ConvParams &g, float4 a, const float4 bz, int nc, size_t pix) {
+// (sk: the shortcut's four elements, asked for by the caller)
+__device__ __forceinline__ uint2 conv_skip4(const ConvParams &g, int nc, size_t pix) {
+    return g.skip ? __ldg(reinterpret_cast<const uint2 *>(g.skip + pix * g.skip_ctot + nc)) : make_uint2(0u, 0u);
+}
+__device__ __forceinline__ void conv_finish_store4(const ConvParams &g, float4 a, const float4 bz, int nc, size_t pix, const uint2 sk) {
     const float lo1 = act_lo(g.act), hi1 = act_hi(g.act), lo2 = act_lo(g.act2), hi2 = act_hi(g.act2);
     float v[4] = {a.x + bz.x, a.y + bz.y, a.z + bz.z, a.w + bz.w};
 #pragma unroll
     for (int c = 0; c < 4; ++c) v[c] = fminf(fmaxf(v[c], lo1), hi1);
     if (g.skip) {
-        const uint2 sk = __ldg(reinterpret_cast<const uint2 *>(g.skip + pix * g.skip_ctot + nc));
         v[0] += __uint_as_float(sk.x << 16); v[1] += __uint_as_float(sk.x & 0xffff0000u);
         v[2] += __uint_as_float(sk.y << 16); v[3] += __uint_as_float(sk.y & 0xffff0000u);
     }
@@ -585,7 +588,7 @@ __device__ __forceinline__ bool conv_epilogue_split(const ConvParams &g, uint8_t
                 const float4 x4 = __ldcg(reinterpret_cast<const float4 *>(src + (size_t)sp * g.split_stride));
                 a.x += x4.x; a.y += x4.y; a.z += x4.z; a.w += x4.w;
             }
-            conv_finish_store4(g, a, ld_shared_f4(bias_s + (uint32_t)nc * 4u), nc, px);
+            conv_finish_store4(g, a, ld_shared_f4(bias_s + (uint32_t)nc * 4u), nc, px, conv_skip4(g, nc, px));
         }
         asm volatile("bar.sync 1, 256;" ::: "memory");
         if (et == 0) {
@@ -608,11 +611,13 @@ __device__ __forceinline__ void cluster_sync() {
 }
 
 // Reduction split over a thread-block cluster: the chunks of a tile are the CTAs of one cluster (rank = chunk).  Each CTA owns
-// an equal share of the tile's rows; every CTA sends its fp32 partial sums of a row to the row's owner through distributed
-// shared memory, and the owner adds the chunks in ascending order and stores.  The exchange buffer is [chunk][row of the
-// share][tile_n + 4] (the 4 words of padding spread a warp's rows over the banks); "arrived" counts the warps of all CTAs.
-// Measured at batch 1: through global memory and counters the exchange took 5 us (fence 0.7, partial sums 0.5, counter 0.9,
-// reads and stores 2.7), as much as the product; the 12 split launches of a batch-1 ResNet-18 gave back 16 of 131 us.
+// an equal share of the tile's rows.  A CTA parks its fp32 partial sums [row][tile_n + 4] in the operand ring, which is free by
+// then, and sends every other owner its rows, which are contiguous, as one bulk copy into chunk t.ks of that owner's exchange
+// buffer [chunk][row of the share][tile_n + 4]; the owner adds the chunks in ascending order and stores.  (The 4 words of padding
+// spread a warp's rows over the banks; "arrived" counts the bytes.)
+// Measured at batch 1: through global memory and counters the exchange took 5 us, as much as the product.  As 16-byte stores to
+// distributed shared memory by all threads it took 4400 to 6000 cycles for 18 KB a CTA (of which 1100 to 2700 for the release
+// behind the stores) and 8900 for 57 KB.
 __device__ __forceinline__ bool conv_epilogue_cluster(const ConvParams &g, uint8_t *sm, uint32_t bar, uint32_t tmem_base, uint32_t arrived) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, e = warp - 4, quarter = warp & 3, half = e >> 2;
     const int row = quarter * 32 + lane, et = threadIdx.x - 128;
@@ -621,11 +626,17 @@ __device__ __forceinline__ bool conv_epilogue_cluster(const ConvParams &g, uint8
     const int n0 = t.nt * g.tile_n, m0 = t.mt * g.tile_rows;
     const int live = min(kTileM, g.rows - m0), per = (live + g.ksplit - 1) / g.ksplit;
     const uint32_t pitch = (uint32_t)(g.tile_n + 4) * 4u;
+    const int r0 = t.ks * per, mine = max(0, min(per, live - r0)), c4n = g.tile_n >> 2, items = mine * c4n;
+    if (et == 0) mbar_arrive_expect_tx(arrived, (uint32_t)((g.ksplit - 1) * mine) * pitch);
+    // this thread's first four columns of the result, and its shortcut elements, which are asked for before the exchange
+    int rr = et / c4n, c4 = et - rr * c4n;
+    const int step_r = 32 * kCvEpiWarps / c4n, step_c = 32 * kCvEpiWarps - step_r * c4n;
+    uint2 sk = make_uint2(0u, 0u);
+    if (et < items && n0 + c4 * 4 < g.N) sk = conv_skip4(g, n0 + c4 * 4, (size_t)(m0 + r0 + rr));
     const bool ok = mbar_wait(bar + 8u * (2 * kCvMaxStages), 0u);
     if (ok) {
         tc_fence_after();
-        const int owner = row / per;
-        const uint32_t dst = cluster_addr(buf, (uint32_t)min(owner, g.ksplit - 1)) + (uint32_t)(t.ks * per + row - owner * per) * pitch;
+        const uint32_t dst = sbase + (uint32_t)row * pitch;
 #pragma unroll 1
         for (int j = half; j < g.nchunks; j += 2) {
             float v[16];
@@ -633,17 +644,21 @@ __device__ __forceinline__ bool conv_epilogue_cluster(const ConvParams &g, uint8
             if (row < live)
 #pragma unroll
                 for (int q4 = 0; q4 < 16; q4 += 4)
-                    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(j * 16 + q4) * 4u), "f"(v[q4]), "f"(v[q4 + 1]),
+                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(j * 16 + q4) * 4u), "f"(v[q4]), "f"(v[q4 + 1]),
                                  "f"(v[q4 + 2]), "f"(v[q4 + 3]) : "memory");
         }
         tc_fence_before();
+        fence_proxy_async();
     }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    // warp e sends owner e its rows (also after a wait that gave up: nobody waits in vain for this CTA)
+    const int theirs = min(per, live - e * per);
+    if (e < g.ksplit && e != t.ks && theirs > 0 && elect_one())
+        asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(cluster_addr(buf, (uint32_t)e) + (uint32_t)(t.ks * per) * pitch), "r"(sbase + (uint32_t)(e * per) * pitch), "r"((uint32_t)theirs * pitch),
+                     "r"(cluster_addr(arrived, (uint32_t)e)) : "memory");
     __syncwarp();
-    // one arrival per warp at every owner (also after a wait that gave up: nobody waits in vain for this CTA)
-    if (lane < g.ksplit)
-        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr(arrived, (uint32_t)lane)) : "memory");
     if (!ok) return false;
-    const int r0 = t.ks * per, mine = min(per, live - r0), c4n = g.tile_n >> 2;
     bool seen = false;
 #pragma unroll 1
     for (int i = 0; i < kSpinLimit && !seen; ++i) {
@@ -657,16 +672,23 @@ __device__ __forceinline__ bool conv_epilogue_cluster(const ConvParams &g, uint8
     }
     if (!seen) return false;
 #pragma unroll 1
-    for (int idx = et; idx < mine * c4n; idx += 32 * kCvEpiWarps) {
-        const int rr = idx / c4n, c4 = idx - rr * c4n, nc = n0 + c4 * 4;
-        if (nc >= g.N) continue;
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int idx = et; idx < items; idx += 32 * kCvEpiWarps) {
+        const int nc = n0 + c4 * 4;
+        const size_t px = (size_t)(m0 + r0 + rr);
+        int rn = rr + step_r, cn = c4 + step_c;
+        if (cn >= c4n) { cn -= c4n; ++rn; }
+        uint2 next = make_uint2(0u, 0u);
+        if (idx + 32 * kCvEpiWarps < items && n0 + cn * 4 < g.N) next = conv_skip4(g, n0 + cn * 4, (size_t)(m0 + r0 + rn));
+        if (nc < g.N) {
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-        for (int s = 0; s < g.ksplit; ++s) {
-            const float4 x = ld_shared_f4(buf + (uint32_t)(s * per + rr) * pitch + (uint32_t)c4 * 16u);
-            a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+            for (int s = 0; s < g.ksplit; ++s) {
+                const float4 x = ld_shared_f4(s == t.ks ? sbase + (uint32_t)(r0 + rr) * pitch + (uint32_t)c4 * 16u : buf + (uint32_t)(s * per + rr) * pitch + (uint32_t)c4 * 16u);
+                a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+            }
+            conv_finish_store4(g, a, ld_shared_f4(bias_s + (uint32_t)nc * 4u), nc, px, sk);
         }
-        conv_finish_store4(g, a, ld_shared_f4(bias_s + (uint32_t)nc * 4u), nc, (size_t)(m0 + r0 + rr));
+        rr = rn; c4 = cn; sk = next;
     }
     return true;
 }
@@ -694,7 +716,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
         // (a lane per barrier: one thread takes half a microsecond for all of them)
         constexpr int acce = 2 * kCvMaxStages + 2, first_skip = 2 * kCvMaxStages + 8, n_bars = kEpi == CE_SKIP ? first_skip + kMaxSkipSlots * kCvEpiWarps : first_skip + 1;
         for (int i = lane; i < n_bars; i += 32)
-            mbar_init(bar + 8u * i, i < kCvMaxStages ? (g.b_resident ? 1u : 2u) : i == acce || i == acce + 1 ? kCvEpiWarps : kEpi == CE_CLUSTER && i == first_skip ? kCvEpiWarps * g.ksplit : 1u);
+            mbar_init(bar + 8u * i, i < kCvMaxStages ? (g.b_resident ? 1u : 2u) : i == acce || i == acce + 1 ? kCvEpiWarps : 1u);
         if (lane == 0) fail_flag[0] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA0) : "memory");
