@@ -210,54 +210,72 @@ f32_chain_kernel(const F32ChainParams p) {
     const int rp = p.pool_stride * p.hp, mp = p.halo_h * rp;      // pitches of a middle row and of a middle channel
     float *s_in = f32_smem;                                       // [C][max_ih][iwp]
     float *s_mid = s_in + p.C * max_ih * p.iwp;                   // [mpad][halo_h][pool_stride][hp]
-    float *s_w1 = s_mid + p.mpad * mp;                            // [C][k][k][mpad]
     const int kper = p.K2 / p.parts_outc, kperp = (kper + 7) & ~7;
+    float *s_b1 = s_mid + p.mpad * mp;                            // [mpad]
+    float *s_b2 = s_b1 + p.mpad;                                  // [kperp], the part's slice
+    float *s_w1 = s_b2 + kperp;                                   // [C][k][k][mpad]
     float *s_w2 = s_w1 + p.C * p.k * p.k * p.mpad;               // [Cmid][kperp], the part's slice
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (kWS) {
         const int n4 = p.C * p.k * p.k * p.mpad / 4;
         for (int i = threadIdx.x; i < n4; i += T) cp_async16_f32(s_w1 + 4 * i, p.w1 + 4 * i);
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");      // (the image may be the predecessor's result)
-    int cur_part = -1;
+    for (int i = threadIdx.x; i < p.mpad; i += T) s_b1[i] = i < p.Cmid ? __ldg(p.b1 + i) : 0.0f;
     const int total = p.N * p.parts_outc * p.tiles_h * p.tiles_w;
-    for (int cta0 = blockIdx.x; cta0 < total; cta0 += gridDim.x) {
-        int cta = cta0;
+    struct Tile { int n, part, py0, px0, th, tw, rh, rw, ih; };
+    auto tile_of = [&](int cta) {
+        Tile t;
         const int tx = cta % p.tiles_w; cta /= p.tiles_w;
         const int ty = cta % p.tiles_h; cta /= p.tiles_h;
-        const int part = cta % p.parts_outc, n = cta / p.parts_outc;
+        t.part = cta % p.parts_outc; t.n = cta / p.parts_outc;
         // pool tile -> stage-1 patch -> input patch
-        const int py0 = ty * p.tile_h, px0 = tx * p.tile_w;
-        const int th = min(p.tile_h, p.PP - py0), tw = min(p.tile_w, p.PQ - px0);
-        const int rh = (th - 1) * p.pool_stride + p.pool_k, rw = (tw - 1) * p.pool_stride + p.pool_k;
-        const int ih = (rh - 1) * p.stride + p.k;
-        const int i0 = py0 * p.pool_stride * p.stride - p.pad, j0 = px0 * p.pool_stride * p.stride - p.pad;      // may be negative
-        if (rh > p.halo_h || rw > p.halo_w || ih > max_ih) {
+        t.py0 = ty * p.tile_h; t.px0 = tx * p.tile_w;
+        t.th = min(p.tile_h, p.PP - t.py0); t.tw = min(p.tile_w, p.PQ - t.px0);
+        t.rh = (t.th - 1) * p.pool_stride + p.pool_k; t.rw = (t.tw - 1) * p.pool_stride + p.pool_k;
+        t.ih = (t.rh - 1) * p.stride + p.k;
+        return t;
+    };
+    // A tile's input patch, asked for: 8, 16 or 32 lanes along a row, as many rows of a (channel, row) walk at once as that
+    // leaves.  (With a warp and two divisions per row the requests of a 32-channel patch took 11 thousand cycles, of a
+    // 16-channel one of 4 x 8 elements 4200.)
+    auto ask_patch = [&](const Tile &t) {
+        const int lr = p.iwp <= 8 ? 3 : p.iwp <= 16 ? 4 : 5, rows = T >> lr, lane = threadIdx.x & ((1 << lr) - 1);
+        const int i0 = t.py0 * p.pool_stride * p.stride - p.pad, j0 = t.px0 * p.pool_stride * p.stride - p.pad;      // may be negative
+        int a = threadIdx.x >> lr, c = 0;
+        while (a >= t.ih) { a -= t.ih; ++c; }
+        const float *img = p.x + (size_t)t.n * p.C * p.H * p.W;
+        for (; c < p.C;) {
+            const int gy = i0 + a;
+            const bool row_in = gy >= 0 && gy < p.H;
+            const float *src = img + ((size_t)c * p.H + (row_in ? gy : 0)) * p.W;
+            float *dst = s_in + (c * max_ih + a) * p.iwp;
+            for (int b = lane; b < p.iwp; b += 1 << lr) {
+                const int gx = j0 + b;
+                const bool live = row_in && gx >= 0 && gx < p.W;
+                cp_async4(dst + b, live ? src + gx : p.x, live);
+            }
+            a += rows;
+            while (a >= t.ih) { a -= t.ih; ++c; }
+        }
+    };
+    int cur_part = -1;
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // (the image may be the predecessor's result)
+    if ((int)blockIdx.x < total) ask_patch(tile_of(blockIdx.x));
+    for (int cta = blockIdx.x; cta < total; cta += gridDim.x) {
+        const Tile tile = tile_of(cta);
+        const int n = tile.n, part = tile.part, py0 = tile.py0, px0 = tile.px0, th = tile.th, tw = tile.tw, rh = tile.rh, rw = tile.rw;
+        if (rh > p.halo_h || rw > p.halo_w || tile.ih > max_ih) {
             if (threadIdx.x == 0) atomicCAS(p.status, 0u, 0x80000000u | 10u);
+            asm volatile("cp.async.wait_all;" ::: "memory");
             return;
         }
-        {
-            // a warp per (channel, row): lanes along the row
-            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = T >> 5;
-            for (int cr = warp; cr < p.C * ih; cr += warps) {
-                const int c = cr / ih, a = cr - c * ih, gy = i0 + a;
-                const bool row_in = gy >= 0 && gy < p.H;
-                const float *src = p.x + (((size_t)n * p.C + c) * p.H + (row_in ? gy : 0)) * p.W;
-                float *dst = s_in + (c * max_ih + a) * p.iwp;
-                for (int b = lane; b < p.iwp; b += 32) {
-                    const int gx = j0 + b;
-                    const bool live = row_in && gx >= 0 && gx < p.W;
-                    cp_async4(dst + b, live ? src + gx : p.x, live);
-                }
-            }
-        }
         const float *w2 = p.w2 + (size_t)part * p.Cmid * kperp;
-        if (kWS && part != cur_part) {
+        if (part != cur_part) {
             cur_part = part;
-            for (int i = threadIdx.x; i < p.Cmid * kperp / 4; i += T) cp_async16_f32(s_w2 + 4 * i, w2 + 4 * i);
+            if (kWS) for (int i = threadIdx.x; i < p.Cmid * kperp / 4; i += T) cp_async16_f32(s_w2 + 4 * i, w2 + 4 * i);
+            for (int i = threadIdx.x; i < kperp; i += T) s_b2[i] = i < kper ? __ldg(p.b2 + part * kper + i) : 0.0f;
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         // stage 1
         {
@@ -320,7 +338,7 @@ f32_chain_kernel(const F32ChainParams p) {
 #pragma unroll
                 for (int i = 0; i < TM / 2; ++i) {
                     const int m = mg * TM + 2 * i;
-                    const float b0 = m < p.Cmid ? __ldg(p.b1 + m) : 0.0f, b1 = m + 1 < p.Cmid ? __ldg(p.b1 + m + 1) : 0.0f;
+                    const float b0 = s_b1[m], b1 = s_b1[m + 1];
                     float *o = s_mid + m * mp + a * rp;
 #pragma unroll
                     for (int j = 0; j < TP; ++j) {
@@ -334,6 +352,8 @@ f32_chain_kernel(const F32ChainParams p) {
             }
         }
         __syncthreads();
+        // the next tile's patch arrives while this tile's second stage runs
+        if (cta + (int)gridDim.x < total) ask_patch(tile_of(cta + gridDim.x));
         // stage 2 + pool
         if (p.pool_k == 2) {
             // a thread takes TM channels of one pool output: the window's four pixels are its pixel tile
@@ -352,8 +372,25 @@ f32_chain_kernel(const F32ChainParams p) {
                 for (int i = 0; i < TM / 2; ++i)
 #pragma unroll
                     for (int d = 0; d < 4; ++d) acc[i][d] = make_float2(0.0f, 0.0f);
+                int m = 0;
+                if (TP == 1) {
+                    // (all of eight channels' reads before their products, as in stage 1)
+                    for (; m + 8 <= p.Cmid; m += 8) {
+                        float2 w[8][TM / 2];
+                        float xs[8][4];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            f32_load_w<TM>(w[i], wp + i * kperp);
+#pragma unroll
+                            for (int d = 0; d < 4; ++d) xs[i][d] = src[d][(m + i) * mp];
+                        }
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) f32_fma<TM, 4>(acc, w[i], xs[i]);
+                        wp += 8 * kperp;
+                    }
+                }
 #pragma unroll 4
-                for (int m = 0; m < p.Cmid; ++m) {
+                for (; m < p.Cmid; ++m) {
                     float2 w[TM / 2];
                     float xs[4];
                     f32_load_w<TM>(w, wp);
@@ -365,7 +402,7 @@ f32_chain_kernel(const F32ChainParams p) {
 #pragma unroll
                 for (int i = 0; i < TM / 2; ++i) {
                     const int kl = kg * TM + 2 * i;
-                    const float bx = kl < kper ? __ldg(p.b2 + kk0 + 2 * i) : 0.0f, by = kl + 1 < kper ? __ldg(p.b2 + kk0 + 2 * i + 1) : 0.0f;
+                    const float bx = s_b2[kl], by = s_b2[kl + 1];
                     const float pool0 = p.pool_kind == 0 ? -INFINITY : 0.0f;
                     float2 res = make_float2(pool0, pool0);
 #pragma unroll
@@ -390,8 +427,7 @@ f32_chain_kernel(const F32ChainParams p) {
                 float2 res[TM / 2][TP], bias[TM / 2];
 #pragma unroll
                 for (int i = 0; i < TM / 2; ++i) {
-                    bias[i].x = kg * TM + 2 * i < kper ? __ldg(p.b2 + kk0 + 2 * i) : 0.0f;
-                    bias[i].y = kg * TM + 2 * i + 1 < kper ? __ldg(p.b2 + kk0 + 2 * i + 1) : 0.0f;
+                    bias[i] = make_float2(s_b2[kg * TM + 2 * i], s_b2[kg * TM + 2 * i + 1]);
 #pragma unroll
                     for (int j = 0; j < TP; ++j) res[i][j] = make_float2(pool0, pool0);
                 }

@@ -629,7 +629,7 @@ struct Lower {
         auto mid_pitch = [&](int tw) { return round_up(tw, 4) + round_up((C.k - 1) / C.stride, 4); };
         auto smem_need = [&](int th, int tw, int po, bool ws) {
             const int rh = region(th), ih = (rh - 1) * A.stride + A.k;
-            size_t f = (size_t)A.cin * ih * patch_pitch(tw) + (size_t)mpad * rh * C.stride * mid_pitch(tw);
+            size_t f = (size_t)A.cin * ih * patch_pitch(tw) + (size_t)mpad * rh * C.stride * mid_pitch(tw) + mpad + round_up(B.cout / po, 8);
             if (ws) f += (size_t)taps * mpad + (size_t)A.cout * round_up(B.cout / po, 8);
             return 4 * f;
         };
