@@ -143,8 +143,7 @@ __global__ void f32_fc_kernel(const float *__restrict__ x, const float *__restri
 // ------------------------------------------------------------------------------------------------
 // Linked chain ConvX(+act) -> Conv1x1(+act) -> pool (Table 1), a CTA per (image, outC part, pool tile), walking over
 // them when there are more than fit.
-//   stage 0: the input patch the tile needs goes to shared memory (cp.async, zeros outside the image and in the padding of
-//            the row pitch)
+//   stage 0: the input patch the tile needs goes to shared memory (zeros outside the image and in the padding of the row pitch)
 //   stage 1: ConvX on the patch -> shared memory [Cmid][row][column % pool_stride][column / pool_stride], so that the
 //            outputs of one pool tap are adjacent: the order stage 2 reads
 //   stage 2: Conv1x1 over the CTA's slice of output channels, pooled in registers
@@ -235,32 +234,55 @@ f32_chain_kernel(const F32ChainParams p) {
         t.ih = (t.rh - 1) * p.stride + p.k;
         return t;
     };
-    // A tile's input patch, asked for: 8, 16 or 32 lanes along a row, as many rows of a (channel, row) walk at once as that
-    // leaves.  (With a warp and two divisions per row the requests of a 32-channel patch took 11 thousand cycles, of a
-    // 16-channel one of 4 x 8 elements 4200.)
-    auto ask_patch = [&](const Tile &t) {
-        const int lr = p.iwp <= 8 ? 3 : p.iwp <= 16 ? 4 : 5, rows = T >> lr, lane = threadIdx.x & ((1 << lr) - 1);
+    // A tile's input patch: 8, 16 or 32 lanes along a row, as many rows of a (channel, row) walk at once as that leaves.  (With a
+    // warp and two divisions per row the requests of a 32-channel patch of 8 x 40 took 11 thousand cycles, of a 16-channel one of
+    // 4 x 8 4200.)  Small tiles ask for theirs as asynchronous copies, which travel with the weights (one 32 x 32 map 9.1 us, by
+    // way of registers 9.9); a warp's 4-byte copies cost some 20 cycles each, 9200 for the larger patch, which large tiles
+    // therefore load through registers, up to eight loads of a thread under way (75 x 75, batch 32: 232 us, as copies 237).
+    auto load_patch = [&](const Tile &t) {
+        const int lr = p.iwp <= 8 ? 3 : p.iwp <= 16 ? 4 : 5, lanes = 1 << lr, rows = T >> lr;
         const int i0 = t.py0 * p.pool_stride * p.stride - p.pad, j0 = t.px0 * p.pool_stride * p.stride - p.pad;      // may be negative
-        int a = threadIdx.x >> lr, c = 0;
-        while (a >= t.ih) { a -= t.ih; ++c; }
         const float *img = p.x + (size_t)t.n * p.C * p.H * p.W;
-        for (; c < p.C;) {
-            const int gy = i0 + a;
-            const bool row_in = gy >= 0 && gy < p.H;
-            const float *src = img + ((size_t)c * p.H + (row_in ? gy : 0)) * p.W;
-            float *dst = s_in + (c * max_ih + a) * p.iwp;
-            for (int b = lane; b < p.iwp; b += 1 << lr) {
-                const int gx = j0 + b;
-                const bool live = row_in && gx >= 0 && gx < p.W;
-                cp_async4(dst + b, live ? src + gx : p.x, live);
-            }
-            a += rows;
+        for (int b = threadIdx.x & (lanes - 1); b < p.iwp; b += 2 * lanes) {
+            int a = threadIdx.x >> lr, c = 0;
             while (a >= t.ih) { a -= t.ih; ++c; }
+            const bool in0 = (unsigned)(j0 + b) < (unsigned)p.W, in1 = (unsigned)(j0 + b + lanes) < (unsigned)p.W, two = b + lanes < p.iwp;
+            while (TP == 1 && c < p.C) {
+                const int gy = i0 + a;
+                const bool row_in = (unsigned)gy < (unsigned)p.H;
+                const float *src = img + ((size_t)c * p.H + (row_in ? gy : 0)) * p.W + j0 + b;
+                float *dst = s_in + (c * max_ih + a) * p.iwp + b;
+                cp_async4(dst, row_in && in0 ? src : p.x, row_in && in0);
+                if (two) cp_async4(dst + lanes, row_in && in1 ? src + lanes : p.x, row_in && in1);
+                a += rows;
+                while (a >= t.ih) { a -= t.ih; ++c; }
+            }
+            while (TP != 1 && c < p.C) {
+                float v[4][2];
+                int d[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int gy = i0 + a;
+                    const bool row_in = c < p.C && (unsigned)gy < (unsigned)p.H;
+                    const float *src = img + ((size_t)c * p.H + gy) * p.W + j0 + b;
+                    v[i][0] = row_in && in0 ? __ldg(src) : 0.0f;
+                    v[i][1] = row_in && in1 && two ? __ldg(src + lanes) : 0.0f;
+                    d[i] = c < p.C ? (c * max_ih + a) * p.iwp + b : -1;
+                    a += rows;
+                    while (a >= t.ih) { a -= t.ih; ++c; }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (d[i] >= 0) {
+                        s_in[d[i]] = v[i][0];
+                        if (two) s_in[d[i] + lanes] = v[i][1];
+                    }
+            }
         }
     };
     int cur_part = -1;
     asm volatile("griddepcontrol.wait;" ::: "memory");      // (the image may be the predecessor's result)
-    if ((int)blockIdx.x < total) ask_patch(tile_of(blockIdx.x));
+    if ((int)blockIdx.x < total) load_patch(tile_of(blockIdx.x));
     for (int cta = blockIdx.x; cta < total; cta += gridDim.x) {
         const Tile tile = tile_of(cta);
         const int n = tile.n, part = tile.part, py0 = tile.py0, px0 = tile.px0, th = tile.th, tw = tile.tw, rh = tile.rh, rw = tile.rw;
@@ -352,8 +374,8 @@ f32_chain_kernel(const F32ChainParams p) {
             }
         }
         __syncthreads();
-        // the next tile's patch arrives while this tile's second stage runs
-        if (cta + (int)gridDim.x < total) ask_patch(tile_of(cta + gridDim.x));
+        // (the patch is free from here on)
+        if (cta + (int)gridDim.x < total) load_patch(tile_of(cta + gridDim.x));
         // stage 2 + pool
         if (p.pool_k == 2) {
             // a thread takes TM channels of one pool output: the window's four pixels are its pixel tile
@@ -373,30 +395,29 @@ f32_chain_kernel(const F32ChainParams p) {
 #pragma unroll
                     for (int d = 0; d < 4; ++d) acc[i][d] = make_float2(0.0f, 0.0f);
                 int m = 0;
-                if (TP == 1) {
-                    // (all of eight channels' reads before their products, as in stage 1)
-                    for (; m + 8 <= p.Cmid; m += 8) {
-                        float2 w[8][TM / 2];
-                        float xs[8][4];
+                // (the reads of several channels before their products, as in stage 1)
+                constexpr int kAhead = TP == 1 ? 8 : 2;
+                for (; m + kAhead <= p.Cmid; m += kAhead) {
+                    float2 w[kAhead][TM / 2];
+                    float xs[kAhead][4];
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            f32_load_w<TM>(w[i], wp + i * kperp);
+                    for (int i = 0; i < kAhead; ++i) {
+                        f32_load_w<TM>(w[i], wp + i * kperp);
 #pragma unroll
-                            for (int d = 0; d < 4; ++d) xs[i][d] = src[d][(m + i) * mp];
-                        }
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) f32_fma<TM, 4>(acc, w[i], xs[i]);
-                        wp += 8 * kperp;
+                        for (int d = 0; d < 4; ++d) { xs[i][d] = *src[d]; src[d] += mp; }
                     }
+#pragma unroll
+                    for (int i = 0; i < kAhead; ++i) f32_fma<TM, 4>(acc, w[i], xs[i]);
+                    wp += kAhead * kperp;
                 }
-#pragma unroll 4
+#pragma unroll 1
                 for (; m < p.Cmid; ++m) {
                     float2 w[TM / 2];
                     float xs[4];
                     f32_load_w<TM>(w, wp);
                     wp += kperp;
 #pragma unroll
-                    for (int d = 0; d < 4; ++d) xs[d] = src[d][m * mp];
+                    for (int d = 0; d < 4; ++d) { xs[d] = *src[d]; src[d] += mp; }
                     f32_fma<TM, 4>(acc, w, xs);
                 }
 #pragma unroll
