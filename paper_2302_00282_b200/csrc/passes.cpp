@@ -777,6 +777,12 @@ struct Lower {
         }
         const int rows = pooln ? L.PP : L.P, cols = pooln ? L.PQ : L.Q;
         L.st_pairs = k / 2 * C + (k % 2 ? (C + 1) / 2 : 0);
+        // Rows that are whole 16-byte pieces travel by bulk copies, several per producer warp under way (strides 1 and 2): a slot
+        // holds a row between zeros for the padding, and the region starts with a row of zeros.
+        const int es = src.io_dtype == XENOS_DTYPE_F32 ? 4 : 2;
+        const bool by_rows = src.w * es % 16 == 0 && src.w * es <= 4096 && (S == 1 || L.st_vec);
+        L.st_raw_lead = round_up((M.pad + L.st_lead) * es, 16);
+        L.st_raw_stride = L.st_raw_lead + src.w * es + round_up(M.pad * es, 16);
         const int wbytes = L.st_pairs * 2 * L.tile_n * 16, pc = L.tile_n <= 16 ? 1 : L.tile_n <= 32 ? 2 : 3;
         const int cap = std::min(g.hw.smem_bytes_per_cta, 227 * 1024) - 1024 - 512;
         // (a producer warp makes at most 128 lanes' worth of a row: two columns each, or one for strides above 2)
@@ -789,16 +795,26 @@ struct Lower {
             if (width > most) return false;
             L.st_qp = round_up(width, 8);
             const int row = C * L.st_qp * 16, stage = pooln ? 2 * width << (4 + pc) : 0;
-            const int base = wbytes + 2048 + 256 + (int)align_up((size_t)stage, 128);
-            for (int D = 6; D >= 2; --D) {
-                L.st_slots = (D - 1) * std::min(S, k) + k;
-                if ((L.st_slots + 1) * row + base > cap) continue;
-                L.hstages = D;
-                L.off_b = (int)align_up((size_t)(L.st_slots + 1) * row + 2048, 128);       // (zeros of one chunk; a tile's last rows read past its pieces)
+            const int base = wbytes + 2048 + 256 + 512 + (int)align_up((size_t)stage, 128);
+            // four rows of a warp under way before more steps of the ring; two where four do not fit; else loads into registers
+            auto deepest = [&](int raw) {
+                const int rbytes = raw ? (int)align_up((size_t)(1 + 7 * raw) * L.st_raw_stride, 128) : 0;
+                for (int D = 6; D >= 2; --D) {
+                    L.st_slots = (D - 1) * std::min(S, k) + k;
+                    if ((L.st_slots + 1) * row + rbytes + base <= cap) { L.hstages = D; L.st_raw = raw; return rbytes; }
+                }
+                return -1;
+            };
+            int rbytes = -1;
+            if (by_rows) { rbytes = deepest(4); if (rbytes < 0) rbytes = deepest(2); }
+            if (rbytes < 0) rbytes = deepest(0);
+            if (rbytes >= 0) {
+                L.off_raw = (int)align_up((size_t)(L.st_slots + 1) * row + 2048, 128);       // (zeros of one chunk; a tile's last rows read past its pieces)
+                L.off_b = L.off_raw + rbytes;
                 L.off_bias = L.off_b + wbytes;
                 L.off_stg = L.off_bias + 256;
                 L.off_bar = (int)align_up((size_t)(L.off_stg + stage), 128);
-                L.smem_bytes = L.off_bar + 512 + 1024;
+                L.smem_bytes = L.off_bar + 768 + 1024;
                 return true;
             }
             return false;

@@ -242,20 +242,21 @@ static DwKernel dw_kernel_of(int stride, int br) {
 }
 // Convolution of an image: how its rows are loaded, the image's type, with or without a pool.
 using StemKernel = void (*)(xk::StemParams);
-template <int kMode>
+template <int kMode, bool kRows>
 static StemKernel stem_kernel_of(bool f32, bool pool) {
-    return f32 ? (pool ? xk::stem_tc_kernel<kMode, true, true> : xk::stem_tc_kernel<kMode, true, false>)
-               : (pool ? xk::stem_tc_kernel<kMode, false, true> : xk::stem_tc_kernel<kMode, false, false>);
+    return f32 ? (pool ? xk::stem_tc_kernel<kMode, true, true, kRows> : xk::stem_tc_kernel<kMode, true, false, kRows>)
+               : (pool ? xk::stem_tc_kernel<kMode, false, true, kRows> : xk::stem_tc_kernel<kMode, false, false, kRows>);
 }
-static StemKernel stem_kernel(int mode, bool f32, bool pool) {
-    return mode == xk::SM_S1 ? stem_kernel_of<xk::SM_S1>(f32, pool) : mode == xk::SM_S2 ? stem_kernel_of<xk::SM_S2>(f32, pool)
-         : mode == xk::SM_S2X ? stem_kernel_of<xk::SM_S2X>(f32, pool) : stem_kernel_of<xk::SM_ANY>(f32, pool);
+static StemKernel stem_kernel(int mode, bool f32, bool pool, bool rows) {
+    if (rows) return mode == xk::SM_S1 ? stem_kernel_of<xk::SM_S1, true>(f32, pool) : stem_kernel_of<xk::SM_S2, true>(f32, pool);
+    return mode == xk::SM_S1 ? stem_kernel_of<xk::SM_S1, false>(f32, pool) : mode == xk::SM_S2 ? stem_kernel_of<xk::SM_S2, false>(f32, pool)
+         : mode == xk::SM_S2X ? stem_kernel_of<xk::SM_S2X, false>(f32, pool) : stem_kernel_of<xk::SM_ANY, false>(f32, pool);
 }
 
 // Whole groups of elements where rows are made of them (images are 16-byte aligned); else element by element.
 static StemKernel stem_kernel(const Launch &L) {
     const int mode = L.stride == 2 ? (L.st_vec ? xk::SM_S2 : xk::SM_S2X) : L.stride == 1 ? xk::SM_S1 : xk::SM_ANY;
-    return stem_kernel(mode, L.seg[0].src_dtype == XENOS_DTYPE_F32, L.epi == EPI_POOL);
+    return stem_kernel(mode, L.seg[0].src_dtype == XENOS_DTYPE_F32, L.epi == EPI_POOL, L.st_raw > 0);
 }
 
 static auto *conv_kernel(const Launch &L) {
@@ -673,6 +674,7 @@ static xenos_status_t issue_pass(Graph &g, int batch, const void *const *in, voi
                 p.act = L.act; p.out_ctot = L.out_ctot; p.out_coff = L.out_coff;
                 p.idesc = make_idesc(L.tile_n);
                 p.off_w = L.off_b; p.off_bias = L.off_bias; p.off_stage = L.off_stg; p.stage_bytes = (L.off_bar - L.off_stg) / 2 & ~15; p.off_bar = L.off_bar;
+                p.raw_slots = L.st_raw; p.raw_stride = L.st_raw_stride; p.raw_lead = L.st_raw_lead; p.off_raw = L.off_raw;
                 p.launch_id = (int)li;
                 const int gx = std::min(p.units, std::max(1, sms / L.n_tiles));
                 le = to.pdl(stem_kernel(L), dim3(gx, L.n_tiles), L.block, L.smem_bytes, p);

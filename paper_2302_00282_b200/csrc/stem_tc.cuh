@@ -45,8 +45,12 @@ struct StemParams {
     int act, out_ctot, out_coff;
     uint32_t idesc;
     int off_w, off_bias, off_stage, stage_bytes, off_bar;
+    int raw_slots, raw_stride, raw_lead, off_raw;      // image rows on their way: slots per producer warp, bytes of a slot and of the zeros in front
     int launch_id;
 };
+constexpr int kStMaxRaw = 6;
+constexpr int kStRawBar = 2 * kStMaxSteps + 2 * kStMaxAcc + 2;      // barriers of the row slots, kStMaxRaw per producer warp
+static_assert(8 * (kStRawBar + kStMaxRaw * kStProdWarps) <= 768, "barriers exceed their place");
 
 struct StemRun { int n, out0, out1, row, len, p0, p1, base, width; };
 
@@ -248,6 +252,143 @@ __device__ __forceinline__ bool stem_produce(const StemParams &g, uint32_t sbase
             start = false;
             have = d < k;
             if (have) load(ih0 + d);
+        }
+    }
+    return true;
+}
+
+// The rows of a producer warp in the order it makes them.
+template <bool kPool>
+struct StemCursor {
+    int u, n, p, p1, d, ih0;
+    bool more;
+    __device__ __forceinline__ void run(const StemParams &g, int u1, int j0, int stride, int pad) {
+        const StemRun r = stem_run<kPool>(g, u, u1);
+        u += r.len; n = r.n; p = r.p0; p1 = r.p1; d = j0; ih0 = p * stride - pad;
+    }
+    __device__ __forceinline__ void next(const StemParams &g, int u1, int j0, int rstep, int k, int nr, int stride, int pad) {
+        d += rstep;
+        while (d >= k) {
+            if (++p < p1) { ih0 += stride; d = j0 < nr ? k - nr + j0 : k; }
+            else if (u < u1) run(g, u1, j0, stride, pad);
+            else { more = false; return; }
+        }
+    }
+};
+
+// The same where rows are whole 16-byte pieces of memory: a warp keeps raw_slots of its rows on their way by bulk copies and
+// reads them from shared memory, between zeros for the padding (a row outside the image is a slot of zeros).  With the loads of
+// one row ahead in registers every step cost the latency of a load from memory, 1000 to 1900 cycles.
+template <int kMode, bool kF32>
+__device__ __forceinline__ void stem_read(uint32_t (&raw)[4][StemForm<kMode, kF32>::words], uint32_t s, int passes, int stride) {
+    using F = StemForm<kMode, kF32>;
+    constexpr int es = kF32 ? 4 : 2;
+    const int S = F::S ? F::S : stride;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (i >= passes) break;
+        const uint32_t a = s + (uint32_t)(32 * F::run * S * i * es);
+        uint32_t *r = raw[i];
+        auto ld2 = [](uint32_t *d, uint32_t at) { asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(d[0]), "=r"(d[1]) : "r"(at)); };
+        if (kMode == SM_S2 && kF32) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[4 * j]), "=r"(r[4 * j + 1]), "=r"(r[4 * j + 2]), "=r"(r[4 * j + 3]) : "r"(a + 16u * j));
+            ld2(r + F::words - 2, a + 32u);
+        } else if (kMode == SM_S2) {
+            ld2(r, a);
+            ld2(r + 2, a + 8u);
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(r[4]) : "r"(a + 16u));
+        } else {
+            r[F::words - 1] = 0u;
+            r[F::words - 2] = 0u;
+#pragma unroll
+            for (int j = 0; j < F::elems; ++j) {
+                if (kF32) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(r[j % F::words]) : "r"(a + 4u * j));
+                else {
+                    unsigned short h;
+                    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(h) : "r"(a + 2u * j));
+                    r[j % F::words] = h;
+                }
+            }
+        }
+    }
+}
+template <int kMode, bool kF32, bool kPool>
+__device__ __forceinline__ bool stem_produce_rows(const StemParams &g, uint32_t sbase, uint32_t bar, int u0, int u1, int w, int lane) {
+    using F = StemForm<kMode, kF32>;
+    constexpr int es = kF32 ? 4 : 2;
+    const int C = in_reg(g.C), k = in_reg(g.k), stride = F::S ? F::S : in_reg(g.stride), R = in_reg(g.R), D = in_reg(g.D), H = in_reg(g.H);
+    const int pad = in_reg(g.pad), rstep = kStProdWarps / C, nr = min(stride, k);
+    int j0 = w / C;
+    const int c = w - j0 * C;
+    if (j0 >= rstep) j0 = k;                              // a warp without rows only keeps the steps' counts
+    const uint32_t slot_bytes = in_reg((uint32_t)(g.qp * C * 16)), ring = in_reg(sbase + (uint32_t)((c * g.qp + F::run * lane) * 16)), wrap = (uint32_t)R * slot_bytes;
+    const uint32_t row_bytes = in_reg((uint32_t)(g.W * es)), raw_stride = in_reg((uint32_t)g.raw_stride), lead = (uint32_t)g.raw_lead;
+    const uint32_t zeros = sbase + (uint32_t)g.off_raw + lead;                                    // slot 0 of the region: a row of zeros
+    const uint32_t mine = zeros + raw_stride * (uint32_t)(1 + w * g.raw_slots), mine_end = mine + raw_stride * (uint32_t)g.raw_slots;
+    const uint32_t bar0 = bar + 8u * (uint32_t)(kStRawBar + kStMaxRaw * w);
+    auto both = [&](int j) {                              // which of elements j, j + 1 of a piece the window takes
+        const uint32_t x = (unsigned)(j - g.lead) < (unsigned)k, y = (unsigned)(j + 1 - g.lead) < (unsigned)k;
+        return in_reg(x * 0xffffu | y * 0xffff0000u);
+    };
+    const uint4 in_window = make_uint4(both(0), both(2), both(4), both(6));
+    StemCursor<kPool> ahead;
+    ahead.u = u0; ahead.more = u0 < u1 && j0 < k;
+    if (ahead.more) ahead.run(g, u1, j0, stride, pad);
+    uint32_t raw_at = mine, raw_bar = bar0, raw_ph = 0u;      // the slot that is read next; it is filled again behind the read
+    auto ask = [&](uint32_t at, uint32_t b) {
+        while (ahead.more && (unsigned)(ahead.ih0 + ahead.d) >= (unsigned)H) ahead.next(g, u1, j0, rstep, k, nr, stride, pad);
+        if (!ahead.more) return;
+        const uint8_t *src = reinterpret_cast<const uint8_t *>(g.src) + ((size_t)(ahead.n * C + c) * H + (ahead.ih0 + ahead.d)) * row_bytes;
+        if (lane == 0) {
+            mbar_arrive_expect_tx(b, row_bytes);
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(at), "l"(src), "r"(row_bytes), "r"(b) : "memory");
+        }
+        __syncwarp();
+        ahead.next(g, u1, j0, rstep, k, nr, stride, pad);
+    };
+    for (int i = 0; i < g.raw_slots; ++i) ask(mine + raw_stride * (uint32_t)i, bar0 + 8u * i);
+    uint32_t raw[4][F::words];
+    int t = 0, sl = 0, slot = 0;                          // step, its barrier, ring slot of its window row 0
+    uint32_t ph = 0;
+#pragma unroll 1
+    for (int u = u0; u < u1;) {
+        const StemRun r = stem_run<kPool>(g, u, u1);
+        u += r.len;
+        const int e = ((r.base + F::run * lane) * stride - pad - g.lead) * es;
+        const int lanes = (r.width + F::run - 1) / F::run, passes = (lanes + 31) >> 5, left = lanes - lane;
+        int d = j0, ih0 = r.p0 * stride - pad;
+#pragma unroll 1
+        for (int p = r.p0; p < r.p1; ++p, ih0 += stride) {
+            // (the slots of a step's rows are free when the step D before it has been multiplied; the first rows of another image
+            // wait for all of the last one's)
+            if (p == r.p0 && t > 0) {
+                if (!mbar_wait(bar + 8u * (kStMaxSteps + (sl ? sl - 1 : D - 1)), sl ? ph : ph ^ 1u)) return false;
+            } else if (t >= D) {
+                if (!mbar_wait(bar + 8u * (kStMaxSteps + sl), ph ^ 1u)) return false;
+            }
+#pragma unroll 1
+            for (; d < k; d += rstep) {
+                const bool in = (unsigned)(ih0 + d) < (unsigned)H;
+                if (in && !mbar_wait(raw_bar, raw_ph)) return false;
+                stem_read<kMode, kF32>(raw, (in ? raw_at : zeros) + (uint32_t)e, passes, stride);
+                int s = slot + d;
+                if (s >= R) s -= R;
+                stem_store<kMode, kF32>(raw, ring + (uint32_t)s * slot_bytes, s == 0 ? wrap : 0u, left, passes, lane, in_window);
+                if (in) {
+                    __syncwarp();
+                    ask(raw_at, raw_bar);
+                    raw_at += raw_stride; raw_bar += 8u;
+                    if (raw_at == mine_end) { raw_at = mine; raw_bar = bar0; raw_ph ^= 1u; }
+                }
+            }
+            warp_arrive(bar + 8u * sl, lane);
+            if (++sl == D) { sl = 0; ph ^= 1u; }
+            ++t;
+            slot += p + 1 == r.p1 ? k : nr;
+            if (slot >= R) slot -= R;
+            d = j0 < nr ? k - nr + j0 : k;
         }
     }
     return true;
@@ -507,7 +648,8 @@ __device__ __forceinline__ bool stem_epilogue_pool(const StemParams &g, uint32_t
     return ok;
 }
 
-template <int kMode, bool kF32, bool kPool>
+// kRows: image rows by bulk copies
+template <int kMode, bool kF32, bool kPool, bool kRows>
 __global__ void __launch_bounds__(kStThreads, 1)
 stem_tc_kernel(const __grid_constant__ StemParams g) {
     extern __shared__ uint8_t smem_raw[];
@@ -524,6 +666,7 @@ stem_tc_kernel(const __grid_constant__ StemParams g) {
             for (int s = 0; s < g.D; ++s) { mbar_init(bar + 8u * s, kStProdWarps); mbar_init(bar + 8u * (kStMaxSteps + s), 1); }
             mbar_init(bar + 8u * (2 * kStMaxSteps + 2 * kStMaxAcc), 1);
             for (int b = 0; b < g.nacc; ++b) { mbar_init(bar + 8u * (2 * kStMaxSteps + b), 1); mbar_init(bar + 8u * (2 * kStMaxSteps + kStMaxAcc + b), kStEpiWarps); }
+            if (kRows) for (int b = 0; b < kStMaxRaw * kStProdWarps; ++b) mbar_init(bar + 8u * (kStRawBar + b), 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             // the weights: parameters, which no earlier kernel writes
             const uint32_t bytes = (uint32_t)(g.npairs * 2 * g.tile_n * 16), wbar = bar + 8u * (2 * kStMaxSteps + 2 * kStMaxAcc);
@@ -537,6 +680,11 @@ stem_tc_kernel(const __grid_constant__ StemParams g) {
     } else {
         // (zeros of one chunk, 128 pieces, behind the ring)
         if (threadIdx.x < 128) st_shared16(sbase + (uint32_t)((g.R + 1) * g.qp * g.C * 16) + threadIdx.x * 16u, make_uint4(0u, 0u, 0u, 0u));
+        // (the row slots' zeros, before any copy into them)
+        if (kRows) {
+            for (int i = threadIdx.x; i < (1 + g.raw_slots * kStProdWarps) * g.raw_stride / 16; i += 32 * 15) st_shared16(sbase + (uint32_t)g.off_raw + i * 16u, make_uint4(0u, 0u, 0u, 0u));
+            fence_proxy_async();
+        }
         if ((int)threadIdx.x < g.tile_n) reinterpret_cast<float *>(sm + g.off_bias)[threadIdx.x] = __ldg(g.bias + blockIdx.y * g.tile_n + threadIdx.x);
     }
     tc_fence_before();
@@ -553,7 +701,8 @@ stem_tc_kernel(const __grid_constant__ StemParams g) {
         if (!ok && lane == 0) atomicCAS(g.status, 0u, gave_up | (5u << 8));
     } else if (warp < 15) {
         pdl_wait();
-        ok = stem_produce<kMode, kF32, kPool>(g, sbase, bar, u0, u1, warp - kStEpiWarps, lane);
+        ok = kRows ? stem_produce_rows<kMode, kF32, kPool>(g, sbase, bar, u0, u1, warp - kStEpiWarps, lane)
+                   : stem_produce<kMode, kF32, kPool>(g, sbase, bar, u0, u1, warp - kStEpiWarps, lane);
         if (!ok && lane == 0) atomicCAS(g.status, 0u, gave_up | (3u << 8));
     } else {
         if (elect_one()) {
