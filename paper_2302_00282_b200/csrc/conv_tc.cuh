@@ -132,20 +132,23 @@ __device__ __forceinline__ int conv_row0(const ConvParams &g, int mt) {
 __device__ __forceinline__ int in_reg(int x) { asm volatile("" : "+r"(x)); return x; }
 __device__ __forceinline__ uint32_t in_reg(uint32_t x) { asm volatile("" : "+r"(x)); return x; }
 
-// The ring as its issuing thread sees it: slot, phase, and the addresses of the slot's barrier and data.  Barriers
-// are asked as little and as early as possible (see mbar_test): `ready` is what is known of the slot at hand.
+// The ring as a thread that walks all of it sees it: the slot's barrier, data and phase; ready: what is known of its barrier,
+// which is asked as early as possible (see mbar_test).  No branches: a lone thread needs some eight cycles an instruction and
+// more for a branch.
 struct ConvRing {
-    int s, n, step;
-    uint32_t ph, fb, data, fb0, data0, ready;
+    uint32_t ph, fb, data, fb0, data0, fb_last, step, ready;
     __device__ __forceinline__ void init(const ConvParams &g, uint32_t sbase, uint32_t bar) {
-        s = 0; n = in_reg(g.stages); step = in_reg(g.stage_bytes); ph = 0; ready = 0;
-        fb = fb0 = bar; data = data0 = sbase;
+        step = in_reg((uint32_t)g.stage_bytes); ph = 0u; ready = 0u;
+        fb = fb0 = in_reg(bar); data = data0 = in_reg(sbase);
+        fb_last = in_reg(bar + 8u * (uint32_t)(g.stages - 1));
     }
     __device__ __forceinline__ uint32_t empty() const { return fb + 8u * kCvMaxStages; }
     __device__ __forceinline__ bool full() const { return ready || mbar_wait(fb, ph); }
     __device__ __forceinline__ void next() {
-        ++s; fb += 8u; data += (uint32_t)step;
-        if (s == n) { s = 0; ph ^= 1u; fb = fb0; data = data0; }
+        const bool wrap = fb == fb_last;
+        fb = wrap ? fb0 : fb + 8u;
+        data = wrap ? data0 : data + step;
+        ph ^= wrap ? 1u : 0u;
     }
 };
 
@@ -278,8 +281,9 @@ __device__ __forceinline__ bool conv_mma(const ConvParams &g, ConvRing &st, uint
         for (int kb = kb0; kb < kb1; ++kb) {
             const uint32_t a4 = 0x10000u | (st.data >> 4), used = st.empty();      // (shared addresses are below 2^18)
             if (!kRes) b4 = a4 + (kABytes >> 4);
-            int steps = 4;
-            if (++cb == cblocks) { cb = 0; steps = last; }
+            const bool end = ++cb == cblocks;
+            const int steps = end ? last : 4;
+            cb = end ? 0 : cb;
             if (!st.full()) return false;
             st.next();
             st.ready = umma_block(d_tmem, a_hi, a4, 2u, 4u, 6u, b_hi, b4, idesc, acc, steps, used, st.fb, st.ph);
@@ -780,7 +784,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                 ConvRing st;
                 st.init(g, sbase, bar);
                 const int total = in_reg(g.total);
-                int fresh = st.n;      // slots that nothing has been put in yet
+                int fresh = in_reg(g.stages);      // slots that nothing has been put in yet
 #pragma unroll 1
                 for (int ti = blockIdx.x; ti < total && ok; ti += gridDim.x) {
                     const ConvTile t = conv_tile(g, ti);
