@@ -48,6 +48,16 @@ def test_reduction_split_over_clusters(cin, hw, cout, k, parts_k, batch):
     assert gg.g.plan()["launches"][0]["ksplit"] == parts_k
 
 
+# stages of several 16- or 32-channel boxes, filled by two threads in turn: one stage, odd and even numbers of them, a last stage
+# with fewer boxes, several tiles per CTA, weights that stay and that are streamed, chunks of a split reduction
+@pytest.mark.parametrize("cin,h,w,cout,k,pad,batch,parts_k", [(8, 9, 5, 24, 2, 0, 1, 1), (16, 21, 23, 40, 5, 2, 3, 1), (32, 30, 31, 64, 3, 1, 40, 1), (24, 7, 7, 520, 7, 3, 2, 1),
+                                                             (16, 55, 55, 128, 3, 1, 7, 1), (32, 6, 6, 32, 5, 2, 2, 3)])
+def test_convolution_stages_of_several_boxes(cin, h, w, cout, k, pad, batch, parts_k):
+    spec = _spec((cin, h, w), lambda g: g.cbr("c", "input", cout, k, 1, pad))
+    check_bf16(f"boxes{(cin, h, w, cout, k, parts_k)}", spec, batch, in_mode="bf16_nhwc", images=[0, batch - 1],
+               splits=[("c", dict(parts_k=parts_k))] if parts_k > 1 else ())
+
+
 # middle tiles of 8 to 256 channels, one row to many tiles, output blocks that end inside 128 columns, with and without shortcut
 @pytest.mark.parametrize("cin,h,w,k,cmid,cout,add,batch", [(64, 1, 1, 1, 8, 8, False, 1), (64, 8, 16, 3, 64, 64, True, 1), (128, 3, 43, 1, 256, 136, False, 2),
                                                            (192, 5, 27, 3, 192, 192, True, 3), (64, 40, 40, 3, 40, 392, False, 13)])
@@ -76,6 +86,19 @@ def test_depthwise_pointwise_tiles(c, h, w, cout, st, gap, batch):
     assert gg.g.launch_count() == 1
 
 
+# tiles of 4 to 32 rows, whose operand slots are as short, with fewer and more channel blocks than the ring has slots, weights that
+# stay in shared memory and that are streamed, a last block of fewer channels; a tile's rows in all quarters of the accumulator
+@pytest.mark.parametrize("c,h,w,cout,st,gap,batch", [(576, 2, 3, 64, 1, False, 1), (1024, 2, 2, 72, 1, True, 1), (520, 3, 7, 512, 2, False, 2), (192, 1, 16, 1024, 1, False, 1),
+                                                     (512, 14, 14, 512, 1, False, 1), (256, 6, 20, 256, 1, False, 3), (968, 9, 9, 1024, 2, False, 4)])
+def test_depthwise_tiles_of_few_rows(c, h, w, cout, st, gap, batch):
+    def build(g):
+        y = g.cbr("pw", g.cbr("dw", "input", c, 3, st, 1, groups=c, act="relu6"), cout, 1, act="relu6")
+        if gap:
+            g.gap("gap", y)
+    _, _, gg = check_bf16(f"dw_rows{(c, h, w, cout, st, gap)}", _spec((c, h, w), build), batch, in_mode="bf16_nhwc")
+    assert gg.g.launch_count() == 1 and gg.g.plan()["launches"][0]["tile_rows"] <= 32
+
+
 # 1 to 7 channels, windows of 2 to 8, strides 1, 2 (rows of whole groups of four elements and not) and 3, several column blocks,
 # output channels that end inside a tile and in a second one; pools that overlap by one row, that do not, and over wide images
 @pytest.mark.parametrize("cin,h,w,cout,k,st,pad,pool,batch", [
@@ -92,6 +115,22 @@ def test_image_convolution(cin, h, w, cout, k, st, pad, pool, batch, in_mode):
     if not pool and k == 3 and cout <= 64 and batch <= 8:
         batch = 9          # (smaller batches of a 3 x 3 window run on the CUDA cores)
     _, _, gg = check_bf16(f"stem{(cin, h, w, cout, k, st, pad, pool)}{in_mode}", _spec((cin, h, w), build), batch, in_mode=in_mode, links=links)
+    assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
+
+
+# image rows by bulk copies (whole 16-byte pieces, up to 4096 bytes) and by loads: both sides of either limit, rows of padding above
+# and below, more rows of a producer than are under way, fewer rows than that, several images and column blocks
+@pytest.mark.parametrize("cin,h,w,cout,k,st,pad,pool,batch", [
+    (3, 9, 1024, 16, 3, 2, 1, None, 9), (3, 7, 1028, 16, 3, 2, 1, None, 9), (1, 5, 2048, 8, 7, 2, 3, None, 1), (1, 40, 8, 24, 5, 1, 2, None, 3), (1, 40, 12, 24, 5, 1, 2, None, 3),
+    (7, 33, 64, 40, 7, 2, 3, (3, 2, 1), 2), (2, 50, 24, 64, 4, 2, 1, (2, 2, 0), 20), (3, 3, 16, 8, 8, 1, 3, None, 30)])
+@pytest.mark.parametrize("in_mode", ["f32_nchw", "bf16_nchw"])
+def test_image_rows(cin, h, w, cout, k, st, pad, pool, batch, in_mode):
+    def build(g):
+        y = g.cbr("stem", "input", cout, k, st, pad)
+        if pool:
+            g.pool("mp", y, "maxpool", *pool)
+    _, _, gg = check_bf16(f"rows{(cin, h, w, cout, k, st, pad, pool)}{in_mode}", _spec((cin, h, w), build), batch, in_mode=in_mode,
+                          links=[["stem", "mp"]] if pool else None)
     assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
 
 
@@ -144,6 +183,20 @@ def test_fp32_chain_tiles(cin, hw, cmid, cout, k, st, pool, batch):
     y = gg.run(x)
     assert gg.g.launch_count() == 1 and not np.isnan(y).any()
     assert rel_err_fp32(y, interp.run_graph(spec, P, x)) <= FP32_TOL
+
+
+# input patches of 8, 16, 32 and more lanes a row, fewer and more rows than a walk covers at once, middle channels that are no
+# multiple of those read ahead, several tiles and parts per CTA
+@pytest.mark.parametrize("cin,h,w,cmid,cout,pool,batch", [(2, 9, 150, 7, 8, ("maxpool", 2, 2, 0), 1), (5, 75, 40, 17, 24, ("maxpool", 2, 2, 0), 16), (31, 64, 64, 33, 40, ("avgpool", 2, 2, 0), 12),
+                                                         (16, 12, 200, 9, 16, ("maxpool", 3, 3, 0), 9)])
+def test_fp32_chain_patches(cin, h, w, cmid, cout, pool, batch):
+    def build(g):
+        g.pool("mp", g.cbr("c1", g.cbr("c3", "input", cmid, 3, 1, 1), cout, 1), *pool)
+    spec = _spec((cin, h, w), build, "fp32")
+    P, x = graphs.make_params(spec), graphs.make_input(spec, batch)
+    gg = GpuGraph(spec, P, batch)
+    y = gg.run(x)
+    assert gg.g.launch_count() == 1 and rel_err_fp32(y, interp.run_graph(spec, P, x)) <= FP32_TOL
 
 
 # the recorded form of a pass: repeated calls, images that change in place, other buffers and batches in turn, a call inside the
