@@ -16,11 +16,12 @@
 //   warps 4-11  epilogue of tile i while tile i + 1 is multiplied: two warps per quarter of the accumulator's lanes take
 //               alternate column chunks: bias, activation [, + shortcut, activation], bf16, a swizzled 32-row box in
 //               shared memory, one bulk tensor store.  A shortcut tile arrives in the same boxes the result leaves from.
-// All roles run warp-uniformly and elect one lane per request: measured here, a copy request issued from inside an
-// `if (lane == 0)` branch with address divisions costs 535 cycles of that lane, 240 to 260 when elected and without divisions,
-// and an MMA 61 against 40-48 (M = 128, N <= 64; 64 at N = 128, 128 at N = 256, the pipe's own time).
-// What bounds it: L2 -> shared memory for A (16 KB per block at the measured 71-76 B per cycle and SM: about 220 cycles,
-// against 192 / 256 / 512 cycles of the tensor pipe for N = 64 / 128 / 256), and for 1x1 products HBM.
+// A role is one elected lane.  Measured: a request with its announcement takes that lane 50 to 120 cycles, the look at a barrier
+// 190 (mbar_test), other work some eight cycles an instruction; an MMA takes the pipe 40-48 cycles (M = 128, N <= 64; 64 at N =
+// 128, 128 at N = 256).  The copy engine brings 16 KB of A in 150 to 180 cycles alone and in 200 to 256 with all SMs at it.
+// What bounds it: at N = 64 the products' issue (some 260 cycles a block, 400 before umma_block and the early look at the ring)
+// and shared memory, which an MMA of N <= 128 reads at its full 128 B per cycle while the copies write; at N = 256 the tensor
+// pipe (550 of 512 cycles at 72 blocks of a 3 x 3 window over 512 channels); for 1x1 products HBM.
 //
 // Channels: C in (32, 64] and above uses 64-channel boxes (128-byte swizzle), C <= 32 and C <= 16 use boxes of 32 and 16
 // channels (64- and 32-byte swizzle; 2 or 4 taps share a stage), and MMA steps over channels beyond C are not issued.

@@ -13,9 +13,12 @@
 // slots of the rings are its own (ring sizes are multiples of G: a group meets every phase of its slots' barriers).  A
 // thread owns BR x 4 pixels of a channel pair; G is chosen so that a group covers a tile: small tiles have all their channel
 // blocks under way at once, large ones two, which hides the shared-memory latency of the stencil.
-// Bound: issue slots and the FMA pipe of the stencil (4 x 4 pixels: about 340 instructions of a warp for 1024 results, 12 per
-// cycle and SM).  MobileNet at batch 32: issue slots 59 % busy in the first chain, 37 to 56 % in the others, DRAM 3 to 21 %, tensor
-// pipe 2 to 21 %; the rest is boxes (see layout_dw) and waits between the roles.
+// Bound: issue slots (4 x 4 pixels: some 400 instructions of a warp for 1024 results; a result box some 120 per 32 columns; the
+// walk over a batch's tiles by all workers the rest of the first chain's 16.7 million), and at small batches the latencies of
+// one tile: window, stencil, products, box.  MobileNet at batch 32: issue slots 58 % busy in the first chain, 28 to 53 % in the
+// others.  A launch on 14 x 14 x 512 at batch 1 takes 5 to 6 us between its predecessor's end and its own, 5.8 to 7.2 before
+// operand slots became as short as the tile (all of a tile's blocks fit, so the stencils do not wait for the products), weights
+// stayed in shared memory and the products of a block were issued in one sequence (umma_block; 750 cycles a block before).
 #pragma once
 
 #include "pair_tc.cuh"
