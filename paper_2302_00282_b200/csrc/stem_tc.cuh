@@ -16,7 +16,7 @@
 //                  maximum over columns through a staged row
 //   warps 8..14  : image rows -> operand pieces
 //   warp 15      : issues the products; a convolution row is one accumulator per 128 columns
-// What bounds it: the producers, some 1300 cycles a step and warp for one row (reading and storing its pieces 400, asking for
+// What bounds it: the producers, some 1000 cycles a step and warp for one row (reading and storing its pieces 400, asking for
 // the row four ahead and the walk 600, the ring's barrier 200), then the products' thread, 900 a row of 128 columns and 3 x 3 taps;
 // the products themselves read 6 KB of shared memory each for 64 channels (48 cycles), 11 per 128 columns for a 7 x 7 window of
 // 3 channels.  MobileNet's stem at batch 32: 1500 cycles a row, 1750 with the rows loaded through registers one ahead.
@@ -339,16 +339,29 @@ __device__ __forceinline__ bool stem_produce_rows(const StemParams &g, uint32_t 
     ahead.u = u0; ahead.more = u0 < u1 && j0 < k;
     if (ahead.more) ahead.run(g, u1, j0, stride, pad);
     uint32_t raw_at = mine, raw_bar = bar0, raw_ph = 0u;      // the slot that is read next; it is filled again behind the read
+    // A row into a slot.  Behind the first step of a run a warp's rows of it lie a stride apart, one per step: `again` of them
+    // follow without another look at the walk (which made the request 700 cycles of a step).
+    const uint8_t *src = nullptr;
+    int again = 0;
     auto ask = [&](uint32_t at, uint32_t b) {
-        while (ahead.more && (unsigned)(ahead.ih0 + ahead.d) >= (unsigned)H) ahead.next(g, u1, j0, rstep, k, nr, stride, pad);
-        if (!ahead.more) return;
-        const uint8_t *src = reinterpret_cast<const uint8_t *>(g.src) + ((size_t)(ahead.n * C + c) * H + (ahead.ih0 + ahead.d)) * row_bytes;
+        if (again > 0) {
+            --again;
+            src += (uint32_t)stride * row_bytes;
+        } else {
+            while (ahead.more && (unsigned)(ahead.ih0 + ahead.d) >= (unsigned)H) ahead.next(g, u1, j0, rstep, k, nr, stride, pad);
+            if (!ahead.more) return;
+            const int ih = ahead.ih0 + ahead.d;
+            src = reinterpret_cast<const uint8_t *>(g.src) + ((size_t)(ahead.n * C + c) * H + ih) * row_bytes;
+            if (ahead.d == k - nr + j0 && ahead.d + rstep >= k) {
+                again = min(ahead.p1 - 1 - ahead.p, (H - 1 - ih) >> (F::S == 2 ? 1 : 0));
+                ahead.p += again; ahead.ih0 += again * stride;
+            }
+            ahead.next(g, u1, j0, rstep, k, nr, stride, pad);
+        }
         if (lane == 0) {
             mbar_arrive_expect_tx(b, row_bytes);
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(at), "l"(src), "r"(row_bytes), "r"(b) : "memory");
         }
-        __syncwarp();
-        ahead.next(g, u1, j0, rstep, k, nr, stride, pad);
     };
     for (int i = 0; i < g.raw_slots; ++i) ask(mine + raw_stride * (uint32_t)i, bar0 + 8u * i);
     uint32_t raw[4][F::words];
