@@ -16,10 +16,11 @@
 //                  maximum over columns through a staged row
 //   warps 8..14  : image rows -> operand pieces
 //   warp 15      : issues the products; a convolution row is one accumulator per 128 columns
-// What bounds it: the producers, some 1000 cycles a step and warp for one row (reading and storing its pieces 400, asking for
-// the row four ahead and the walk 600, the ring's barrier 200), then the products' thread, 900 a row of 128 columns and 3 x 3 taps;
-// the products themselves read 6 KB of shared memory each for 64 channels (48 cycles), 11 per 128 columns for a 7 x 7 window of
-// 3 channels.  MobileNet's stem at batch 32: 1500 cycles a row, 1750 with the rows loaded through registers one ahead.
+// What bounds it: the producers (one row a step and warp: 400 cycles for reading and storing its pieces, the rest for the request
+// of the row four ahead and the barriers; 1530 in all while every request walked to its row), then the products' thread, 900 a
+// row of 128 columns and 3 x 3 taps; the products themselves read 6 KB of shared memory each for 64 channels (48 cycles), 11 per
+// 128 columns for a 7 x 7 window of 3 channels.  With rows loaded through registers one ahead a row of MobileNet's stem at batch
+// 32 took 1750 cycles.
 #pragma once
 
 #include "conv_tc.cuh"
