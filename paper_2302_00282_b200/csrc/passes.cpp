@@ -1469,7 +1469,9 @@ struct Lower {
             const int stg = 8 * L.s_slots * 2048;
             const int room = cap - 1024 - mid - stg - bias;
             const int weights = L.kblocks * L.n1pad * 128 + L.kblocks2 * L.n_tiles * 16384;
-            L.b_resident = room - weights >= 3 * 16384;
+            // (the kernel keeps one 128-row weight block per operand block: wider middle tiles take theirs in two halves, which travel
+            // through the ring)
+            L.b_resident = L.n1pad <= 128 && room - weights >= 3 * 16384;
             const int slots = (room - (L.b_resident ? weights : 0)) / 16384;
             L.a_slots = L.b_resident ? std::min(8, slots) : slots * 2 / 5;
             L.b_slots = L.b_resident ? 0 : std::min(8, slots - L.a_slots);
@@ -1871,7 +1873,7 @@ void emit_plan_json(Graph &g) {
             jint(s, "k2", L.k2); jint(s, "cmid", L.Cmid); jint(s, "n1pad", L.n1pad); jint(s, "kblocks", L.kblocks); jint(s, "kblocks2", L.kblocks2);
             jint(s, "tile_n", L.tile_n); jint(s, "n_tiles", L.n_tiles); jint(s, "m_tiles", L.m_tiles); jint(s, "npad", L.npad);
             jint(s, "patch_rh", L.patch_rh); jint(s, "patch_rw", L.patch_rw); jint(s, "rh2", L.rh2); jint(s, "rw2", L.rw2);
-            jint(s, "tiles_y", L.tiles_y); jint(s, "tiles_x", L.tiles_x); jint(s, "stages", L.stages);
+            jint(s, "tiles_y", L.tiles_y); jint(s, "tiles_x", L.tiles_x); jint(s, "stages", L.stages); jint(s, "b_resident", L.b_resident);
         }
         if (L.kind == LK_F32_CONV_CONV_POOL) {
             jint(s, "parts_outc", L.parts_outc); jint(s, "tile_h", L.tile_h); jint(s, "tile_w", L.tile_w);

@@ -72,6 +72,17 @@ def test_two_convolutions_with_a_1x1_consumer(cin, h, w, k, cmid, cout, add, bat
     assert gg.g.launch_count() == 1
 
 
+# middle tiles of more than 128 channels whose weights would fit beside the rings: one tile, several per CTA
+@pytest.mark.parametrize("cmid,cout,add,batch", [(192, 64, True, 2), (192, 128, False, 1), (256, 8, False, 140)])
+def test_two_convolutions_with_a_wide_middle(cmid, cout, add, batch):
+    def build(g):
+        y = g.cbr("c2", g.cbr("c1", "input", cmid, 1), cout, 1, act=None if add else "relu")
+        if add:
+            g.act("relu", g.add("add", y, "input"), "relu")
+    check_bf16(f"pair_wide{(cmid, cout)}", _spec((64, 9, 17), build), batch, in_mode="bf16_nhwc", images=[0, batch - 1],
+               links=[["c1", "c2"] + (["add"] if add else [])])
+
+
 # both strides, maps smaller than a tile and much wider, channel counts that end inside an 8-channel piece's K block, one and
 # many tiles per CTA, the global average of one and of many images per tile
 @pytest.mark.parametrize("c,h,w,cout,st,gap,batch", [(8, 1, 1, 8, 1, False, 1), (24, 3, 5, 40, 2, False, 2), (16, 79, 79, 32, 1, False, 3), (72, 17, 66, 136, 2, False, 2),

@@ -602,3 +602,13 @@ def test_plan_names_the_kernel_of_every_launch():
     assert kernels(graphs.single_chain(), 1) == ["f32_chain_kernel"]
     assert kernels(graphs.single_chain(), 1, linked=False) == ["f32_conv_kernel", "f32_conv_kernel", "f32_pool_kernel"]
     assert set(kernels(graphs.resnet50_stress(), 8)) == {"stem_tc_kernel", "conv_tc_kernel", "pair_tc_kernel"}
+
+
+@pytest.mark.parametrize("cmid,cout", [(64, 64), (128, 64), (192, 64), (192, 128), (256, 64)])
+def test_wide_middle_tiles_stream_their_weights(cmid, cout):
+    """Weights of two linked convolutions stay in shared memory as one block of at most 128 rows per operand block; a middle tile of
+    more columns takes its weights in halves, through the ring."""
+    spec = GraphSpec("unit", (64, 9, 17))
+    spec.cbr("c2", spec.cbr("c1", "input", cmid, 1), cout, 1)
+    L = compiled(spec, 2, links=[["c1", "c2"]], nhwc=True)[0].plan()["launches"]
+    assert len(L) == 1 and L[0]["kernel"] == "pair_tc_kernel" and L[0]["b_resident"] == (L[0]["n1pad"] <= 128)
