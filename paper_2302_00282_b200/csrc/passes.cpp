@@ -718,7 +718,7 @@ struct Lower {
         static const int one[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15}, two[9] = {0, 296, 148, 93, 71, 56, 45, 37, 33};
         return (int)((long)(half ? two[ks] : one[ks]) * g.hw.sm_count / 148);
     }
-    static int conv_smem_cap(bool half) { return half ? kClusterSmem : 227 * 1024; }
+    int conv_smem_cap(bool half) const { return std::min(g.hw.smem_bytes_per_cta, half ? kClusterSmem : 227 * 1024); }
     static constexpr int kClusterSmem = 112 * 1024;      // what two CTAs of an SM can have each
     // Exchange buffer of a cluster's partial sums.
     static int cluster_bytes(int rows, int tile_n, int ks) { return (int)align_up((size_t)ks * ceil_div(rows, ks) * (tile_n + 4) * 4, 1024); }
@@ -889,7 +889,8 @@ struct Lower {
     xenos_status_t layout_conv(Launch &L, const Tensor &ot) {
         const bool vec = L.out_dtype == XENOS_DTYPE_F32 || ot.c % 8;
         // (up to eight chunks are the CTAs of a cluster while the exchange buffer leaves room for the ring; other splits go
-        // through the workspace)
+        // through the workspace).  The exchange parks a tile's partial sums, 128 rows of tile_n + 4 words, in the ring: three stages
+        // hold them at every width, two do so only below 124 columns.
         const int xbytes = cluster_bytes(std::min(128, g.max_batch * L.rows_per_image), L.tile_n, L.ksplit);
         const bool cluster = L.ksplit > 1 && L.ksplit <= 8 && xbytes + 3 * (16384 + L.tile_n * 128) + L.npad * 4 + 2048 <= conv_smem_cap(L.half);
         L.cv_epi = L.epi == EPI_GAP ? 3 : cluster ? 5 : L.ksplit > 1 ? 4 : vec ? 2 : L.skip >= 0 ? 1 : 0;
@@ -915,7 +916,7 @@ struct Lower {
         // (a CTA with one tile takes half an SM when four stages fit there: the next kernel's CTAs can then set up beside it)
         const bool half = (L.cv_epi == 5 && L.half) || (L.ksplit == 1 && (long)L.m_tiles * L.n_tiles <= g.hw.sm_count &&
                                                         kClusterSmem - 1536 - bias - stg >= std::min(4, std::max(2, L.kblocks)) * (16384 + L.tile_n * 128));
-        const int room = std::min(g.hw.smem_bytes_per_cta, half ? kClusterSmem : 227 * 1024) - 1024 - 512 - bias - stg;
+        const int room = conv_smem_cap(half) - 1024 - 512 - bias - stg;
         const int bbytes = L.kblocks * L.tile_n * 128;
         // weights stay in shared memory when a CTA meets more than one tile of its channel tile and four operand stages
         // still fit beside them

@@ -28,7 +28,7 @@ def to_nhwc_bf16(x_nchw: np.ndarray):
 class GpuGraph:
     """Compiled + bound graph with its device buffers (all memory owned by PyTorch)."""
 
-    def __init__(self, spec, params, max_batch, linked=True, in_mode="f32_nchw", splits=(), links=None):
+    def __init__(self, spec, params, max_batch, linked=True, in_mode="f32_nchw", splits=(), links=None, hw=None):
         import torch
         from paper_2302_00282_b200 import binding as xb
         from xenos_workloads.feed import graph_from_spec
@@ -36,7 +36,7 @@ class GpuGraph:
         dt, lay = {"f32_nchw": (xb.DTYPE_F32, xb.LAYOUT_NCHW), "bf16_nchw": (xb.DTYPE_BF16, xb.LAYOUT_NCHW),
                    "bf16_nhwc": (xb.DTYPE_BF16, xb.LAYOUT_NHWC)}[in_mode]
         self.in_mode = in_mode
-        self.g, self.ids = graph_from_spec(spec, params, in_dtype=dt, in_layout=lay)
+        self.g, self.ids = graph_from_spec(spec, params, in_dtype=dt, in_layout=lay, hw=hw)
         if links is not None:
             for chain in links:
                 self.g.link([self.ids[n] for n in chain])

@@ -13,7 +13,7 @@ from oracle import interp
 from xenos_workloads import graphs
 from xenos_workloads.graphs import GraphSpec
 
-from gpu_util import GpuGraph, rel_err_fp32
+from gpu_util import GpuGraph, abs_err_scaled, rel_err_fp32
 from test_gpu_parity import BF16_TOL, FP32_TOL, check_bf16
 
 pytestmark = pytest.mark.gpu
@@ -46,6 +46,16 @@ def test_reduction_split_over_clusters(cin, hw, cout, k, parts_k, batch):
     spec = _spec((cin, hw, hw), lambda g: g.cbr("c", "input", cout, k, 1, k // 2))
     _, _, gg = check_bf16(f"cluster_split{(cin, hw, cout, k, parts_k)}", spec, batch, in_mode="bf16_nhwc", splits=[("c", dict(parts_k=parts_k))])
     assert gg.g.plan()["launches"][0]["ksplit"] == parts_k
+
+
+# a description of units with less shared memory: splits whose exchange or ring no longer fits take another form
+@pytest.mark.parametrize("smem,cout,parts_k", [(132, 128, 8), (160, 128, 2), (164, 128, 4)])
+def test_reduction_split_in_less_shared_memory(smem, cout, parts_k):
+    from paper_2302_00282_b200 import HwInfo
+    spec = _spec((512, 16, 16), lambda g: g.cbr("c", "input", cout, 1))
+    P, x = graphs.make_params(spec), xo.round_bf16(graphs.make_input(spec, 2))
+    gg = GpuGraph(spec, P, 2, in_mode="bf16_nhwc", splits=[("c", dict(parts_outc=1, parts_k=parts_k))], hw=HwInfo(148, smem * 1024, 512, 126 << 20))
+    assert abs_err_scaled(gg.run(x), interp.run_graph(spec, P, x)) <= BF16_TOL
 
 
 # stages of several 16- or 32-channel boxes, filled by two threads in turn: one stage, odd and even numbers of them, a last stage

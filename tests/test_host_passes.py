@@ -612,3 +612,19 @@ def test_wide_middle_tiles_stream_their_weights(cmid, cout):
     spec.cbr("c2", spec.cbr("c1", "input", cmid, 1), cout, 1)
     L = compiled(spec, 2, links=[["c1", "c2"]], nhwc=True)[0].plan()["launches"]
     assert len(L) == 1 and L[0]["kernel"] == "pair_tc_kernel" and L[0]["b_resident"] == (L[0]["n1pad"] <= 128)
+
+
+@pytest.mark.parametrize("smem", [132, 144, 160, 164, 227])
+@pytest.mark.parametrize("cout,parts_outc,parts_k", [(128, 1, 2), (128, 1, 8), (64, 1, 4), (128, 4, 4)])
+def test_cluster_splits_have_room_for_the_rows_they_exchange(smem, cout, parts_outc, parts_k):
+    """A reduction split over a cluster parks its fp32 partial sums, 128 rows of tile_n + 4 words, in the operand ring; a unit with
+    less shared memory than that takes the split through the workspace, which then holds the chunks' sums."""
+    spec = GraphSpec("unit", (512, 16, 16))
+    spec.cbr("c", "input", cout, 1)
+    whole, _ = compiled(spec, 2, hw=xb.HwInfo(148, smem * 1024, 512, 126 << 20), nhwc=True, splits=[("c", dict(parts_outc=parts_outc))])
+    g, _ = compiled(spec, 2, hw=xb.HwInfo(148, smem * 1024, 512, 126 << 20), nhwc=True, splits=[("c", dict(parts_outc=parts_outc, parts_k=parts_k))])
+    L = g.plan()["launches"][0]
+    assert L["ksplit"] == parts_k and L["smem_bytes"] <= smem * 1024
+    ring, parked = L["stages"] * (16384 + L["tile_n"] * 128), 128 * (L["tile_n"] + 4) * 4
+    through_workspace = g.plan()["workspace_bytes"] - whole.plan()["workspace_bytes"] >= parts_k * 512 * L["npad"] * 4
+    assert ring >= parked or through_workspace
