@@ -754,7 +754,9 @@ static xenos_status_t issue_pass(Graph &g, int batch, const void *const *in, voi
                     if (st != XENOS_OK) return st;
                     maps = &now;
                 }
-                const int limit = L.b_resident ? std::max(1, sms / L.n_tiles) * L.n_tiles : sms;
+                // A plan with a tile for every unit of its description lets a tile's results leave through the operand ring: its tiles
+                // are a CTA's only ones, also on a device with fewer units.
+                const int limit = L.off_stg == 0 && L.cv_epi != xk::DE_SPLIT ? p.total : L.b_resident ? std::max(1, sms / L.n_tiles) * L.n_tiles : sms;
                 auto *k = dw_kernel(L.cv_epi, a.stride, L.dw_br, L.halo_cb);
                 le = to.pdl(k, std::min(p.total, limit), L.block, L.smem_bytes, maps->a0, rt->tmaps[li], maps->o, p);
                 break;

@@ -120,6 +120,25 @@ def test_depthwise_tiles_of_few_rows(c, h, w, cout, st, gap, batch):
     assert gg.g.launch_count() == 1 and gg.g.plan()["launches"][0]["tile_rows"] <= 32
 
 
+# plans for more units than the device has: a tile's results may leave through the ring that its operands came by
+@pytest.mark.parametrize("c,h,w,cout,gap,batch,sms", [(64, 56, 56, 64, False, 8, 296), (512, 7, 7, 512, False, 32, 296), (256, 4, 4, 128, True, 600, 1184)])
+def test_depthwise_plans_for_more_units(c, h, w, cout, gap, batch, sms):
+    from paper_2302_00282_b200 import HwInfo
+    def build(g):
+        y = g.cbr("pw", g.cbr("dw", "input", c, 3, 1, 1, groups=c), cout, 1)
+        if gap:
+            g.gap("ap", y)
+    spec = _spec((c, h, w), build)
+    P, x = graphs.make_params(spec), xo.round_bf16(graphs.make_input(spec, batch))
+    gg = GpuGraph(spec, P, batch, in_mode="bf16_nhwc", hw=HwInfo(sms, 227 * 1024, 512, 126 << 20))
+    L = gg.g.plan()["launches"][0]
+    assert L["kernel"] == "dw_tc_kernel" and L["grid"] > 148
+    y = gg.run(x)
+    sel = [0, batch // 2, batch - 1]
+    assert not np.isnan(y).any()
+    assert abs_err_scaled(y[sel], interp.run_graph(spec, P, x[sel])) <= BF16_TOL
+
+
 # 1 to 7 channels, windows of 2 to 8, strides 1, 2 (rows of whole groups of four elements and not) and 3, several column blocks,
 # output channels that end inside a tile and in a second one; pools that overlap by one row, that do not, and over wide images
 @pytest.mark.parametrize("cin,h,w,cout,k,st,pad,pool,batch", [
