@@ -215,6 +215,15 @@ __device__ __forceinline__ void stem_store(const uint32_t (&raw)[kPasses][StemFo
     }
 }
 
+// The slots of another run's first rows lie anywhere in the ring: all earlier steps have been multiplied.  Two threads issue them, and a
+// commit covers the products of its own thread only: the last step is behind the barrier before this one's, and the step before it,
+// the other thread's last, behind the one before that.
+__device__ __forceinline__ bool stem_drained(uint32_t bar, int t, int sl, int D, uint32_t ph) {
+    const int s1 = sl > 0 ? sl - 1 : D - 1, s2 = sl > 1 ? sl - 2 : sl + D - 2;
+    if (!mbar_wait(bar + 8u * (kStMaxSteps + s1), sl > 0 ? ph : ph ^ 1u)) return false;
+    return t < 2 || mbar_wait(bar + 8u * (kStMaxSteps + s2), sl > 1 ? ph : ph ^ 1u);
+}
+
 // A producer warp: one channel, every rstep-th new row of a step (three channels: two rows each of a step of two convolution rows
 // of stride 2).
 template <int kMode, bool kF32, bool kPool>
@@ -246,20 +255,15 @@ __device__ __forceinline__ bool stem_produce(const StemParams &g, uint32_t sbase
         auto load = [&](int ih) {
             stem_load<kMode, kF32>(raw, col + (long long)ih * (long long)pitch, e, (unsigned)ih < (unsigned)H ? W : 0, passes, stride);
         };
-        // (the slots of a step's rows are free when the step D before it has been multiplied; the first rows of another image
-        // wait for all of the last one's)
+        // (the slots of a step's rows are free when the step D before it has been multiplied)
         uint32_t room = bar + 8u * (kStMaxSteps + sl), room_ph = ph ^ 1u;
-        if (t > 0) {
-            room = bar + 8u * (kStMaxSteps + (sl ? sl - 1 : D - 1));
-            room_ph = sl ? ph : ph ^ 1u;
-        }
         int p = r.p0, d = j0, ih0 = p * stride - pad, nb = min(spr, r.p1 - p), kk = k + (nb - 1) * nr;
         bool start = true, fresh = true, have = false;
 #pragma unroll 1
         for (;;) {
             if (!start) {
                 if (fresh) {
-                    if (!mbar_wait(room, room_ph)) return false;
+                    if (!(p == r.p0 && t > 0 ? stem_drained(bar, t, sl, D, ph) : mbar_wait(room, room_ph))) return false;
                     fresh = false;
                 }
                 if (have) {
@@ -446,26 +450,18 @@ __device__ __forceinline__ bool stem_produce_rows(const StemParams &g, uint32_t 
         for (int p = r.p0; p < r.p1; p += nb, ih0 += nb * stride) {
             nb = min(spr, r.p1 - p);
             const int kk = k + (nb - 1) * nr;
-            // (the slots of a step's rows are free when the step D before it has been multiplied; the first rows of another image
-            // wait for all of the last one's)
+            // (the slots of a step's rows are free when the step D before it has been multiplied)
             const bool first = p == r.p0 && t > 0;
-            const uint32_t room = bar + 8u * (kStMaxSteps + (first ? (sl ? sl - 1 : D - 1) : sl)), room_ph = first && sl ? ph : ph ^ 1u;
+            const uint32_t room = bar + 8u * (kStMaxSteps + sl), room_ph = ph ^ 1u;
             const uint32_t known = mbar_test2(room, room_ph, raw_bar, raw_ph);
             bool here = (known & 2u) != 0;
-            if (!(known & 1u) && (first || t >= D) && !mbar_wait(room, room_ph)) return false;
+            if (first ? !stem_drained(bar, t, sl, D, ph) : !(known & 1u) && t >= D && !mbar_wait(room, room_ph)) return false;
 #pragma unroll 1
             while (d < kk) {
                 if (!here && !mbar_wait(raw_bar, raw_ph)) return false;
                 here = false;
                 uint32_t at = raw_at + (uint32_t)e;
                 const int end = min(d + rows * rstep, kk);
-                auto from = [&](int i) { return (unsigned)(ih0 + i) < (unsigned)H ? at : zeros + (uint32_t)e; };
-                auto to = [&](int i, uint32_t &twice) {
-                    int s = slot + i;
-                    if (s >= R) s -= R;
-                    twice = s == 0 ? wrap : 0u;
-                    return ring + (uint32_t)s * slot_bytes;
-                };
 #pragma unroll 1
                 for (; d < end; d += rstep, at += raw_stride) {
                     const uint32_t from = (unsigned)(ih0 + d) < (unsigned)H ? at : zeros + (uint32_t)e;

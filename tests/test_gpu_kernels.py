@@ -191,6 +191,25 @@ def test_image_convolution_two_rows_a_step(cin, h, w, cout, k, st, pad, pool, ba
     assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
 
 
+# Many short images to a CTA: the first rows of an image enter the ring behind all steps of the last one, which two threads multiply.
+# Equal images have equal results, in every pass
+@pytest.mark.parametrize("cin,h,w,cout,k,st,pad,pool", [(3, 8, 64, 64, 7, 2, 3, (3, 2, 1)), (3, 9, 48, 32, 3, 2, 1, None), (3, 7, 50, 64, 3, 1, 1, (2, 2, 0)), (1, 5, 30, 16, 5, 1, 2, None)])
+def test_many_short_images(cin, h, w, cout, k, st, pad, pool):
+    def build(g):
+        y = g.cbr("stem", "input", cout, k, st, pad)
+        if pool:
+            g.pool("mp", y, "maxpool", *pool)
+    spec, batch = _spec((cin, h, w), build), 1500
+    P, few = graphs.make_params(spec), xo.round_bf16(graphs.make_input(spec, 5))
+    gg = GpuGraph(spec, P, batch, in_mode="bf16_nchw", links=[["stem", "mp"]] if pool else None)
+    assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
+    x = np.tile(few, (batch // 5, 1, 1, 1))
+    for _ in range(5):
+        y = gg.run(x)
+        assert np.array_equal(y, np.tile(y[:5], (batch // 5, 1, 1, 1)))
+    assert abs_err_scaled(y[:5], interp.run_graph(spec, P, few)) <= BF16_TOL
+
+
 # Pixels that are infinite or no number reach exactly the outputs whose window holds them, as they are: windows shorter than the
 # eight elements the operand is made of, aligned (lead elements before the window) and not, odd and even window rows and channels
 @pytest.mark.parametrize("cin,h,w,cout,k,st,pad,act,pool,batch", [
