@@ -135,6 +135,13 @@ struct LinkCtx {
     int rows(int n) const { const Tensor &t = g.tensors[g.nodes[n].out]; return t.h * t.w; }
 };
 
+// Max pools that stem_tc_kernel forms row by row, over a map of `rows` rows: windows overlap by one row at most, and no two end with
+// the same row (the padding below the map can hold the ends of the last two where it is a whole stride).
+static bool pool_in_registers(const Node &p, int rows) {
+    const int count = (rows + 2 * p.pad - p.k) / p.stride + 1, below = (count - 1) * p.stride - p.pad + p.k - rows;
+    return p.k - p.stride <= 1 && p.pad < p.k && below < p.stride;
+}
+
 // largest pool-output tile whose conv-output patch fits the 128-row M tile
 static bool pool_patch(int k, int s, int PP, int PQ, int &th, int &tw, int &rh, int &rw) {
     int best = 0;
@@ -369,7 +376,7 @@ static bool try_match(const LinkCtx &cx, int a, Allowed allowed, Chain &out, boo
             // (Convolutions and pools outside stem_tc_kernel's range keep the rule of the kernel that runs them: two kernels at batch 8
             // and above for images up to 256 pixels wide.)
             const Tensor &image = g.tensors[A.in[0]];
-            const bool in_registers = A.k >= 2 && A.k <= 8 && image.c <= 7 && B.k - B.stride <= 1 && B.pad <= B.stride && B.pad < B.k;
+            const bool in_registers = A.k >= 2 && A.k <= 8 && image.c <= 7 && pool_in_registers(B, g.tensors[A.out].h);
             const bool apart = in_registers ? g.max_batch >= 16 && A.k <= 3 && A.stride > 1 && g.tensors[A.out].w <= 64
                                             : g.max_batch >= 8 && image.w <= 256 && image.h <= 256;
             if (by_model && nchw_in && apart) return false;
@@ -770,7 +777,7 @@ struct Lower {
     bool layout_stem(Launch &L, const Node &M, const Tensor &src, const Node *pooln, int N, const SplitRequest &rq) {
         const int C = src.c, k = M.k, S = M.stride;
         if (k < 2 || k > 8 || C > 7 || (rq.user && (rq.h > 1 || rq.w > 1 || rq.k > 1))) return false;
-        if (pooln && (pooln->k - pooln->stride > 1 || pooln->pad > pooln->stride || pooln->pad >= pooln->k)) return false;
+        if (pooln && !pool_in_registers(*pooln, L.P)) return false;
         L.n_tiles = rq.user && rq.outc > 0 ? rq.outc : ceil_div(N, 64);
         L.tile_n = round_up(ceil_div(N, L.n_tiles), 16);
         if (L.tile_n > 64 || (L.n_tiles - 1) * L.tile_n >= N) return false;

@@ -191,6 +191,15 @@ def test_image_convolution_two_rows_a_step(cin, h, w, cout, k, st, pad, pool, ba
     assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
 
 
+# Padding of a whole stride: the last two windows of a pool may end with the same row
+@pytest.mark.parametrize("h,w,cout,k,st,pool,batch", [(20, 24, 16, 5, 1, (2, 1, 1), 2), (21, 21, 24, 7, 2, (3, 2, 2), 3), (20, 33, 64, 3, 1, (2, 1, 1), 9), (22, 21, 64, 3, 1, (3, 2, 2), 16)])
+def test_image_convolution_and_a_pool_with_wide_padding(h, w, cout, k, st, pool, batch):
+    def build(g):
+        g.pool("mp", g.cbr("stem", "input", cout, k, st, k // 2), "maxpool", *pool)
+    check_bf16(f"wide_padding{(h, w, cout, k, st, pool)}", _spec((3, h, w), build), batch, links=[["stem", "mp"]])
+    check_bf16(f"wide_padding{(h, w, cout, k, st, pool)}", _spec((3, h, w), build), batch)
+
+
 # Many short images to a CTA: the first rows of an image enter the ring behind all steps of the last one, which two threads multiply.
 # Equal images have equal results, in every pass
 @pytest.mark.parametrize("cin,h,w,cout,k,st,pad,pool", [(3, 8, 64, 64, 7, 2, 3, (3, 2, 1)), (3, 9, 48, 32, 3, 2, 1, None), (3, 7, 50, 64, 3, 1, 1, (2, 2, 0)), (1, 5, 30, 16, 5, 1, 2, None)])

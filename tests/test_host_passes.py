@@ -628,3 +628,13 @@ def test_cluster_splits_have_room_for_the_rows_they_exchange(smem, cout, parts_o
     ring, parked = L["stages"] * (16384 + L["tile_n"] * 128), 128 * (L["tile_n"] + 4) * 4
     through_workspace = g.plan()["workspace_bytes"] - whole.plan()["workspace_bytes"] >= parts_k * 512 * L["npad"] * 4
     assert ring >= parked or through_workspace
+
+
+@pytest.mark.parametrize("hw,k,stride,pad,rows", [(20, 2, 1, 1, False), (21, 3, 2, 2, False), (20, 3, 2, 2, True), (21, 3, 2, 1, True), (20, 2, 2, 0, True)])
+def test_pool_windows_that_end_with_the_same_row_are_not_formed_row_by_row(hw, k, stride, pad, rows):
+    """The kernel that forms a pool row by row emits one row at each end of a window: padding of a whole stride below the map makes
+    the last two windows end together, which another kernel runs."""
+    spec = GraphSpec("unit", (3, hw, hw))
+    spec.pool("mp", spec.cbr("c", "input", 16, 5, 1, 2), "maxpool", k, stride, pad)
+    L = compiled(spec, 2, links=[["c", "mp"]])[0].plan()["launches"]
+    assert len(L) == 1 and L[0]["stem_tc"] == rows
