@@ -663,7 +663,7 @@ __device__ __forceinline__ bool conv_epilogue_cluster(const ConvParams &g, uint8
                      ::"r"(cluster_addr(buf, (uint32_t)e) + (uint32_t)(t.ks * per) * pitch), "r"(sbase + (uint32_t)(e * per) * pitch), "r"((uint32_t)theirs * pitch),
                      "r"(cluster_addr(arrived, (uint32_t)e)) : "memory");
     __syncwarp();
-    if (!ok) return false;
+    // (behind a wait that gave up, too: the other CTAs' copies are on their way into this CTA's buffer until they have arrived)
     bool seen = false;
 #pragma unroll 1
     for (int i = 0; i < kSpinLimit && !seen; ++i) {
@@ -675,7 +675,7 @@ __device__ __forceinline__ bool conv_epilogue_cluster(const ConvParams &g, uint8
             : "=r"(done) : "r"(arrived), "r"(kSuspendHintNs) : "memory");
         seen = done != 0;
     }
-    if (!seen) return false;
+    if (!ok || !seen) return false;
 #pragma unroll 1
     for (int idx = et; idx < items; idx += 32 * kCvEpiWarps) {
         const int nc = n0 + c4 * 4;
@@ -928,7 +928,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     }
     tc_fence_before();
     __syncthreads();
-    if (kEpi == CE_CLUSTER) cluster_sync();      // (no CTA leaves while another may still write to its shared memory)
+    // (a cluster barrier does not wait for bulk copies: every CTA has seen all that was announced to it arrive, so nothing is on its
+    // way into its buffer, and behind the barrier nothing out of its ring either)
+    if (kEpi == CE_CLUSTER) cluster_sync();
     if (warp == 3) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)g.tmem_cols) : "memory");
