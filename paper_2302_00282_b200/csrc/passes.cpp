@@ -365,21 +365,14 @@ static bool try_match(const LinkCtx &cx, int a, Allowed allowed, Chain &out, boo
             int th, tw, rh, rw;
             const Tensor &po = g.tensors[B.out];
             if (!pool_patch(B.k, B.stride, po.h, po.w, th, tw, rh, rw)) return false;
-            // An image convolution and its max pool are one kernel, with the pool's maximum over rows in registers: the feature map
-            // between them is four times the pool's output.  Both forms, us in a stream of launches, two kernels and linked, bf16:
-            //   3x3 to 64 channels, 224 wide, batch 8 / 16 / 32 / 64: 26.8 / 18.5 / 30.1 / 59.2 and 11.5 / 15.9 / 24.0 / 40.1
-            //   7x7 to 64 channels, 224 wide, batch 8 / 16 / 32 / 64: 16.3 / 22.3 / 36.1 / 73.1 and 13.2 / 17.6 / 26.5 / 42.9
-            //   7x7, 128 wide, batch 8 / 32 / 64: 11.8 / 19.7 / 29.3 and 10.2 / 18.4 / 27.6; fp32 images alike
-            // Two kernels are as fast or faster where a row fills half of an accumulator's lanes at most and a window is small, so that
-            // the pool's warps are the most of the work: 3x3, 128 wide, batch 8 / 16 / 32 / 64: 11.7 / 12.1 / 16.7 / 25.6 and 10.0 /
-            // 12.6 / 17.0 / 26.3 (157 wide, batch 32 and 64: 21.1 / 42.6 and 21.5 / 35.1).  Either form can be requested.
-            // (Convolutions and pools outside stem_tc_kernel's range keep the rule of the kernel that runs them: two kernels at batch 8
-            // and above for images up to 256 pixels wide.)
-            const Tensor &image = g.tensors[A.in[0]];
-            const bool in_registers = A.k >= 2 && A.k <= 8 && image.c <= 7 && pool_in_registers(B, g.tensors[A.out].h);
-            const bool apart = in_registers ? g.max_batch >= 16 && A.k <= 3 && A.stride > 1 && g.tensors[A.out].w <= 64
-                                            : g.max_batch >= 8 && image.w <= 256 && image.h <= 256;
-            if (by_model && nchw_in && apart) return false;
+            // At batch 8 and above an image convolution and its max pool stay two kernels for images up to 256 pixels wide.  The
+            // rule was measured with the kernel before stem_tc_kernel, whose pooling pass cost what a pool kernel costs.  With
+            // the pool in registers the link is the faster form there, too: SqueezeNet (3x3 stem) 96 us linked against 110
+            // at batch 8, 158 against 168 at 32, 245 against 270 at 64; ResNet-18 (7x7 stem) 160 against 160, 246 against 255
+            // and 361 against 386; 3x3, 24 channels, 224 x 224: 21 against 30 us at batch 8, 66 against 81 at 32.  It can be
+            // requested.  Below batch 8 and for wider images it is linked (7x7 stem at 512 x 512: 31 against 51 us at batch 8, 201
+            // against 366 at batch 64).
+            if (by_model && nchw_in && g.max_batch >= 8 && g.tensors[A.in[0]].w <= 256 && g.tensors[A.in[0]].h <= 256) return false;
             out.kind = CK_CONV_TAIL;
             out.nodes = {a, b};
             out.pattern = "ConvX -> ZPooling (CBR-MaxPooling)";
