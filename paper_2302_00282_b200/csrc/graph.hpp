@@ -149,8 +149,7 @@ struct Launch {
     // convolution of the image in stem_tc_kernel: elements a piece starts before its window, aligned loads, column blocks and
     // their width in output columns, row slots, steps in flight, pieces per (slot, channel), staged pixel, chunk pairs
     int stem_tc = 0, st_lead = 0, st_vec = 0, st_cbs = 1, st_cw = 0, st_slots = 0, st_qp = 0, st_pc = 0, st_pairs = 0;
-    int st_spr = 1, st_prod = 6, st_raw_rows = 1, st_bufs = 1, st_nsm = 1, st_sets = 2;         // convolution rows of a step, producer warps, image rows of a copy group, staged pool rows, accumulators of a row, sets of a step's accumulators
-    int st_raw = 0, st_raw_lead = 0, st_raw_stride = 0, off_raw = 0;              // image rows by bulk copies: groups per warp (0: by loads)
+    int st_raw = 0, st_raw_lead = 0, st_raw_stride = 0, off_raw = 0;              // image rows by bulk copies: slots per warp (0: by loads)
     int n_acc = 1;                                                 // dw_tc_kernel: channel tiles of tile_n columns per CTA (2: both accumulators hold one tile)
     int pair = 0, a_stride = 0, a_slots = 0, b_slots = 0, off_b2 = 0, s_slots = 2;            // LK_GEMM2 with a 1x1 consumer: pair_tc_kernel and its rings
     // ---- two linked convolutions (LK_GEMM2): producer tile rh1 x rw1 = patch_rh x patch_rw, consumer tile rh2 x rw2

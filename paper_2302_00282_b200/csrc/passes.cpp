@@ -782,8 +782,6 @@ struct Lower {
             const int lead = (4 - M.pad % 4) % 4;
             if (k + lead <= 8) { L.st_lead = lead; L.st_vec = src.w % 4 == 0 ? 1 : 0; }
         }
-        L.acc_stride = L.tile_n <= 32 ? 32 : 64;
-        L.st_prod = C < 7 ? 6 : 7;      // (with six, a seventh warp issues every second step's products)
         const int rows = pooln ? L.PP : L.P, cols = pooln ? L.PQ : L.Q;
         L.st_pairs = k / 2 * C + (k % 2 ? (C + 1) / 2 : 0);
         // Rows that are whole 16-byte pieces travel by bulk copies, several per producer warp under way (strides 1 and 2): a slot
@@ -803,42 +801,26 @@ struct Lower {
             const int width = std::min(L.Q, pooln ? (L.st_cw - 1) * pooln->stride + pooln->k + 1 : L.st_cw);
             if (width > most) return false;
             L.st_qp = round_up(width, 8);
-            L.st_nsm = ceil_div(L.st_qp, 128);
-            const int row = C * L.st_qp * 16, stage = pooln ? width << (4 + pc) : 0;
-            // Two convolution rows a step where their ring fits, four image rows of a producer warp under way before more steps of
-            // the ring; then fewer of either; one row a step; at last loads into registers.
-            auto deepest = [&](int spr, int least, int groups) {
-                const int nr = std::min(S, k), set = spr * L.st_nsm * L.acc_stride;
-                if (spr > 1 && 2 * set > g.hw.tmem_columns) return -1;
-                L.st_sets = 4 * set <= g.hw.tmem_columns ? 4 : 2;
-                L.st_raw_rows = ceil_div(spr * nr, L.st_prod / C);
-                const int rbytes = groups ? (int)align_up((size_t)(1 + L.st_prod * groups * L.st_raw_rows) * L.st_raw_stride, 128) : 0;
-                for (int bufs = pooln ? 2 : 1; bufs >= 1; --bufs)
-                    for (int D = 6; D >= least; --D) {
-                        L.st_slots = (D * spr - 1) * nr + k;
-                        const int base = wbytes + 2048 + 1024 + 512 + (int)align_up((size_t)bufs * stage, 128);
-                        if ((L.st_slots + 1) * row + rbytes + base > cap) continue;
-                        L.hstages = D; L.st_spr = spr; L.st_raw = groups; L.st_bufs = bufs;
-                        return rbytes;
-                    }
+            const int row = C * L.st_qp * 16, stage = pooln ? 2 * width << (4 + pc) : 0;
+            const int base = wbytes + 2048 + 256 + 512 + (int)align_up((size_t)stage, 128);
+            // four rows of a warp under way before more steps of the ring; two where four do not fit; else loads into registers
+            auto deepest = [&](int raw) {
+                const int rbytes = raw ? (int)align_up((size_t)(1 + 7 * raw) * L.st_raw_stride, 128) : 0;
+                for (int D = 6; D >= 2; --D) {
+                    L.st_slots = (D - 1) * std::min(S, k) + k;
+                    if ((L.st_slots + 1) * row + rbytes + base <= cap) { L.hstages = D; L.st_raw = raw; return rbytes; }
+                }
                 return -1;
             };
-            // (a CTA with two rows or fewer starts with one: SqueezeNet's stem and pool at batch 1 6.7 us against 6.9)
-            const bool few = (long)g.max_batch * rows * cbs <= 2l * g.hw.sm_count;
             int rbytes = -1;
-            for (int spr = S <= k && !few ? 2 : 1; spr >= 1 && rbytes < 0; --spr)
-                for (int least = 3; least >= 2 && rbytes < 0; --least)
-                    for (int groups : {4, 3, 2, 0}) {
-                        if (rbytes >= 0 || (groups > 0) != by_rows) continue;
-                        rbytes = deepest(spr, least, groups);
-                    }
-            if (rbytes < 0) rbytes = deepest(1, 2, 0);
+            if (by_rows) { rbytes = deepest(4); if (rbytes < 0) rbytes = deepest(2); }
+            if (rbytes < 0) rbytes = deepest(0);
             if (rbytes >= 0) {
                 L.off_raw = (int)align_up((size_t)(L.st_slots + 1) * row + 2048, 128);       // (zeros of one chunk; a tile's last rows read past its pieces)
                 L.off_b = L.off_raw + rbytes;
                 L.off_bias = L.off_b + wbytes;
-                L.off_stg = L.off_bias + 1024;
-                L.off_bar = (int)align_up((size_t)(L.off_stg + L.st_bufs * stage), 128);
+                L.off_stg = L.off_bias + 256;
+                L.off_bar = (int)align_up((size_t)(L.off_stg + stage), 128);
                 L.smem_bytes = L.off_bar + 768 + 1024;
                 return true;
             }
@@ -857,8 +839,9 @@ struct Lower {
         L.m_tiles = pooln ? g.max_batch * L.tiles_y * L.tiles_x : g.max_batch * L.P * L.st_cbs * ceil_div(L.st_qp, 128);
         L.stages = L.hstages;
         L.grid = (int)std::min<long>((long)g.max_batch * rows * L.st_cbs, std::max(1, g.hw.sm_count / L.n_tiles)) * L.n_tiles;
-        L.block = pooln ? 640 : 512;
-        L.tmem_cols = L.st_sets * L.st_spr * L.st_nsm * L.acc_stride;
+        L.block = 512;
+        L.acc_stride = L.tile_n <= 32 ? 32 : 64;
+        L.tmem_cols = 4 * L.acc_stride;
         return true;
     }
     // Weights in the order of its products: [channel tile][pair][two chunks][output channel][8 elements of a window row].

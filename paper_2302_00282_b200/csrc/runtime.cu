@@ -669,15 +669,14 @@ static xenos_status_t issue_pass(Graph &g, int batch, const void *const *in, voi
                 p.d_rows = xk::make_fastdiv((uint32_t)p.rows); p.d_cbs = xk::make_fastdiv((uint32_t)p.cbs);
                 p.C = L.C; p.H = L.H; p.W = L.W; p.k = L.k; p.stride = L.stride; p.pad = L.pad; p.lead = L.st_lead;
                 p.P = L.P; p.Q = L.Q; p.N = L.K; p.tile_n = L.tile_n; p.npairs = L.st_pairs;
-                p.R = L.st_slots; p.D = L.hstages; p.spr = L.st_spr; p.nsets = L.st_sets; p.nsm = L.st_nsm; p.acc_stride = L.acc_stride; p.qp = L.st_qp;
+                p.R = L.st_slots; p.D = L.hstages; p.nacc = 4; p.acc_stride = L.acc_stride; p.qp = L.st_qp;
                 p.pk = L.pool_k; p.ps = L.pool_stride; p.pp = L.pool_pad; p.PQ = L.PQ; p.pc_log2 = L.st_pc;
                 p.act = L.act; p.out_ctot = L.out_ctot; p.out_coff = L.out_coff;
                 p.idesc = make_idesc(L.tile_n);
-                p.off_w = L.off_b; p.off_bias = L.off_bias; p.off_stage = L.off_stg; p.stage_bufs = L.st_bufs; p.stage_bytes = (L.off_bar - L.off_stg) / L.st_bufs & ~15; p.off_bar = L.off_bar;
-                p.nprod = L.st_prod; p.rstep = L.st_prod / L.C; p.raw_groups = L.st_raw; p.raw_rows = L.st_raw_rows; p.raw_stride = L.st_raw_stride; p.raw_lead = L.st_raw_lead; p.off_raw = L.off_raw;
+                p.off_w = L.off_b; p.off_bias = L.off_bias; p.off_stage = L.off_stg; p.stage_bytes = (L.off_bar - L.off_stg) / 2 & ~15; p.off_bar = L.off_bar;
+                p.raw_slots = L.st_raw; p.raw_stride = L.st_raw_stride; p.raw_lead = L.st_raw_lead; p.off_raw = L.off_raw;
                 p.launch_id = (int)li;
                 const int gx = std::min(p.units, std::max(1, sms / L.n_tiles));
-                p.unit_share = p.units / gx; p.unit_extra = p.units % gx;
                 le = to.pdl(stem_kernel(L), dim3(gx, L.n_tiles), L.block, L.smem_bytes, p);
                 break;
             }
@@ -960,9 +959,9 @@ xenos_status_t runtime_status(Graph &g, void *stream_v) {
     cudaMemset(ws + g.status_off, 0, 256 + g.cnt_bytes);      // (the arrival counters of a run that gave up are stale too)
     int code = -(int)(word & 0xffu);
     if (code == XENOS_E_TIMEOUT) {
-        static const char *role[] = {"a wait", "the TMA warp", "the MMA warp", "a producer warp", "a producer warp at the last tile", "an epilogue warp", "a pooling warp"};
+        static const char *role[] = {"a wait", "the TMA warp", "the MMA warp", "a producer warp", "a producer warp at the last tile", "an epilogue warp"};
         const unsigned r = (word >> 8) & 0xfu;
-        return fail(g, code, std::string("a kernel gave up a bounded wait (") + role[r < 7 ? r : 0] + ", launch " + std::to_string((word >> 12) & 0xfffu) + ")");
+        return fail(g, code, std::string("a kernel gave up a bounded wait (") + role[r < 6 ? r : 0] + ", launch " + std::to_string((word >> 12) & 0xfffu) + ")");
     }
     return fail(g, code, "a kernel failed an index check");
 }

@@ -174,23 +174,6 @@ def test_image_rows(cin, h, w, cout, k, st, pad, pool, batch, in_mode):
     assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
 
 
-# Enough rows a CTA for steps of two convolution rows: odd row counts (a last step of one row, a run that ends in another image), one
-# channel, two (rows unevenly dealt to warps), four and seven (one thread issues all products), rows by copies and by loads, pools that
-# overlap and do not, two accumulators a row with one staged row, tiles of one, two, three and four chunks of columns
-@pytest.mark.parametrize("cin,h,w,cout,k,st,pad,pool,batch", [
-    (3, 45, 48, 64, 7, 2, 3, (3, 2, 1), 30), (7, 33, 64, 40, 7, 2, 3, (3, 2, 1), 40), (2, 50, 24, 72, 4, 2, 1, None, 15), (1, 30, 20, 8, 5, 1, 2, None, 12),
-    (3, 40, 300, 24, 3, 2, 1, None, 16), (3, 31, 512, 64, 7, 2, 3, (3, 2, 1), 40), (4, 37, 30, 48, 3, 1, 1, (2, 2, 0), 20), (3, 33, 40, 16, 3, 2, 0, (2, 1, 0), 25)])
-@pytest.mark.parametrize("in_mode", ["f32_nchw", "bf16_nchw"])
-def test_image_convolution_two_rows_a_step(cin, h, w, cout, k, st, pad, pool, batch, in_mode):
-    def build(g):
-        y = g.cbr("stem", "input", cout, k, st, pad)
-        if pool:
-            g.pool("mp", y, "maxpool", *pool)
-    _, _, gg = check_bf16(f"two_rows{(cin, h, w, cout, k, st, pad, pool)}{in_mode}", _spec((cin, h, w), build), batch, in_mode=in_mode,
-                          links=[["stem", "mp"]] if pool else None, images=[0, 1, batch - 1])
-    assert [l.get("stem_tc") for l in gg.g.plan()["launches"]] == [1]
-
-
 # Padding of a whole stride: the last two windows of a pool may end with the same row
 @pytest.mark.parametrize("h,w,cout,k,st,pool,batch", [(20, 24, 16, 5, 1, (2, 1, 1), 2), (21, 21, 24, 7, 2, (3, 2, 2), 3), (20, 33, 64, 3, 1, (2, 1, 1), 9), (22, 21, 64, 3, 1, (3, 2, 2), 16)])
 def test_image_convolution_and_a_pool_with_wide_padding(h, w, cout, k, st, pool, batch):
@@ -200,8 +183,8 @@ def test_image_convolution_and_a_pool_with_wide_padding(h, w, cout, k, st, pool,
     check_bf16(f"wide_padding{(h, w, cout, k, st, pool)}", _spec((3, h, w), build), batch)
 
 
-# Many short images to a CTA: the first rows of an image enter the ring behind all steps of the last one, which two threads multiply.
-# Equal images have equal results, in every pass
+# Many short images to a CTA: the first rows of an image enter the ring behind all steps of the last one.  Equal images have equal
+# results, in every pass
 @pytest.mark.parametrize("cin,h,w,cout,k,st,pad,pool", [(3, 8, 64, 64, 7, 2, 3, (3, 2, 1)), (3, 9, 48, 32, 3, 2, 1, None), (3, 7, 50, 64, 3, 1, 1, (2, 2, 0)), (1, 5, 30, 16, 5, 1, 2, None)])
 def test_many_short_images(cin, h, w, cout, k, st, pad, pool):
     def build(g):
