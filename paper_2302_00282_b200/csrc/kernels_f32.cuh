@@ -287,6 +287,7 @@ f32_chain_kernel(const F32ChainParams p) {
     for (int cta = blockIdx.x; cta < total; cta += gridDim.x) {
         const Tile tile = tile_of(cta);
         const int n = tile.n, part = tile.part, py0 = tile.py0, px0 = tile.px0, th = tile.th, tw = tile.tw, rh = tile.rh, rw = tile.rw;
+        // (patches are filled ahead of this: binding refuses a plan whose largest tile does not fit)
         if (rh > p.halo_h || rw > p.halo_w || tile.ih > max_ih) {
             if (threadIdx.x == 0) atomicCAS(p.status, 0u, 0x80000000u | 10u);
             asm volatile("cp.async.wait_all;" ::: "memory");

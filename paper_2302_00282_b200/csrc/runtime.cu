@@ -377,7 +377,12 @@ static xenos_status_t attach(Graph &g, void *ws, void *stream_v) {
     for (const Launch &L : g.launches) {
         if (L.kind == LK_GEMM2) { any_gemm = true; max_gemm_smem = std::max(max_gemm_smem, L.smem_bytes); }
         if (L.kind == LK_GEMM) { any_gemm = true; max_gemm_smem = std::max(max_gemm_smem, L.smem_bytes); }
-        if (L.kind == LK_F32_CONV_CONV_POOL) max_chain_smem = std::max(max_chain_smem, L.smem_bytes);
+        if (L.kind == LK_F32_CONV_CONV_POOL) {
+            max_chain_smem = std::max(max_chain_smem, L.smem_bytes);
+            // (the kernel fills a tile's patch before it looks at the tile's extents)
+            if ((L.tile_h - 1) * L.pool_stride + L.pool_k > L.halo_h || (L.tile_w - 1) * L.pool_stride + L.pool_k > L.halo_w)
+                return fail(g, XENOS_E_BAD_SPLIT, "internal: a tile's patch exceeds its place in shared memory");
+        }
     }
     rt->tmaps.resize(g.launches.size());
     rt->hmaps.resize(g.launches.size());

@@ -635,3 +635,15 @@ def test_pool_windows_that_end_with_the_same_row_are_not_formed_row_by_row(hw, k
     spec.pool("mp", spec.cbr("c", "input", 16, 5, 1, 2), "maxpool", k, stride, pad)
     L = compiled(spec, 2, links=[["c", "mp"]])[0].plan()["launches"]
     assert len(L) == 1 and L[0]["stem_tc"] == rows
+
+
+@pytest.mark.parametrize("hw,cin,cmid,cout,k,pool,batch", [(32, 16, 32, 32, 3, ("maxpool", 2, 2, 0), 1), (75, 32, 64, 64, 3, ("maxpool", 3, 2, 0), 32),
+                                                           (9, 2, 7, 8, 5, ("avgpool", 3, 1, 0), 2), (5, 1, 1, 3, 3, ("maxpool", 5, 5, 0), 40)])
+def test_fp32_chain_tiles_fit_their_patch(hw, cin, cmid, cout, k, pool, batch):
+    """The fp32 chain's kernel fills a tile's patch before it looks at the tile: the plan's place for a patch holds the largest tile's."""
+    spec = GraphSpec("unit", (cin, hw, hw), precision="fp32")
+    spec.pool("mp", spec.cbr("c1", spec.cbr("c0", "input", cmid, k, 1, k // 2), cout, 1), *pool)
+    L = compiled(spec, batch)[0].plan()["launches"]
+    assert len(L) == 1
+    L = L[0]
+    assert (L["tile_h"] - 1) * pool[2] + pool[1] <= L["halo_h"] and (L["tile_w"] - 1) * pool[2] + pool[1] <= L["halo_w"]
