@@ -90,8 +90,8 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// Whether the phase with the given parity is complete.  The answer takes some 190 cycles however long ago that was (a wait that
-// finds its phase complete costs 240, four MMAs of N = 64 with their commit 190; measured): a multiplying thread asks for the
+// Whether the phase with the given parity is complete.  The answer takes some 190 cycles however long ago that was (205 by a
+// poll that may sleep; four MMAs of N = 64 with their commit take 190; measured): a multiplying thread asks for the
 // next block before it issues this one (umma_block), and nobody asks for ring slots that nothing has been put in yet.
 __device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
     uint32_t done;

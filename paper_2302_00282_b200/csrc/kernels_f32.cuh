@@ -237,9 +237,9 @@ f32_chain_kernel(const F32ChainParams p) {
     };
     // A tile's input patch: 8, 16 or 32 lanes along a row, as many rows of a (channel, row) walk at once as that leaves.  (With a
     // warp and two divisions per row the requests of a 32-channel patch of 8 x 40 took 11 thousand cycles, of a 16-channel one of
-    // 4 x 8 4200.)  Small tiles ask for theirs as asynchronous copies, which travel with the weights (one 32 x 32 map 9.1 us, by
-    // way of registers 9.9); a warp's 4-byte copies cost some 20 cycles each, 9200 for the larger patch, which large tiles
-    // therefore load through registers, up to eight loads of a thread under way (75 x 75, batch 32: 232 us, as copies 237).
+    // 4 x 8 4200.)  Small tiles ask for theirs as asynchronous copies, which travel with the weights (one 32 x 32 map 9.1 us when
+    // this was chosen, by way of registers 9.9); a warp's 4-byte copies cost some 20 cycles each, 9200 for the larger patch, which large tiles
+    // therefore load through registers, up to eight loads of a thread under way (75 x 75, batch 32: then 232 us, as copies 237).
     auto load_patch = [&](const Tile &t) {
         const int lr = p.iwp <= 8 ? 3 : p.iwp <= 16 ? 4 : 5, lanes = 1 << lr, rows = T >> lr;
         const int i0 = t.py0 * p.pool_stride * p.stride - p.pad, j0 = t.px0 * p.pool_stride * p.stride - p.pad;      // may be negative

@@ -725,8 +725,9 @@ struct Lower {
     // Modelled cycles of a plan with tile_n columns and ksplit chunks on `units` SMs.  Per 64-wide K block a CTA waits for
     // the slower of the tensor pipe (max(48, tile_n / 2) cycles per K = 16 step) and the operand traffic from L2 (75
     // bytes per cycle and SM); a tile's epilogue overlaps the next tile's product; a split adds the exchange of the partial
-    // sums.  The constants are measurements on B200 (see conv_tc.cuh), but a stage of several copy requests is charged like one:
-    // four im2col boxes of 16 channels are 300 cycles here and some 1000 on the device.
+    // sums.  The constants are measurements on B200 (see conv_tc.cuh), but a stage of several copy requests is charged like one
+    // (four im2col boxes of 16 channels are 300 cycles here and 720 of a filling thread, of which there are two), and the exchange is that
+    // of 16-byte stores through distributed shared memory, before the bulk copies.
     double conv_cycles(const Launch &L, int tile_n, int n_tiles, int ksplit, bool half) const {
         const double units = g.hw.sm_count;
         const double tiles = (double)L.m_tiles * n_tiles;

@@ -573,8 +573,8 @@ def test_graph_image_rejects_what_is_not_an_intact_image():
 
 
 def test_image_convolution_and_max_pool_link_by_measured_cost():
-    """At batch 8 and above an image convolution and its max pool run as two kernels (measured faster), unless the image is
-    wider than 256 pixels or the link is requested; at small batch they are linked.  An unlinked image convolution's tiles
+    """At batch 8 and above an image convolution and its max pool run as two kernels (a rule measured with an earlier kernel), unless
+    the image is wider than 256 pixels or the link is requested; at small batch they are linked.  An unlinked image convolution's tiles
     keep their input patch within the copy engine's 256 x 256 box, also for a 512 x 512 image."""
     spec = graphs.resnet18()
     def first_chain(batch, **kw):
